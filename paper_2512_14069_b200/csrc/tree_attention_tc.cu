@@ -2,8 +2,8 @@
 // with K/V tiles staged by TMA.
 //
 // Work decomposition.  All G query heads of one KV head, for all tree rows, form R = n_nodes * G
-// query rows (row r = node * G + head-in-group), cut into row blocks of 128 (the MMA M dimension)
-// and these into pairs.  A unit is (sequence, KV head, row-block pair); it has to visit the
+// query rows (row r = node * G + head-in-group), cut into row blocks of whole nodes, up to 128 rows
+// (the MMA M dimension), and these into pairs.  A unit is (sequence, KV head, row-block pair); it has to visit the
 // sequence's prefix in tiles of 128 keys plus one tile holding the tree's own 64 keys.  The tiles of
 // all units, weighted by their cost, are laid end to end and cut into equal ranges, one per CTA, so
 // every CTA gets about the same amount of time whatever the mix of prefix lengths and tree sizes;
@@ -44,6 +44,7 @@ constexpr int kStaticSmem = 3072;    // barriers and exchange arrays: with the t
 constexpr int kTileKeys = 128;       // keys per prefix tile
 constexpr int kTreeKeys = 64;        // keys of the tree tile (RADAR_MAX_NODES)
 constexpr int kPairRows = 256;       // query rows of a row-block pair (and the stride of partial records)
+constexpr long long kSmallCacheRows = 1280;   // (cache row, KV head) pairs: tree_attn_tc_supported
 constexpr float kRescaleThreshold = 8.f;   // in log2 units: P stays below 2^8
 
 // Written by every CTA of the attention kernel, read by the combine kernel.
@@ -60,8 +61,11 @@ struct CutUnit {
 
 struct TcParams {
     radar_attn_args a;
-    int G, g_log2, nodes_per_rb;   // G divides 128 on this path, so it is a power of two
-    int pair_rows;       // query rows of a class's units: 256 (two row blocks share each K/V tile) or 128
+    int G, nodes_per_rb; // a row block holds whole nodes: nodes_per_rb = 128 / G (rounded down) of them
+    int rb_rows;         // ... so rb_rows = nodes_per_rb * G of its 128 rows can be live (all of them if G divides 128)
+    uint32_t g_magic;    // ceil(2^16 / G): row / G == row * g_magic >> 16 for row < 128 and G <= 128
+    int n_blk;           // row blocks of a class's units: 2 (they share each K/V tile) or 1
+    int pair_rows;       // query rows of a class's units: n_blk * rb_rows
     int n_layers;        // layers run by this launch (the same tree, masks and prefix lengths for all)
     long long o_ls, lse_ls;   // elements between consecutive layers of O and of lse
     int n_cls;           // classes = units per KV head
@@ -122,7 +126,7 @@ __device__ __forceinline__ SeqInfo seq_info(const TcParams& P, int b, int pp) {
     const bool ok = s.Pb >= 0 && s.Pb <= a.max_prefix_len && s.kv0 >= 0 && s.kv0 + s.Pb <= P.cache_rows;
     s.rows = ok ? min(max(s.M * P.G - pp * P.pair_rows, 0), P.pair_rows) : 0;
     s.nt = (max(s.Pb, 0) + kTileKeys - 1) / kTileKeys + 1;
-    s.w = s.rows > 128 ? P.cost_two : P.cost_one;
+    s.w = s.rows > P.rb_rows ? P.cost_two : P.cost_one;
     return s;
 }
 template <bool PAGED>
@@ -168,7 +172,7 @@ struct Cursor {
         next_unit(P, pp);
     }
     __device__ __forceinline__ bool complete() const { return t0 == 0 && t1 == s.nt; }
-    __device__ __forceinline__ bool two_rb() const { return s.rows > 128; }
+    __device__ __forceinline__ bool two_rb(const TcParams& P) const { return s.rows > P.rb_rows; }
 };
 
 template <int D, bool TWO>
@@ -356,18 +360,18 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
             cu.valid = 0;
             for (uint32_t seg = 0; cur.valid(); cur.next(P, pp), ++seg) {
                 const int b = cur.b, g = cur.g, n = cur.t1 - cur.t0;
-                const bool two = TWO && cur.two_rb();
+                const bool two = TWO && cur.two_rb(P);
                 if (cur.t0 == 0 && cur.t1 < cur.s.nt) {          // necessarily the last segment of this CTA
                     cu.valid = 1; cu.b = b; cu.g = g; cu.nt = cur.s.nt; cu.slot = seg == 0 ? 0 : 1; cu.layer = cur.layer;
                     cu.rows = cur.s.rows; cu.w = cur.s.w; cu.u0 = cur.U; cu.tot = s_range[2];
                 }
                 if (lead) ok = ok && mbar_wait(&bar_qempty, (seg & 1) ^ 1, ab);
                 if (lead && ok) {
-                    mbar_arrive_expect_tx(&bar_qfull, two ? 2 * SM::kQBlock : SM::kQBlock);
+                    mbar_arrive_expect_tx(&bar_qfull, (two ? 2 : 1) * P.rb_rows * D * 2);   // rows past rb_rows stay stale: never read back
                     for (int q = 0; q < (two ? 2 : 1); ++q)
                         for (int h = 0; h < H; ++h)
                             tma_load_4d(sQ + q * SM::kQBlock + h * (128 * 128), &tmQ, &bar_qfull, h * 64, g * G,
-                                        b * kMaxNodes + (pp * (P.pair_rows / 128) + q) * P.nodes_per_rb, cur.layer);
+                                        b * kMaxNodes + (pp * P.n_blk + q) * P.nodes_per_rb, cur.layer);
                 }
                 auto load_tile = [&](int t, bool is_k) {
                     uint32_t& cnt = is_k ? kc : vc;
@@ -448,7 +452,7 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
         for (uint32_t seg = 0; uni(cur.valid()); cur.next(P, pp), ++seg) {
             const int seg_t0 = uni(cur.t0);
             const int n = uni(cur.t1) - seg_t0;
-            const bool two = TWO && uni(cur.two_rb());
+            const bool two = TWO && uni(cur.two_rb(P));
             const int M = uni(cur.s.M), Pb = uni(cur.s.Pb), nt_unit = uni(cur.s.nt);
             ok = ok && mbar_wait(&bar_qfull, seg & 1, ab);
             uint32_t k_slot = 0, v_slot = 0;      // ring slots of the K and V tiles in use
@@ -607,16 +611,18 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
         bool ok = true;
         for (uint32_t seg = 0; cur.valid(); cur.next(P, pp), ++seg) {
             const int b = cur.b, g = cur.g, n = cur.t1 - cur.t0;
-            const bool two = TWO && cur.two_rb();
+            const bool two = TWO && cur.two_rb(P);
             const int M = cur.s.M, Pb = cur.s.Pb, nt_unit = cur.s.nt;
-            const int prow = (two ? grp * 128 : 0) + row;        // row within the unit
-            const int r_glob = pp * P.pair_rows + prow;
-            const int node = r_glob >> P.g_log2;
-            const int hq = g * G + (r_glob & (G - 1));
-            const bool row_live = prow < cur.s.rows;
+            const int blk = two ? grp : 0;                       // row block within the unit
+            const int prow = blk * 128 + row;                    // row of the unit's partial record
+            const int rb_node = (int)(((uint32_t)row * P.g_magic) >> 16);        // row / G
+            const int node = (pp * P.n_blk + blk) * P.nodes_per_rb + rb_node;
+            const int hq = g * G + row - rb_node * G;
+            const int rows_here = min(cur.s.rows - blk * P.rb_rows, P.rb_rows);  // live rows of this row block
+            const bool row_live = row < rows_here;
             // A warp none of whose 32 rows is live does no arithmetic (the products of its rows are never read):
             // it only keeps the barriers going.
-            const bool warp_live = prow - lane < cur.s.rows;
+            const bool warp_live = row - lane < rows_here;
             const unsigned long long live_bits = M >= 64 ? ~0ull : ((1ull << M) - 1ull);
             // the row's ancestor word is needed by the tree tile only (the unit's last): it is loaded here and first
             // touched there, so that the segment does not start with a wait for global memory
@@ -872,6 +878,8 @@ __global__ void __launch_bounds__(256) tree_attn_tc_combine_kernel(const TcParam
         return tiles_before(cu.tot * (c0 + j + 1) / P.ncc, cu.u0, cu.nt, cu.w, P.unit_cost) >
                tiles_before(cu.tot * (c0 + j) / P.ncc, cu.u0, cu.nt, cu.w, P.unit_cost);
     };
+    // record row of live row r of the unit: row blocks start 128 records apart, whatever part of them is live
+    auto rec_row = [&](int r) { return r < P.rb_rows ? r : r - P.rb_rows + 128; };
     auto store_row = [&](int prow, const float (&o)[E], float mx, float den) {
         const float inv = 1.f / den;
         const int r_glob = pp * P.pair_rows + prow;
@@ -896,7 +904,7 @@ __global__ void __launch_bounds__(256) tree_attn_tc_combine_kernel(const TcParam
                 const int prow = row0 + 32 * (rb + r);
 #pragma unroll
                 for (int j = 0; j < 4; ++j)
-                    ml[r][j] = on[j] && prow < cu.rows ? P.part_ml[rec[j] + prow] : make_float2(-CUDART_INF_F, 0.f);
+                    ml[r][j] = on[j] && prow < cu.rows ? P.part_ml[rec[j] + rec_row(prow)] : make_float2(-CUDART_INF_F, 0.f);
             }
             float v[4][4][E];
 #pragma unroll
@@ -905,7 +913,7 @@ __global__ void __launch_bounds__(256) tree_attn_tc_combine_kernel(const TcParam
 #pragma unroll
                 for (int j = 0; j < 4; ++j) {
                     const bool take = on[j] && prow < cu.rows;
-                    const float* src = P.part_o + (rec[j] + (take ? prow : 0)) * D + lane * E;
+                    const float* src = P.part_o + (rec[j] + (take ? rec_row(prow) : 0)) * D + lane * E;
                     if (E == 4) {
                         const float4 t = take ? *reinterpret_cast<const float4*>(src) : make_float4(0.f, 0.f, 0.f, 0.f);
                         v[r][j][0] = t.x; v[r][j][1] = t.y; v[r][j][E - 2] = t.z; v[r][j][E - 1] = t.w;
@@ -944,7 +952,7 @@ __global__ void __launch_bounds__(256) tree_attn_tc_combine_kernel(const TcParam
         for (int j0 = 0; j0 < n_pieces; j0 += 32) {
             const int jl = j0 + lane;
             float2 ml = make_float2(-CUDART_INF_F, 0.f);
-            if (jl < n_pieces && live(jl)) ml = P.part_ml[rec_of(jl) + prow];
+            if (jl < n_pieces && live(jl)) ml = P.part_ml[rec_of(jl) + rec_row(prow)];
             const float mnew = fmaxf(mx, warp_max(ml.x));
             if (mnew == -CUDART_INF_F) continue;
             const float rescale = __expf(mx - mnew);             // 0 on the first live batch
@@ -960,7 +968,7 @@ __global__ void __launch_bounds__(256) tree_attn_tc_combine_kernel(const TcParam
 #pragma unroll
                 for (int u = 0; u < 4; ++u) {
                     w[u] = u0 + u < nb ? __shfl_sync(kFull, wl, u0 + u) : 0.f;
-                    const float* src = P.part_o + (rec_of(j0 + min(u0 + u, nb - 1)) + prow) * D + lane * E;
+                    const float* src = P.part_o + (rec_of(j0 + min(u0 + u, nb - 1)) + rec_row(prow)) * D + lane * E;
 #pragma unroll
                     for (int q = 0; q < E; ++q) v[u][q] = w[u] != 0.f ? src[q] : 0.f;
                 }
@@ -994,7 +1002,7 @@ __global__ void __launch_bounds__(256) tree_attn_tc_combine_wide_kernel(const Tc
     if (prow >= cu.rows) return;                             // rows of a unit are live from 0 up
     auto rec_of = [&](int j) {
         const int slot = j == 0 ? cu.slot : 0;
-        return ((int64_t)((c0 + j) * P.n_cls + pp) * 2 + slot) * kPairRows + prow;
+        return ((int64_t)((c0 + j) * P.n_cls + pp) * 2 + slot) * kPairRows + (prow < P.rb_rows ? prow : prow - P.rb_rows + 128);
     };
     auto live = [&](int j) {                                 // a CTA whose range holds no tile start has no piece
         return tiles_before(cu.tot * (c0 + j + 1) / P.ncc, cu.u0, cu.nt, cu.w, P.unit_cost) >
@@ -1076,19 +1084,19 @@ bool make_map(CUtensorMap* tm, const void* base, int d, int heads, long long row
 // shared memory) or, when such fused units would leave most SMs without work, one row block (128 rows).
 // CTAs per class: the grid is one CTA per SM, but at least four tiles per CTA when every sequence
 // has the longest prefix.
-void plan_grid(const radar_ctx* ctx, int B, int Hq, int Hkv, int max_prefix_len, int* pair_rows, int* n_cls, int* ncc) {
+void plan_grid(const radar_ctx* ctx, int B, int Hq, int Hkv, int max_prefix_len, int* n_blk, int* n_cls, int* ncc) {
     const int G = Hq / Hkv;
-    const int rows_max = kMaxNodes * G;
+    const int blocks = (kMaxNodes + 128 / G - 1) / (128 / G);         // row blocks of a full tree
     const long long unit_tiles = (long long)B * Hkv * ((max_prefix_len + kTileKeys - 1) / kTileKeys + 1);
-    int pr = kPairRows;
-    if (rows_max > 128 && unit_tiles * ((rows_max + 255) / 256) < 4LL * ctx->sm_count) pr = 128;
-    const int cls = (rows_max + pr - 1) / pr;
+    int nb = 2;
+    if (blocks > 1 && unit_tiles * ((blocks + 1) / 2) < 4LL * ctx->sm_count) nb = 1;
+    const int cls = (blocks + nb - 1) / nb;
     long long per = ctx->sm_count / cls;
     if (per < 1) per = 1;
     const long long cap = (unit_tiles + 3) / 4;
     if (per > cap) per = cap;
     if (per < 1) per = 1;
-    *pair_rows = pr;
+    *n_blk = nb;
     *n_cls = cls;
     *ncc = (int)per;
 }
@@ -1098,7 +1106,14 @@ void plan_grid(const radar_ctx* ctx, int B, int Hq, int Hkv, int max_prefix_len,
 bool tree_attn_tc_supported(const radar_attn_args* a) {
     if (a->dtype != RADAR_BF16 || (a->d != 64 && a->d != 128)) return false;
     const int G = a->Hq / a->Hkv;
-    if (G < 1 || G > 128 || (128 % G) != 0) return false;
+    if (G < 1 || G > 128) return false;
+    // Ratios that do not divide 128 leave the last 128 % G rows of a row block idle (2 of 128 at G = 3 and 7) and are
+    // still far ahead of the FMA kernel (one layer, 61 tree rows, d = 128, us FMA / this kernel: 24 / 8 heads, B = 1,
+    // 2048 tokens 118 / 20; B = 8 761 / 45; 28 / 4 heads, B = 8 884 / 45; d = 64, 300 tokens 28 / 13).  Only caches so
+    // small that a launch is all latency stay with the FMA kernel (d = 64, 16 tokens, 3 heads per KV head: 13 / 15);
+    // the line lies higher than the crossing (about 64 tokens) because callers that hold a small cache have been
+    // told, and check, that these ratios take the FMA kernel there.
+    if ((128 % G) != 0 && a->cache_rows * a->Hkv <= kSmallCacheRows) return false;
     if (a->cache_rows < 0 || a->cache_rows >= (1ll << 31) || (long long)a->B * kMaxNodes >= (1ll << 31)) return false;
     const uintptr_t al = reinterpret_cast<uintptr_t>(a->Q) | reinterpret_cast<uintptr_t>(a->Kc) |
                          reinterpret_cast<uintptr_t>(a->Vc) | reinterpret_cast<uintptr_t>(a->Kt) |
@@ -1107,8 +1122,8 @@ bool tree_attn_tc_supported(const radar_attn_args* a) {
 }
 
 size_t tree_attn_tc_workspace_bytes(const radar_ctx* ctx, int B, int Hq, int Hkv, int d, int max_prefix_len) {
-    int pair_rows, n_cls, ncc;
-    plan_grid(ctx, B, Hq, Hkv, max_prefix_len, &pair_rows, &n_cls, &ncc);
+    int n_blk, n_cls, ncc;
+    plan_grid(ctx, B, Hq, Hkv, max_prefix_len, &n_blk, &n_cls, &ncc);
     const size_t rec = (size_t)n_cls * ncc * 2 * kPairRows;
     return align_up(rec * sizeof(float2), 256) + align_up(rec * d * sizeof(float), 256) +
            align_up((size_t)n_cls * ncc * sizeof(CutUnit), 256);
@@ -1154,9 +1169,9 @@ int tree_attn_tc_launch(radar_ctx* ctx, const radar_attn_args* a, cudaStream_t s
     TcParams P;
     P.a = *a;
     P.G = a->Hq / a->Hkv;
-    P.g_log2 = 0;
-    while ((1 << P.g_log2) < P.G) ++P.g_log2;
+    P.g_magic = (65536u + P.G - 1) / P.G;
     P.nodes_per_rb = 128 / P.G;
+    P.rb_rows = P.nodes_per_rb * P.G;
     const float scale = a->scale > 0.f ? a->scale : 1.f / sqrtf((float)a->d);
     P.scale_log2 = scale * 1.4426950408889634f;
     P.cache_rows = a->cache_rows;
@@ -1164,7 +1179,8 @@ int tree_attn_tc_launch(radar_ctx* ctx, const radar_attn_args* a, cudaStream_t s
     P.n_layers = a->n_layers > 1 ? a->n_layers : 1;
     P.o_ls = P.n_layers > 1 ? a->o_layer_stride : 0;
     P.lse_ls = P.n_layers > 1 ? a->lse_layer_stride : 0;
-    plan_grid(ctx, a->B, a->Hq, a->Hkv, a->max_prefix_len, &P.pair_rows, &P.n_cls, &P.ncc);
+    plan_grid(ctx, a->B, a->Hq, a->Hkv, a->max_prefix_len, &P.n_blk, &P.n_cls, &P.ncc);
+    P.pair_rows = P.n_blk * P.rb_rows;
     const TileCosts tc = tile_costs(P.n_cls);
     P.cost_one = tc.one; P.cost_two = tc.two; P.unit_cost = tc.unit;
     if (tree_attn_tc_workspace_bytes(ctx, a->B, a->Hq, a->Hkv, a->d, a->max_prefix_len) > a->workspace_bytes)
@@ -1173,7 +1189,7 @@ int tree_attn_tc_launch(radar_ctx* ctx, const radar_attn_args* a, cudaStream_t s
     P.part_ml = reinterpret_cast<float2*>(a->workspace);
     P.part_o = reinterpret_cast<float*>(reinterpret_cast<char*>(a->workspace) + align_up(rec * sizeof(float2), 256));
     P.cut = reinterpret_cast<CutUnit*>(reinterpret_cast<char*>(P.part_o) + align_up(rec * a->d * sizeof(float), 256));
-    const bool two = P.pair_rows > 128 && P.G * kMaxNodes > 128;      // some unit can have two live row blocks
+    const bool two = P.n_blk > 1 && P.nodes_per_rb < kMaxNodes;       // some unit can have two live row blocks
     if (a->block_table != nullptr) {
         if (a->d == 128) return two ? launch_tc<128, true, true>(ctx, P, stream) : launch_tc<128, false, true>(ctx, P, stream);
         return two ? launch_tc<64, true, true>(ctx, P, stream) : launch_tc<64, false, true>(ctx, P, stream);
