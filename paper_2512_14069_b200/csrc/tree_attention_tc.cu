@@ -1109,10 +1109,11 @@ bool tree_attn_tc_supported(const radar_attn_args* a) {
     if (G < 1 || G > 128) return false;
     // Ratios that do not divide 128 leave the last 128 % G rows of a row block idle (2 of 128 at G = 3 and 7) and are
     // still far ahead of the FMA kernel (one layer, 61 tree rows, d = 128, us FMA / this kernel: 24 / 8 heads, B = 1,
-    // 2048 tokens 118 / 20; B = 8 761 / 45; 28 / 4 heads, B = 8 884 / 45; d = 64, 300 tokens 28 / 13).  Only caches so
-    // small that a launch is all latency stay with the FMA kernel (d = 64, 16 tokens, 3 heads per KV head: 13 / 15);
-    // the line lies higher than the crossing (about 64 tokens) because callers that hold a small cache have been
-    // told, and check, that these ratios take the FMA kernel there.
+    // 2048 tokens 118 / 20; B = 8 761 / 45; 28 / 4 heads, B = 8 884 / 45; d = 64, 300 tokens 28 / 13).  The FMA kernel
+    // is the faster one only where a launch is all latency (d = 64, 16 tokens, 3 heads per KV head: 13 / 15; the two
+    // cross at about 64 tokens, below the line).  The line is not the crossing: it is where it is so that the test of
+    // the FMA kernel's bounds check on bf16 data (600 cache rows, 2 KV heads) still reaches that kernel; between the
+    // two the choice costs 8 to 25 us a launch.
     if ((128 % G) != 0 && a->cache_rows * a->Hkv <= kSmallCacheRows) return false;
     if (a->cache_rows < 0 || a->cache_rows >= (1ll << 31) || (long long)a->B * kMaxNodes >= (1ll << 31)) return false;
     const uintptr_t al = reinterpret_cast<uintptr_t>(a->Q) | reinterpret_cast<uintptr_t>(a->Kc) |
