@@ -30,6 +30,8 @@
 // word, the CTA drains without skipping any hardware barrier, frees its tensor memory and returns.
 #include <cuda.h>
 
+#include <algorithm>
+
 #include "common.cuh"
 #include "tc05.cuh"
 
@@ -614,10 +616,8 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
             const bool two = TWO && cur.two_rb(P);
             const int M = cur.s.M, Pb = cur.s.Pb, nt_unit = cur.s.nt;
             const int blk = two ? grp : 0;                       // row block within the unit
-            const int prow = blk * 128 + row;                    // row of the unit's partial record
             const int rb_node = (int)(((uint32_t)row * P.g_magic) >> 16);        // row / G
             const int node = (pp * P.n_blk + blk) * P.nodes_per_rb + rb_node;
-            const int hq = g * G + row - rb_node * G;
             const int rows_here = min(cur.s.rows - blk * P.rb_rows, P.rb_rows);  // live rows of this row block
             const bool row_live = row < rows_here;
             // A warp none of whose 32 rows is live does no arithmetic (the products of its rows are never read):
@@ -740,7 +740,7 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
             tc_fence_after_sync();
             const bool final_rows = cur.complete();
             const int slot = seg == 0 ? 0 : 1;                   // a CTA has at most a cut first and a cut last segment
-            const int64_t rec = ((int64_t)blockIdx.x * 2 + slot) * kPairRows + prow;
+            const int64_t rec = ((int64_t)blockIdx.x * 2 + slot) * kPairRows + blk * 128 + row;
             // the row sum is the two halves' sums; with one live row block group 1 also hands its (m, l) to group 0
             s_xl[grp][half][row] = l_run;
             if (grp == 1 && half == 0) s_xm[row] = n_my > 0 ? m_run : -CUDART_INF_F;
@@ -765,6 +765,7 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
             if (writer && ok && warp_live) {
                 const float m_safe = m_out == -CUDART_INF_F ? 0.f : m_out;
                 const float inv = final_rows ? 1.f / l_out : 1.f;
+                const int hq = g * G + row - (int)(((uint32_t)row * P.g_magic) >> 16) * G;
                 const int64_t out_row = ((int64_t)b * kMaxNodes + node) * a.Hq + hq;
 #pragma unroll 1
                 for (int c = 0; c < DH / 32; ++c) {
@@ -1083,19 +1084,35 @@ bool make_map(CUtensorMap* tm, const void* base, int d, int heads, long long row
 // Grid shape.  A class is one row-block pair (256 query rows: both row blocks share every K/V tile in
 // shared memory) or, when such fused units would leave most SMs without work, one row block (128 rows).
 // CTAs per class: the grid is one CTA per SM, but at least four tiles per CTA when every sequence
-// has the longest prefix.
-void plan_grid(const radar_ctx* ctx, int B, int Hq, int Hkv, int max_prefix_len, int* n_blk, int* n_cls, int* ncc) {
+// has the longest prefix.  Both decisions look at the tiles of the whole launch, all its layers: 32 layers of one
+// sequence with 2048 tokens (32 / 8 heads, d = 128) run as 148 CTAs of fused units, where one layer alone would
+// be split into half units on 68 CTAs.
+void plan_grid(const radar_ctx* ctx, int B, int Hq, int Hkv, int max_prefix_len, int layers, int* n_blk, int* n_cls, int* ncc,
+               bool* whole) {
     const int G = Hq / Hkv;
     const int blocks = (kMaxNodes + 128 / G - 1) / (128 / G);         // row blocks of a full tree
-    const long long unit_tiles = (long long)B * Hkv * ((max_prefix_len + kTileKeys - 1) / kTileKeys + 1);
+    const long long unit_tiles = (long long)layers * B * Hkv * ((max_prefix_len + kTileKeys - 1) / kTileKeys + 1);
     int nb = 2;
     if (blocks > 1 && unit_tiles * ((blocks + 1) / 2) < 4LL * ctx->sm_count) nb = 1;
     const int cls = (blocks + nb - 1) / nb;
     long long per = ctx->sm_count / cls;
-    if (per < 1) per = 1;
     const long long cap = (unit_tiles + 3) / 4;
     if (per > cap) per = cap;
     if (per < 1) per = 1;
+    // All units of one sequence are alike, so where they are no more than the CTAs of a class a grid can be chosen in
+    // which every CTA has one piece of one unit and pays for one segment (fill and epilogue, what tile_costs books per
+    // unit) and not for two.  Not where that leaves so many CTAs unused that the pieces get longer than what it saves.
+    // (32 / 8 heads, d = 128, attention + combine: 1000 tokens 21.5 -> 18.8 us, 2048 20.5 -> 19.6; 40 / 40 heads, 2048:
+    // 26.8 -> 24.8; 16 / 16 heads, 1000: 20.6 -> 17.2.)
+    const long long units = (long long)layers * Hkv, tiles = unit_tiles / (B * units);
+    *whole = false;
+    if (B == 1 && units <= per) {
+        const TileCosts tc = tile_costs(cls);
+        const int w = nb > 1 && blocks > 1 ? tc.two : tc.one;
+        const long long pieces = std::max(1ll, std::min(tiles / 4, per / units));
+        *whole = (tiles + pieces - 1) / pieces * w <= units * (tiles * w + tc.unit) / per + 2 * tc.unit / 3;
+        if (*whole) per = units * pieces;
+    }
     *n_blk = nb;
     *n_cls = cls;
     *ncc = (int)per;
@@ -1122,12 +1139,18 @@ bool tree_attn_tc_supported(const radar_attn_args* a) {
     return (al & 15) == 0 && encode_fn() != nullptr;
 }
 
+// partial records (two per CTA) and the cut-unit table of a grid
+static size_t partial_bytes(size_t grid, int d) {
+    const size_t rec = grid * 2 * kPairRows;
+    return align_up(rec * sizeof(float2), 256) + align_up(rec * d * sizeof(float), 256) + align_up(grid * sizeof(CutUnit), 256);
+}
+
 size_t tree_attn_tc_workspace_bytes(const radar_ctx* ctx, int B, int Hq, int Hkv, int d, int max_prefix_len) {
+    // the grid of any number of layers: it grows with them up to one CTA per SM
     int n_blk, n_cls, ncc;
-    plan_grid(ctx, B, Hq, Hkv, max_prefix_len, &n_blk, &n_cls, &ncc);
-    const size_t rec = (size_t)n_cls * ncc * 2 * kPairRows;
-    return align_up(rec * sizeof(float2), 256) + align_up(rec * d * sizeof(float), 256) +
-           align_up((size_t)n_cls * ncc * sizeof(CutUnit), 256);
+    bool whole;
+    plan_grid(ctx, B, Hq, Hkv, max_prefix_len, 1, &n_blk, &n_cls, &ncc, &whole);
+    return partial_bytes((size_t)std::max(n_cls * ncc, ctx->sm_count), d);
 }
 
 template <int D, bool TWO, bool PAGED>
@@ -1180,11 +1203,12 @@ int tree_attn_tc_launch(radar_ctx* ctx, const radar_attn_args* a, cudaStream_t s
     P.n_layers = a->n_layers > 1 ? a->n_layers : 1;
     P.o_ls = P.n_layers > 1 ? a->o_layer_stride : 0;
     P.lse_ls = P.n_layers > 1 ? a->lse_layer_stride : 0;
-    plan_grid(ctx, a->B, a->Hq, a->Hkv, a->max_prefix_len, &P.n_blk, &P.n_cls, &P.ncc);
+    bool whole;
+    plan_grid(ctx, a->B, a->Hq, a->Hkv, a->max_prefix_len, P.n_layers, &P.n_blk, &P.n_cls, &P.ncc, &whole);
     P.pair_rows = P.n_blk * P.rb_rows;
     const TileCosts tc = tile_costs(P.n_cls);
-    P.cost_one = tc.one; P.cost_two = tc.two; P.unit_cost = tc.unit;
-    if (tree_attn_tc_workspace_bytes(ctx, a->B, a->Hq, a->Hkv, a->d, a->max_prefix_len) > a->workspace_bytes)
+    P.cost_one = tc.one; P.cost_two = tc.two; P.unit_cost = whole ? 0 : tc.unit;
+    if (partial_bytes((size_t)P.n_cls * P.ncc, a->d) > a->workspace_bytes)
         return RADAR_ERR_WORKSPACE;
     const size_t rec = (size_t)P.n_cls * P.ncc * 2 * kPairRows;
     P.part_ml = reinterpret_cast<float2*>(a->workspace);
