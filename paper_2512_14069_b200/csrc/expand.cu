@@ -3,6 +3,8 @@
 // scores, appends them to the pool, selects the k best over all parents and runs the
 // prediction model (LSTM cell + MLP head) on their confidence scores.  The block is built for
 // latency: everything it reads from global memory is fetched in a few wide, independent batches.
+#include <algorithm>
+
 #include "common.cuh"
 
 namespace radar {
@@ -13,7 +15,7 @@ constexpr int kSelWarps = kSelThreads / 32;
 constexpr int kMergeWarps = 16;                      // warps 0..15 merge chunk records, warps 16..31 prepare the gate
 constexpr int kMaxF = 32;
 constexpr size_t kStageLimit = 96 * 1024;            // chunk records are staged in shared memory up to this size
-constexpr int kSurvCap = 256;                        // per-row survivor list of the parallel merge
+constexpr int kSurvCap = 256;                        // per-row survivor list of the parallel merge (even: read in pairs)
 constexpr int kSelCluster = 4;                       // blocks per sequence when the recurrent product is shared out
 constexpr long long kShortPassLogits = 4 << 20;      // ... which is done while a vocabulary pass reads at most this many logits
 
@@ -91,7 +93,6 @@ __device__ __forceinline__ void cp_async16(void* smem, const void* gmem) {
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(smem)), "l"(gmem) : "memory");
 }
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
-__host__ __device__ inline size_t up16(size_t x) { return (x + 15) & ~(size_t)15; }
 
 // Thread-block cluster pieces of the select + gate block: stores and barrier arrivals into block 0's shared memory.
 __device__ __forceinline__ uint32_t smem_addr(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
@@ -126,6 +127,14 @@ __device__ __forceinline__ float key_value(unsigned long long key) {
     return __uint_as_float((u & 0x80000000u) ? (u ^ 0x80000000u) : ~u);
 }
 __device__ __forceinline__ int key_index(unsigned long long key) { return 0x7fffffff - (int)(uint32_t)key; }
+
+// smallest of the lanes' values (redux on a monotone unsigned image of the floats)
+__device__ __forceinline__ float warp_min_value(float v) {
+    uint32_t u = __float_as_uint(v + 0.f);
+    u = (u & 0x80000000u) ? ~u : (u | 0x80000000u);
+    u = __reduce_min_sync(kFull, u);
+    return __uint_as_float((u & 0x80000000u) ? (u ^ 0x80000000u) : ~u);
+}
 
 // One block per sequence.  Phase 1 runs two things side by side: warps 0-15 merge the vocabulary pass's
 // chunk records into each row's top-k and log-normaliser, warps 16-31 do everything of the prediction
@@ -195,12 +204,11 @@ __global__ void __launch_bounds__(kSelThreads, 1) expand_select_gate_kernel(cons
     const int policy = a.policy;
     const int kx = policy == RADAR_POLICY_LSTM_HIDDEN ? 0 : k;      // input columns the block itself multiplies
 
-    const size_t stage_elems = P.staged ? (size_t)F * per_row : 0;
-    float* st_v = reinterpret_cast<float*>(sel_smem);                              // [F][n_chunks][k] if staged
-    int* st_i = reinterpret_cast<int*>(sel_smem + up16(stage_elems * 4));
-    float* sv_v = reinterpret_cast<float*>(sel_smem + 2 * up16(stage_elems * 4));   // [kMergeWarps][kSurvCap]
-    int* sv_i = reinterpret_cast<int*>(sv_v + kMergeWarps * kSurvCap);
-    float* s_wih = reinterpret_cast<float*>(sv_i + kMergeWarps * kSurvCap);         // [4H][k]
+    const int stage_stride = P.staged ? (per_row + 3) & ~3 : 0;                     // elements of a merge warp's record copy
+    unsigned long long* sv_key = reinterpret_cast<unsigned long long*>(sel_smem);   // [kMergeWarps][kSurvCap] survivors
+    float* st_v = reinterpret_cast<float*>(sv_key + kMergeWarps * kSurvCap);        // [merge warps in use][stage_stride]
+    int* st_i = reinterpret_cast<int*>(st_v + (size_t)min(F, kMergeWarps) * stage_stride);
+    float* s_wih = reinterpret_cast<float*>(st_i + (size_t)min(F, kMergeWarps) * stage_stride);   // [4H][k]
     float* s_w1 = s_wih + 4 * H * k;                                                // [H][H + k]
 
     // The gate's weights are constants: their copies into shared memory are issued before the wait where that is
@@ -245,8 +253,6 @@ __global__ void __launch_bounds__(kSelThreads, 1) expand_select_gate_kernel(cons
     __shared__ float s_b1[kHidden], s_w2[2 * kHidden], s_b2[2];
     __shared__ float s_y[2];
     __shared__ int s_base;
-    __shared__ float s_tv[kMergeWarps], s_rv[kMergeWarps][32];
-    __shared__ int s_ti[kMergeWarps], s_ri[kMergeWarps][32];
 
     if (tid == 0) s_base = a.t > 1 ? a.pool_len[b] : 0;
     // previous call's state, needed late: requested now so that nothing waits for it (F * k <= the block's threads)
@@ -254,100 +260,111 @@ __global__ void __launch_bounds__(kSelThreads, 1) expand_select_gate_kernel(cons
     const int forced = a.force_calls != nullptr ? a.force_calls[b] : -1;     // read now, needed at the very end
 
     if (warp < kMergeWarps) {
-        // ---- 1a. chunk records -> shared memory (coalesced), then per row: top-k, log-normaliser, scores ----
+        // ---- 1a. per row: chunk records -> this warp's shared memory, log-normaliser, top-k, candidate scores ----
+        // A warp works on its row alone (no block barrier), and on its own its time is the number of instructions it
+        // issues one after the other plus what its shuffles wait for the ones of the other rows (an SM passes one
+        // warp's shuffle a clock).  So the chunk heads and the survivors are ranked from shared memory, four and two
+        // to a broadcast load, the records are filtered flat (a lane takes every 32nd entry, whatever its chunk), and
+        // the only shuffles left are those of the log-normaliser.
         const size_t row0 = (size_t)b * F;
-        const float* gv = P.vp.part_v + row0 * per_row;
-        const int* gi = P.vp.part_i + row0 * per_row;
+        float* pv_s = st_v + (size_t)warp * stage_stride;
+        int* pi_s = st_i + (size_t)warp * stage_stride;
+        unsigned long long* lk = sv_key + warp * kSurvCap;
+        float* s_heads = reinterpret_cast<float*>(lk);              // (done with before the first survivor is written)
         chain_sync();
-        if (P.staged) {
-            if ((per_row & 3) == 0) {       // rows of records are 16-byte aligned (the partial arrays are 256-byte aligned)
-                for (int e = tid; e < F * per_row / 4; e += kMergeWarps * 32) { cp_async16(st_v + 4 * e, gv + 4 * e); cp_async16(st_i + 4 * e, gi + 4 * e); }
-            } else {
-                for (int e = tid; e < F * per_row; e += kMergeWarps * 32) { cp_async4(st_v + e, gv + e); cp_async4(st_i + e, gi + e); }
-            }
-            cp_async_wait_all();
-            group_barrier(2);
-        }
         for (int f = warp; f < F; f += kMergeWarps) {
             const size_t row = row0 + f;
-            // log-sum-exp over the chunks in fp64: the first loads are issued here and consumed after the merge
-            // (always from a valid address, and not looked at before the merge is done: nothing below waits for them)
-            const float pm0_raw = P.vp.part_m[row * n_chunks + min(lane, n_chunks - 1)];
-            const float ps0_raw = P.vp.part_s[row * n_chunks + min(lane, n_chunks - 1)];
-            const float parent_sc = a.parent_score[(size_t)b * F + f];
-            WarpTopList<float> top;
-            top.reset();
+            const float* gv = P.vp.part_v + row * per_row;
+            const int* gi = P.vp.part_i + row * per_row;
+            __syncwarp();                                            // the previous row's lists have been read
+            if (P.staged) {
+                if ((per_row & 3) == 0) {                            // rows of records are 16-byte aligned then
+                    for (int e = lane; e < per_row / 4; e += 32) { cp_async16(pv_s + 4 * e, gv + 4 * e); cp_async16(pi_s + 4 * e, gi + 4 * e); }
+                } else {
+                    for (int e = lane; e < per_row; e += 32) { cp_async4(pv_s + e, gv + e); cp_async4(pi_s + e, gi + e); }
+                }
+            }
+            // log-sum-exp over the chunks in fp64
+            const float parent_sc = a.parent_score[row];
+            const float pm0 = lane < n_chunks ? P.vp.part_m[row * n_chunks + lane] : -CUDART_INF_F;
+            const float ps0 = lane < n_chunks ? P.vp.part_s[row * n_chunks + lane] : 0.f;
+            float mloc = pm0;
+            for (int c = lane + 32; c < n_chunks; c += 32) mloc = fmaxf(mloc, P.vp.part_m[row * n_chunks + c]);
+            const float M = warp_max(mloc);
+            double sloc = pm0 > -CUDART_INF_F ? (double)ps0 * exp((double)pm0 - (double)M) : 0.0;
+            for (int c = lane + 32; c < n_chunks; c += 32) {
+                const float mc = P.vp.part_m[row * n_chunks + c];
+                if (mc > -CUDART_INF_F) sloc += (double)P.vp.part_s[row * n_chunks + c] * exp((double)mc - (double)M);
+            }
+            const double S = warp_sum(sloc);
+            const double lse = (double)M + log(S);
+            auto put = [&](int rank, float v, int tok) {             // the row's candidate number `rank`
+                const double logp = (double)v - lse;
+                a.topk_tok[row * k + rank] = tok;
+                a.topk_logp[row * k + rank] = (float)logp;
+                s_cand[f * k + rank] = (double)parent_sc + logp;
+                s_ctok[f * k + rank] = tok;
+            };
             bool merged = false;
             if (P.staged) {
-                // Parallel merge of the sorted chunk lists.  The k-th best chunk head bounds the row's k-th
-                // best from below; what is not after it survives, and survivors are ranked by counting.
-                const float* pv = st_v + (size_t)f * per_row;
-                const int* pi = st_i + (size_t)f * per_row;
-                // survivors as order keys, in the space of this warp's value and index lists
-                unsigned long long* lk = reinterpret_cast<unsigned long long*>(sv_v) + warp * kSurvCap;
-                if (lane == 0) { s_tv[warp] = -CUDART_INF_F; s_ti[warp] = 0x7fffffff; }
-                s_rv[warp][lane] = -CUDART_INF_F;
-                s_ri[warp][lane] = 0x7fffffff;
+                cp_async_wait_all();
                 __syncwarp();
-                if (n_chunks <= 32) {
-                    // lane c holds the head of chunk c; its rank among the heads by shuffling the heads' order keys
-                    // (one 64-bit comparison per pair: the warp's instruction count is what this phase costs)
-                    const float hv = lane < n_chunks ? pv[lane * k] : -CUDART_INF_F;
-                    const int hi = lane < n_chunks ? pi[lane * k] : 0x7fffffff;
-                    const unsigned long long hk = order_key(hv, hi);
-                    int rank = 0;
-#pragma unroll 4
-                    for (int o = 0; o < n_chunks; ++o) rank += __shfl_sync(kFull, hk, o) > hk ? 1 : 0;
-                    if (lane < n_chunks && rank == k - 1) { s_tv[warp] = hv; s_ti[warp] = hi; }
-                } else {
-                    for (int c = lane; c < n_chunks; c += 32) {
-                        const float hv = pv[c * k];
-                        const int hi = pi[c * k];
-                        int rank = 0;
-                        for (int o = 0; o < n_chunks; ++o) rank += precedes(pv[o * k], pi[o * k], hv, hi) ? 1 : 0;
-                        if (rank == k - 1) { s_tv[warp] = hv; s_ti[warp] = hi; }
-                    }
-                }
-                __syncwarp();
-                const float tv = s_tv[warp];
-                const int ti = s_ti[warp];
-                int total = 0;
-                for (int c0 = 0; c0 < n_chunks; c0 += 32) {
-                    const int c = c0 + lane;
-                    int cnt = 0;
-                    if (c < n_chunks)
-                        while (cnt < k && !precedes(tv, ti, pv[c * k + cnt], pi[c * k + cnt])) ++cnt;
-                    int incl = cnt;
+                // The k-th best chunk head (best head of every 32nd chunk, if there are more than 32) bounds the row's
+                // k-th best value from below; without that many chunks, the worst of all lists' j-th entries does,
+                // where the lists' first j entries are at least k.
+                float tv;
+                if (n_chunks >= k) {
+                    float hv = lane < n_chunks ? pv_s[lane * k] : -CUDART_INF_F;
+                    for (int c = lane + 32; c < n_chunks; c += 32) hv = fmaxf(hv, pv_s[c * k]);
+                    s_heads[lane] = hv;
+                    __syncwarp();
+                    int above = 0;
 #pragma unroll
-                    for (int o = 1; o < 32; o <<= 1) {
-                        const int v = __shfl_up_sync(kFull, incl, o);
-                        if (lane >= o) incl += v;
+                    for (int o = 0; o < 32; o += 4) {
+                        const float4 h4 = *reinterpret_cast<const float4*>(s_heads + o);
+                        above += (h4.x > hv ? 1 : 0) + (h4.y > hv ? 1 : 0) + (h4.z > hv ? 1 : 0) + (h4.w > hv ? 1 : 0);
                     }
-                    const int off = total + incl - cnt;
-                    for (int e = 0; e < cnt; ++e)
-                        if (off + e < kSurvCap) lk[off + e] = order_key(pv[c * k + e], pi[c * k + e]);
-                    total += __shfl_sync(kFull, incl, 31);
+                    tv = warp_min_value(lane < n_chunks && above < k ? hv : CUDART_INF_F);
+                    __syncwarp();
+                } else {
+                    const int jth = (k + n_chunks - 1) / n_chunks;
+                    tv = warp_min_value(lane < n_chunks ? pv_s[lane * k + jth - 1] : CUDART_INF_F);
                 }
-                __syncwarp();
+                int total = 0;
+#pragma unroll 4
+                for (int e0 = 0; e0 < per_row; e0 += 32) {
+                    const int e = e0 + lane;
+                    const float v = e < per_row ? pv_s[e] : 0.f;
+                    const bool keep = e < per_row && v >= tv;
+                    const unsigned m = __ballot_sync(kFull, keep);
+                    const int at = total + __popc(m & ((1u << lane) - 1u));
+                    if (keep && at < kSurvCap) lk[at] = order_key(v, pi_s[e]);
+                    total += __popc(m);
+                }
                 if (total <= kSurvCap) {
+                    if (lane == 0 && (total & 1)) lk[total] = 0ull;   // read in pairs: a key that precedes nothing
+                    __syncwarp();
                     for (int e = lane; e < total; e += 32) {
                         const unsigned long long ck = lk[e];
                         int rank = 0;
 #pragma unroll 4
-                        for (int j = 0; j < total; ++j) rank += lk[j] > ck ? 1 : 0;
-                        if (rank < k) { s_rv[warp][rank] = key_value(ck); s_ri[warp][rank] = key_index(ck); }
+                        for (int j = 0; j < total; j += 2) {
+                            const ulonglong2 kk = *reinterpret_cast<const ulonglong2*>(lk + j);
+                            rank += (kk.x > ck ? 1 : 0) + (kk.y > ck ? 1 : 0);
+                        }
+                        if (rank < k) put(rank, key_value(ck), key_index(ck));
                     }
-                    __syncwarp();
-                    top.v = s_rv[warp][lane];
-                    top.i = s_ri[warp][lane];
+                    for (int e = total + lane; e < k; e += 32) put(e, -CUDART_INF_F, 0x7fffffff);   // (only with NaN logits)
                     merged = true;
                 }
                 __syncwarp();
             }
             if (!merged) {
                 // serial merge (records too large to stage, or a survivor list that overflowed)
-                const float* pv = (P.staged ? st_v : gv) + (size_t)f * per_row;
-                const int* pi = (P.staged ? st_i : gi) + (size_t)f * per_row;
+                const float* pv = P.staged ? pv_s : gv;
+                const int* pi = P.staged ? pi_s : gi;
+                WarpTopList<float> top;
+                top.reset();
                 float thr = -CUDART_INF_F;
                 int thr_i = 0x7fffffff;
                 for (int c = 0; c < n_chunks; ++c) {
@@ -360,26 +377,7 @@ __global__ void __launch_bounds__(kSelThreads, 1) expand_select_gate_kernel(cons
                         thr_i = top.index_at(k - 1);
                     }
                 }
-            }
-            const float pm0 = lane < n_chunks ? pm0_raw : -CUDART_INF_F;
-            const float ps0 = lane < n_chunks ? ps0_raw : 0.f;
-            float mloc = pm0;
-            for (int c = lane + 32; c < n_chunks; c += 32) mloc = fmaxf(mloc, P.vp.part_m[row * n_chunks + c]);
-            const float M = warp_max(mloc);
-            double sloc = pm0 > -CUDART_INF_F ? (double)ps0 * exp((double)pm0 - (double)M) : 0.0;
-            for (int c = lane + 32; c < n_chunks; c += 32) {
-                const float mc = P.vp.part_m[row * n_chunks + c];
-                if (mc > -CUDART_INF_F) sloc += (double)P.vp.part_s[row * n_chunks + c] * exp((double)mc - (double)M);
-            }
-            const double S = warp_sum(sloc);
-            const double lse = (double)M + log(S);
-            if (lane < k) {
-                const double logp = (double)top.v - lse;
-                const double sc = (double)parent_sc + logp;
-                a.topk_tok[row * k + lane] = top.i;
-                a.topk_logp[row * k + lane] = (float)logp;
-                s_cand[f * k + lane] = sc;
-                s_ctok[f * k + lane] = top.i;
+                if (lane < k) put(lane, top.v, top.i);
             }
         }
     } else if (run_gate) {
@@ -633,12 +631,12 @@ extern "C" int radar_expand_step(radar_ctx* ctx, const radar_expand_args* a, voi
     if (a->phase == RADAR_EXPAND_VOCAB) return RADAR_OK;
     sp.split = a->phase == RADAR_EXPAND_SELECT ? 1 : 0;
     // The chunk records are staged in shared memory only if they fit next to the survivor lists and the gate
-    // weights inside the 227 KB a block may have; otherwise the merge reads them from global memory.
-    const size_t stage_bytes = (size_t)a->F * vp.n_chunks * a->k * 8;
+    // weights inside the 227 KB a block may have (18 KB of them static); otherwise the merge reads them from global memory.
+    const size_t stage_bytes = (size_t)std::min(a->F, kMergeWarps) * ((vp.n_chunks * a->k + 3) & ~3) * 8;
     const size_t fixed_smem = (size_t)kMergeWarps * kSurvCap * 8 +
                               sizeof(float) * ((size_t)4 * kHidden * a->k + (size_t)kHidden * (kHidden + a->k));
-    sp.staged = stage_bytes <= kStageLimit && 2 * up16(stage_bytes / 2) + fixed_smem <= 227 * 1024 ? 1 : 0;
-    const size_t smem = 2 * up16(sp.staged ? stage_bytes / 2 : 0) + fixed_smem;
+    sp.staged = stage_bytes <= kStageLimit && stage_bytes + fixed_smem <= 208 * 1024 ? 1 : 0;
+    const size_t smem = fixed_smem + (sp.staged ? stage_bytes : 0);
     // Blocks per sequence.  With a recurrent policy, three more blocks per sequence hold W_hh (256 KB, more than
     // one block has room for) in their shared memory, loaded while the predecessor still runs, and deliver
     // W_hh h + biases into block 0: the block then streams none of it after the wait (measured: 1.3 us less per
