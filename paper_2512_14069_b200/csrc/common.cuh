@@ -33,7 +33,9 @@ enum radar_smem_slot {
     RADAR_SMEM_SELECT_GATE = 0,
     RADAR_SMEM_SELECT_GATE_CLUSTER,   // the instantiation with helper blocks
     RADAR_SMEM_TREE_BUILD,
-    RADAR_SMEM_ATTN_FMA,        // + 2 * (bf16) + (d == 128)
+    RADAR_SMEM_WALK,            // + 2 * (bf16) + CTAs per SM - 1
+    RADAR_SMEM_ACCLEN = RADAR_SMEM_WALK + 4,        // the same
+    RADAR_SMEM_ATTN_FMA = RADAR_SMEM_ACCLEN + 4,        // + 2 * (bf16) + (d == 128)
     RADAR_SMEM_ATTN_TC = RADAR_SMEM_ATTN_FMA + 4,   // + 4 * (d == 128) + 2 * two + paged
     RADAR_SMEM_COUNT = RADAR_SMEM_ATTN_TC + 8
 };
@@ -45,6 +47,7 @@ struct radar_ctx {
     // is per device: a second device in the same process needs its own opt-in)
     size_t smem_opt_in[RADAR_SMEM_COUNT];
     int* d_status;          // sticky device status word
+    int acclen_clusters[4][4];   // clusters of 1, 2, 4, 8 of each per-row kernel of Eq. 11-13 that are resident at once (0: not asked yet)
     // launch accounting (host side)
     long long launches[RADAR_K_COUNT];
     // optional per-kernel CUDA-event timing

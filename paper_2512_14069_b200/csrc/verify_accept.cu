@@ -3,14 +3,15 @@
 //                the live tree rows, then one warp per sequence walks the tree with ballots.
 //   stochastic - one thread-block cluster per sequence walks the tree lazily: only rows on the accepted
 //                path are read, and each CTA of the cluster owns a slice of the vocabulary in every pass.
-//                Probabilities are fp64.  exp((z - max) / T) of the current node's target and draft rows
-//                is cached in the workspace (p, q = cached value / row sum); after j rejections the residual pair is, for every token v that has
+//                Probabilities are fp64.  exp((z - reference) / T) of the current node's target and draft rows
+//                is cached on chip and, what has no room there, in the workspace (p, q = cached value / row sum); after j rejections the residual pair is, for every token v that has
 //                not been proposed yet,  p_j(v) = max(0, p(v) - a_j q(v)) / W_j,  q_j(v) = c_j q(v),
 //                and for the token proposed at trial i <= j,  p_j(x_i) = max(0, p(x_i) - a_i q(x_i)) / W_j,
 //                q_j(x_i) = 0, with a_{j+1} = a_j + c_j W_j,  c_{j+1} = c_j / (1 - q_j(x_{j+1})) and
 //                W_{j+1} = sum_v max(0, p(v) - a(v) q(v)).  This is the rectify / remove / renormalise
 //                recursion of Eq. 2 unrolled, so each rejection costs one read-only pass.
 #include <algorithm>
+#include <cmath>
 
 #include "common.cuh"
 
@@ -81,278 +82,600 @@ __global__ void __launch_bounds__(64) greedy_walk_kernel(const GreedyParams P) {
 // ------------------------------------------------------------------------------------------
 // stochastic walk
 // ------------------------------------------------------------------------------------------
-constexpr int kSThreads = 1024;
+// Few warps: all of them carry the walk's scalars, so its steps between two passes wait for what every warp issues, and
+// the exponentials get their overlap from eight chains a thread (512 threads: 40 us for four sequences of 32000
+// tokens, 256: 31).  kernels<1>: one CTA per SM, 255 registers a thread, for launches that leave room; kernels<2>: two, so
+// that one's passes run while the other exchanges.
+constexpr int kSThreads = 256;
+constexpr int kSWarps = kSThreads / 32;
 constexpr int kMaxCluster = 8;           // portable cluster size limit
+constexpr int kMinSlice = 1024;          // tokens of a CTA's slice below which a larger cluster is not worth its exchanges
+constexpr int kAccMinSlice = 4096;       // ... where there are rows enough to fill the device anyway
+
+// A CTA's slice of the vocabulary is worked on in tiles of 128 tokens, a contiguous run of tiles to each warp, a quad of
+// tokens to a lane: a warp's partial sum is the mass of a run of tokens, and the partial sums of the pass that settles the
+// last weights are all that the final draw needs to find the warp that owns the sampled point.
+// The exponentials of both rows are cached tile by tile (128 of the target row, 128 of the draft row): a slice's first tiles
+// in shared memory, what has no room there in the workspace.  Inside a tile come the first pairs of its
+// quads, then their second pairs, so that a warp's two 16-byte accesses each cover 512 bytes without gaps.  A slice's
+// last tile may be only partly real (its padding holds zeros); in the workspace CTA r's tiles start 128 r tokens
+// behind its first one's index, which keeps the slices apart.
+constexpr int kTileTokens = 128;
+constexpr int kTileDoubles = 2 * kTileTokens;
+constexpr size_t kTileBytes = kTileDoubles * sizeof(double);
+// shared memory left for cached tiles when `per_sm` CTAs share an SM's 228 KB (1 KB of each is the system's, 20 KB static)
+constexpr size_t cache_room(int per_sm) { return ((228 * 1024 / per_sm - 1024 - 20 * 1024 - 512) / kTileBytes) * kTileBytes; }
+__host__ __device__ inline size_t cache_stride(int V) { return (((size_t)V + 3) & ~(size_t)3) + kTileTokens * 8; }
+extern __shared__ __align__(16) double s_cache[];
+struct Cache {
+    double* g;                           // this CTA's tiles in the workspace
+    int st;                              // tiles [0, st) are in shared memory
+    __device__ __forceinline__ double* tile(int t) const { return (t < st ? s_cache : g) + (size_t)t * kTileDoubles; }
+    __device__ __forceinline__ double& token(int o, int which) const {       // o: offset in the slice
+        return tile(o / kTileTokens)[which * kTileTokens + 2 * ((o >> 2) & 31) + 32 * (o & 2) + (o & 1)];
+    }
+};
+struct Tiles { int t0, t1; };            // a warp's run
+__device__ __forceinline__ Tiles warp_tiles(int n, int warp) {       // n: tokens of the slice
+    const int T = (n + kTileTokens - 1) / kTileTokens;
+    return {T * warp / kSWarps, T * (warp + 1) / kSWarps};
+}
+
+struct ExpTable { double t[64]; };       // 2^(j/64)
+// 64 / ln 2; ln 2 / 64 and what its rounding left; 1/5!, 1/4!, 1/3!: instructions take them from the constant bank
+__constant__ double c_exp[6] = {92.33248261689366, 0.010830424696249145, 3.623510646634843e-19, 1.0 / 120.0, 1.0 / 24.0, 1.0 / 6.0};
+// The table in shared memory, sixteen copies side by side: lane l reads the one in its own pair of banks, so that a
+// warp's 32 look-ups never conflict (one copy: 3 of 16 lanes on the same banks on average).
+struct ExpShared {
+    double t[64][16];
+    __device__ __forceinline__ void fill(const ExpTable& T) {
+        for (int i = threadIdx.x; i < 64 * 16; i += blockDim.x) t[i >> 4][i & 15] = T.t[i >> 4];
+    }
+    __device__ __forceinline__ const double* mine() const { return &t[0][threadIdx.x & 15]; }
+};
 
 struct StochParams {
     radar_accept_args a;
-    double* p_cache;     // [B][V] unnormalised exp((z_target - max) / T)
-    double* q_cache;     // [B][V] same for the draft row
+    double* cache;       // [B][2 * cache_stride] exponentials of the current node's target and draft rows that have no room on chip
+    int smem_tiles;      // tiles of a slice whose exponentials are kept in shared memory
     int* status;
+    ExpTable tab;
 };
 
-// The walk of one sequence is shared by the CTAs of a thread-block cluster: CTA r owns the vocabulary
-// slice [V r / n, V (r + 1) / n) of every full-vocabulary pass.  Every scalar that steers the walk is
-// reduced over the cluster into every CTA in a fixed order, so all CTAs take identical decisions and
-// meet at the same cluster barriers.
-struct ClusterRed {
-    double* block_scratch;   // [32] shared
-    double* slots;           // [2][kMaxCluster] shared; the same array exists in every CTA of the cluster
-    unsigned rank, n;
-    unsigned phase;
-
-    __device__ double block_sum(double v) {
-        v = warp_sum(v);
-        __syncthreads();
-        if ((threadIdx.x & 31) == 0) block_scratch[threadIdx.x >> 5] = v;
-        __syncthreads();
-        double t = 0.0;
-        for (int w = 0; w < kSThreads / 32; ++w) t += block_scratch[w];     // same order in every thread
-        return t;
-    }
-    __device__ double block_max(double v) {
-        v = warp_max(v);
-        __syncthreads();
-        if ((threadIdx.x & 31) == 0) block_scratch[threadIdx.x >> 5] = v;
-        __syncthreads();
-        double t = block_scratch[0];
-        for (int w = 1; w < kSThreads / 32; ++w) t = fmax(t, block_scratch[w]);
-        return t;
-    }
-    // every CTA's value lands in out[0..n) of every CTA (rank order)
-    __device__ void all_gather(double mine, double* out) {
-        double* my = slots + (phase & 1) * kMaxCluster;
-        if (threadIdx.x < n) {
-            asm volatile(
-                "{\n\t.reg .u32 ra;\n\t"
-                "mapa.shared::cluster.u32 ra, %0, %1;\n\t"
-                "st.shared::cluster.f64 [ra], %2;\n\t}"
-                ::"r"((uint32_t)__cvta_generic_to_shared(my + rank)), "r"(threadIdx.x), "d"(mine)
-                : "memory");
+// exp(x) in fp64 by table look-up (P. T. P. Tang, "Table-driven implementation of the exponential function in IEEE
+// floating-point arithmetic", ACM TOMS 15(2), 1989): x = (64 m + j) ln2/64 + r with |r| <= ln2/128, so
+// exp(x) = 2^m 2^(j/64) exp(r), and the Taylor series of exp(r) is exact to 4e-17 after its r^5 term.  Ten fp64
+// instructions and a shared-memory read; the results are within 1.1 ulp.  tab: ExpShared::mine()
+// exp_split: the factor 2^(j/64) exp(r), and m.
+__device__ __forceinline__ double exp_split(double x, const double* tab, int& m) {
+    constexpr double kShift = 6755399441055744.0;                 // 1.5 * 2^52: the sum's low word is the rounded integer
+    const double t = fma(x, c_exp[0], kShift);
+    const int n = __double2loint(t);
+    const double nd = t - kShift;
+    const double r = fma(-nd, c_exp[2], fma(-nd, c_exp[1], x));
+    double s = fma(r, c_exp[3], c_exp[4]);
+    s = fma(s, r, c_exp[5]);
+    s = fma(s, r, 0.5);
+    s = fma(s * r, r, r);
+    const double tj = tab[(n & 63) * 16];
+    m = n >> 6;
+    return fma(tj, s, tj);
+}
+__device__ __forceinline__ double times_2_to(double y, int m) { return __hiloint2double(__double2hiint(y) + (m << 20), __double2loint(y)); }
+// ... over the whole range: 2 ulp below -700, where 2^m leaves the normal numbers; infinite above 700
+__device__ __forceinline__ double exp64(double x, const double* tab) {
+    int m;
+    const double y = exp_split(x, tab, m);
+    if (fabs(x) > 700.0) return x > 0.0 ? CUDART_INF : x < -760.0 ? 0.0 : times_2_to(y, m + 512) * 7.458340731200207e-155;   // 2^-512
+    return times_2_to(y, m);
+}
+// exp(z[i] / T + shift) for 4 Q logits, with one fp32 test and one branch for the rare ranges (an fp64 comparison behind each
+// exponential costs the pipe that bounds this, and a branch behind each keeps the chains from overlapping)
+struct ExpRange {
+    double invT, shift;
+    float lo, hi;                        // logits between which |z / T + shift| stays below 700
+    __device__ __forceinline__ double arg(float z) const { return fma((double)z, invT, shift); }
+};
+template <int Q>
+__device__ __forceinline__ void exp64_quads(const float (&z)[Q][4], const ExpRange& X, const double* tab, double (&e)[Q][4]) {
+    float lo = z[0][0], hi = z[0][0];
+#pragma unroll
+    for (int q = 0; q < Q; ++q)
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            int m;
+            const double y = exp_split(X.arg(z[q][i]), tab, m);
+            e[q][i] = times_2_to(y, m);
+            lo = fminf(lo, z[q][i]);
+            hi = fmaxf(hi, z[q][i]);
         }
-        cluster_sync();
-        for (unsigned r = 0; r < n; ++r) out[r] = my[r];
-        ++phase;                         // the other half is written next: no second barrier is needed
+    if (!(lo >= X.lo && hi <= X.hi)) {
+#pragma unroll
+        for (int q = 0; q < Q; ++q)
+#pragma unroll
+            for (int i = 0; i < 4; ++i) e[q][i] = exp64(X.arg(z[q][i]), tab);
     }
+}
+
+__device__ __forceinline__ float max_nan(float a, float b) {
+    float y;
+    asm("max.NaN.f32 %0, %1, %2;" : "=f"(y) : "f"(a), "f"(b));
+    return y;
+}
+// logits v .. v + 3 of a row; -inf from v1 on.  `wide`: the row starts on a boundary of four
+__device__ __forceinline__ void load_quad(const float* row, int v, int v1, bool wide, float (&o)[4]) {
+    if (wide && v + 4 <= v1) {
+        const float4 x = *reinterpret_cast<const float4*>(row + v);
+        o[0] = x.x; o[1] = x.y; o[2] = x.z; o[3] = x.w;
+    } else {
+#pragma unroll
+        for (int e = 0; e < 4; ++e) o[e] = v + e < v1 ? row[v + e] : -CUDART_INF_F;
+    }
+}
+__device__ __forceinline__ void load_quad(const __nv_bfloat16* row, int v, int v1, bool wide, float (&o)[4]) {
+    if (wide && v + 4 <= v1) {
+        const uint2 x = *reinterpret_cast<const uint2*>(row + v);
+        o[0] = __uint_as_float(x.x << 16); o[1] = __uint_as_float(x.x & 0xffff0000u);
+        o[2] = __uint_as_float(x.y << 16); o[3] = __uint_as_float(x.y & 0xffff0000u);
+    } else {
+#pragma unroll
+        for (int e = 0; e < 4; ++e) o[e] = v + e < v1 ? to_float(row[v + e]) : -CUDART_INF_F;
+    }
+}
+template <typename T>
+__device__ __forceinline__ bool row_is_wide(const T* row) { return (reinterpret_cast<uintptr_t>(row) & (4 * sizeof(T) - 1)) == 0; }
+// this lane's quad of a cached tile
+__device__ __forceinline__ void store_quad(double* tile, const double (&e)[4]) {
+    const int lane = threadIdx.x & 31;
+    reinterpret_cast<double2*>(tile)[lane] = make_double2(e[0], e[1]);
+    reinterpret_cast<double2*>(tile)[lane + 32] = make_double2(e[2], e[3]);
+}
+__device__ __forceinline__ void load_quad(const double* tile, double (&e)[4]) {
+    const int lane = threadIdx.x & 31;
+    const double2 x = reinterpret_cast<const double2*>(tile)[lane], y = reinterpret_cast<const double2*>(tile)[lane + 32];
+    e[0] = x.x; e[1] = x.y; e[2] = y.x; e[3] = y.y;
+}
+
+// Asks for this CTA's slice of a row to be brought into L2 (one instruction of one thread; the 16-byte granules that lie
+// wholly inside the slice).
+template <typename T>
+__device__ __forceinline__ void prefetch_slice(const T* row, int v0, int v1) {
+    const uintptr_t lo = (reinterpret_cast<uintptr_t>(row + v0) + 15) & ~(uintptr_t)15, hi = reinterpret_cast<uintptr_t>(row + v1) & ~(uintptr_t)15;
+    if (hi > lo) asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(lo), "r"((uint32_t)(hi - lo)) : "memory");
+}
+
+// The walk of one sequence (and the evaluation of one tree row) is shared by the CTAs of a thread-block cluster: CTA r
+// owns a slice of whole quads of tokens in every full-vocabulary pass.  Every scalar that steers the walk is reduced
+// over the cluster into every CTA in a fixed order, so all CTAs take identical decisions and make the same exchanges.
+// What a pass over a small slice costs is its exchange.  Every warp sends its partial pair into every CTA's slots with
+// asynchronous stores that complete on the receiver's mbarrier, and every warp adds all of them up by itself: one way
+// across the cluster, and no barrier whose release would first wait for the pass's stores to global memory (a cluster
+// barrier in its place: 2000 cycles an exchange, at one CTA as at eight).
+// Use k of a half of the slots follows use k - 2 safely: whoever sends in use k has waited for everyone's use k - 1,
+// and a warp sends there only after it has read its use k - 2.
+struct RedShared {
+    double2 slots[2][kMaxCluster * kSWarps];
+    uint64_t bar[2];                         // kSWarps local arrivals and the bytes of all warps of the cluster
+};
+struct ClusterRed {
+    RedShared& R;
+    int* status;
+    unsigned rank, n, phase;
+
     __device__ static void cluster_sync() {
         asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
     }
-    __device__ double sum(double local) {
-        double all[kMaxCluster];
-        all_gather(block_sum(local), all);
-        double t = 0.0;
-        for (unsigned r = 0; r < n; ++r) t += all[r];
-        return t;
+    // by all threads, before the first exchange
+    __device__ void start() {
+        if (threadIdx.x == 0) {
+            for (int h = 0; h < 2; ++h)
+                asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"((uint32_t)__cvta_generic_to_shared(&R.bar[h])), "r"(kSWarps) : "memory");
+            asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        }
+        __syncthreads();
+        cluster_sync();
     }
-    __device__ double max(double local) {
-        double all[kMaxCluster];
-        all_gather(block_max(local), all);
-        double t = all[0];
-        for (unsigned r = 1; r < n; ++r) t = fmax(t, all[r]);
-        return t;
+    // this warp's pair (the same in every lane) to slot (rank, warp) of every CTA.  What the warp has written to shared or
+    // global memory before is visible to this CTA's other warps once they have received.
+    __device__ __forceinline__ void send(double a, double b) {
+        const unsigned lane = threadIdx.x & 31, warp = threadIdx.x >> 5, h = phase & 1;
+        const uint32_t bar = (uint32_t)__cvta_generic_to_shared(&R.bar[h]);
+        if (n == 1) {
+            if (lane == 0) R.slots[h][warp] = make_double2(a, b);
+        } else if (lane < n) {
+            asm volatile(
+                "{\n\t.reg .u32 ra, rb;\n\t"
+                "mapa.shared::cluster.u32 ra, %0, %2;\n\t"
+                "mapa.shared::cluster.u32 rb, %1, %2;\n\t"
+                "st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v2.f64 [ra], {%3, %4}, [rb];\n\t}"
+                ::"r"((uint32_t)__cvta_generic_to_shared(&R.slots[h][rank * kSWarps + warp])), "r"(bar), "r"(lane), "d"(a), "d"(b)
+                : "memory");
+        }
+        __syncwarp();
+        if (lane == 0) {
+            if (warp == 0 && n > 1) asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(n * kSWarps * 16) : "memory");
+            else asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
+        }
+    }
+    // the slots, filled (rank-major: token order of the slices)
+    __device__ __forceinline__ const double2* receive() {
+        const unsigned h = phase & 1, parity = (phase >> 1) & 1;
+        const uint32_t bar = (uint32_t)__cvta_generic_to_shared(&R.bar[h]);
+        uint32_t ok = 0;
+        // (test_wait: a thread that try_wait has put to sleep takes longer to come back than the partials take to arrive)
+        for (uint32_t it = 0; it < (1u << 24) && !ok; ++it)
+            asm volatile("{\n\t.reg .pred p;\n\tmbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
+                         : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
+        if (!ok) set_status(status, RADAR_ERR_TIMEOUT);
+        __syncwarp();
+        ++phase;
+        return R.slots[h];
+    }
+    // the slots of the last exchange received (until the next but one is sent)
+    __device__ __forceinline__ const double2* last() const { return R.slots[(phase - 1) & 1]; }
+    __device__ double2 receive_sum2() {
+        const double2* all = receive();
+        double2 t = make_double2(0.0, 0.0);
+        for (unsigned i = threadIdx.x & 31; i < n * kSWarps; i += 32) { t.x += all[i].x; t.y += all[i].y; }
+        return make_double2(warp_sum(t.x), warp_sum(t.y));
+    }
+    __device__ double receive_sum() {
+        const double2* all = receive();
+        double t = 0.0;
+        for (unsigned i = threadIdx.x & 31; i < n * kSWarps; i += 32) t += all[i].x;
+        return warp_sum(t);
+    }
+    __device__ float2 max(float a, float b) {
+        send((double)warp_max(a), (double)warp_max(b));
+        const double2* all = receive();
+        float2 t = make_float2(-CUDART_INF_F, -CUDART_INF_F);
+        for (unsigned i = threadIdx.x & 31; i < n * kSWarps; i += 32) { t.x = fmaxf(t.x, (float)all[i].x); t.y = fmaxf(t.y, (float)all[i].y); }
+        return make_float2(warp_max(t.x), warp_max(t.y));
     }
 };
 
-// cache[v] = exp(z[v] / T - max) over this CTA's slice; returns 1 / sum over the whole row
-template <typename T>
-__device__ double softmax_to_cache(const T* z, int v0, int v1, double invT, double* cache, ClusterRed& red, bool* nan_seen) {
-    double m = -CUDART_INF;
-    for (int v = v0 + threadIdx.x; v < v1; v += kSThreads) {
-        const float zf = to_float(z[v]);
-        if (zf != zf) *nan_seen = true;
-        m = fmax(m, (double)zf * invT);
-    }
-    m = red.max(m);
-    double s = 0.0;
-    for (int v = v0 + threadIdx.x; v < v1; v += kSThreads) {
-        const double e = exp((double)to_float(z[v]) * invT - m);
-        cache[v] = e;
-        s += e;
-    }
-    s = red.sum(s);                      // its cluster barrier also publishes every slice of the cache
-    return 1.0 / s;
+struct NodeShared {
+    ExpShared exps;
+    RedShared red;
+    int tok[kMaxNodes], par[kMaxNodes], drow[kMaxNodes];
+    double pe[kMaxNodes], qe[kMaxNodes];     // exponentials of the node's children, by tree row
+};
+
+// children of row c as a 64-bit set, in every thread
+__device__ __forceinline__ unsigned long long children_of(const NodeShared& S, int c) {
+    const int lane = threadIdx.x & 31;
+    const unsigned lo = __ballot_sync(kFull, S.par[lane] == c && lane > c), hi = __ballot_sync(kFull, S.par[lane + 32] == c && lane + 32 > c);
+    return (unsigned long long)hi << 32 | lo;
 }
 
+// this CTA's slice of one row: this thread's maximum (NaN if it has seen one)
 template <typename T>
-__global__ void __launch_bounds__(kSThreads) stochastic_walk_kernel(const StochParams P) {
-    chain_wait();
+__device__ __forceinline__ float slice_max(const T* row, int v0, int v1) {
+    const bool wide = row_is_wide(row);
+    const Tiles w = warp_tiles(v1 - v0, threadIdx.x >> 5);
+    float m = -CUDART_INF_F;
+#pragma unroll 1
+    for (int t = w.t0; t < w.t1; ++t) {
+        float z[4];
+        load_quad(row, v0 + t * kTileTokens + 4 * (threadIdx.x & 31), v1, wide, z);
+        m = max_nan(max_nan(m, max_nan(z[0], z[1])), max_nan(z[2], z[3]));
+    }
+    return m;
+}
+
+// This CTA's slice of one row into the cache (which: 0 target, 1 draft): exp(z / T + shift); returns this thread's sum.
+// Two tiles at a time, eight chains of exponentials side by side, the next two tiles' quads on their way meanwhile.
+// z: the thread's first quad.  Not inlined: with the caller's state in the same registers the loop would spill.
+template <typename T>
+__device__ __forceinline__ double slice_exp(const T* row, int v0, int v1, const ExpRange X, const double* tab, const Cache C, int which, float4 first) {
+    const bool wide = row_is_wide(row);
+    const Tiles w = warp_tiles(v1 - v0, threadIdx.x >> 5);
+    const int mine = v0 + 4 * (threadIdx.x & 31);
+    double s0 = 0.0, s1 = 0.0;
+    float z[2][4] = {{first.x, first.y, first.z, first.w}, {-CUDART_INF_F, -CUDART_INF_F, -CUDART_INF_F, -CUDART_INF_F}};
+    if (w.t0 + 1 < w.t1) load_quad(row, mine + (w.t0 + 1) * kTileTokens, v1, wide, z[1]);
+    int t = w.t0;
+    for (; t + 1 < w.t1; t += 2) {
+        float zn[2][4];
+        load_quad(row, t + 2 < w.t1 ? mine + (t + 2) * kTileTokens : v1, v1, wide, zn[0]);
+        load_quad(row, t + 3 < w.t1 ? mine + (t + 3) * kTileTokens : v1, v1, wide, zn[1]);
+        double e[2][4];
+        exp64_quads<2>(z, X, tab, e);
+        store_quad(C.tile(t) + which * kTileTokens, e[0]);
+        store_quad(C.tile(t + 1) + which * kTileTokens, e[1]);
+        s0 += (e[0][0] + e[0][1]) + (e[0][2] + e[0][3]);
+        s1 += (e[1][0] + e[1][1]) + (e[1][2] + e[1][3]);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) { z[0][i] = zn[0][i]; z[1][i] = zn[1][i]; }
+    }
+    if (t < w.t1) {
+        const float zl[1][4] = {{z[0][0], z[0][1], z[0][2], z[0][3]}};
+        double e[1][4];
+        exp64_quads<1>(zl, X, tab, e);
+        store_quad(C.tile(t) + which * kTileTokens, e[0]);
+        s0 += (e[0][0] + e[0][1]) + (e[0][2] + e[0][3]);
+    }
+    return s0 + s1;
+}
+template <typename T>
+__device__ __forceinline__ float4 first_quad(const T* row, int v0, int v1) {
+    const Tiles w = warp_tiles(v1 - v0, threadIdx.x >> 5);
+    float z[4] = {0.f, 0.f, 0.f, 0.f};
+    if (w.t0 < w.t1) load_quad(row, v0 + w.t0 * kTileTokens + 4 * (threadIdx.x & 31), v1, row_is_wide(row), z);
+    return make_float4(z[0], z[1], z[2], z[3]);
+}
+
+// this CTA's slice of the two rows (draft may be NULL): this thread's maxima, NaN if it has seen one
+template <typename T>
+__device__ __forceinline__ float2 slice_maxima(const T* target, const T* draft, int v0, int v1) {
+    return make_float2(slice_max(target, v0, v1), draft != nullptr ? slice_max(draft, v0, v1) : 0.f);
+}
+
+// One tree node's rows: cache[v] = exp((z[v] - ref) / T) of the target row and, unless `draft` is NULL, of the draft
+// row, over this CTA's slice [v0, v1); the exponentials at the node's children into S.pe / S.qe.  Returns the
+// two row sums (1 for a missing draft row).  `meanwhile` runs while the sums are on their way.
+// The reference of a row need not be its maximum: fp64 has room for exp(700), and relative precision does not depend on
+// the scale.  It is the largest of 32 of the row's logits, the same ones in every warp, so a row is read once
+// and its two rows take one exchange.  Only if a sum shows that some logit lies so far above (or that the sample held
+// nothing finite) the pass is repeated from the exact maxima.
+template <typename T, typename F>
+__device__ double2 softmax_rows(NodeShared& S, ClusterRed& red, const T* target, const T* draft, int V, int v0, int v1,
+                                double invT, const Cache C, unsigned long long children, bool* nan_seen,
+                                F&& meanwhile) {
+    const int tid = threadIdx.x;
+    const bool two = draft != nullptr;
+    const int x = tid < kMaxNodes && ((children >> tid) & 1) ? S.tok[tid] : -1;
+    const bool child = x >= 0 && x < V;
+    const float xt = child ? to_float(target[x]) : 0.f, xd = child && two ? to_float(draft[x]) : 0.f;
+    const int at = (int)((long long)(V - 1) * (tid & 31) / 31);
+    float rt = to_float(target[at]), rd = two ? to_float(draft[at]) : 0.f;
+    const float4 ft = first_quad(target, v0, v1), fd = two ? first_quad(draft, v0, v1) : make_float4(0.f, 0.f, 0.f, 0.f);
+    rt = warp_max(rt);
+    rd = warp_max(rd);
+    const double* tab = S.exps.mine();
+    // logits within 690 T of the reference are in range
+    const float reach = (float)(690.0 / invT);
+    for (int pass = 0;; ++pass) {
+        const double nt = -((double)rt * invT), nd = -((double)rd * invT);
+        const double st = slice_exp(target, v0, v1, ExpRange{invT, nt, rt - reach, rt + reach}, tab, C, 0, ft);
+        const double sd = two ? slice_exp(draft, v0, v1, ExpRange{invT, nd, rd - reach, rd + reach}, tab, C, 1, fd) : 1.0 / (kMaxCluster * kSThreads);
+        if (child) {
+            S.pe[tid] = exp64(fma((double)xt, invT, nt), tab);
+            S.qe[tid] = two ? exp64(fma((double)xd, invT, nd), tab) : 0.0;
+        }
+        red.send(warp_sum(st), warp_sum(sd));
+        if (pass == 0) meanwhile();
+        const double2 s = red.receive_sum2();                      // ... and S.pe and S.qe
+        if ((s.x > 0.0 && s.x < 1e250 && s.y > 0.0 && s.y < 1e250) || pass == 1) return make_double2(s.x, two ? s.y : 1.0);
+        const float2 mine = slice_maxima(target, draft, v0, v1);
+        if (mine.x != mine.x || mine.y != mine.y) *nan_seen = true;
+        const float2 m = red.max(mine.x, mine.y);
+        rt = m.x;
+        rd = m.y;
+    }
+}
+
+// this thread's share of the sum over the slice (n tokens) of max(0, e_p - rho e_q), the exponentials from the caches
+__device__ __forceinline__ double residual_of_tiles(const double* base, int t0, int t1, double rho) {
+    double g0 = 0.0, g1 = 0.0;
+#pragma unroll 2
+    for (int t = t0; t < t1; ++t) {
+        double p[4], q[4];
+        load_quad(base + (size_t)t * kTileDoubles, p);
+        load_quad(base + (size_t)t * kTileDoubles + kTileTokens, q);
+        const double d0 = fma(-rho, q[0], p[0]), d1 = fma(-rho, q[1], p[1]), d2 = fma(-rho, q[2], p[2]), d3 = fma(-rho, q[3], p[3]);
+        if (d0 > 0.0) g0 += d0;                              // (a compare and a predicated add: fewer instructions than fmax)
+        if (d1 > 0.0) g1 += d1;
+        if (d2 > 0.0) g0 += d2;
+        if (d3 > 0.0) g1 += d3;
+    }
+    return g0 + g1;
+}
+__device__ __forceinline__ double slice_residual(const Cache C, int n, double rho) {
+    const Tiles w = warp_tiles(n, threadIdx.x >> 5);
+    const int mid = min(max(C.st, w.t0), w.t1);
+    return residual_of_tiles(s_cache, w.t0, mid, rho) + residual_of_tiles(C.g, mid, w.t1, rho);
+}
+
+// The residual pair of a node while its children are tried in order (file header), in units of the target row's sum:
+// with the row sums s_p and s_q, rho = a s_p / s_q and G = W s_p, the residual of a token is max(0, e_p - rho e_q) / G
+// and rho grows by c G / s_q.  Every thread carries it.
+struct Residual {
+    double rho = 0.0, G, c = 1.0, inv_sq;
+    bool any = false;                    // some child has been rejected
+    bool settled = true;                 // the last exchange carried the masses of the present weights
+    __device__ Residual(double sp, double sq) : G(sp), inv_sq(1.0 / sq) {}
+    __device__ double left(double ep, double eq) const { return fmax(0.0, fma(-rho, eq, ep)); }    // a token's residual (over G: its probability)
+    __device__ double draft(double eq) const { return c * (eq * inv_sq); }                         // its probability under the draft left
+    // reject the child with token x, of probability qj under the draft left; false once the draft's mass is used up.
+    // `meanwhile` runs while the partial sums are on their way.
+    template <typename F>
+    __device__ bool reject(ClusterRed& red, const Cache C, int v0, int v1, int x, double ep, double eq, double qj, F&& meanwhile) {
+        const double rho_new = fma(c * inv_sq, G, rho);
+        red.send(warp_sum(slice_residual(C, v1 - v0, rho_new)), 0.0);
+        meanwhile();
+        const double rest = 1.0 - qj;                        // draft mass left after removing x
+        c = c / rest;
+        const double g = red.receive_sum();
+        settled = g > 0.0;
+        if (settled) { rho = rho_new; G = g; }               // else: residual empty, p stays as it is
+        any = true;
+        // From here on x keeps its own coefficient: its cached pair becomes (residual, 0), which every later pass takes as
+        // it is.  The thread that writes it is the one that reads it in them.
+        const int o = x - v0, t = o / kTileTokens;
+        const Tiles w = warp_tiles(v1 - v0, threadIdx.x >> 5);
+        if (o >= 0 && x < v1 && t >= w.t0 && t < w.t1 && ((o >> 2) & 31) == (int)(threadIdx.x & 31)) {
+            C.token(o, 0) = left(ep, eq);
+            C.token(o, 1) = 0.0;
+        }
+        return rest > 0.0;
+    }
+};
+
+template <typename T, int kPerSm>
+__global__ void __launch_bounds__(kSThreads, kPerSm) stochastic_walk_kernel(const __grid_constant__ StochParams P) {
     const radar_accept_args& a = P.a;
     unsigned crank, csize;
     asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(crank));
     asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(csize));
-    const int b = blockIdx.x / csize, tid = threadIdx.x;
+    const int b = blockIdx.x / csize, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int V = a.V, W = a.t_max + 1;
-    __shared__ double s_red[32];
-    __shared__ double s_slots[2 * kMaxCluster];
-    __shared__ int s_tok[kMaxNodes], s_par[kMaxNodes], s_drow[kMaxNodes], s_child[kMaxNodes];
-    __shared__ int s_nchild;
-    __shared__ int s_rx[RADAR_MAX_NODES];        // tokens proposed and rejected at the current node
-    __shared__ double s_ra[RADAR_MAX_NODES];     // their frozen coefficients a_i
-    __shared__ int s_pick, s_last_pos;
-    ClusterRed red{s_red, s_slots, crank, csize, 0};
-    const int v0 = (int)((long long)V * crank / csize), v1 = (int)((long long)V * (crank + 1) / csize);
+    __shared__ NodeShared S;
+    __shared__ float s_ua[kMaxNodes];
+    S.exps.fill(P.tab);
+    ClusterRed red{S.red, P.status, crank, csize, 0};
+    red.start();
+    chain_wait();
+    const int nq = (V + 3) / 4;
+    const int v0 = 4 * (int)((long long)nq * crank / csize), v1 = min(V, 4 * (int)((long long)nq * (crank + 1) / csize));
     const bool lead = crank == 0;                 // writes the per-sequence outputs
 
-    const int M = min(max(a.n_nodes[b], 1), kMaxNodes);
+    const int nl = a.n_leaves[b];
+    const int retr = a.N * W;                     // the retrieve rows, needed at the very end: into L1 by then
+    if (lead && tid >= 64 && (tid - 64) * 32 < retr) asm volatile("prefetch.global.L1 [%0];" ::"l"(a.retrieve + (size_t)b * retr + (tid - 64) * 32));
     if (tid < kMaxNodes) {
-        s_tok[tid] = tid < M ? a.tree_tok[(size_t)b * kMaxNodes + tid] : -1;
-        s_par[tid] = tid < M ? a.tree_parent[(size_t)b * kMaxNodes + tid] : -2;
-        s_drow[tid] = tid < M ? a.tree_draft_row[(size_t)b * kMaxNodes + tid] : -1;
+        const size_t o = (size_t)b * kMaxNodes + tid;
+        const int M = min(max(a.n_nodes[b], 1), kMaxNodes);
+        const int tok = a.tree_tok[o], par = a.tree_parent[o], dr = a.tree_draft_row[o];
+        s_ua[tid] = a.u_accept[o];
+        S.tok[tid] = tid < M ? tok : -1;
+        S.par[tid] = tid < M ? par : -2;
+        S.drow[tid] = tid < M ? dr : -1;
     }
-    __syncthreads();
-    ClusterRed::cluster_sync();                   // every CTA's shared memory is live before the first remote store
-
     const T* target = reinterpret_cast<const T*>(a.target_logits) + (size_t)b * kMaxNodes * V;
     const T* draft = reinterpret_cast<const T*>(a.draft_logits) + (size_t)b * a.R * V;
-    double* pc = P.p_cache + (size_t)b * V;
-    double* qc = P.q_cache + (size_t)b * V;
+    const Cache C{P.cache + 2 * ((size_t)b * cache_stride(V) + v0 + kTileTokens * crank), P.smem_tiles};
+    if (tid == 0) prefetch_slice(target, v0, v1);                 // the root's rows
+    if (tid == 0) prefetch_slice(draft, v0, v1);
+    __syncthreads();
     const double invT = 1.0 / (double)a.temperature;
-    const float* ua = a.u_accept + (size_t)b * kMaxNodes;
-    bool nan_seen = false;
+    bool nan_seen = false, bad_tree = false;
 
     int32_t* pn = a.path_nodes + (size_t)b * W;
     int32_t* pt = a.path_tokens + (size_t)b * W;
     int cur = 0, len = 0;
-    if (lead && tid == 0) { pn[0] = 0; pt[0] = s_tok[0]; }
+    if (lead && tid == 0) { pn[0] = 0; pt[0] = S.tok[0]; }
 
-    int n_rej = 0;           // rejections at the final node (0 => weights are p itself)
-    double a_coef = 0.0;     // p_j(v) = max(0, p(v) - a q(v)) / W_j for tokens not yet proposed
-    double ip = 1.0, iq = 1.0;   // 1 / sum of the cached exponentials: p(v) = pc[v] * ip, q(v) = qc[v] * iq
-    bool bad_tree = false;
+    Residual res(1.0, 1.0);
     for (;;) {
-        ip = softmax_to_cache<T>(target + (size_t)cur * V, v0, v1, invT, pc, red, &nan_seen);
-        if (tid == 0) {
-            int n = 0;
-            for (int j = cur + 1; j < M; ++j)
-                if (s_par[j] == cur) s_child[n++] = j;
-            s_nchild = n;
-        }
-        __syncthreads();
-        const int nchild = s_nchild;
-        n_rej = 0;
-        a_coef = 0.0;
-        if (nchild == 0 || len >= a.t_max) break;
-        const int drow = s_drow[cur];
-        if (drow < 0 || drow >= a.R) { bad_tree = true; break; }
-        iq = softmax_to_cache<T>(draft + (size_t)drow * V, v0, v1, invT, qc, red, &nan_seen);
-
-        double Wn = 1.0, cq = 1.0;
+        unsigned long long kids = len >= a.t_max ? 0ull : children_of(S, cur);
+        const int drow = S.drow[cur];
+        if (kids != 0 && (drow < 0 || drow >= a.R)) { bad_tree = true; kids = 0; }
+        // The rows of the child that is tried next are asked for ahead: if it is accepted they are the next node's, and a
+        // row's first access otherwise waits for memory and address translation (2500 cycles).
+        auto fetch_ahead = [&](unsigned long long next) {
+            if (tid == 0 && next != 0) {
+                const int j = __ffsll(next) - 1, dr = S.drow[j];
+                prefetch_slice(target + (size_t)j * V, v0, v1);
+                if (dr >= 0 && dr < a.R) prefetch_slice(draft + (size_t)dr * V, v0, v1);
+            }
+        };
+        const double2 sums = softmax_rows<T>(S, red, target + (size_t)cur * V, kids != 0 ? draft + (size_t)drow * V : nullptr, V, v0, v1, invT,
+                                             C, kids, &nan_seen, [&] { fetch_ahead(kids); });
+        res = Residual(sums.x, sums.y);
         int accepted = -1;
-        for (int ci = 0; ci < nchild; ++ci) {
-            const int j = s_child[ci];
-            const int x = s_tok[j];
+        for (; kids != 0; kids &= kids - 1) {
+            const int j = __ffsll(kids) - 1;
+            const int x = S.tok[j];
             if (x < 0 || x >= V) { bad_tree = true; break; }
-            const double px = pc[x] * ip, qx = qc[x] * iq;
-            const double pj = fmax(0.0, px - a_coef * qx) / Wn;      // x has not been proposed before
-            const double qj = cq * qx;
-            bool acc;
-            if (qj <= 0.0) acc = pj > 0.0;
-            else {
-                const double ratio = pj / qj;
-                acc = (double)ua[j] < (ratio < 1.0 ? ratio : 1.0);
-            }
-            if (acc) { accepted = j; break; }
-            // reject: one pass for the new residual mass
-            const double a_new = a_coef + cq * Wn;
-            double g = 0.0;
-            for (int v = v0 + tid; v < v1; v += kSThreads) g += fmax(0.0, pc[v] * ip - a_new * (qc[v] * iq));
-            g = red.sum(g);
-            // tokens rejected earlier keep their own coefficient: swap their terms
-            for (int r = 0; r < n_rej; ++r) {
-                const int xr = s_rx[r];
-                const double pr = pc[xr] * ip, qr = qc[xr] * iq;
-                g += fmax(0.0, pr - s_ra[r] * qr) - fmax(0.0, pr - a_new * qr);
-            }
-            double frozen = a_coef;
-            if (g > 0.0) { a_coef = a_new; Wn = g; frozen = a_new; }   // else: residual empty, p stays as it is
-            __syncthreads();
-            if (tid == 0) { s_rx[n_rej] = x; s_ra[n_rej] = frozen; }
-            __syncthreads();
-            ++n_rej;
-            const double rest = 1.0 - qj;                               // draft mass left after removing x
-            if (rest <= 0.0) break;
-            cq = cq / rest;
+            const double ep = S.pe[j], eq = S.qe[j];
+            const double pj = res.left(ep, eq);                      // x has not been proposed before
+            const double qj = res.draft(eq);
+            // u < min(1, (pj / G) / qj) without the divisions; u is below 1
+            if (qj <= 0.0 ? pj > 0.0 : (double)s_ua[j] * (qj * res.G) < pj) { accepted = j; break; }
+            if (!res.reject(red, C, v0, v1, x, ep, eq, qj, [&] { fetch_ahead(kids & (kids - 1)); })) break;
         }
         if (bad_tree || accepted < 0) break;
         cur = accepted;
         ++len;
-        if (lead && tid == 0) { pn[len] = cur; pt[len] = s_tok[cur]; }
+        if (lead && tid == 0) { pn[len] = cur; pt[len] = S.tok[cur]; }
     }
 
     // ---- final draw: inverse CDF over w(v) = max(0, p(v) - a(v) q(v)) (or p(v) when nothing was rejected) ----
-    const int nv = v1 - v0;
-    const int per = (nv + kSThreads - 1) / kSThreads;
-    const int t0 = v0 + min(tid * per, nv), t1 = v0 + min(tid * per + per, nv);
-    auto weight = [&](int v) -> double {
-        if (n_rej == 0) return pc[v] * ip;
-        double av = a_coef;
-        for (int r = 0; r < n_rej; ++r)
-            if (s_rx[r] == v) av = s_ra[r];
-        return fmax(0.0, pc[v] * ip - av * (qc[v] * iq));
+    // The warps' masses, in token order, tell every warp which one holds the point; that warp then goes through its tiles.
+    // The last exchange has carried them: the sums of the exponentials if nothing was rejected, else those of the last
+    // residual (unless that was empty, and the weights are still the ones before it).
+    auto weights = [&](int t, double (&w)[4]) {   // (of a tile's quad, in units of G)
+        load_quad(C.tile(t), w);
+        if (res.any) {
+            double q[4];
+            load_quad(C.tile(t) + kTileTokens, q);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) w[i] = res.left(w[i], q[i]);
+        }
     };
-    if (tid == 0) { s_pick = 0x7fffffff; s_last_pos = -1; }
-    double seg = 0.0;
-    int last_pos = -1;
-    for (int v = t0; v < t1; ++v) {
-        const double w = weight(v);
-        seg += w;
-        if (w > 0.0) last_pos = v;
+    const Tiles mine_t = warp_tiles(v1 - v0, warp);
+    if (!res.settled) {
+        double mass = 0.0;
+        for (int t = mine_t.t0; t < mine_t.t1; ++t) {
+            double w[4];
+            weights(t, w);
+            mass += (w[0] + w[1]) + (w[2] + w[3]);
+        }
+        red.send(warp_sum(mass), 0.0);
+        red.receive();
     }
-    // scan of seg over the threads of this CTA (fp64).  A thread's end and its successor's start are the
-    // same expression, so at most one thread owns a point.
-    double incl = seg;
-    const int lane = tid & 31, warp = tid >> 5;
+    const double2* all = red.last();
+    // running sums over all warps of the cluster, four consecutive ones to a lane
+    const int nw = (int)csize * kSWarps;
+    double m4[4], own = 0.0;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        m4[i] = 4 * lane + i < nw ? all[4 * lane + i].x : 0.0;
+        own += m4[i];
+    }
+    double incl = own;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
         const double t = __shfl_up_sync(kFull, incl, o);
         if (lane >= o) incl += t;
     }
-    double excl = __shfl_up_sync(kFull, incl, 1);
-    if (lane == 0) excl = 0.0;
-    __syncthreads();
-    if (lane == 31) s_red[warp] = incl;
-    __syncthreads();
-    double woff = 0.0, slice_total = 0.0;
-    for (int w = 0; w < kSThreads / 32; ++w) {
-        if (w == warp) woff = slice_total;
-        slice_total += s_red[w];
-    }
-    __syncthreads();
-    // slice totals of every CTA, in rank order: the running sum gives each slice's start, and the same
-    // expression is the previous slice's end
-    double tots[kMaxCluster];
-    red.all_gather(slice_total, tots);
-    double total = 0.0, my_start = 0.0;
-    for (unsigned r = 0; r < csize; ++r) {
-        if (r == crank) my_start = total;
-        total += tots[r];
-    }
+    const double total = __shfl_sync(kFull, incl, 31);
     const double tgt = (double)a.u_sample[b] * total;
-    // owner: the first slice whose end exceeds the point; if rounding leaves none, the last slice with mass
-    int owner = -1, last_live = 0;
-    {
-        double run = 0.0;
-        for (unsigned r = 0; r < csize; ++r) {
-            run += tots[r];
-            if (tots[r] > 0.0) last_live = (int)r;
-            if (owner < 0 && tgt < run) owner = (int)r;
-        }
-        if (owner < 0) owner = last_live;
+    // owner: the first warp whose end exceeds the point; if rounding leaves none, the last one with mass
+    int first = 0x7fffffff, last_live = -1;
+    double start = 0.0, run = incl - own;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const double before = run;
+        run += m4[i];
+        if (m4[i] > 0.0) last_live = 4 * lane + i;
+        if (first == 0x7fffffff && tgt < run && m4[i] > 0.0) { first = 4 * lane + i; start = before; }
     }
-    if ((int)crank == owner) {
-        const double start = my_start + (woff + excl), end = my_start + (woff + incl);
-        if (last_pos >= 0) atomicMax(&s_last_pos, last_pos);
-        if (start <= tgt && tgt < end) {
-            double run = start;
-            int pick = last_pos;                                            // rounding guard: the crossing is in here
-            for (int v = t0; v < t1; ++v) {
-                run += weight(v);
-                if (run > tgt) { pick = v; break; }
+    const int who = __reduce_min_sync(kFull, first);
+    const int live = __reduce_max_sync(kFull, last_live);
+    start = __shfl_sync(kFull, start, who != 0x7fffffff ? who >> 2 : 0);
+    const int owner = who != 0x7fffffff ? who : max(live, 0);
+    if (owner == (int)crank * kSWarps + warp) {
+        double at = start;
+        int pick = -1, last_pos = -1;
+        for (int t = mine_t.t0; t < mine_t.t1; ++t) {
+            const int v = v0 + t * kTileTokens + 4 * lane;
+            double w[4];
+            weights(t, w);
+            const double mine = (w[0] + w[1]) + (w[2] + w[3]);
+            double in = mine;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const double u = __shfl_up_sync(kFull, in, o);
+                if (lane >= o) in += u;
             }
-            if (pick >= 0) atomicMin(&s_pick, pick);
+            double c = at + (in - mine);
+            int hit = 0x7fffffff, pos = -1;
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                c += w[i];
+                if (w[i] > 0.0) {
+                    pos = v + i;
+                    if (hit == 0x7fffffff && c > tgt) hit = v + i;
+                }
+            }
+            hit = __reduce_min_sync(kFull, hit);
+            last_pos = max(last_pos, __reduce_max_sync(kFull, pos));
+            if (who != 0x7fffffff && hit != 0x7fffffff) { pick = hit; break; }
+            at += __shfl_sync(kFull, in, 31);
         }
-        __syncthreads();
-        if (tid == 0) a.next_token[b] = s_pick != 0x7fffffff ? s_pick : s_last_pos;
+        if (lane == 0) a.next_token[b] = pick >= 0 ? pick : last_pos;     // (rounding guard: the crossing is in this run)
     }
     if (lead && tid == 0) {
         a.accept_len[b] = len;
@@ -363,15 +686,13 @@ __global__ void __launch_bounds__(kSThreads) stochastic_walk_kernel(const StochP
         for (int dd = len + 1 + tid; dd < W; dd += kSThreads) { pn[dd] = -1; pt[dd] = -1; }
         if (tid < 32) {
             int best = 0x7fffffff;
-            const int nl = a.n_leaves[b];
             for (int r = tid; r < nl; r += 32)
                 if (a.retrieve[((size_t)b * a.N + r) * W + len] == cur) best = min(best, r);
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) best = min(best, __shfl_xor_sync(kFull, best, o));
+            best = __reduce_min_sync(kFull, best);
             if (tid == 0) a.best_retrieve_row[b] = best == 0x7fffffff ? -1 : best;
         }
     }
-    ClusterRed::cluster_sync();                   // no CTA leaves while another may still store into its shared memory
+    // (every CTA has received all that was sent to it: none leaves before a store into its shared memory has landed)
 }
 
 // ------------------------------------------------------------------------------------------
@@ -379,132 +700,250 @@ __global__ void __launch_bounds__(kSThreads) stochastic_walk_kernel(const StochP
 // ------------------------------------------------------------------------------------------
 struct AccLenParams {
     radar_acclen_args a;
-    double* p_cache;     // [grid][V]
-    double* q_cache;     // [grid][V]
+    double* cache;       // [clusters][2 * cache_stride]
+    int smem_tiles;
     double* cond;        // [B][64]: P_acc(row | its parent), in the workspace
     int* status;
+    ExpTable tab;
 };
 
-// One item = one tree row of one sequence; rows without children have nothing to do.  A persistent
-// grid walks the items; each block evaluates its row's children in order with the same closed-form
-// residual recursion as the stochastic walk, but follows every rejection branch: child j gets
-// reach_j a_j with reach_j = prod_{i<j} (1 - a_i).
-template <typename T>
-__global__ void __launch_bounds__(kSThreads) accept_length_nodes_kernel(const AccLenParams P) {
-    chain_wait();
+// One item = one tree row with children of one sequence, evaluated by a cluster of CTAs (slices of the vocabulary, as in
+// the walk above).  The resident clusters take the items in turn; a row's children are tried in order with the same
+// closed-form residual recursion, but every rejection branch is followed: child j gets reach_j a_j with
+// reach_j = prod_{i<j} (1 - a_i).  Clusters of 8 at V = 128256 keep at most 36 pairs of cached rows alive (74 MB,
+// inside L2; one CTA per row had 300 MB of them and went to HBM with every pass).
+template <typename T, int kPerSm>
+__global__ void __launch_bounds__(kSThreads, kPerSm) accept_length_nodes_kernel(const __grid_constant__ AccLenParams P) {
     const radar_acclen_args& a = P.a;
-    const int tid = threadIdx.x, V = a.V;
-    __shared__ double s_red[32];
-    __shared__ double s_slots[2 * kMaxCluster];
-    __shared__ int s_tok[kMaxNodes], s_par[kMaxNodes];
-    __shared__ int s_rx[RADAR_MAX_NODES];
-    __shared__ double s_ra[RADAR_MAX_NODES];
-    ClusterRed red{s_red, s_slots, 0u, 1u, 0};       // launched without clusters: every block is its own
-    double* pc = P.p_cache + (size_t)blockIdx.x * V;
-    double* qc = P.q_cache + (size_t)blockIdx.x * V;
+    unsigned crank, csize;
+    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(crank));
+    asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(csize));
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, V = a.V;
+    __shared__ NodeShared S;
+    constexpr int kBatch = 8, kRows = kBatch * kMaxNodes, kEach = kRows / kSThreads;      // sequences whose trees are looked at together
+    __shared__ __align__(16) int s_count[kRows + 4];         // children of each of their rows, then the order's keys
+    __shared__ int s_group[kRows / 32];
+    __shared__ short s_order[kRows];
+    __shared__ int s_tok[kRows], s_par[kRows], s_drow[kRows];      // the batch's trees
+    S.exps.fill(P.tab);
+    ClusterRed red{S.red, P.status, crank, csize, 0};
+    red.start();
+    chain_wait();
+    const int cluster = blockIdx.x / csize, n_clusters = gridDim.x / csize;
+    const int nq = (V + 3) / 4;
+    const int v0 = 4 * (int)((long long)nq * crank / csize), v1 = min(V, 4 * (int)((long long)nq * (crank + 1) / csize));
+    const Cache C{P.cache + 2 * ((size_t)cluster * cache_stride(V) + v0 + kTileTokens * crank), P.smem_tiles};
     const double invT = 1.0 / (double)a.temperature;
     bool nan_seen = false, bad_tree = false;
 
-    for (int item = blockIdx.x; item < a.B * kMaxNodes; item += gridDim.x) {
-        const int b = item / kMaxNodes, c = item % kMaxNodes;
-        const int M = min(max(a.n_nodes[b], 1), kMaxNodes);
-        if (c >= M) {
-            if (tid == 0) P.cond[item] = 0.0;
-            continue;
-        }
-        __syncthreads();                                  // previous item's readers are done with s_tok / s_par
-        if (tid < kMaxNodes) {
-            s_tok[tid] = tid < M ? a.tree_tok[(size_t)b * kMaxNodes + tid] : -1;
-            s_par[tid] = tid < M ? a.tree_parent[(size_t)b * kMaxNodes + tid] : -2;
-        }
-        __syncthreads();
-        if (c == 0 && tid == 0) P.cond[item] = 1.0;       // the root is always "accepted"
-        int nchild = 0;
-        for (int j = c + 1; j < M; ++j) nchild += s_par[j] == c ? 1 : 0;
-        if (nchild == 0) continue;
-        const int drow = a.tree_draft_row[(size_t)b * kMaxNodes + c];
-        if (drow < 0 || drow >= a.R) { bad_tree = true; continue; }
-        const T* target = reinterpret_cast<const T*>(a.target_logits) + ((size_t)b * kMaxNodes + c) * V;
-        const T* draft = reinterpret_cast<const T*>(a.draft_logits) + ((size_t)b * a.R + drow) * V;
-        const double ip = softmax_to_cache<T>(target, 0, V, invT, pc, red, &nan_seen);
-        const double iq = softmax_to_cache<T>(draft, 0, V, invT, qc, red, &nan_seen);
-
-        double a_coef = 0.0, Wn = 1.0, cq = 1.0, reach = 1.0;
-        int n_rej = 0;
-        bool exhausted = false;
-        for (int j = c + 1; j < M; ++j) {
-            if (s_par[j] != c) continue;
-            if (exhausted) {
-                if (tid == 0) P.cond[(size_t)b * kMaxNodes + j] = 0.0;
-                continue;
+    for (int b0 = 0; b0 < a.B; b0 += kBatch) {
+        int n_items;
+        // Rows with children of up to eight sequences, those with the most children first (a row's time is two passes
+        // over its logits and one per child but the last), dealt out over the clusters back and forth: thread (b, c)
+        // counts row c's children and finds its own place in that order.
+        {
+            // (every thread does kEach rows: row e = tid + i * kSThreads of the batch)
+            int tok[kEach], up[kEach], dr[kEach], M[kEach];
+#pragma unroll
+            for (int i = 0; i < kEach; ++i) {
+                const int e = tid + i * kSThreads, b = b0 + e / kMaxNodes;
+                const size_t o = (size_t)(b < a.B ? b : 0) * kMaxNodes + e % kMaxNodes;
+                tok[i] = a.tree_tok[o]; up[i] = a.tree_parent[o]; dr[i] = a.tree_draft_row[o];
+                M[i] = b < a.B ? min(max(a.n_nodes[b], 1), kMaxNodes) : 0;
             }
-            const int x = s_tok[j];
-            if (x < 0 || x >= V) { bad_tree = true; break; }
-            const double px = pc[x] * ip, qx = qc[x] * iq;
-            const double pj = fmax(0.0, px - a_coef * qx) / Wn;
-            const double qj = cq * qx;
-            double acc;
-            if (qj <= 0.0) acc = pj > 0.0 ? 1.0 : 0.0;
-            else { acc = pj / qj; if (acc > 1.0) acc = 1.0; }
-            if (tid == 0) P.cond[(size_t)b * kMaxNodes + j] = reach * acc;
-            reach *= 1.0 - acc;
-            // the rejection branch: new residual, x leaves the draft distribution
-            const double a_new = a_coef + cq * Wn;
-            double g = 0.0;
-            for (int v = tid; v < V; v += kSThreads) g += fmax(0.0, pc[v] * ip - a_new * (qc[v] * iq));
-            g = red.sum(g);
-            for (int r = 0; r < n_rej; ++r) {
-                const int xr = s_rx[r];
-                const double pr = pc[xr] * ip, qr = qc[xr] * iq;
-                g += fmax(0.0, pr - s_ra[r] * qr) - fmax(0.0, pr - a_new * qr);
+            __syncthreads();                                 // the previous batch's readers are done
+#pragma unroll
+            for (int i = 0; i < kEach; ++i) {
+                const int e = tid + i * kSThreads, c = e % kMaxNodes;
+                s_count[e] = 0;
+                s_tok[e] = c < M[i] ? tok[i] : -1;
+                s_par[e] = c < M[i] ? up[i] : -2;
+                s_drow[e] = dr[i];
             }
-            double frozen = a_coef;
-            if (g > 0.0) { a_coef = a_new; Wn = g; frozen = a_new; }
             __syncthreads();
-            if (tid == 0) { s_rx[n_rej] = x; s_ra[n_rej] = frozen; }
+#pragma unroll
+            for (int i = 0; i < kEach; ++i) {
+                const int e = tid + i * kSThreads, c = e % kMaxNodes;
+                if (c > 0 && c < M[i] && up[i] >= 0 && up[i] < c) atomicAdd(&s_count[e - c + up[i]], 1);
+            }
             __syncthreads();
-            ++n_rej;
-            const double rest = 1.0 - qj;
-            if (rest <= 0.0) exhausted = true;
-            else cq = cq / rest;
+            int mine[kEach];
+            unsigned has[kEach];
+#pragma unroll
+            for (int i = 0; i < kEach; ++i) {
+                mine[i] = s_count[tid + i * kSThreads];
+                has[i] = __ballot_sync(kFull, mine[i] > 0);
+                if (lane == 0) s_group[warp + i * kSWarps] = __popc(has[i]);
+            }
+            __syncthreads();
+            n_items = 0;
+            int before[kEach];
+#pragma unroll
+            for (int g = 0; g < kRows / 32; ++g) {           // groups of 32 rows, in order
+#pragma unroll
+                for (int i = 0; i < kEach; ++i)
+                    if (g == warp + i * kSWarps) before[i] = n_items;
+                n_items += s_group[g];
+            }
+#pragma unroll
+            for (int i = 0; i < kEach; ++i)                  // (all counts have been read)
+                if (mine[i] > 0) s_count[before[i] + __popc(has[i] & ((1u << lane) - 1u))] = (kMaxNodes - mine[i]) * kRows + tid + i * kSThreads;
+            if (tid < 3) s_count[n_items + tid] = 0x7fffffff;
+            __syncthreads();
+            for (int x = tid; x < n_items; x += kSThreads) {
+                const int key = s_count[x];
+                int place = 0;
+                for (int o = 0; o < n_items; o += 4) {
+                    const int4 k4 = *reinterpret_cast<const int4*>(s_count + o);
+                    place += (k4.x < key ? 1 : 0) + (k4.y < key ? 1 : 0) + (k4.z < key ? 1 : 0) + (k4.w < key ? 1 : 0);
+                }
+                s_order[place] = (short)(key % kRows);
+            }
+            __syncthreads();
+        }
+        for (int round = 0; round * n_clusters < n_items; ++round) {
+            const int place = round * n_clusters + ((round & 1) ? n_clusters - 1 - cluster : cluster);
+            if (place < n_items) {
+                const int item = s_order[place], first = item & ~(kMaxNodes - 1);
+                const int b = b0 + item / kMaxNodes, c = item % kMaxNodes;
+                const int drow = s_drow[item];
+                __syncthreads();                             // the previous item's readers are done with S
+                if (tid < kMaxNodes) {
+                    S.tok[tid] = s_tok[first + tid];
+                    S.par[tid] = s_par[first + tid];
+                }
+                __syncthreads();
+                if (drow < 0 || drow >= a.R) { bad_tree = true; continue; }
+                unsigned long long kids = children_of(S, c);
+                const T* target = reinterpret_cast<const T*>(a.target_logits) + ((size_t)b * kMaxNodes + c) * V;
+                const T* draft = reinterpret_cast<const T*>(a.draft_logits) + ((size_t)b * a.R + drow) * V;
+                // the rows of this cluster's next item are asked for while this one's are worked on
+                const int next = (round + 1) * n_clusters + ((round & 1) ? cluster : n_clusters - 1 - cluster);
+                const double2 sums = softmax_rows<T>(S, red, target, draft, V, v0, v1, invT, C, kids, &nan_seen, [&] {
+                    if (tid == 0 && next < n_items) {
+                        const size_t bn = b0 + s_order[next] / kMaxNodes, cn = s_order[next] % kMaxNodes;
+                        const int dn = s_drow[s_order[next]];
+                        prefetch_slice(reinterpret_cast<const T*>(a.target_logits) + (bn * kMaxNodes + cn) * V, v0, v1);
+                        if (dn >= 0 && dn < a.R) prefetch_slice(reinterpret_cast<const T*>(a.draft_logits) + (bn * a.R + dn) * V, v0, v1);
+                    }
+                });
+                Residual res(sums.x, sums.y);
+                double reach = 1.0;
+                bool exhausted = false;
+                for (; kids != 0; kids &= kids - 1) {
+                    const int j = __ffsll(kids) - 1;
+                    if (exhausted) {
+                        if (crank == 0 && tid == 0) P.cond[(size_t)b * kMaxNodes + j] = 0.0;
+                        continue;
+                    }
+                    const int x = S.tok[j];
+                    if (x < 0 || x >= V) { bad_tree = true; break; }
+                    const double ep = S.pe[j], eq = S.qe[j];
+                    const double pj = res.left(ep, eq), qj = res.draft(eq);
+                    auto book = [&] {
+                        double acc;
+                        if (qj <= 0.0) acc = pj > 0.0 ? 1.0 : 0.0;
+                        else { acc = pj / (qj * res.G); if (acc > 1.0) acc = 1.0; }
+                        if (crank == 0 && tid == 0) P.cond[(size_t)b * kMaxNodes + j] = reach * acc;
+                        reach *= 1.0 - acc;
+                    };
+                    // the rejection branch: new residual, x leaves the draft distribution (nobody is left to see the last one's)
+                    if ((kids & (kids - 1)) != 0) exhausted = !res.reject(red, C, v0, v1, x, ep, eq, qj, book);
+                    else book();
+                }
+            }
         }
     }
+    // (every CTA has received all that was sent to it: none leaves before a store into its shared memory has landed)
     if (nan_seen) set_status(P.status, RADAR_ERR_NUMERIC);
     if (bad_tree && tid == 0) set_status(P.status, RADAR_ERR_TREE);
 }
 
-// one warp per sequence: P_acc along the paths (parents precede children), P_stop, p_i
+// one warp per sequence: P_acc along the paths, P_stop, p_i.  Lane l owns rows l and l + 32 (and length l).
 __global__ void __launch_bounds__(32) accept_length_dist_kernel(const AccLenParams P) {
     chain_wait();
     const radar_acclen_args& a = P.a;
     const int b = blockIdx.x, lane = threadIdx.x;
     const int M = min(max(a.n_nodes[b], 1), kMaxNodes);
-    __shared__ double s_pacc[kMaxNodes], s_sum[kMaxNodes], s_dist[64];
-    for (int i = lane; i < kMaxNodes; i += 32) { s_pacc[i] = 0.0; s_sum[i] = 0.0; }
-    for (int i = lane; i < 64; i += 32) s_dist[i] = 0.0;
-    __syncwarp();
-    if (lane == 0) {
-        s_pacc[0] = 1.0;
-        for (int j = 1; j < M; ++j) {
-            const int par = a.tree_parent[(size_t)b * kMaxNodes + j];
-            const double cj = (par >= 0 && par < j) ? P.cond[(size_t)b * kMaxNodes + j] : 0.0;
-            s_pacc[j] = (par >= 0 && par < j ? s_pacc[par] : 0.0) * cj;
-            if (par >= 0 && par < j) s_sum[par] += cj;
-        }
-        for (int c = 0; c < M; ++c) {
-            const int dep = a.tree_depth[(size_t)b * kMaxNodes + c];
-            if (dep >= 0 && dep <= a.t_max) s_dist[dep] += s_pacc[c] * (1.0 - s_sum[c]);
-        }
+    __shared__ double s_cond[kMaxNodes], s_stop[kMaxNodes];
+    __shared__ int s_par[kMaxNodes], s_dep[kMaxNodes];
+#pragma unroll
+    for (int j = lane; j < kMaxNodes; j += 32) {
+        const size_t o = (size_t)b * kMaxNodes + j;
+        const int par = j > 0 && j < M ? a.tree_parent[o] : -1;
+        s_par[j] = par < j ? par : -1;
+        s_dep[j] = j < M ? a.tree_depth[o] : -1;
+        s_cond[j] = s_par[j] >= 0 ? P.cond[o] : (j == 0 ? 1.0 : 0.0);       // the root is always "accepted"
     }
     __syncwarp();
-    for (int i = lane; i < kMaxNodes; i += 32) a.p_acc_node[(size_t)b * kMaxNodes + i] = s_pacc[i];
-    for (int i = lane; i <= a.t_max; i += 32) a.dist[(size_t)b * (a.t_max + 1) + i] = s_dist[i];
+#pragma unroll
+    for (int c = lane; c < kMaxNodes; c += 32) {
+        double p = s_cond[c];
+        for (int q = s_par[c]; q > 0; q = s_par[q]) p *= s_cond[q];
+        double acc = 0.0;                                                   // children in row order
+        for (int j = c + 1; j < M; ++j) acc += s_par[j] == c ? s_cond[j] : 0.0;
+        if (c >= M) p = 0.0;
+        a.p_acc_node[(size_t)b * kMaxNodes + c] = p;
+        s_stop[c] = p * (1.0 - acc);
+    }
+    __syncwarp();
+    for (int i = lane; i <= a.t_max; i += 32) {
+        double d = 0.0;
+        for (int c = 0; c < M; ++c) d += s_dep[c] == i ? s_stop[c] : 0.0;
+        a.dist[(size_t)b * (a.t_max + 1) + i] = d;
+    }
+}
+
+// correctly rounded from 64-bit mantissas
+ExpTable exp_table() {
+    static const ExpTable t = [] {
+        ExpTable x;
+        for (int j = 0; j < 64; ++j) x.t[j] = (double)exp2l((long double)j / 64.0L);
+        return x;
+    }();
+    return t;
 }
 
 }  // namespace
 }  // namespace radar
 
 using namespace radar;
+
+// shared memory for the cached tiles of a slice, all of them or as many as fit
+static size_t cache_smem(int V, int cs, int per_sm) {
+    const int slice = 4 * (((V + 3) / 4 + cs - 1) / cs);
+    return std::min(cache_room(per_sm), (size_t)(slice + kTileTokens - 1) / kTileTokens * kTileBytes);
+}
+
+// launch configuration of the cluster kernels (attr: two attributes that outlive it)
+static cudaLaunchConfig_t cluster_config(int ctas, int cs, size_t smem, cudaStream_t stream, cudaLaunchAttribute* attr) {
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = (unsigned)cs;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)ctas);
+    cfg.blockDim = dim3(kSThreads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = stream;
+    cfg.attrs = attr;
+    cfg.numAttrs = 2;
+    return cfg;
+}
+
+template <typename T, int kPerSm>
+static cudaError_t launch_walk(radar_ctx* ctx, StochParams& sp, int cs, cudaStream_t stream) {
+    const size_t smem = cache_smem(sp.a.V, cs, kPerSm);
+    sp.smem_tiles = (int)(smem / kTileBytes);
+    cudaError_t e = radar_opt_in_smem(ctx, RADAR_SMEM_WALK + 2 * (sizeof(T) == 2) + kPerSm - 1, stochastic_walk_kernel<T, kPerSm>, cache_room(kPerSm));
+    if (e != cudaSuccess) return e;
+    cudaLaunchAttribute attr[2];
+    const cudaLaunchConfig_t cfg = cluster_config(sp.a.B * cs, cs, smem, stream, attr);
+    radar_launch_scope scope(ctx, RADAR_K_STOCH_WALK, stream);
+    return cudaLaunchKernelEx(&cfg, stochastic_walk_kernel<T, kPerSm>, sp);
+}
 
 extern "C" size_t radar_accept_workspace_bytes(const radar_ctx* ctx, int B, int V, int mode) {
     if (!ctx || B <= 0 || V <= 0) return 0;
@@ -513,7 +952,7 @@ extern "C" size_t radar_accept_workspace_bytes(const radar_ctx* ctx, int B, int 
         const int n_chunks = vocab_pass_plan_chunks(ctx->sm_count, B * kMaxNodes, V, &chunk);
         return vocab_pass_partial_bytes(B * kMaxNodes, n_chunks, 1);
     }
-    return align_up((size_t)B * V * sizeof(double), 256) * 2;
+    return align_up((size_t)B * cache_stride(V) * sizeof(double), 256) * 2;
 }
 
 extern "C" int radar_verify_accept(radar_ctx* ctx, const radar_accept_args* a, void* stream_) {
@@ -559,41 +998,60 @@ extern "C" int radar_verify_accept(radar_ctx* ctx, const radar_accept_args* a, v
     if (!(a->temperature > 0.f)) return RADAR_ERR_INVALID_ARG;
     StochParams sp;
     sp.a = *a;
-    sp.p_cache = reinterpret_cast<double*>(a->workspace);
-    sp.q_cache = reinterpret_cast<double*>(reinterpret_cast<char*>(a->workspace) +
-                                           align_up((size_t)a->B * a->V * sizeof(double), 256));
+    sp.cache = reinterpret_cast<double*>(a->workspace);
     sp.status = ctx->d_status;
-    // cluster size: as many CTAs per sequence as keep the whole batch resident at once (at most 8)
+    sp.tab = exp_table();
+    // Cluster size: as many CTAs per sequence as keep the whole batch resident at once, two to an SM, while a CTA's slice
+    // of the vocabulary is worth an exchange between them.  One CTA per SM where that still leaves SMs over (clusters need
+    // their SMs in one GPC, so not all SMs can be used that way): B = 4, V = 32000 28 / 34 us for one / two; B = 16,
+    // V = 17000 42 / 35; B = 32, V = 128256 128 (clusters of 4) / 107.
     int cs = 1;
-    while (cs < kMaxCluster && (long long)a->B * cs * 2 <= ctx->sm_count) cs *= 2;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)(a->B * cs));
-    cfg.blockDim = dim3(kSThreads);
-    cfg.dynamicSmemBytes = 0;
-    cfg.stream = stream;
-    cudaLaunchAttribute attr[2];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = (unsigned)cs;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
-    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[1].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 2;
-    {
-        radar_launch_scope scope(ctx, RADAR_K_STOCH_WALK, stream);
-        if (a->logits_dtype == RADAR_F32) RADAR_CUDA_CHECK(cudaLaunchKernelEx(&cfg, stochastic_walk_kernel<float>, sp));
-        else RADAR_CUDA_CHECK(cudaLaunchKernelEx(&cfg, stochastic_walk_kernel<__nv_bfloat16>, sp));
-    }
+    while (cs < kMaxCluster && (long long)a->B * cs * 2 <= 2 * ctx->sm_count && a->V >= cs * 2 * kMinSlice) cs *= 2;
+    const bool one = 4ll * a->B * cs <= 3ll * ctx->sm_count;
+    if (a->logits_dtype == RADAR_F32) RADAR_CUDA_CHECK((one ? launch_walk<float, 1>(ctx, sp, cs, stream) : launch_walk<float, 2>(ctx, sp, cs, stream)));
+    else RADAR_CUDA_CHECK((one ? launch_walk<__nv_bfloat16, 1>(ctx, sp, cs, stream) : launch_walk<__nv_bfloat16, 2>(ctx, sp, cs, stream)));
     RADAR_CUDA_CHECK(cudaGetLastError());
     return RADAR_OK;
 }
 
-static int acclen_grid(const radar_ctx* ctx, int B) { return std::min(B * kMaxNodes, ctx->sm_count); }
+// CTAs per tree row: a slice of at least kAccMinSlice tokens each
+static int acclen_cluster(int V) {
+    int cs = 1;
+    while (cs < kMaxCluster && V >= cs * 2 * kAccMinSlice) cs *= 2;
+    return cs;
+}
+static int acclen_max_clusters(const radar_ctx* ctx, int B, int cs) { return std::min(B * kMaxNodes, std::max(1, 2 * ctx->sm_count / cs)); }
 
 extern "C" size_t radar_acclen_workspace_bytes(const radar_ctx* ctx, int B, int V) {
     if (!ctx || B <= 0 || V <= 0) return 0;
-    return 2 * align_up((size_t)acclen_grid(ctx, B) * V * sizeof(double), 256) + align_up((size_t)B * kMaxNodes * sizeof(double), 256);
+    return 2 * align_up((size_t)acclen_max_clusters(ctx, B, acclen_cluster(V)) * cache_stride(V) * sizeof(double), 256) +
+           align_up((size_t)B * kMaxNodes * sizeof(double), 256);
+}
+
+template <typename T, int kPerSm>
+static cudaError_t launch_acclen(radar_ctx* ctx, AccLenParams& P, int cs, int max_clusters, cudaStream_t stream) {
+    constexpr int kind = 2 * (sizeof(T) == 2) + kPerSm - 1;
+    cudaError_t e = radar_opt_in_smem(ctx, RADAR_SMEM_ACCLEN + kind, accept_length_nodes_kernel<T, kPerSm>, cache_room(kPerSm));
+    if (e != cudaSuccess) return e;
+    // As many clusters as are resident at once: the rows are dealt out over them in advance.  How many that is, is a
+    // property of the kernel and the device, asked for once per cluster size (with the most shared memory it may get).
+    int log_cs = 0;
+    while ((1 << log_cs) < cs) ++log_cs;
+    cudaLaunchAttribute attr[2];
+    int& resident = ctx->acclen_clusters[kind][log_cs];
+    if (resident == 0) {
+        cudaLaunchConfig_t q = cluster_config(2 * ctx->sm_count / cs * cs, cs, cache_room(kPerSm), stream, attr);
+        q.numAttrs = 1;
+        int n = 0;
+        e = cudaOccupancyMaxActiveClusters(&n, accept_length_nodes_kernel<T, kPerSm>, &q);
+        if (e != cudaSuccess) return e;
+        resident = n > 0 ? n : 1;
+    }
+    const size_t smem = cache_smem(P.a.V, cs, kPerSm);
+    P.smem_tiles = (int)(smem / kTileBytes);
+    const cudaLaunchConfig_t cfg = cluster_config(std::min(max_clusters, resident) * cs, cs, smem, stream, attr);
+    radar_launch_scope scope(ctx, RADAR_K_ACCLEN_NODES, stream);
+    return cudaLaunchKernelEx(&cfg, accept_length_nodes_kernel<T, kPerSm>, P);
 }
 
 extern "C" int radar_accept_length_distribution(radar_ctx* ctx, const radar_acclen_args* a, void* stream_) {
@@ -607,20 +1065,21 @@ extern "C" int radar_accept_length_distribution(radar_ctx* ctx, const radar_accl
         return RADAR_ERR_INVALID_ARG;
     if ((reinterpret_cast<uintptr_t>(a->workspace) & 255) != 0) return RADAR_ERR_WORKSPACE;
     if (radar_acclen_workspace_bytes(ctx, a->B, a->V) > a->workspace_bytes) return RADAR_ERR_WORKSPACE;
-    const int grid = acclen_grid(ctx, a->B);
+    const int cs = acclen_cluster(a->V), max_clusters = acclen_max_clusters(ctx, a->B, cs);
     AccLenParams P;
     P.a = *a;
     char* w = reinterpret_cast<char*>(a->workspace);
-    const size_t cache = align_up((size_t)grid * a->V * sizeof(double), 256);
-    P.p_cache = reinterpret_cast<double*>(w);
-    P.q_cache = reinterpret_cast<double*>(w + cache);
+    const size_t cache = align_up((size_t)max_clusters * cache_stride(a->V) * sizeof(double), 256);
+    P.cache = reinterpret_cast<double*>(w);
     P.cond = reinterpret_cast<double*>(w + 2 * cache);
     P.status = ctx->d_status;
-    {
-        radar_launch_scope scope(ctx, RADAR_K_ACCLEN_NODES, stream);
-        if (a->logits_dtype == RADAR_F32) RADAR_CUDA_CHECK(launch_chained(accept_length_nodes_kernel<float>, dim3(grid), dim3(kSThreads), 0, stream, P));
-        else RADAR_CUDA_CHECK(launch_chained(accept_length_nodes_kernel<__nv_bfloat16>, dim3(grid), dim3(kSThreads), 0, stream, P));
-    }
+    P.tab = exp_table();
+    // One CTA per SM while the rows (about twenty with children to a tree) are few waves, two when their passes are what
+    // takes the time: 4 trees, V = 32000 (16 CTAs times rows) 31 / 36 us for one / two; 4 trees, V = 70000 (32) 52 / 44;
+    // 16 trees, V = 32000 (64) 88 / 72; 8 trees, V = 128256 (64) 191 / 135.
+    const bool one = a->B * cs <= 16;
+    if (a->logits_dtype == RADAR_F32) RADAR_CUDA_CHECK((one ? launch_acclen<float, 1>(ctx, P, cs, max_clusters, stream) : launch_acclen<float, 2>(ctx, P, cs, max_clusters, stream)));
+    else RADAR_CUDA_CHECK((one ? launch_acclen<__nv_bfloat16, 1>(ctx, P, cs, max_clusters, stream) : launch_acclen<__nv_bfloat16, 2>(ctx, P, cs, max_clusters, stream)));
     RADAR_CUDA_CHECK(cudaGetLastError());
     {
         radar_launch_scope scope(ctx, RADAR_K_ACCLEN_DIST, stream);
