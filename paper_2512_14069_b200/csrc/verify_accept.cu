@@ -26,27 +26,45 @@ struct GreedyParams {
     VocabPassParams vp;
 };
 
-__global__ void __launch_bounds__(64) greedy_walk_kernel(const GreedyParams P) {
+// Latency is all there is to it: eight threads share a row's chunk records, and what the end needs (leaf count, retrieve
+// rows) is asked for at the start.
+constexpr int kGreedyThreads = 8 * kMaxNodes;
+__global__ void __launch_bounds__(kGreedyThreads) greedy_walk_kernel(const GreedyParams P) {
     chain_wait();
     const radar_accept_args& a = P.a;
     const int b = blockIdx.x, tid = threadIdx.x, lane = tid & 31;
     __shared__ int s_arg[kMaxNodes], s_tok[kMaxNodes], s_par[kMaxNodes];
     const int M = min(max(a.n_nodes[b], 1), kMaxNodes);
+    const int nl = a.n_leaves[b];
     const int nc = P.vp.n_chunks;
-    {   // argmax of row tid: best chunk record by (value desc, token asc)
+    const int retr = a.N * (a.t_max + 1);
+    if (tid * 32 < retr) asm volatile("prefetch.global.L1 [%0];" ::"l"(a.retrieve + (size_t)b * retr + tid * 32));
+    {   // argmax of row tid / 8: best chunk record by (value desc, token asc)
+        const int r = tid >> 3;
         int best_i = 0x7fffffff;
         float best_v = -CUDART_INF_F;
-        if (tid < M) {
-            const size_t rec0 = ((size_t)b * kMaxNodes + tid) * nc;
-            for (int c = 0; c < nc; ++c) {
+        if (r < M) {
+            const size_t rec0 = ((size_t)b * kMaxNodes + r) * nc;
+#pragma unroll 4
+            for (int c = tid & 7; c < nc; c += 8) {
                 const float v = P.vp.part_v[rec0 + c];
                 const int i = P.vp.part_i[rec0 + c];
                 if (precedes(v, i, best_v, best_i)) { best_v = v; best_i = i; }
             }
         }
-        s_arg[tid] = best_i;
-        s_tok[tid] = tid < M ? a.tree_tok[(size_t)b * kMaxNodes + tid] : -1;
-        s_par[tid] = tid < M ? a.tree_parent[(size_t)b * kMaxNodes + tid] : -2;
+        if (tid < kMaxNodes) {
+            const size_t o = (size_t)b * kMaxNodes + tid;
+            const int tok = a.tree_tok[o], par = a.tree_parent[o];
+            s_tok[tid] = tid < M ? tok : -1;
+            s_par[tid] = tid < M ? par : -2;
+        }
+#pragma unroll
+        for (int o = 4; o > 0; o >>= 1) {
+            const float ov = __shfl_xor_sync(kFull, best_v, o);
+            const int oi = __shfl_xor_sync(kFull, best_i, o);
+            if (precedes(ov, oi, best_v, best_i)) { best_v = ov; best_i = oi; }
+        }
+        if ((tid & 7) == 0) s_arg[r] = best_i;
     }
     __syncthreads();
     if (tid >= 32) return;
@@ -67,7 +85,6 @@ __global__ void __launch_bounds__(64) greedy_walk_kernel(const GreedyParams P) {
     }
     for (int dd = len + 1 + lane; dd < W; dd += 32) { pn[dd] = -1; pt[dd] = -1; }
     int best = 0x7fffffff;
-    const int nl = a.n_leaves[b];
     for (int r = lane; r < nl; r += 32)
         if (a.retrieve[((size_t)b * a.N + r) * W + len] == cur) best = min(best, r);
 #pragma unroll
@@ -989,7 +1006,7 @@ extern "C" int radar_verify_accept(radar_ctx* ctx, const radar_accept_args* a, v
         RADAR_CUDA_CHECK(vocab_pass_launch(ctx, RADAR_K_VOCAB_ACCEPT, vp, stream));
         {
             radar_launch_scope scope(ctx, RADAR_K_GREEDY_WALK, stream);
-            RADAR_CUDA_CHECK(launch_chained(greedy_walk_kernel, dim3(a->B), dim3(64), 0, stream, gp));
+            RADAR_CUDA_CHECK(launch_chained(greedy_walk_kernel, dim3(a->B), dim3(kGreedyThreads), 0, stream, gp));
         }
         RADAR_CUDA_CHECK(cudaGetLastError());
         return RADAR_OK;
@@ -1197,7 +1214,7 @@ extern "C" int radar_verify_accept_greedy_noalloc(radar_ctx* ctx, const radar_ac
     RADAR_CUDA_CHECK(vocab_pass_launch(ctx, RADAR_K_VOCAB_ACCEPT, vp, stream));
     {
         radar_launch_scope scope(ctx, RADAR_K_GREEDY_WALK, stream);
-        RADAR_CUDA_CHECK(launch_chained(greedy_walk_kernel, dim3(a->B), dim3(64), 0, stream, gp));
+        RADAR_CUDA_CHECK(launch_chained(greedy_walk_kernel, dim3(a->B), dim3(kGreedyThreads), 0, stream, gp));
     }
     RADAR_CUDA_CHECK(cudaGetLastError());
     return RADAR_OK;
