@@ -49,16 +49,16 @@ constexpr int kPairRows = 256;       // query rows of a row-block pair (and the 
 constexpr long long kSmallCacheRows = 1280;   // (cache row, KV head) pairs: tree_attn_tc_supported
 constexpr float kRescaleThreshold = 8.f;   // in log2 units: P stays below 2^8
 
-// Written by every CTA of the attention kernel, read by the combine kernel.
-struct CutUnit {
+// Written by every CTA of the attention kernel, read by the combine kernel: the pieces are worked out by the producer warp
+// behind its last load, where nothing waits for it, and not by every warp of the combine (two 64-bit divisions a piece).
+constexpr int kMaxPerClass = 160;    // CTAs of a class at most (plan_grid)
+struct __align__(16) CutUnit {
     int valid;           // 1: this CTA's last segment starts a unit that continues in the following CTAs
-    int b, g, nt;        // the unit and its number of tiles
-    int layer;           // the layer it belongs to
+    int b, g, layer;     // the unit
     int slot;            // partial slot of that first piece in this CTA (0 or 1)
     int rows;            // live query rows of the unit
-    int w;               // cost of one of its tiles
-    long long u0;        // position of the unit's first tile in the class's space
-    long long tot;       // size of that space
+    int n_pieces;        // CTAs of the class from this one on whose range begins before the unit's end
+    uint32_t live[kMaxPerClass / 32];    // bit j: piece j's range holds the start of a tile of the unit
 };
 
 struct TcParams {
@@ -354,18 +354,20 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
         // One lane does everything for the contiguous cache.  With a paged cache the whole warp walks the same
         // loop and lane p looks up and fetches page p of a tile (up to eight boxes per tile), the leading lane
         // still doing the waits, the byte counts, Q and the tree tile.
+        CutUnit cu;
+        cu.valid = 0;
+        int cut_nt = 0, cut_w = 0;
+        long long cut_u0 = 0;
         if (PAGED || lane == 0) {
             const bool lead = lane == 0;
             uint32_t kc = 0, vc = 0;
             bool ok = true;
-            CutUnit cu;
-            cu.valid = 0;
             for (uint32_t seg = 0; cur.valid(); cur.next(P, pp), ++seg) {
                 const int b = cur.b, g = cur.g, n = cur.t1 - cur.t0;
                 const bool two = TWO && cur.two_rb(P);
                 if (cur.t0 == 0 && cur.t1 < cur.s.nt) {          // necessarily the last segment of this CTA
-                    cu.valid = 1; cu.b = b; cu.g = g; cu.nt = cur.s.nt; cu.slot = seg == 0 ? 0 : 1; cu.layer = cur.layer;
-                    cu.rows = cur.s.rows; cu.w = cur.s.w; cu.u0 = cur.U; cu.tot = s_range[2];
+                    cu.valid = 1; cu.b = b; cu.g = g; cu.slot = seg == 0 ? 0 : 1; cu.layer = cur.layer; cu.rows = cur.s.rows;
+                    cut_nt = cur.s.nt; cut_w = cur.s.w; cut_u0 = cur.U;
                 }
                 if (lead) ok = ok && mbar_wait(&bar_qempty, (seg & 1) ^ 1, ab);
                 if (lead && ok) {
@@ -425,7 +427,28 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
                     if (i + la < n) load_tile(cur.t0 + i + la, true);
                 }
             }
-            if (lead) P.cut[blockIdx.x] = cu;
+        }
+        __syncwarp();
+        if (__shfl_sync(kFull, cu.valid, 0)) {
+            const int nt = __shfl_sync(kFull, cut_nt, 0), w = __shfl_sync(kFull, cut_w, 0);
+            const long long u0 = __shfl_sync(kFull, cut_u0, 0), u1 = u0 + (long long)nt * w + P.unit_cost, tot = s_range[2];
+            cu.n_pieces = 0;
+#pragma unroll 1
+            for (int k = 0; k < kMaxPerClass / 32; ++k) {
+                const int c = ci + k * 32 + lane;
+                const long long lo = tot * c / P.ncc, hi = tot * (c + 1) / P.ncc;
+                const bool piece = c < P.ncc && lo < u1;
+                const bool on = piece && tiles_before(hi, u0, nt, w, P.unit_cost) > tiles_before(lo, u0, nt, w, P.unit_cost);
+                const uint32_t pieces = __ballot_sync(kFull, piece), live = __ballot_sync(kFull, on);
+                cu.n_pieces += __popc(pieces);
+                if (lane == 0) P.cut[blockIdx.x].live[k] = live;
+                if (pieces != 0xffffffffu) break;
+            }
+        }
+        if (lane == 0) {
+            CutUnit* out = P.cut + blockIdx.x;
+            out->valid = cu.valid; out->b = cu.b; out->g = cu.g; out->layer = cu.layer;
+            out->slot = cu.slot; out->rows = cu.rows; out->n_pieces = cu.n_pieces;
         }
         __syncwarp();
     } else if (warp == kMmaWarp) {
@@ -849,206 +872,117 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
     }
 }
 
-// Merges the pieces of the units that were cut across CTAs.  Block (c, y): CTA c of the attention
-// kernel holds the first piece of a cut unit (or the block exits); the following CTAs of the same
-// class hold the rest, each as its first segment.  A warp owns up to eight query rows
-// (y * 8 + warp + 32 r); it works out the unit's pieces once and fetches four rows at a time, every
-// piece of them in flight together.
-constexpr int kCombineY = 4;                 // blocks per cut unit: 4 * 8 warps * 8 rows = 256 rows
+// Merges the pieces of the units that were cut across CTAs.  Blocks (c, *): CTA c of the attention kernel holds the first
+// piece of a cut unit (or the blocks exit); the following CTAs of the same class hold the rest, each as its first
+// segment.  A warp merges one query row, every piece of it in flight together: the work is a chain of three trips to L2,
+// and many warps hide it better than many rows a warp do (148 cut units of 256 rows: 17.1 us event-timed with one row a
+// warp, 18.4 with two, 20.6 with four; 72 cut units of 128 rows: 10.0, 10.8, 14.7).
 template <int D>
 __global__ void __launch_bounds__(256) tree_attn_tc_combine_kernel(const TcParams P) {
     chain_wait();
     const radar_attn_args& a = P.a;
-    const CutUnit cu = P.cut[blockIdx.x];
-    if (!cu.valid) return;
+    const CutUnit& cu = P.cut[blockIdx.x];
+    const int valid = cu.valid, b = cu.b, g = cu.g, layer = cu.layer, slot = cu.slot, rows = cu.rows, n_pieces = cu.n_pieces;
+    const uint32_t live0 = cu.live[0];
+    if (!valid) return;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int pp = blockIdx.x % P.n_cls, c0 = blockIdx.x / P.n_cls;
-    const long long u1 = cu.u0 + (long long)cu.nt * cu.w + P.unit_cost;
-    const int row0 = blockIdx.y * 8 + warp;
-    if (row0 >= cu.rows) return;                             // rows of a unit are live from 0 up
-    // pieces: class-local CTAs c0, c0 + 1, ... while their range starts before the unit's end
-    int n_pieces = 1;
-    while (c0 + n_pieces < P.ncc && cu.tot * (c0 + n_pieces) / P.ncc < u1) ++n_pieces;
-    const int G = P.G;
+    const int r = blockIdx.y * 8 + warp;
+    if (r >= rows) return;                                   // rows of a unit are live from 0 up
     constexpr int E = D / 32;                                // output elements per lane
-    auto rec_of = [&](int j) {                               // record of row 0 of piece j
-        const int slot = j == 0 ? cu.slot : 0;
-        return ((int64_t)((c0 + j) * P.n_cls + pp) * 2 + slot) * kPairRows;
+    // the row's record in piece j's partials (row blocks start 128 records apart, whatever part of them is live)
+    const int blk = r < P.rb_rows ? 0 : 1, in_blk = r - blk * P.rb_rows;
+    auto rec_of = [&](int j) {
+        const int64_t cta = (int64_t)blockIdx.x + (int64_t)j * P.n_cls;
+        return (cta * 2 + (j == 0 ? slot : 0)) * kPairRows + blk * 128 + in_blk;
     };
-    auto live = [&](int j) {                                 // a CTA whose range holds no tile start has no piece
-        return tiles_before(cu.tot * (c0 + j + 1) / P.ncc, cu.u0, cu.nt, cu.w, P.unit_cost) >
-               tiles_before(cu.tot * (c0 + j) / P.ncc, cu.u0, cu.nt, cu.w, P.unit_cost);
-    };
-    // record row of live row r of the unit: row blocks start 128 records apart, whatever part of them is live
-    auto rec_row = [&](int r) { return r < P.rb_rows ? r : r - P.rb_rows + 128; };
-    auto store_row = [&](int prow, const float (&o)[E], float mx, float den) {
+    auto store_row = [&](const float (&o)[E], float mx, float den) {
         const float inv = 1.f / den;
-        const int r_glob = pp * P.pair_rows + prow;
-        const int node = r_glob / G, hq = cu.g * G + r_glob % G;
-        __nv_bfloat16* dst = reinterpret_cast<__nv_bfloat16*>(a.O) + cu.layer * P.o_ls + (((int64_t)cu.b * kMaxNodes + node) * a.Hq + hq) * D + lane * E;
+        const int rb_node = (int)(((uint32_t)in_blk * P.g_magic) >> 16);
+        const int node = ((blockIdx.x % P.n_cls) * P.n_blk + blk) * P.nodes_per_rb + rb_node, hq = g * P.G + in_blk - rb_node * P.G;
+        __nv_bfloat16* dst = reinterpret_cast<__nv_bfloat16*>(a.O) + layer * P.o_ls + (((int64_t)b * kMaxNodes + node) * a.Hq + hq) * D + lane * E;
+        __nv_bfloat162 w[E / 2];
 #pragma unroll
-        for (int q = 0; q < E; q += 2) *reinterpret_cast<__nv_bfloat162*>(dst + q) = __floats2bfloat162_rn(o[q] * inv, o[q + 1] * inv);
-        if (a.lse != nullptr && lane == 0) a.lse[cu.layer * P.lse_ls + ((int64_t)cu.b * a.Hq + hq) * kMaxNodes + node] = mx + logf(den);
+        for (int q = 0; q < E; q += 2) w[q / 2] = __floats2bfloat162_rn(o[q] * inv, o[q + 1] * inv);
+        if (E == 4) *reinterpret_cast<uint2*>(dst) = *reinterpret_cast<const uint2*>(w);
+        else *reinterpret_cast<uint32_t*>(dst) = *reinterpret_cast<const uint32_t*>(w);
+        if (a.lse != nullptr && lane == 0) a.lse[layer * P.lse_ls + ((int64_t)b * a.Hq + hq) * kMaxNodes + node] = mx + logf(den);
+    };
+    auto load_row = [&](const float* src, float (&v)[E]) {
+        if (E == 4) {
+            const float4 t = *reinterpret_cast<const float4*>(src);
+            v[0] = t.x; v[1] = t.y; v[E - 2] = t.z; v[E - 1] = t.w;
+        } else {
+            const float2 t = *reinterpret_cast<const float2*>(src);
+            v[0] = t.x; v[1] = t.y;
+        }
     };
 
     if (n_pieces <= 4) {
-        // ---- the usual case: a unit spread over a few CTAs ----
-        int64_t rec[4];
-        bool on[4];
+        // ---- the usual case: a unit spread over a few CTAs.  (A CTA whose range holds no tile start has no piece.) ----
+        float2 ml[4];
+        float v[4][E], o[E];
 #pragma unroll
-        for (int j = 0; j < 4; ++j) { on[j] = j < n_pieces && live(j); rec[j] = rec_of(min(j, n_pieces - 1)); }
-        for (int rb = 0; rb < 8; rb += 4) {
-            if (row0 + 32 * rb >= cu.rows) break;
-            float2 ml[4][4];
-#pragma unroll
-            for (int r = 0; r < 4; ++r) {
-                const int prow = row0 + 32 * (rb + r);
-#pragma unroll
-                for (int j = 0; j < 4; ++j)
-                    ml[r][j] = on[j] && prow < cu.rows ? P.part_ml[rec[j] + rec_row(prow)] : make_float2(-CUDART_INF_F, 0.f);
-            }
-            float v[4][4][E];
-#pragma unroll
-            for (int r = 0; r < 4; ++r) {
-                const int prow = row0 + 32 * (rb + r);
-#pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    const bool take = on[j] && prow < cu.rows;
-                    const float* src = P.part_o + (rec[j] + (take ? rec_row(prow) : 0)) * D + lane * E;
-                    if (E == 4) {
-                        const float4 t = take ? *reinterpret_cast<const float4*>(src) : make_float4(0.f, 0.f, 0.f, 0.f);
-                        v[r][j][0] = t.x; v[r][j][1] = t.y; v[r][j][E - 2] = t.z; v[r][j][E - 1] = t.w;
-                    } else {
-                        const float2 t = take ? *reinterpret_cast<const float2*>(src) : make_float2(0.f, 0.f);
-                        v[r][j][0] = t.x; v[r][j][1] = t.y;
-                    }
-                }
-            }
-#pragma unroll
-            for (int r = 0; r < 4; ++r) {
-                const int prow = row0 + 32 * (rb + r);
-                if (prow >= cu.rows) break;
-                const float mx = fmaxf(fmaxf(ml[r][0].x, ml[r][1].x), fmaxf(ml[r][2].x, ml[r][3].x));
-                float den = 0.f, o[E];
-#pragma unroll
-                for (int q = 0; q < E; ++q) o[q] = 0.f;
-#pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    const float w = ml[r][j].x == -CUDART_INF_F ? 0.f : __expf(ml[r][j].x - mx);
-                    den = fmaf(ml[r][j].y, w, den);
-#pragma unroll
-                    for (int q = 0; q < E; ++q) o[q] = fmaf(v[r][j][q], w, o[q]);
-                }
-                store_row(prow, o, mx, den);
-            }
+        for (int j = 0; j < 4; ++j) {
+            const bool on = ((live0 >> j) & 1u) && j < n_pieces;
+            const int64_t rec = rec_of(on ? j : 0);
+            ml[j] = P.part_ml[rec];
+            load_row(P.part_o + rec * D + lane * E, v[j]);
+            if (!on) ml[j] = make_float2(-CUDART_INF_F, 0.f);
         }
+        const float mx = fmaxf(fmaxf(ml[0].x, ml[1].x), fmaxf(ml[2].x, ml[3].x));
+        float den = 0.f;
+#pragma unroll
+        for (int q = 0; q < E; ++q) o[q] = 0.f;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            if (ml[j].x == -CUDART_INF_F) continue;
+            const float w = __expf(ml[j].x - mx);
+            den = fmaf(ml[j].y, w, den);
+#pragma unroll
+            for (int q = 0; q < E; ++q) o[q] = fmaf(v[j][q], w, o[q]);
+        }
+        store_row(o, mx, den);
         return;
     }
 
-    // ---- a unit spread over many CTAs (very long prefixes): one row at a time, lane j holds piece j's (m, l) ----
-    for (int prow = row0; prow < cu.rows; prow += 32) {
-        float den = 0.f, mx = -CUDART_INF_F, o[E];
+    // ---- a unit spread over many CTAs (few units, long prefixes): lane j holds piece j's (m, l) ----
+    float den = 0.f, mx = -CUDART_INF_F, o[E];
 #pragma unroll
-        for (int q = 0; q < E; ++q) o[q] = 0.f;
-        for (int j0 = 0; j0 < n_pieces; j0 += 32) {
-            const int jl = j0 + lane;
-            float2 ml = make_float2(-CUDART_INF_F, 0.f);
-            if (jl < n_pieces && live(jl)) ml = P.part_ml[rec_of(jl) + rec_row(prow)];
-            const float mnew = fmaxf(mx, warp_max(ml.x));
-            if (mnew == -CUDART_INF_F) continue;
-            const float rescale = __expf(mx - mnew);             // 0 on the first live batch
-            den *= rescale;
-#pragma unroll
-            for (int q = 0; q < E; ++q) o[q] *= rescale;
-            mx = mnew;
-            const float wl = ml.x == -CUDART_INF_F ? 0.f : __expf(ml.x - mx);
-            den += warp_sum(ml.y * wl);
-            const int nb = min(32, n_pieces - j0);
-            for (int u0 = 0; u0 < nb; u0 += 4) {
-                float v[4][E], w[4];
-#pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                    w[u] = u0 + u < nb ? __shfl_sync(kFull, wl, u0 + u) : 0.f;
-                    const float* src = P.part_o + (rec_of(j0 + min(u0 + u, nb - 1)) + rec_row(prow)) * D + lane * E;
-#pragma unroll
-                    for (int q = 0; q < E; ++q) v[u][q] = w[u] != 0.f ? src[q] : 0.f;
-                }
-#pragma unroll
-                for (int u = 0; u < 4; ++u)
-#pragma unroll
-                    for (int q = 0; q < E; ++q) o[q] = fmaf(v[u][q], w[u], o[q]);
-            }
-        }
-        store_row(prow, o, mx, den);
-    }
-}
-
-// The same merge for launches with few cut units, where latency counts: block (c, y): CTA c of the attention
-// kernel holds the first piece of a cut unit (or the block exits); the following CTAs of the same
-// class hold the rest, each as its first segment.  One warp per query row, 8 rows per block.
-template <int D>
-__global__ void __launch_bounds__(256) tree_attn_tc_combine_wide_kernel(const TcParams P) {
-    chain_wait();
-    const radar_attn_args& a = P.a;
-    const CutUnit cu = P.cut[blockIdx.x];
-    if (!cu.valid) return;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int pp = blockIdx.x % P.n_cls, c0 = blockIdx.x / P.n_cls;
-    const long long u1 = cu.u0 + (long long)cu.nt * cu.w + P.unit_cost;
-    // pieces: class-local CTAs c0, c0 + 1, ... while their range starts before the unit's end
-    int n_pieces = 1;
-    while (c0 + n_pieces < P.ncc && cu.tot * (c0 + n_pieces) / P.ncc < u1) ++n_pieces;
-    const int G = P.G;
-    const int prow = blockIdx.y * 8 + warp;
-    if (prow >= cu.rows) return;                             // rows of a unit are live from 0 up
-    auto rec_of = [&](int j) {
-        const int slot = j == 0 ? cu.slot : 0;
-        return ((int64_t)((c0 + j) * P.n_cls + pp) * 2 + slot) * kPairRows + (prow < P.rb_rows ? prow : prow - P.rb_rows + 128);
-    };
-    auto live = [&](int j) {                                 // a CTA whose range holds no tile start has no piece
-        return tiles_before(cu.tot * (c0 + j + 1) / P.ncc, cu.u0, cu.nt, cu.w, P.unit_cost) >
-               tiles_before(cu.tot * (c0 + j) / P.ncc, cu.u0, cu.nt, cu.w, P.unit_cost);
-    };
-    float den = 0.f, mx = -CUDART_INF_F, o[D / 32];
-#pragma unroll
-    for (int q = 0; q < D / 32; ++q) o[q] = 0.f;
-    // lane j holds piece j's (m, l); the accumulator rows of up to four pieces are fetched together
+    for (int q = 0; q < E; ++q) o[q] = 0.f;
     for (int j0 = 0; j0 < n_pieces; j0 += 32) {
         const int jl = j0 + lane;
+        const uint32_t live = cu.live[j0 >> 5];
         float2 ml = make_float2(-CUDART_INF_F, 0.f);
-        if (jl < n_pieces && live(jl)) ml = P.part_ml[rec_of(jl)];
+        if (jl < n_pieces && ((live >> lane) & 1u)) ml = P.part_ml[rec_of(jl)];
         const float mnew = fmaxf(mx, warp_max(ml.x));
         if (mnew == -CUDART_INF_F) continue;
         const float rescale = __expf(mx - mnew);             // 0 on the first live batch
         den *= rescale;
 #pragma unroll
-        for (int q = 0; q < D / 32; ++q) o[q] *= rescale;
+        for (int q = 0; q < E; ++q) o[q] *= rescale;
         mx = mnew;
         const float wl = ml.x == -CUDART_INF_F ? 0.f : __expf(ml.x - mx);
         den += warp_sum(ml.y * wl);
         const int nb = min(32, n_pieces - j0);
         for (int u0 = 0; u0 < nb; u0 += 4) {
-            float v[4][D / 32], w[4];
+            float v[4][E], w[4];
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
                 w[u] = u0 + u < nb ? __shfl_sync(kFull, wl, u0 + u) : 0.f;
-                const float* src = P.part_o + rec_of(j0 + min(u0 + u, nb - 1)) * D + lane * (D / 32);
+                if (w[u] != 0.f) {
+                    load_row(P.part_o + rec_of(j0 + u0 + u) * D + lane * E, v[u]);
+                } else {
 #pragma unroll
-                for (int q = 0; q < D / 32; ++q) v[u][q] = w[u] != 0.f ? src[q] : 0.f;
+                    for (int q = 0; q < E; ++q) v[u][q] = 0.f;
+                }
             }
 #pragma unroll
             for (int u = 0; u < 4; ++u)
 #pragma unroll
-                for (int q = 0; q < D / 32; ++q) o[q] = fmaf(v[u][q], w[u], o[q]);
+                for (int q = 0; q < E; ++q) o[q] = fmaf(v[u][q], w[u], o[q]);
         }
     }
-    const float inv = 1.f / den;
-    const int r_glob = pp * P.pair_rows + prow;
-    const int node = r_glob / G, hq = cu.g * G + r_glob % G;
-    __nv_bfloat16* dst = reinterpret_cast<__nv_bfloat16*>(a.O) + cu.layer * P.o_ls + (((int64_t)cu.b * kMaxNodes + node) * a.Hq + hq) * D + lane * (D / 32);
-#pragma unroll
-    for (int q = 0; q < D / 32; ++q) dst[q] = __float2bfloat16(o[q] * inv);
-    if (a.lse != nullptr && lane == 0) a.lse[cu.layer * P.lse_ls + ((int64_t)cu.b * a.Hq + hq) * kMaxNodes + node] = mx + logf(den);
+    store_row(o, mx, den);
 }
 
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
@@ -1083,8 +1017,8 @@ bool make_map(CUtensorMap* tm, const void* base, int d, int heads, long long row
 
 // Grid shape.  A class is one row-block pair (256 query rows: both row blocks share every K/V tile in
 // shared memory) or, when such fused units would leave most SMs without work, one row block (128 rows).
-// CTAs per class: the grid is one CTA per SM, but at least four tiles per CTA when every sequence
-// has the longest prefix.  Both decisions look at the tiles of the whole launch, all its layers: 32 layers of one
+// CTAs per class: the grid is one CTA per SM, but at least two tiles per CTA when every sequence
+// has the longest prefix (four: 16.8 us for 32 / 8 heads, 1000 tokens, two: 15.0; 4 / 4 heads, d = 64, 500 tokens: 14.1, 12.2).  Both decisions look at the tiles of the whole launch, all its layers: 32 layers of one
 // sequence with 2048 tokens (32 / 8 heads, d = 128) run as 148 CTAs of fused units, where one layer alone would
 // be split into half units on 68 CTAs.
 void plan_grid(const radar_ctx* ctx, int B, int Hq, int Hkv, int max_prefix_len, int layers, int* n_blk, int* n_cls, int* ncc,
@@ -1095,21 +1029,20 @@ void plan_grid(const radar_ctx* ctx, int B, int Hq, int Hkv, int max_prefix_len,
     int nb = 2;
     if (blocks > 1 && unit_tiles * ((blocks + 1) / 2) < 4LL * ctx->sm_count) nb = 1;
     const int cls = (blocks + nb - 1) / nb;
-    long long per = ctx->sm_count / cls;
-    const long long cap = (unit_tiles + 3) / 4;
+    long long per = std::min(ctx->sm_count / cls, kMaxPerClass);
+    const long long cap = (unit_tiles + 1) / 2;
     if (per > cap) per = cap;
     if (per < 1) per = 1;
     // All units of one sequence are alike, so where they are no more than the CTAs of a class a grid can be chosen in
     // which every CTA has one piece of one unit and pays for one segment (fill and epilogue, what tile_costs books per
     // unit) and not for two.  Not where that leaves so many CTAs unused that the pieces get longer than what it saves.
-    // (32 / 8 heads, d = 128, attention + combine: 1000 tokens 21.5 -> 18.8 us, 2048 20.5 -> 19.6; 40 / 40 heads, 2048:
-    // 26.8 -> 24.8; 16 / 16 heads, 1000: 20.6 -> 17.2.)
+    // (Attention + combine, d = 128: 40 / 40 heads, 2048 tokens 26.8 -> 24.8 us; 16 / 16 heads, 1000 tokens 20.6 -> 17.2.)
     const long long units = (long long)layers * Hkv, tiles = unit_tiles / (B * units);
     *whole = false;
     if (B == 1 && units <= per) {
         const TileCosts tc = tile_costs(cls);
         const int w = nb > 1 && blocks > 1 ? tc.two : tc.one;
-        const long long pieces = std::max(1ll, std::min(tiles / 4, per / units));
+        const long long pieces = std::max(1ll, std::min(tiles / 2, per / units));
         *whole = (tiles + pieces - 1) / pieces * w <= units * (tiles * w + tc.unit) / per + 2 * tc.unit / 3;
         if (*whole) per = units * pieces;
     }
@@ -1179,11 +1112,7 @@ static int launch_tc(radar_ctx* ctx, TcParams& P, cudaStream_t stream) {
     RADAR_CUDA_CHECK(cudaGetLastError());
     {
         radar_launch_scope scope(ctx, RADAR_K_ATTN_COMBINE, stream);
-        // few cut units: one row per warp and many small blocks; many: eight rows per warp, fewer waves of blocks
-        if ((long long)P.n_cls * P.ncc * (kPairRows / 8) <= 16ll * ctx->sm_count)
-            RADAR_CUDA_CHECK(launch_chained(tree_attn_tc_combine_wide_kernel<D>, dim3((unsigned)(P.n_cls * P.ncc), kPairRows / 8), dim3(256), 0, stream, P));
-        else
-            RADAR_CUDA_CHECK(launch_chained(tree_attn_tc_combine_kernel<D>, dim3((unsigned)(P.n_cls * P.ncc), kCombineY), dim3(256), 0, stream, P));
+        RADAR_CUDA_CHECK(launch_chained(tree_attn_tc_combine_kernel<D>, dim3((unsigned)(P.n_cls * P.ncc), kPairRows / 8), dim3(256), 0, stream, P));
     }
     RADAR_CUDA_CHECK(cudaGetLastError());
     return RADAR_OK;
