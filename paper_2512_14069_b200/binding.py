@@ -1,6 +1,6 @@
-"""Thin ctypes binding of libradar_b200.so: same names as include/radar.h, argument
-marshalling only.  torch tensors are used for device memory and streams; every step of
-the path runs in the library's CUDA kernels.  There is no CPU fallback: if the library
+"""Thin binding of libradar_b200.so: same names as include/radar.h, argument marshalling only.  The four calls
+of a step fill their argument structs natively (csrc/marshal.cpp), the others through ctypes.  torch
+tensors are used for device memory and streams; every step of the path runs in the library's CUDA kernels.  There is no CPU fallback: if the library
 is missing or a call fails, an exception is raised.
 """
 from __future__ import annotations
@@ -189,6 +189,39 @@ def dtype_code(t: torch.Tensor) -> int:
     raise ValueError("unsupported dtype %s" % t.dtype)
 
 
+def _raw_stream(stream) -> int:
+    if stream is None:
+        return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+    return stream.cuda_stream
+
+
+class _Call:
+    """One entry point of the library whose argument struct is filled natively from a dictionary {field: value}.
+    `dtypes` gives the dtype a tensor must have for a pointer field (absent: any); `optional` the fields that may be
+    left out (0 / NULL then)."""
+
+    def __init__(self, name, struct, dtypes, optional):
+        self.name, self.struct, self.dtypes, self.optional = name, struct, dtypes, frozenset(optional)
+        self.address = self.fill = None
+
+    def _load(self):
+        from . import _marshal
+        kinds = {_c_int: 0, _c_i64: 1, _sz: 1, _c_f: 2, _vp: 3}
+        like = {dt: torch.empty(0, dtype=dt) for dt in set(self.dtypes.values())}
+        fields = [(f, getattr(self.struct, f).offset, kinds[t], like.get(self.dtypes.get(f)), f not in self.optional)
+                  for f, t in self.struct._fields_]
+        self.address = ctypes.cast(getattr(lib(), self.name), _vp).value
+        self.fill = _marshal.Filler(ctypes.sizeof(self.struct), fields)        # last: another thread may test it
+
+    def __call__(self, ctx, stream, kw):
+        if self.fill is None:
+            self._load()
+        handle = ctx.handle
+        status = self.fill(self.address, handle.value if handle else 0, _raw_stream(stream), kw)
+        if status != RADAR_OK:
+            raise RadarError(self.name, status)
+
+
 class Context:
     """radar_create / radar_destroy."""
 
@@ -248,56 +281,46 @@ def radar_accept_workspace_bytes(ctx: Context, B, V, mode) -> int:
     return int(lib().radar_accept_workspace_bytes(ctx.handle, B, V, mode))
 
 
-def radar_expand_step(ctx: Context, *, B, F, V, k, t, t_max, logits, logits_row_stride, logits_seq_stride,
-                      logits_offset_elems=0, parent_score, parent_pool_idx, active, force_calls=None, gate,
-                      h, c, pool_capacity, pool_tok, pool_parent, pool_depth, pool_draft_row, pool_score, pool_len,
-                      frontier_tok, frontier_score, frontier_pool_idx, frontier_src_row, topk_tok, topk_logp,
-                      gate_logits, cont, workspace, stream=None, policy=RADAR_POLICY_LSTM_SCORES, features=None,
-                      phase=RADAR_EXPAND_ALL):
+_f32, _i32, _u8, _i64 = torch.float32, torch.int32, torch.uint8, torch.int64
+_GATE = ("w_ih", "w_hh", "b_ih", "b_hh", "w1", "b1", "w2", "b2")
+_expand = _Call(
+    "radar_expand_step", ExpandArgs,
+    dict({n: _f32 for n in _GATE}, parent_score=_f32, parent_pool_idx=_i32, active=_u8, force_calls=_i32, h=_f32, c=_f32, pool_tok=_i32,
+         pool_parent=_i32, pool_depth=_i32, pool_draft_row=_i32, pool_score=_f32, pool_len=_i32, frontier_tok=_i32, frontier_score=_f32,
+         frontier_pool_idx=_i32, frontier_src_row=_i32, topk_tok=_i32, topk_logp=_f32, gate_logits=_f32, cont=_u8, features=_f32),
+    _GATE + ("force_calls", "policy", "feat_dim", "features", "phase"))
+
+
+def radar_expand_step(ctx: Context, *, logits, gate, workspace, logits_offset_elems=0, features=None, stream=None, **kw):
     """One draft call's expansion.  `logits` is a CUDA tensor; the rows of this call start
     `logits_offset_elems` elements into it.  `gate` is a dict of the weight tensors (all eight for the
     LSTM policies; w1, b1, w2, b2 for RADAR_POLICY_MLP_SCORES); `features` [B, feat_dim] float32 is the
-    input of RADAR_POLICY_LSTM_HIDDEN."""
-    f32, i32, u8 = torch.float32, torch.int32, torch.uint8
-    a = ExpandArgs()
-    a.B, a.F, a.V, a.k, a.t, a.t_max = B, F, V, k, t, t_max
-    a.logits = _ptr(logits) + logits_offset_elems * logits.element_size()
-    a.logits_dtype = dtype_code(logits)
-    a.logits_row_stride, a.logits_seq_stride = logits_row_stride, logits_seq_stride
-    a.parent_score, a.parent_pool_idx = _ptr(parent_score, f32), _ptr(parent_pool_idx, i32)
-    a.active, a.force_calls = _ptr(active, u8), _ptr(force_calls, i32)
-    for n in ("w_ih", "w_hh", "b_ih", "b_hh", "w1", "b1", "w2", "b2"):
-        setattr(a, n, _ptr(gate.get(n), f32))
-    a.policy, a.phase = policy, phase
+    input of RADAR_POLICY_LSTM_HIDDEN.  The other keyword arguments are the fields of radar_expand_args: B, F, V, k, t, t_max,
+    logits_row_stride, logits_seq_stride, parent_score, parent_pool_idx, active, h, c, pool_capacity, pool_tok, pool_parent,
+    pool_depth, pool_draft_row, pool_score, pool_len, frontier_tok, frontier_score, frontier_pool_idx, frontier_src_row,
+    topk_tok, topk_logp, gate_logits, cont, and, with defaults, force_calls (None), policy (RADAR_POLICY_LSTM_SCORES) and
+    phase (RADAR_EXPAND_ALL)."""
+    kw["logits"] = _ptr(logits) + logits_offset_elems * logits.element_size()
+    kw["logits_dtype"] = dtype_code(logits)
+    for n in _GATE:
+        kw[n] = gate.get(n)
     if features is not None:
-        a.features, a.feat_dim = _ptr(features, f32), features.shape[-1]
-    a.h, a.c = _ptr(h, f32), _ptr(c, f32)
-    a.pool_capacity = pool_capacity
-    a.pool_tok, a.pool_parent, a.pool_depth = _ptr(pool_tok, i32), _ptr(pool_parent, i32), _ptr(pool_depth, i32)
-    a.pool_draft_row, a.pool_score, a.pool_len = _ptr(pool_draft_row, i32), _ptr(pool_score, f32), _ptr(pool_len, i32)
-    a.frontier_tok, a.frontier_score = _ptr(frontier_tok, i32), _ptr(frontier_score, f32)
-    a.frontier_pool_idx, a.frontier_src_row = _ptr(frontier_pool_idx, i32), _ptr(frontier_src_row, i32)
-    a.topk_tok, a.topk_logp = _ptr(topk_tok, i32), _ptr(topk_logp, f32)
-    a.gate_logits, a.cont = _ptr(gate_logits, f32), _ptr(cont, u8)
-    a.workspace, a.workspace_bytes = _ptr(workspace), workspace.numel() * workspace.element_size()
-    _check("radar_expand_step", lib().radar_expand_step(ctx.handle, ctypes.byref(a), _stream(stream)))
+        kw["features"], kw["feat_dim"] = features, features.shape[-1]
+    kw["workspace"], kw["workspace_bytes"] = workspace, workspace.numel() * workspace.element_size()
+    _expand(ctx, stream, kw)
 
 
-def radar_rerank_build_tree(ctx: Context, *, B, N, t_max, pool_capacity, pool_tok, pool_parent, pool_depth,
-                            pool_draft_row, pool_score, pool_len, n_keep=None, root_tok, prefix_len, tree_tok,
-                            tree_parent, tree_depth, tree_pos, tree_pool_idx, tree_draft_row, tree_score, tree_mask,
-                            n_nodes, retrieve, n_leaves, stream=None):
-    f32, i32 = torch.float32, torch.int32
-    a = TreeArgs()
-    a.B, a.N, a.t_max, a.pool_capacity = B, N, t_max, pool_capacity
-    a.pool_tok, a.pool_parent, a.pool_depth = _ptr(pool_tok, i32), _ptr(pool_parent, i32), _ptr(pool_depth, i32)
-    a.pool_draft_row, a.pool_score, a.pool_len = _ptr(pool_draft_row, i32), _ptr(pool_score, f32), _ptr(pool_len, i32)
-    a.n_keep, a.root_tok, a.prefix_len = _ptr(n_keep, i32), _ptr(root_tok, i32), _ptr(prefix_len, i32)
-    a.tree_tok, a.tree_parent, a.tree_depth = _ptr(tree_tok, i32), _ptr(tree_parent, i32), _ptr(tree_depth, i32)
-    a.tree_pos, a.tree_pool_idx, a.tree_draft_row = _ptr(tree_pos, i32), _ptr(tree_pool_idx, i32), _ptr(tree_draft_row, i32)
-    a.tree_score, a.tree_mask = _ptr(tree_score, f32), _ptr(tree_mask, torch.int64)
-    a.n_nodes, a.retrieve, a.n_leaves = _ptr(n_nodes, i32), _ptr(retrieve, i32), _ptr(n_leaves, i32)
-    _check("radar_rerank_build_tree", lib().radar_rerank_build_tree(ctx.handle, ctypes.byref(a), _stream(stream)))
+_tree = _Call(
+    "radar_rerank_build_tree", TreeArgs,
+    dict({f: _i32 for f, t in TreeArgs._fields_ if t is _vp}, pool_score=_f32, tree_score=_f32, tree_mask=_i64), ("n_keep",))
+
+
+def radar_rerank_build_tree(ctx: Context, *, stream=None, **kw):
+    """Rerank and serialisation.  The keyword arguments are the fields of radar_tree_args: B, N, t_max, pool_capacity,
+    pool_tok, pool_parent, pool_depth, pool_draft_row, pool_score, pool_len, root_tok, prefix_len, tree_tok, tree_parent,
+    tree_depth, tree_pos, tree_pool_idx, tree_draft_row, tree_score, tree_mask, n_nodes, retrieve, n_leaves, and n_keep
+    (default None)."""
+    _tree(ctx, stream, kw)
 
 
 def _attn_args(*, B, Hq, Hkv, d, Q, Kc, Vc, kv_start, prefix_len, max_prefix_len, Kt, Vt, mask, n_nodes, O, workspace,
@@ -327,11 +350,29 @@ def _attn_args(*, B, Hq, Hkv, d, Q, Kc, Vc, kv_start, prefix_len, max_prefix_len
     return a
 
 
-def radar_tree_attention(ctx: Context, *, stream=None, **kw):
+_attention = _Call(
+    "radar_tree_attention", AttnArgs,
+    dict(kv_start=_i64, prefix_len=_i32, mask=_i64, n_nodes=_i32, lse=_f32, block_table=_i32),
+    ("scale", "lse", "block_table", "page_size", "max_pages", "n_layers", "q_layer_stride", "cache_layer_stride", "tree_kv_layer_stride",
+     "o_layer_stride", "lse_layer_stride"))
+
+
+def radar_tree_attention(ctx: Context, *, Hkv, d, Q, Kc, Vc, Kt, Vt, O, workspace, lse=None, block_table=None, page_size=0, n_layers=1,
+                         stream=None, **kw):
     """Arguments as in `_attn_args` (the fields of radar_attn_args as tensors).  `block_table` [B, max_pages] int32
     with `page_size` selects the paged prefix cache (kv_start may then be None)."""
-    a = _attn_args(**kw)
-    _check("radar_tree_attention", lib().radar_tree_attention(ctx.handle, ctypes.byref(a), _stream(stream)))
+    for t in (Kc, Vc, Kt, Vt, O):
+        if t is not None and t.dtype != Q.dtype:
+            raise ValueError("Q, K, V and O must share one dtype")
+    kw.update(Hkv=Hkv, d=d, dtype=dtype_code(Q), Q=Q, Kc=Kc, Vc=Vc, Kt=Kt, Vt=Vt, O=O, lse=lse, workspace=workspace,
+              workspace_bytes=workspace.numel() * workspace.element_size(),
+              cache_rows=0 if Kc is None else min(Kc.numel(), Vc.numel()) // (Hkv * d * max(n_layers, 1)))      # token rows per layer
+    if n_layers > 1:
+        kw.update(n_layers=n_layers, q_layer_stride=Q[0].numel(), o_layer_stride=O[0].numel(), tree_kv_layer_stride=Kt[0].numel(),
+                  cache_layer_stride=0 if Kc is None else Kc[0].numel(), lse_layer_stride=0 if lse is None else lse[0].numel())
+    if block_table is not None:
+        kw.update(block_table=block_table, page_size=page_size, max_pages=block_table.shape[-1])
+    _attention(ctx, stream, kw)
 
 
 def radar_tree_attention_path(**kw) -> int:
@@ -343,24 +384,23 @@ def radar_tree_attention_path(**kw) -> int:
     return int(L.radar_tree_attention_path(ctypes.byref(a)))
 
 
-def radar_verify_accept(ctx: Context, *, B, V, t_max, N, mode, target_logits, tree_tok, tree_parent, tree_draft_row,
-                        n_nodes, retrieve, n_leaves, accept_len, path_nodes, path_tokens, next_token,
-                        best_retrieve_row, workspace, temperature=1.0, draft_logits=None, R=0, u_accept=None,
-                        u_sample=None, stream=None):
-    i32, f32 = torch.int32, torch.float32
-    a = AcceptArgs()
-    a.B, a.V, a.t_max, a.N, a.mode, a.temperature = B, V, t_max, N, mode, temperature
-    a.target_logits, a.logits_dtype = _ptr(target_logits), dtype_code(target_logits)
+_accept = _Call(
+    "radar_verify_accept", AcceptArgs,
+    dict({f: _i32 for f in ("tree_tok", "tree_parent", "tree_draft_row", "n_nodes", "retrieve", "n_leaves", "accept_len", "path_nodes",
+                            "path_tokens", "next_token", "best_retrieve_row")}, u_accept=_f32, u_sample=_f32),
+    ("draft_logits", "R", "u_accept", "u_sample"))
+
+
+def radar_verify_accept(ctx: Context, *, target_logits, workspace, temperature=1.0, draft_logits=None, stream=None, **kw):
+    """Acceptance of the verified tree.  The other keyword arguments are the fields of radar_accept_args: B, V, t_max, N, mode,
+    tree_tok, tree_parent, tree_draft_row, n_nodes, retrieve, n_leaves, accept_len, path_nodes, path_tokens, next_token,
+    best_retrieve_row, and, for stochastic acceptance, R (default 0), u_accept and u_sample (default None)."""
     if draft_logits is not None and draft_logits.dtype != target_logits.dtype:
         raise ValueError("target and draft logits must share one dtype")
-    a.tree_tok, a.tree_parent, a.tree_draft_row = _ptr(tree_tok, i32), _ptr(tree_parent, i32), _ptr(tree_draft_row, i32)
-    a.n_nodes, a.retrieve, a.n_leaves = _ptr(n_nodes, i32), _ptr(retrieve, i32), _ptr(n_leaves, i32)
-    a.draft_logits, a.R = _ptr(draft_logits), R
-    a.u_accept, a.u_sample = _ptr(u_accept, f32), _ptr(u_sample, f32)
-    a.accept_len, a.path_nodes, a.path_tokens = _ptr(accept_len, i32), _ptr(path_nodes, i32), _ptr(path_tokens, i32)
-    a.next_token, a.best_retrieve_row = _ptr(next_token, i32), _ptr(best_retrieve_row, i32)
-    a.workspace, a.workspace_bytes = _ptr(workspace), workspace.numel() * workspace.element_size()
-    _check("radar_verify_accept", lib().radar_verify_accept(ctx.handle, ctypes.byref(a), _stream(stream)))
+    kw["target_logits"], kw["draft_logits"], kw["logits_dtype"] = target_logits, draft_logits, dtype_code(target_logits)
+    kw["temperature"] = temperature
+    kw["workspace"], kw["workspace_bytes"] = workspace, workspace.numel() * workspace.element_size()
+    _accept(ctx, stream, kw)
 
 
 def radar_acclen_workspace_bytes(ctx: Context, B, V) -> int:

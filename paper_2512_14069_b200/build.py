@@ -1,4 +1,5 @@
-"""Builds the CUDA library in-tree with nvcc for sm_100a (no JIT cache, no torch extension)."""
+"""Builds the CUDA library in-tree with nvcc for sm_100a (no JIT cache), and next to it the native argument marshaller
+of the binding, which is compiled against torch's headers."""
 from __future__ import annotations
 
 import os
@@ -13,6 +14,35 @@ FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-O3", "-lineinfo", "-std
          "-Xcompiler", "-fPIC", "--expt-relaxed-constexpr"]
 
 
+MARSHAL_SRC = os.path.join(CSRC, "marshal.cpp")
+MARSHAL = os.path.join(HERE, "_marshal.so")
+
+
+def _start_marshal(force: bool):
+    """Starts the compiler for the marshaller if it is out of date; (process, temporary file) or None."""
+    if not force and os.path.exists(MARSHAL) and os.path.getmtime(MARSHAL) >= os.path.getmtime(MARSHAL_SRC):
+        return None
+    import sysconfig
+    from importlib.util import find_spec
+    tdir = os.path.dirname(find_spec("torch").origin)
+    tmp = MARSHAL + ".%d.tmp" % os.getpid()
+    cmd = [os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-shared", "-fPIC", "-I" + os.path.join(tdir, "include"),
+           "-I" + os.path.join(tdir, "include", "torch", "csrc", "api", "include"), "-I" + sysconfig.get_paths()["include"], MARSHAL_SRC,
+           "-o", tmp, "-L" + os.path.join(tdir, "lib"), "-lc10", "-ltorch_cpu", "-ltorch", "-ltorch_python"]
+    return subprocess.Popen(cmd, stdout=subprocess.PIPE, stderr=subprocess.STDOUT, text=True), tmp
+
+
+def _finish_marshal(started):
+    if started is None:
+        return
+    proc, tmp = started
+    out, _ = proc.communicate()
+    if proc.returncode != 0:
+        sys.stderr.write(out)
+        raise RuntimeError("g++ failed on marshal.cpp")
+    os.replace(tmp, MARSHAL)
+
+
 def _deps():
     out = [os.path.join(CSRC, s) for s in SOURCES]
     out += [os.path.join(CSRC, f) for f in os.listdir(CSRC) if f.endswith((".cuh", ".h"))]
@@ -21,7 +51,15 @@ def _deps():
 
 
 def build(force: bool = False, verbose: bool = False) -> str:
-    """Compile every .cu into objects under _build/ and link libradar_b200.so next to this file."""
+    """Compile every .cu into objects under _build/ and link libradar_b200.so next to this file; build the marshaller."""
+    marshal = _start_marshal(force)
+    try:
+        return _build_library(force, verbose)
+    finally:
+        _finish_marshal(marshal)
+
+
+def _build_library(force: bool, verbose: bool) -> str:
     newest = max(os.path.getmtime(p) for p in _deps())
     if not force and os.path.exists(LIB) and os.path.getmtime(LIB) >= newest:
         return LIB

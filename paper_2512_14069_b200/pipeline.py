@@ -72,35 +72,47 @@ class SpecStep:
             setattr(self, n, t[off:off + t.numel() - 255])
 
     # ---- expansion -------------------------------------------------------------------
+    def _slots(self):
+        """The addresses of the per-call outputs as one tuple per draft call: (frontier_tok, frontier_score, frontier_pool_idx,
+        frontier_src_row, topk_tok, topk_logp, gate_logits, cont).  Worked out from the buffers each time a step is
+        issued (indexing 64 views out of them instead costs 75 us a step of host time)."""
+        f32, i32 = torch.float32, torch.int32
+        bufs = ((self.frontier_tok, i32), (self.frontier_score, f32), (self.frontier_pool_idx, i32), (self.frontier_src_row, i32),
+                (self.topk_tok, i32), (self.topk_logp, f32), (self.gate_logits, f32), (self.cont_hist, torch.uint8))
+        return list(zip(*(range(p, p + x.numel() * x.element_size(), x.stride(0) * x.element_size())
+                          for x, p in ((x, rb._ptr(x, dt)) for x, dt in bufs))))
+
     def expand(self, t, draft_logits, gate, force_calls=None, policy=rb.RADAR_POLICY_LSTM_SCORES, features=None,
-               phase=rb.RADAR_EXPAND_ALL, vocab_mask=None, workspace=None, stream=None):
+               phase=rb.RADAR_EXPAND_ALL, vocab_mask=None, workspace=None, stream=None, slots=None):
         """Draft call t (1-based) on draft_logits [B,R,V]: row 0 for t = 1, rows 1+(t-2)k.. for t >= 2.
         `features` [t_max-1, B, feat_dim] feeds the hidden-state policy (row t-1 at call t).  `phase`, `vocab_mask`
-        (the mask a RADAR_EXPAND_VOCAB call reads rows by), `workspace` and `stream` serve the pipelined form."""
+        (the mask a RADAR_EXPAND_VOCAB call reads rows by), `workspace` and `stream` serve the pipelined form;
+        `slots` is what `_slots()` returns, for callers that make several calls."""
         k, B, V = self.k, self.B, self.V
         F = 1 if t == 1 else k
         row0 = 0 if t == 1 else 1 + (t - 2) * k
         s = t - 1
+        slots = self._slots() if slots is None else slots
+        frontier_tok, frontier_score, frontier_pool_idx, frontier_src_row, topk_tok, topk_logp, gate_logits, cont = slots[s]
         rb.radar_expand_step(
             self.ctx, B=B, F=F, V=V, k=k, t=t, t_max=self.t_max, logits=draft_logits,
             logits_row_stride=V, logits_seq_stride=self.R * V, logits_offset_elems=row0 * V,
-            parent_score=self.root_score if t == 1 else self.frontier_score[s - 1],
-            parent_pool_idx=self.root_pool_idx if t == 1 else self.frontier_pool_idx[s - 1],
+            parent_score=self.root_score if t == 1 else slots[s - 1][1],
+            parent_pool_idx=self.root_pool_idx if t == 1 else slots[s - 1][2],
             active=vocab_mask if phase == rb.RADAR_EXPAND_VOCAB else self.active, force_calls=force_calls, gate=gate, h=self.h, c=self.c,
             pool_capacity=self.C, pool_tok=self.pool_tok, pool_parent=self.pool_parent, pool_depth=self.pool_depth,
             pool_draft_row=self.pool_draft_row, pool_score=self.pool_score, pool_len=self.pool_len,
-            frontier_tok=self.frontier_tok[s], frontier_score=self.frontier_score[s],
-            frontier_pool_idx=self.frontier_pool_idx[s], frontier_src_row=self.frontier_src_row[s],
-            topk_tok=self.topk_tok1 if t == 1 else self.topk_tok[s],
-            topk_logp=self.topk_logp1 if t == 1 else self.topk_logp[s],
-            gate_logits=self.gate_logits[s], cont=self.cont_hist[s], workspace=self.ws_expand if workspace is None else workspace,
+            frontier_tok=frontier_tok, frontier_score=frontier_score, frontier_pool_idx=frontier_pool_idx,
+            frontier_src_row=frontier_src_row, topk_tok=self.topk_tok1 if t == 1 else topk_tok,
+            topk_logp=self.topk_logp1 if t == 1 else topk_logp, gate_logits=gate_logits, cont=cont, workspace=self.ws_expand if workspace is None else workspace,
             policy=policy, features=None if features is None or t >= self.t_max else features[s], phase=phase, stream=stream)
 
     def run_expansion(self, draft_logits, gate, force_calls=None, policy=rb.RADAR_POLICY_LSTM_SCORES, features=None,
                       pipelined=True):
+        slots = self._slots()
         if not pipelined:
             for t in range(1, self.t_max + 1):      # call 1 restarts the state on the device
-                self.expand(t, draft_logits, gate, force_calls, policy, features)
+                self.expand(t, draft_logits, gate, force_calls, policy, features, slots=slots)
             return
         # Two chains.  The vocabulary pass of call t (side stream, workspace t % 2) needs the select + gate block
         # of call t - 2 done: that block wrote the mask the pass skips rows by (cont of call t - 2; nothing for
@@ -114,12 +126,12 @@ class SpecStep:
         for t in range(1, self.t_max + 1):
             if t - 2 in sel_done:
                 side.wait_event(sel_done[t - 2])
-            mask = self.cont_hist[t - 3] if t >= 3 else None
-            self.expand(t, *args, phase=rb.RADAR_EXPAND_VOCAB, vocab_mask=mask, workspace=ws[t % 2], stream=side)
+            mask = slots[t - 3][7] if t >= 3 else None
+            self.expand(t, *args, phase=rb.RADAR_EXPAND_VOCAB, vocab_mask=mask, workspace=ws[t % 2], stream=side, slots=slots)
             voc = torch.cuda.Event()
             voc.record(side)
             main.wait_event(voc)
-            self.expand(t, *args, phase=rb.RADAR_EXPAND_SELECT, workspace=ws[t % 2], stream=main)
+            self.expand(t, *args, phase=rb.RADAR_EXPAND_SELECT, workspace=ws[t % 2], stream=main, slots=slots)
             sel_done[t] = torch.cuda.Event()
             sel_done[t].record(main)
         main.wait_stream(side)                      # join (the last pass has been waited for already)

@@ -1,0 +1,53 @@
+"""The native argument marshaller: every field of every argument struct lands where ctypes puts it, and what does not fit
+is refused.  No GPU needed (the called function is a Python callback)."""
+import ctypes
+
+import pytest
+import torch
+
+from paper_2512_14069_b200 import binding as rb
+from paper_2512_14069_b200 import build as rbuild
+
+
+@pytest.fixture(scope="module", autouse=True)
+def built():
+    rbuild.build()
+
+
+def _filler(struct, optional=(), like=None):
+    from paper_2512_14069_b200 import _marshal
+    kinds = {ctypes.c_int: 0, ctypes.c_int64: 1, ctypes.c_size_t: 1, ctypes.c_float: 2, ctypes.c_void_p: 3}
+    return _marshal.Filler(ctypes.sizeof(struct), [(f, getattr(struct, f).offset, kinds[t], like, f not in optional) for f, t in struct._fields_])
+
+
+@pytest.mark.parametrize("struct", [rb.ExpandArgs, rb.TreeArgs, rb.AttnArgs, rb.AcceptArgs])
+def test_fields_land_where_ctypes_puts_them(struct):
+    seen = []
+
+    @ctypes.CFUNCTYPE(ctypes.c_int, ctypes.c_void_p, ctypes.c_void_p, ctypes.c_void_p)
+    def callee(ctx, args, stream):
+        seen.append((ctx, ctypes.string_at(args, ctypes.sizeof(struct)), stream))
+        return -3
+
+    values, want = {}, struct()
+    for i, (f, t) in enumerate(struct._fields_):
+        v = {ctypes.c_int: -7 - i, ctypes.c_float: 0.5 * i}.get(t, (1 << 40) + i)
+        values[f] = v
+        setattr(want, f, v)
+    assert _filler(struct)(ctypes.cast(callee, ctypes.c_void_p).value, 11, 13, values) == -3
+    assert seen == [(11, bytes(want), 13)]
+
+
+def test_what_does_not_fit_is_refused():
+    fill = _filler(rb.TreeArgs, optional=("n_keep",), like=torch.zeros(0))
+    good = {f: 1 for f, _ in rb.TreeArgs._fields_}
+    with pytest.raises(TypeError, match="unexpected keyword argument 'extra'"):
+        fill(1, 0, 0, dict(good, extra=1))
+    with pytest.raises(TypeError, match="missing required keyword argument 'root_tok'"):
+        fill(1, 0, 0, {f: v for f, v in good.items() if f not in ("root_tok", "n_keep")})
+    with pytest.raises(OverflowError):
+        fill(1, 0, 0, dict(good, B=1 << 31))
+    with pytest.raises(ValueError, match="contiguous CUDA tensor"):
+        fill(1, 0, 0, dict(good, pool_tok=torch.zeros(3)))
+    with pytest.raises(TypeError):
+        fill(1, 0, 0, dict(good, pool_tok="x"))
