@@ -33,6 +33,7 @@ enum radar_smem_slot {
     RADAR_SMEM_SELECT_GATE = 0,
     RADAR_SMEM_SELECT_GATE_CLUSTER,   // the instantiation with helper blocks
     RADAR_SMEM_TREE_BUILD,
+    RADAR_SMEM_TRAIN_ROLLOUT,   // the instantiation with four points a block
     RADAR_SMEM_WALK,            // + 2 * (bf16) + CTAs per SM - 1
     RADAR_SMEM_ACCLEN = RADAR_SMEM_WALK + 4,        // the same
     RADAR_SMEM_ATTN_FMA = RADAR_SMEM_ACCLEN + 4,        // + 2 * (bf16) + (d == 128)

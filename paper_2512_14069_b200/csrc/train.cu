@@ -1,8 +1,8 @@
 // One REINFORCE step of the prediction model (Sec. 4.2, Eq. 3-10; data points {S, D} of Sec. 4.3).
 //
 // Three kernels:
-//   train_rollout_kernel   one block per data point: rolls the LSTM + MLP out over the states with sampled
-//                          actions, draws the acceptance length from d_T, forms the returns, and runs
+//   train_rollout_kernel   one block per one, two or four data points: rolls the LSTM + MLP out over the states with
+//                          sampled actions, draws the acceptance length from d_T, forms the returns, and runs
 //                          backpropagation through time.  What the parameter gradients need - the deltas of
 //                          every layer and the activations they multiply - goes to a record per (data point,
 //                          decision) in the workspace.
@@ -19,6 +19,7 @@ namespace {
 constexpr int H = kHidden;            // 128
 constexpr int kTrainThreads = 4 * H;  // one thread per LSTM gate row
 constexpr int kMaxSteps = 16;
+constexpr int kGroups = kTrainThreads / 32;   // row groups of the rollout's transposed products
 constexpr int kXPad = 32;             // room for the k scores behind h in the head's input
 constexpr int kSlices = 8;            // the records are summed in this many slices, one block each per output tile
 
@@ -62,90 +63,173 @@ struct TrainParams {
 __device__ __forceinline__ float sigmoidf(float v) { return 1.f / (1.f + __expf(-v)); }
 __device__ __forceinline__ float softplusf(float v) { return v > 0.f ? v + log1pf(expf(-v)) : log1pf(expf(v)); }
 
+// Sums of N values over the warp's 32 lanes, N a power of two: lane l returns the sum of value l / (32 / N).  Halving the
+// values with every exchange costs N - 1 + log2(32 / N) shuffles; N butterflies would cost 5 N, and an SM passes one
+// warp's shuffle a clock.
+template <int N>
+__device__ __forceinline__ float transposed_sum(float (&v)[N]) {
+    const int lane = threadIdx.x & 31;
+    int o = 16;
+#pragma unroll
+    for (int m = N / 2; m > 0; m >>= 1, o >>= 1) {
+        const bool up = (lane & o) != 0;
+#pragma unroll
+        for (int i = 0; i < m; ++i) {
+            const float give = up ? v[i] : v[i + m], keep = up ? v[i + m] : v[i];
+            v[i] = keep + __shfl_xor_sync(kFull, give, o);
+        }
+    }
+    float t = v[0];
+    for (; o > 0; o >>= 1) t += __shfl_xor_sync(kFull, t, o);
+    return t;
+}
+
+// A block takes kP data points side by side.  What bounds it is the way of the weights from L2 into the SM (256 KB of W_hh
+// and 70 KB of W_1 for every decision, forwards and backwards, 64 B a clock) and the latency of that way: the points of
+// a block share every weight that is loaded, and a thread has eight or more loads of a product in flight.  With one point
+// a block, a row at a time and five shuffles a row, n = 148 took 134 us and n = 1024 332; now 65 and 139.
+template <int kP>
 __global__ void __launch_bounds__(kTrainThreads, 1) train_rollout_kernel(const TrainParams P) {
     chain_wait();
     const radar_train_args& a = P.a;
-    const int j = blockIdx.x, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int j0 = blockIdx.x * kP, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int k = a.k, t_max = a.t_max, n = a.n;
     const Theta W = carve_theta(a.theta, k);
-    __shared__ __align__(16) float sh[H], sc[H], sx[kXPad], sg[4 * H], shid[H], sd1[H], sdp[4 * H], sdh[H], sdc[H], spart[4][H];
-    __shared__ float sy[2], spi1[kMaxSteps], sG[kMaxSteps];
-    __shared__ int sact[kMaxSteps];
-    if (tid < H) { sh[tid] = 0.f; sc[tid] = 0.f; }
+    __shared__ __align__(16) float sh[kP][H], sc[kP][H], sx[kP][kXPad], sg[kP][4 * H], shid[kP][H], sd1[kP][H], sdp[kP][4 * H], sdh[kP][H], sdc[kP][H];
+    extern __shared__ __align__(16) float train_smem[];
+    float (*spart)[kGroups][H] = reinterpret_cast<float (*)[kGroups][H]>(train_smem);      // [kP]
+    __shared__ float sy[kP][2], spi1[kP][kMaxSteps], sG[kP][kMaxSteps];
+    __shared__ int sact[kP][kMaxSteps], sT[kP], sndec[kP], s_going[kP];
+    for (int e = tid; e < kP * H; e += kTrainThreads) { (&sh[0][0])[e] = 0.f; (&sc[0][0])[e] = 0.f; }
+    if (tid < kP) { s_going[tid] = j0 + tid < n; sT[tid] = t_max; sndec[tid] = 0; }
     __syncthreads();
-    float* rec0 = P.rec + (size_t)j * (t_max - 1) * R_STRIDE;
+    auto record = [&](int p, int s) { return P.rec + ((size_t)(j0 + p) * (t_max - 1) + s) * R_STRIDE; };
 
     // ---- rollout ----
-    int T = t_max, ndec = 0;
     for (int t = 1; t < t_max; ++t) {
-        float* rec = rec0 + (size_t)(t - 1) * R_STRIDE;
-        if (tid < kXPad) sx[tid] = tid < k ? __expf(a.log_states[((size_t)(t - 1) * n + j) * k + tid]) : 0.f;
-        if (tid < H) { rec[R_HPREV + tid] = sh[tid]; rec[R_CPREV + tid] = sc[tid]; }
-        __syncthreads();
-        // LSTM pre-activations: warp w owns rows 32 w .. 32 w + 31, the lanes share each row's dot products
-        float mine = 0.f;
-        for (int rr = 0; rr < 32; ++rr) {
-            const int row = warp * 32 + rr;
-            const float4 wv = *reinterpret_cast<const float4*>(W.w_hh + (size_t)row * H + 4 * lane);
-            const float4 hv = *reinterpret_cast<const float4*>(sh + 4 * lane);
-            float p = wv.x * hv.x + wv.y * hv.y + wv.z * hv.z + wv.w * hv.w;
-            if (lane < k) p += W.w_ih[(size_t)row * k + lane] * sx[lane];
-            p = warp_sum(p);
-            if (lane == rr) mine = p;
+        bool going[kP], any = false;                          // the same in every thread
+#pragma unroll
+        for (int p = 0; p < kP; ++p) { going[p] = s_going[p] != 0; any |= going[p]; }
+        if (!any) break;
+        for (int e = tid; e < kP * kXPad; e += kTrainThreads) {
+            const int p = e / kXPad, c = e % kXPad;
+            sx[p][c] = c < k && going[p] ? __expf(a.log_states[((size_t)(t - 1) * n + j0 + p) * k + c]) : 0.f;
         }
-        {
-            const float pre = mine + W.b_ih[tid] + W.b_hh[tid];
-            sg[tid] = (tid >= 2 * H && tid < 3 * H) ? tanhf(pre) : sigmoidf(pre);
-            rec[R_GATES + tid] = sg[tid];
-        }
-        __syncthreads();
-        if (tid < H) {
-            const float cn = sg[H + tid] * sc[tid] + sg[tid] * sg[2 * H + tid];
-            const float hn = sg[3 * H + tid] * tanhf(cn);
-            sc[tid] = cn;
-            sh[tid] = hn;
-            rec[R_C + tid] = cn;
-            rec[R_CAT + tid] = hn;
-        } else if (tid < H + kXPad) {
-            rec[R_CAT + tid] = sx[tid - H];
-        }
-        __syncthreads();
-        // head: warp w owns hidden rows 8 w .. 8 w + 7
-        for (int rr = 0; rr < 8; ++rr) {
-            const int row = warp * 8 + rr;
-            const float* wr = W.w1 + (size_t)row * (H + k);
-            float p = 0.f;
-            for (int c = lane; c < H + k; c += 32) p += wr[c] * (c < H ? sh[c] : sx[c - H]);
-            p = warp_sum(p);
-            if (lane == 0) {
-                const float hv = fmaxf(p + W.b1[row], 0.f);
-                shid[row] = hv;
-                rec[R_HID + row] = hv;
+        for (int e = tid; e < kP * H; e += kTrainThreads) {
+            const int p = e / H, c = e % H;
+            if (going[p]) {
+                float* rec = record(p, t - 1);
+                rec[R_HPREV + c] = sh[p][c];
+                rec[R_CPREV + c] = sc[p][c];
             }
         }
         __syncthreads();
-        if (warp < 2) {
-            float p = 0.f;
-            for (int c = lane; c < H; c += 32) p += W.w2[warp * H + c] * shid[c];
-            p = warp_sum(p);
-            if (lane == 0) sy[warp] = p + W.b2[warp];
+        // LSTM pre-activations: warp w owns rows 32 w .. 32 w + 31 in two batches of 16, the lanes share each row's dot
+        // product; even lanes end up with a row of the first batch, odd lanes with one of the second
+        float mine[kP];
+#pragma unroll
+        for (int half = 0; half < 2; ++half) {
+            const int r0 = warp * 32 + half * 16;
+            float4 w[16];
+            float wx[16];
+#pragma unroll
+            for (int i = 0; i < 16; ++i) w[i] = *reinterpret_cast<const float4*>(W.w_hh + (size_t)(r0 + i) * H + 4 * lane);
+#pragma unroll
+            for (int i = 0; i < 16; ++i) wx[i] = lane < k ? W.w_ih[(size_t)(r0 + i) * k + lane] : 0.f;
+#pragma unroll
+            for (int p = 0; p < kP; ++p) {
+                const float4 h4 = *reinterpret_cast<const float4*>(&sh[p][4 * lane]);
+                const float x = sx[p][lane];
+                float v[16];
+#pragma unroll
+                for (int i = 0; i < 16; ++i) v[i] = fmaf(wx[i], x, w[i].x * h4.x + w[i].y * h4.y + w[i].z * h4.z + w[i].w * h4.w);
+                const float sum = transposed_sum<16>(v);
+                if ((lane & 1) == half) mine[p] = sum;
+            }
+        }
+        {
+            const int row = warp * 32 + (lane & 1) * 16 + (lane >> 1);
+            const float b = W.b_ih[row] + W.b_hh[row];
+#pragma unroll
+            for (int p = 0; p < kP; ++p) {
+                const float pre = mine[p] + b;
+                const float g = (row >= 2 * H && row < 3 * H) ? tanhf(pre) : sigmoidf(pre);
+                sg[p][row] = g;
+                if (going[p]) record(p, t - 1)[R_GATES + row] = g;
+            }
         }
         __syncthreads();
-        const float d = sy[1] - sy[0];
-        const float pi1 = 1.f / (1.f + expf(-d));
-        const int act = a.u_action[(size_t)j * t_max + (t - 1)] < pi1 ? 1 : 0;
-        if (tid == 0) {
-            spi1[t - 1] = pi1;
-            sact[t - 1] = act;
-            sG[t - 1] = act ? -softplusf(-d) : -softplusf(d);       // log pi(a_t) for now
+        for (int e = tid; e < kP * (H + kXPad); e += kTrainThreads) {
+            const int p = e / (H + kXPad), c = e % (H + kXPad);
+            if (!going[p]) continue;
+            float* rec = record(p, t - 1);
+            if (c < H) {
+                const float cn = sg[p][H + c] * sc[p][c] + sg[p][c] * sg[p][2 * H + c];
+                const float hn = sg[p][3 * H + c] * tanhf(cn);
+                sc[p][c] = cn;
+                sh[p][c] = hn;
+                rec[R_C + c] = cn;
+                rec[R_CAT + c] = hn;
+            } else {
+                rec[R_CAT + c] = sx[p][c - H];
+            }
         }
-        ndec = t;
-        if (!act) { T = t; break; }                                   // the same in every thread
+        __syncthreads();
+        // head: warp w owns hidden rows 8 w .. 8 w + 7
+        {
+            float w[8][4], wx[8];
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                const float* wr = W.w1 + (size_t)(warp * 8 + i) * (H + k);
+#pragma unroll
+                for (int c = 0; c < 4; ++c) w[i][c] = wr[lane + 32 * c];
+                wx[i] = lane < k ? wr[H + lane] : 0.f;
+            }
+            const int row = warp * 8 + (lane >> 2);
+            const float b1 = W.b1[row];
+#pragma unroll
+            for (int p = 0; p < kP; ++p) {
+                float v[8];
+#pragma unroll
+                for (int i = 0; i < 8; ++i) {
+                    v[i] = wx[i] * sx[p][lane];
+#pragma unroll
+                    for (int c = 0; c < 4; ++c) v[i] = fmaf(w[i][c], sh[p][lane + 32 * c], v[i]);
+                }
+                const float hv = fmaxf(transposed_sum<8>(v) + b1, 0.f);
+                if ((lane & 3) == 0) {
+                    shid[p][row] = hv;
+                    if (going[p]) record(p, t - 1)[R_HID + row] = hv;
+                }
+            }
+        }
+        __syncthreads();
+        if (warp < 2 * kP) {
+            const int p = warp >> 1, o = warp & 1;
+            float v = 0.f;
+            for (int c = lane; c < H; c += 32) v += W.w2[o * H + c] * shid[p][c];
+            v = warp_sum(v);
+            if (lane == 0) sy[p][o] = v + W.b2[o];
+        }
+        __syncthreads();
+        if (tid < kP && going[tid]) {
+            const int p = tid;
+            const float d = sy[p][1] - sy[p][0];
+            const float pi1 = 1.f / (1.f + expf(-d));
+            const int act = a.u_action[(size_t)(j0 + p) * t_max + (t - 1)] < pi1 ? 1 : 0;
+            spi1[p][t - 1] = pi1;
+            sact[p][t - 1] = act;
+            sG[p][t - 1] = act ? -softplusf(-d) : -softplusf(d);       // log pi(a_t) for now
+            sndec[p] = t;
+            if (!act) { sT[p] = t; s_going[p] = 0; }
+        }
+        __syncthreads();
     }
     __syncthreads();
 
-    // ---- acceptance length, reward, returns, loss (one thread, fp64) ----
-    if (tid == 0) {
+    // ---- acceptance length, reward, returns, loss (one thread per point, fp64) ----
+    if (tid < kP && j0 + tid < n) {
+        const int p = tid, j = j0 + p, T = sT[p], ndec = sndec[p];
         const double* drow = a.dists + ((size_t)(T - 1) * n + j) * (t_max + 1);
         double total = 0.0;
         for (int i = 0; i <= t_max; ++i) total += drow[i];
@@ -165,59 +249,98 @@ __global__ void __launch_bounds__(kTrainThreads, 1) train_rollout_kernel(const T
         for (int t = T; t >= 1; --t) {
             if (t < T) g = -(double)a.alpha + (double)a.gamma * g;
             if (t <= ndec) {
-                loss -= g * (double)sG[t - 1];
-                sG[t - 1] = (float)g;
+                loss -= g * (double)sG[p][t - 1];
+                sG[p][t - 1] = (float)g;
             }
         }
         P.point_loss[j] = (float)loss;
         P.ndec[j] = ndec;
         a.calls[j] = T;
         a.l_acc[j] = len;
-        for (int t = 1; t <= t_max; ++t) a.actions[(size_t)j * t_max + (t - 1)] = t <= ndec ? (uint8_t)sact[t - 1] : (uint8_t)255;
+        for (int t = 1; t <= t_max; ++t) a.actions[(size_t)j * t_max + (t - 1)] = t <= ndec ? (uint8_t)sact[p][t - 1] : (uint8_t)255;
     }
-    if (tid < H) { sdh[tid] = 0.f; sdc[tid] = 0.f; }
+    for (int e = tid; e < kP * H; e += kTrainThreads) { (&sdh[0][0])[e] = 0.f; (&sdc[0][0])[e] = 0.f; }
     __syncthreads();
+    int steps = 0;
+#pragma unroll
+    for (int p = 0; p < kP; ++p) steps = max(steps, sndec[p]);
 
-    // ---- backpropagation through time ----
+    // ---- backpropagation through time (a point joins at its own last decision) ----
     const int q = tid >> 7, col = tid & (H - 1);
-    for (int s = ndec - 1; s >= 0; --s) {
-        float* rec = rec0 + (size_t)s * R_STRIDE;
-        const float G = sG[s], pi1 = spi1[s];
-        const int act = sact[s];
-        const float dy0 = -G * ((act == 0 ? 1.f : 0.f) - (1.f - pi1));
-        const float dy1 = -G * ((act == 1 ? 1.f : 0.f) - pi1);
-        if (tid == 0) { rec[R_DY] = dy0; rec[R_DY + 1] = dy1; }
-        if (tid < H) {
-            const float v = rec[R_HID + tid] > 0.f ? W.w2[tid] * dy0 + W.w2[H + tid] * dy1 : 0.f;
-            sd1[tid] = v;
-            rec[R_DPRE1 + tid] = v;
+    for (int s = steps - 1; s >= 0; --s) {
+        for (int e = tid; e < kP * H; e += kTrainThreads) {
+            const int p = e / H, c = e % H;
+            float v = 0.f;
+            if (s < sndec[p]) {
+                float* rec = record(p, s);
+                const float G = sG[p][s], pi1 = spi1[p][s];
+                const int act = sact[p][s];
+                const float dy0 = -G * ((act == 0 ? 1.f : 0.f) - (1.f - pi1));
+                const float dy1 = -G * ((act == 1 ? 1.f : 0.f) - pi1);
+                if (c == 0) { rec[R_DY] = dy0; rec[R_DY + 1] = dy1; }
+                v = rec[R_HID + c] > 0.f ? W.w2[c] * dy0 + W.w2[H + c] * dy1 : 0.f;
+                rec[R_DPRE1 + c] = v;
+            }
+            sd1[p][c] = v;
         }
         __syncthreads();
         {   // dh = W1[:, :H]^T dpre1 + dh from the next step: thread (q, col) sums 32 rows
-            float p = 0.f;
-            for (int r = q * 32; r < q * 32 + 32; ++r) p += W.w1[(size_t)r * (H + k) + col] * sd1[r];
-            spart[q][col] = p;
+            float acc[kP];
+#pragma unroll
+            for (int p = 0; p < kP; ++p) acc[p] = 0.f;
+#pragma unroll 16
+            for (int r = q * 32; r < q * 32 + 32; ++r) {
+                const float w = W.w1[(size_t)r * (H + k) + col];
+#pragma unroll
+                for (int p = 0; p < kP; ++p) acc[p] += w * sd1[p][r];
+            }
+#pragma unroll
+            for (int p = 0; p < kP; ++p) spart[p][q][col] = acc[p];
         }
         __syncthreads();
-        if (tid < H) {
-            const float dh = spart[0][tid] + spart[1][tid] + spart[2][tid] + spart[3][tid] + sdh[tid];
-            const float gi = rec[R_GATES + tid], gf = rec[R_GATES + H + tid], gg = rec[R_GATES + 2 * H + tid], go = rec[R_GATES + 3 * H + tid];
-            const float tc = tanhf(rec[R_C + tid]);
-            const float dc = dh * go * (1.f - tc * tc) + sdc[tid];
-            const float di = dc * gg * gi * (1.f - gi), df = dc * rec[R_CPREV + tid] * gf * (1.f - gf);
-            const float dg = dc * gi * (1.f - gg * gg), dob = dh * tc * go * (1.f - go);
-            sdp[tid] = di; sdp[H + tid] = df; sdp[2 * H + tid] = dg; sdp[3 * H + tid] = dob;
-            rec[R_DPRE + tid] = di; rec[R_DPRE + H + tid] = df; rec[R_DPRE + 2 * H + tid] = dg; rec[R_DPRE + 3 * H + tid] = dob;
-            sdc[tid] = dc * gf;
+        for (int e = tid; e < kP * H; e += kTrainThreads) {
+            const int p = e / H, c = e % H;
+            float di = 0.f, df = 0.f, dg = 0.f, dob = 0.f;
+            if (s < sndec[p]) {
+                float* rec = record(p, s);
+                const float dh = spart[p][0][c] + spart[p][1][c] + spart[p][2][c] + spart[p][3][c] + sdh[p][c];
+                const float gi = rec[R_GATES + c], gf = rec[R_GATES + H + c], gg = rec[R_GATES + 2 * H + c], go = rec[R_GATES + 3 * H + c];
+                const float tc = tanhf(rec[R_C + c]);
+                const float dc = dh * go * (1.f - tc * tc) + sdc[p][c];
+                di = dc * gg * gi * (1.f - gi); df = dc * rec[R_CPREV + c] * gf * (1.f - gf);
+                dg = dc * gi * (1.f - gg * gg); dob = dh * tc * go * (1.f - go);
+                rec[R_DPRE + c] = di; rec[R_DPRE + H + c] = df; rec[R_DPRE + 2 * H + c] = dg; rec[R_DPRE + 3 * H + c] = dob;
+                sdc[p][c] = dc * gf;
+            }
+            sdp[p][c] = di; sdp[p][H + c] = df; sdp[p][2 * H + c] = dg; sdp[p][3 * H + c] = dob;
+        }
+        if (s == 0) break;                                    // the state before the first call is a constant
+        __syncthreads();
+        {   // dh for the step before: W_hh^T dpre; thread (warp, lane) sums 32 rows of four columns
+            float4 acc[kP];
+#pragma unroll
+            for (int p = 0; p < kP; ++p) acc[p] = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 16
+            for (int i = 0; i < 32; ++i) {
+                const int r = warp * 32 + i;
+                const float4 w = *reinterpret_cast<const float4*>(W.w_hh + (size_t)r * H + 4 * lane);
+#pragma unroll
+                for (int p = 0; p < kP; ++p) {
+                    const float d = sdp[p][r];
+                    acc[p].x += w.x * d; acc[p].y += w.y * d; acc[p].z += w.z * d; acc[p].w += w.w * d;
+                }
+            }
+#pragma unroll
+            for (int p = 0; p < kP; ++p) *reinterpret_cast<float4*>(&spart[p][warp][4 * lane]) = acc[p];
         }
         __syncthreads();
-        {   // dh for the step before: W_hh^T dpre, thread (q, col) sums 128 rows
-            float p = 0.f;
-            for (int r = q * H; r < q * H + H; ++r) p += W.w_hh[(size_t)r * H + col] * sdp[r];
-            spart[q][col] = p;
+        for (int e = tid; e < kP * H; e += kTrainThreads) {
+            const int p = e / H, c = e % H;
+            float v = 0.f;
+#pragma unroll
+            for (int g = 0; g < kGroups; ++g) v += spart[p][g][c];
+            sdh[p][c] = v;                                    // (zero for a point that has not joined: its sdp was)
         }
-        __syncthreads();
-        if (tid < H) sdh[tid] = spart[0][tid] + spart[1][tid] + spart[2][tid] + spart[3][tid];
         __syncthreads();
     }
 }
@@ -228,8 +351,10 @@ struct OuterJob {
     int ld_out;                 // row stride of the output (N for matrices, 1 for vectors)
     long long out_off, out_off2;   // offsets into grad (out_off2 >= 0: a second copy, for the two LSTM biases)
 };
+constexpr int kJobs = 7;
 struct OuterParams {
-    OuterJob job[8];
+    OuterJob job[kJobs];
+    int first[kJobs + 1];       // first output tile of each job (and their number)
     const float* rec;
     const int* ndec;
     float* part;                // [kSlices][count]
@@ -237,42 +362,69 @@ struct OuterParams {
     int n, steps;               // records per data point = t_max - 1
 };
 
+// Block (tile, slice): a 32 x 32 tile of one output, summed over the records of the slice's data points.  Only decisions that
+// were taken have a record, on average two of a point's t_max - 1: the block lists them first, 256 points at a time, and
+// goes through the list in batches of 32 (in the order of the points, so the sum does not depend on scheduling).  Visiting
+// every possible record cost 60 us at 256 points and 205 at 1024; the list 23 and 57.
 __global__ void __launch_bounds__(256) train_outer_kernel(const OuterParams P) {
     chain_wait();
-    const OuterJob J = P.job[blockIdx.z % 7];
-    const int slice = blockIdx.z / 7;
-    const int m0 = blockIdx.y * 32, c0 = blockIdx.x * 32;
-    if (m0 >= J.M || c0 >= J.N) return;
+    int job = 0;
+    while ((int)blockIdx.x >= P.first[job + 1]) ++job;
+    const OuterJob J = P.job[job];
+    const int tile = blockIdx.x - P.first[job], tiles_x = (J.N + 31) / 32;
+    const int m0 = tile / tiles_x * 32, c0 = tile % tiles_x * 32;
     __shared__ float As[32][33], Bs[32][33];
+    __shared__ int s_rec[256 * (kMaxSteps - 1)], s_sum[8];
     const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;     // 32 x 8
     float acc[4] = {0.f, 0.f, 0.f, 0.f};
-    const int K = P.n * P.steps;
-    const int per = ((K + kSlices - 1) / kSlices + 31) / 32 * 32;
-    const int r_end = min(K, (slice + 1) * per);
-    for (int r0 = slice * per; r0 < r_end; r0 += 32) {
-        // stage 32 records x 32 columns of each operand (invalid records and columns past the edge: zero)
-        for (int e = ty; e < 32; e += 8) {
-            const int r = r0 + e;
-            const bool live = r < r_end && (r % P.steps) < P.ndec[r / P.steps];
-            const float* rec = P.rec + (size_t)r * R_STRIDE;
-            As[e][tx] = live && m0 + tx < J.M ? rec[J.a_off + m0 + tx] : 0.f;
-            Bs[e][tx] = live && c0 + tx < J.N ? (J.b_off < 0 ? 1.f : rec[J.b_off + c0 + tx]) : 0.f;
-        }
-        __syncthreads();
-#pragma unroll 8
-        for (int e = 0; e < 32; ++e) {
-            const float b = Bs[e][tx];
+    const int p_end = (int)((long long)P.n * (blockIdx.y + 1) / kSlices);
+    for (int p0 = (int)((long long)P.n * blockIdx.y / kSlices); p0 < p_end; p0 += 256) {
+        // list of the records of points p0 .. p0 + 255
+        const int pt = p0 + threadIdx.x;
+        const int mine = pt < p_end ? P.ndec[pt] : 0;
+        int incl = mine;
 #pragma unroll
-            for (int i = 0; i < 4; ++i) acc[i] += As[e][ty + 8 * i] * b;
+        for (int o = 1; o < 32; o <<= 1) {
+            const int v = __shfl_up_sync(kFull, incl, o);
+            if (tx >= o) incl += v;
         }
+        __syncthreads();                                        // the previous list has been read
+        if (tx == 31) s_sum[ty] = incl;
         __syncthreads();
+        int at = incl - mine, total = 0;
+#pragma unroll
+        for (int w = 0; w < 8; ++w) {
+            if (w < ty) at += s_sum[w];
+            total += s_sum[w];
+        }
+        for (int s = 0; s < mine; ++s) s_rec[at + s] = pt * P.steps + s;
+        __syncthreads();
+        for (int r0 = 0; r0 < total; r0 += 32) {
+            // stage 32 records x 32 columns of each operand (past the list and past the edge: zero)
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const int e = ty + 8 * i;
+                const bool live = r0 + e < total;
+                const float* rec = P.rec + (size_t)(live ? s_rec[r0 + e] : 0) * R_STRIDE;
+                As[e][tx] = live && m0 + tx < J.M ? rec[J.a_off + m0 + tx] : 0.f;
+                Bs[e][tx] = live && c0 + tx < J.N ? (J.b_off < 0 ? 1.f : rec[J.b_off + c0 + tx]) : 0.f;
+            }
+            __syncthreads();
+#pragma unroll 8
+            for (int e = 0; e < 32; ++e) {
+                const float b = Bs[e][tx];
+#pragma unroll
+                for (int i = 0; i < 4; ++i) acc[i] += As[e][ty + 8 * i] * b;
+            }
+            __syncthreads();
+        }
     }
     if (c0 + tx < J.N) {
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
             const int m = m0 + ty + 8 * i;
             if (m < J.M) {
-                float* out = P.part + (long long)slice * P.count;
+                float* out = P.part + (long long)blockIdx.y * P.count;
                 out[J.out_off + (long long)m * J.ld_out + c0 + tx] = acc[i];
                 if (J.out_off2 >= 0) out[J.out_off2 + (long long)m * J.ld_out + c0 + tx] = acc[i];
             }
@@ -349,7 +501,21 @@ extern "C" int radar_policy_train_step(radar_ctx* ctx, const radar_train_args* a
     const int k = a->k;
     {
         radar_launch_scope scope(ctx, RADAR_K_TRAIN_ROLLOUT, stream);
-        RADAR_CUDA_CHECK(launch_chained(train_rollout_kernel, dim3((unsigned)a->n), dim3(kTrainThreads), 0, stream, P));
+        // Points per block: one wave of blocks, four points at most.  A block lasts as long as its longest trajectory, so
+        // where trajectories of 1 to 8 calls are mixed (an untrained gate) blocks of one point in several waves do as well
+        // (rollout alone, 1 / 2 / 4 points a block: n = 148 65 / 73 / 96 us, 290 77 / 75 / 95, 420 84 / 83 / 97, 592
+        // 112 / 104 / 99, 4000 484 / 410 / 373); where a trained gate makes them alike the wave decides (n = 256, whole
+        // step: 38 us with one point, 31 with two).
+        const int kp = n <= sms ? 1 : n <= 2 * sms ? 2 : 4;
+        const size_t smem = (size_t)kp * kGroups * H * sizeof(float);
+        if (kp == 1) {
+            RADAR_CUDA_CHECK(launch_chained(train_rollout_kernel<1>, dim3(n), dim3(kTrainThreads), smem, stream, P));
+        } else if (kp == 2) {
+            RADAR_CUDA_CHECK(launch_chained(train_rollout_kernel<2>, dim3((n + 1) / 2), dim3(kTrainThreads), smem, stream, P));
+        } else {                                              // 30 KB static and 32 KB dynamic
+            RADAR_CUDA_CHECK(radar_opt_in_smem(ctx, RADAR_SMEM_TRAIN_ROLLOUT, train_rollout_kernel<4>, 64 * 1024));
+            RADAR_CUDA_CHECK(launch_chained(train_rollout_kernel<4>, dim3((n + 3) / 4), dim3(kTrainThreads), smem, stream, P));
+        }
     }
     {
         // offsets of the tensors inside theta / grad
@@ -364,9 +530,10 @@ extern "C" int radar_policy_train_step(radar_ctx* ctx, const radar_train_args* a
         O.job[4] = {R_DPRE1, H, -1, 1, 1, o_b1, -1};
         O.job[5] = {R_DY, 2, R_HID, H, H, o_w2, -1};                        // w2: dy (x) relu output
         O.job[6] = {R_DY, 2, -1, 1, 1, o_b2, -1};
+        O.first[0] = 0;
+        for (int x = 0; x < kJobs; ++x) O.first[x + 1] = O.first[x] + (O.job[x].M + 31) / 32 * ((O.job[x].N + 31) / 32);
         radar_launch_scope scope(ctx, RADAR_K_TRAIN_OUTER, stream);
-        RADAR_CUDA_CHECK(launch_chained(train_outer_kernel, dim3((unsigned)((H + k + 31) / 32), (unsigned)(4 * H / 32), 7 * kSlices), dim3(256), 0,
-                                        stream, O));
+        RADAR_CUDA_CHECK(launch_chained(train_outer_kernel, dim3((unsigned)O.first[kJobs], kSlices), dim3(256), 0, stream, O));
     }
     {
         const size_t count = param_count(k);
