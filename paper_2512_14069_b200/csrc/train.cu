@@ -501,6 +501,7 @@ extern "C" int radar_policy_train_step(radar_ctx* ctx, const radar_train_args* a
     const int k = a->k;
     {
         radar_launch_scope scope(ctx, RADAR_K_TRAIN_ROLLOUT, stream);
+        const unsigned n = (unsigned)a->n, sms = (unsigned)ctx->sm_count;
         // Points per block: one wave of blocks, four points at most.  A block lasts as long as its longest trajectory, so
         // where trajectories of 1 to 8 calls are mixed (an untrained gate) blocks of one point in several waves do as well
         // (rollout alone, 1 / 2 / 4 points a block: n = 148 65 / 73 / 96 us, 290 77 / 75 / 95, 420 84 / 83 / 97, 592
