@@ -43,6 +43,10 @@ class ExpandArgs(ctypes.Structure):
     ]
 
 
+class ExpandCallsArgs(ctypes.Structure):
+    _fields_ = [("call", ExpandArgs), ("topk_tok_next", _vp), ("topk_logp_next", _vp)]
+
+
 class TreeArgs(ctypes.Structure):
     _fields_ = [
         ("B", _c_int), ("N", _c_int), ("t_max", _c_int), ("pool_capacity", _c_int),
@@ -121,6 +125,10 @@ def lib() -> ctypes.CDLL:
         L.radar_read_device_status.argtypes = [_vp, _vp]
         L.radar_expand_workspace_bytes.restype = _sz
         L.radar_expand_workspace_bytes.argtypes = [_vp, _c_int, _c_int, _c_int, _c_int]
+        L.radar_expand_calls_workspace_bytes.restype = _sz
+        L.radar_expand_calls_workspace_bytes.argtypes = [_vp, _c_int, _c_int, _c_int, _c_int]
+        L.radar_expand_calls.restype = _c_int
+        L.radar_expand_calls.argtypes = [_vp, ctypes.POINTER(ExpandCallsArgs), _vp]
         L.radar_expand_step.restype = _c_int
         L.radar_expand_step.argtypes = [_vp, ctypes.POINTER(ExpandArgs), _vp]
         L.radar_rerank_build_tree.restype = _c_int
@@ -208,8 +216,15 @@ class _Call:
         from . import _marshal
         kinds = {_c_int: 0, _c_i64: 1, _sz: 1, _c_f: 2, _vp: 3}
         like = {dt: torch.empty(0, dtype=dt) for dt in set(self.dtypes.values())}
-        fields = [(f, getattr(self.struct, f).offset, kinds[t], like.get(self.dtypes.get(f)), f not in self.optional)
-                  for f, t in self.struct._fields_]
+
+        def flat(struct, base):                      # a nested struct's fields count as the outer one's
+            for f, t in struct._fields_:
+                at = base + getattr(struct, f).offset
+                if issubclass(t, ctypes.Structure):
+                    yield from flat(t, at)
+                else:
+                    yield f, at, kinds[t]
+        fields = [(f, at, kind, like.get(self.dtypes.get(f)), f not in self.optional) for f, at, kind in flat(self.struct, 0)]
         self.address = ctypes.cast(getattr(lib(), self.name), _vp).value
         self.fill = _marshal.Filler(ctypes.sizeof(self.struct), fields)        # last: another thread may test it
 
@@ -308,6 +323,26 @@ def radar_expand_step(ctx: Context, *, logits, gate, workspace, logits_offset_el
         kw["features"], kw["feat_dim"] = features, features.shape[-1]
     kw["workspace"], kw["workspace_bytes"] = workspace, workspace.numel() * workspace.element_size()
     _expand(ctx, stream, kw)
+
+
+_expand_calls = _Call(
+    "radar_expand_calls", ExpandCallsArgs, dict(_expand.dtypes, topk_tok_next=_i32, topk_logp_next=_f32),
+    tuple(_expand.optional) + ("topk_tok_next", "topk_logp_next"))
+
+
+def radar_expand_calls_workspace_bytes(ctx: Context, B, V, k, t_max) -> int:
+    return int(lib().radar_expand_calls_workspace_bytes(ctx.handle, B, V, k, t_max))
+
+
+def radar_expand_calls(ctx: Context, *, logits, gate, workspace, stream=None, **kw):
+    """All draft calls of a step on `logits` [B, 1+(t_max-1)k, V].  The other keyword arguments are the fields of
+    radar_expand_args for call 1 (F and t are set here), with the per-call outputs as [t_max, ...] buffers, and
+    topk_tok_next, topk_logp_next [t_max-1, B, k, k] (None where t_max is 1)."""
+    kw.update(logits=logits, logits_dtype=dtype_code(logits), F=1, t=1, workspace=workspace,
+              workspace_bytes=workspace.numel() * workspace.element_size())
+    for n in _GATE:
+        kw[n] = gate.get(n)
+    _expand_calls(ctx, stream, kw)
 
 
 _tree = _Call(

@@ -100,6 +100,8 @@ extern "C" const char* radar_kernel_name(int id) {
         case RADAR_K_TRAIN_ROLLOUT: return "train_rollout";
         case RADAR_K_TRAIN_OUTER: return "train_outer";
         case RADAR_K_TRAIN_ADAM: return "train_adam";
+        case RADAR_K_ROW_MERGE: return "row_merge";
+        case RADAR_K_EXPAND_CALLS: return "expand_calls";
         default: return "?";
     }
 }

@@ -25,6 +25,8 @@ enum radar_kernel_id {
     RADAR_K_TRAIN_ROLLOUT,      // REINFORCE step: rollout + backpropagation through time per data point
     RADAR_K_TRAIN_OUTER,        // REINFORCE step: parameter gradients
     RADAR_K_TRAIN_ADAM,         // REINFORCE step: batch loss + Adam update
+    RADAR_K_ROW_MERGE,          // radar_expand_calls: chunk records -> top-k of every row
+    RADAR_K_EXPAND_CALLS,       // radar_expand_calls: the calls of a sequence in one kernel
     RADAR_K_COUNT
 };
 
@@ -32,6 +34,8 @@ enum radar_kernel_id {
 enum radar_smem_slot {
     RADAR_SMEM_SELECT_GATE = 0,
     RADAR_SMEM_SELECT_GATE_CLUSTER,   // the instantiation with helper blocks
+    RADAR_SMEM_EXPAND_CALLS,
+    RADAR_SMEM_EXPAND_CALLS_PLAIN,    // the instantiation without helper blocks
     RADAR_SMEM_TREE_BUILD,
     RADAR_SMEM_TRAIN_ROLLOUT,   // the instantiation with four points a block
     RADAR_SMEM_WALK,            // + 2 * (bf16) + CTAs per SM - 1
@@ -165,6 +169,27 @@ __device__ __forceinline__ T warp_sum(T v) {
     return v;
 }
 
+// Sums of N values over the warp's 32 lanes, N a power of two: lane l returns the sum of value l / (32 / N).  Halving the
+// values with every exchange costs N - 1 + log2(32 / N) shuffles; N butterflies would cost 5 N, and an SM passes one
+// warp's shuffle a clock.
+template <int N>
+__device__ __forceinline__ float transposed_sum(float (&v)[N]) {
+    const int lane = threadIdx.x & 31;
+    int o = 16;
+#pragma unroll
+    for (int m = N / 2; m > 0; m >>= 1, o >>= 1) {
+        const bool up = (lane & o) != 0;
+#pragma unroll
+        for (int i = 0; i < m; ++i) {
+            const float give = up ? v[i] : v[i + m], keep = up ? v[i + m] : v[i];
+            v[i] = keep + __shfl_xor_sync(kFull, give, o);
+        }
+    }
+    float t = v[0];
+    for (; o > 0; o >>= 1) t += __shfl_xor_sync(kFull, t, o);
+    return t;
+}
+
 // Sorted list of the 32 best (value, index) pairs seen by a warp, one per lane (lane 0 = best).
 // V is float or double.  Empty slots hold (-inf, INT_MAX).
 template <typename V>
@@ -210,7 +235,7 @@ struct VocabPassParams {
     int32_t* part_i;                 // [rows][n_chunks][k]
     float* part_m;                   // [rows][n_chunks]
     float* part_s;                   // [rows][n_chunks]
-    int* status;
+    int* status;                     // NULL (with want_lse): a NaN logit is left in part_m for the merge to report
 };
 int vocab_pass_plan_chunks(int sm_count, int rows, int V, int* chunk_out);   // returns n_chunks
 size_t vocab_pass_partial_bytes(int rows, int n_chunks, int k);

@@ -5,18 +5,13 @@
 // latency: everything it reads from global memory is fetched in a few wide, independent batches.
 #include <algorithm>
 
-#include "common.cuh"
+#include "select.cuh"
 
 namespace radar {
 namespace {
 
-constexpr int kSelThreads = 1024;
-constexpr int kSelWarps = kSelThreads / 32;
 constexpr int kMergeWarps = 16;                      // warps 0..15 merge chunk records, warps 16..31 prepare the gate
-constexpr int kMaxF = 32;
 constexpr size_t kStageLimit = 96 * 1024;            // chunk records are staged in shared memory up to this size
-constexpr int kSurvCap = 256;                        // per-row survivor list of the parallel merge (even: read in pairs)
-constexpr int kSelCluster = 4;                       // blocks per sequence when the recurrent product is shared out
 constexpr long long kShortPassLogits = 4 << 20;      // ... which is done while a vocabulary pass reads at most this many logits
 
 struct SelectParams {
@@ -81,59 +76,6 @@ __global__ void __launch_bounds__(1024) gate_features_kernel(const radar_expand_
         }
         __syncthreads();
     }
-}
-
-__device__ __forceinline__ float sigmoidf_(float x) { return 1.f / (1.f + expf(-x)); }
-
-__device__ __forceinline__ void group_barrier(int id) { asm volatile("bar.sync %0, 512;" ::"r"(id) : "memory"); }
-__device__ __forceinline__ void cp_async4(void* smem, const void* gmem) {
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"((uint32_t)__cvta_generic_to_shared(smem)), "l"(gmem) : "memory");
-}
-__device__ __forceinline__ void cp_async16(void* smem, const void* gmem) {
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(smem)), "l"(gmem) : "memory");
-}
-__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
-
-// Thread-block cluster pieces of the select + gate block: stores and barrier arrivals into block 0's shared memory.
-__device__ __forceinline__ uint32_t smem_addr(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
-__device__ __forceinline__ void cluster_barrier() {
-    asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
-}
-__device__ __forceinline__ void st_cluster_f32(const float* local, uint32_t rank, float v) {
-    asm volatile("{\n\t.reg .b32 ra;\n\tmapa.shared::cluster.u32 ra, %0, %1;\n\tst.shared::cluster.f32 [ra], %2;\n\t}" ::"r"(
-                     smem_addr(local)), "r"(rank), "f"(v) : "memory");
-}
-__device__ __forceinline__ void mbar_arrive_cluster(const uint64_t* local, uint32_t rank) {
-    asm volatile("{\n\t.reg .b32 ra;\n\tmapa.shared::cluster.u32 ra, %0, %1;\n\t"
-                 "mbarrier.arrive.release.cluster.shared::cluster.b64 _, [ra];\n\t}" ::"r"(smem_addr(local)), "r"(rank) : "memory");
-}
-__device__ __forceinline__ bool mbar_try_wait_cluster(const uint64_t* bar, uint32_t parity) {
-    uint32_t ok;
-    asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
-                 "selp.u32 %0, 1, 0, p;\n\t}" : "=r"(ok) : "r"(smem_addr(bar)), "r"(parity) : "memory");
-    return ok != 0;
-}
-constexpr int kHelperRows(int n_help) { return (4 * kHidden + n_help - 1) / n_help; }
-
-// (value, index) as one 64-bit word whose unsigned order is the merge's order: a precedes b (larger value, then
-// smaller index) exactly if key(a) > key(b).  -0 is folded into +0 first, as the comparison of values does.
-__device__ __forceinline__ unsigned long long order_key(float v, int i) {
-    uint32_t u = __float_as_uint(v + 0.f);
-    u = (u & 0x80000000u) ? ~u : (u | 0x80000000u);
-    return ((unsigned long long)u << 32) | (uint32_t)(0x7fffffff - i);
-}
-__device__ __forceinline__ float key_value(unsigned long long key) {
-    const uint32_t u = (uint32_t)(key >> 32);
-    return __uint_as_float((u & 0x80000000u) ? (u ^ 0x80000000u) : ~u);
-}
-__device__ __forceinline__ int key_index(unsigned long long key) { return 0x7fffffff - (int)(uint32_t)key; }
-
-// smallest of the lanes' values (redux on a monotone unsigned image of the floats)
-__device__ __forceinline__ float warp_min_value(float v) {
-    uint32_t u = __float_as_uint(v + 0.f);
-    u = (u & 0x80000000u) ? ~u : (u | 0x80000000u);
-    u = __reduce_min_sync(kFull, u);
-    return __uint_as_float((u & 0x80000000u) ? (u ^ 0x80000000u) : ~u);
 }
 
 // One block per sequence.  Phase 1 runs two things side by side: warps 0-15 merge the vocabulary pass's
@@ -261,124 +203,22 @@ __global__ void __launch_bounds__(kSelThreads, 1) expand_select_gate_kernel(cons
 
     if (warp < kMergeWarps) {
         // ---- 1a. per row: chunk records -> this warp's shared memory, log-normaliser, top-k, candidate scores ----
-        // A warp works on its row alone (no block barrier), and on its own its time is the number of instructions it
-        // issues one after the other plus what its shuffles wait for the ones of the other rows (an SM passes one
-        // warp's shuffle a clock).  So the chunk heads and the survivors are ranked from shared memory, four and two
-        // to a broadcast load, the records are filtered flat (a lane takes every 32nd entry, whatever its chunk), and
-        // the only shuffles left are those of the log-normaliser.
+        // (a warp works on its row alone: no block barrier)
         const size_t row0 = (size_t)b * F;
         float* pv_s = st_v + (size_t)warp * stage_stride;
         int* pi_s = st_i + (size_t)warp * stage_stride;
         unsigned long long* lk = sv_key + warp * kSurvCap;
-        float* s_heads = reinterpret_cast<float*>(lk);              // (done with before the first survivor is written)
         chain_sync();
         for (int f = warp; f < F; f += kMergeWarps) {
             const size_t row = row0 + f;
-            const float* gv = P.vp.part_v + row * per_row;
-            const int* gi = P.vp.part_i + row * per_row;
-            __syncwarp();                                            // the previous row's lists have been read
-            if (P.staged) {
-                if ((per_row & 3) == 0) {                            // rows of records are 16-byte aligned then
-                    for (int e = lane; e < per_row / 4; e += 32) { cp_async16(pv_s + 4 * e, gv + 4 * e); cp_async16(pi_s + 4 * e, gi + 4 * e); }
-                } else {
-                    for (int e = lane; e < per_row; e += 32) { cp_async4(pv_s + e, gv + e); cp_async4(pi_s + e, gi + e); }
-                }
-            }
-            // log-sum-exp over the chunks in fp64
             const float parent_sc = a.parent_score[row];
-            const float pm0 = lane < n_chunks ? P.vp.part_m[row * n_chunks + lane] : -CUDART_INF_F;
-            const float ps0 = lane < n_chunks ? P.vp.part_s[row * n_chunks + lane] : 0.f;
-            float mloc = pm0;
-            for (int c = lane + 32; c < n_chunks; c += 32) mloc = fmaxf(mloc, P.vp.part_m[row * n_chunks + c]);
-            const float M = warp_max(mloc);
-            double sloc = pm0 > -CUDART_INF_F ? (double)ps0 * exp((double)pm0 - (double)M) : 0.0;
-            for (int c = lane + 32; c < n_chunks; c += 32) {
-                const float mc = P.vp.part_m[row * n_chunks + c];
-                if (mc > -CUDART_INF_F) sloc += (double)P.vp.part_s[row * n_chunks + c] * exp((double)mc - (double)M);
-            }
-            const double S = warp_sum(sloc);
-            const double lse = (double)M + log(S);
-            auto put = [&](int rank, float v, int tok) {             // the row's candidate number `rank`
+            merge_row(P.vp, row, P.staged != 0, pv_s, pi_s, lk, [&](int rank, float v, int tok, double lse) {     // candidate `rank` of the row
                 const double logp = (double)v - lse;
                 a.topk_tok[row * k + rank] = tok;
                 a.topk_logp[row * k + rank] = (float)logp;
                 s_cand[f * k + rank] = (double)parent_sc + logp;
                 s_ctok[f * k + rank] = tok;
-            };
-            bool merged = false;
-            if (P.staged) {
-                cp_async_wait_all();
-                __syncwarp();
-                // The k-th best chunk head (best head of every 32nd chunk, if there are more than 32) bounds the row's
-                // k-th best value from below; without that many chunks, the worst of all lists' j-th entries does,
-                // where the lists' first j entries are at least k.
-                float tv;
-                if (n_chunks >= k) {
-                    float hv = lane < n_chunks ? pv_s[lane * k] : -CUDART_INF_F;
-                    for (int c = lane + 32; c < n_chunks; c += 32) hv = fmaxf(hv, pv_s[c * k]);
-                    s_heads[lane] = hv;
-                    __syncwarp();
-                    int above = 0;
-#pragma unroll
-                    for (int o = 0; o < 32; o += 4) {
-                        const float4 h4 = *reinterpret_cast<const float4*>(s_heads + o);
-                        above += (h4.x > hv ? 1 : 0) + (h4.y > hv ? 1 : 0) + (h4.z > hv ? 1 : 0) + (h4.w > hv ? 1 : 0);
-                    }
-                    tv = warp_min_value(lane < n_chunks && above < k ? hv : CUDART_INF_F);
-                    __syncwarp();
-                } else {
-                    const int jth = (k + n_chunks - 1) / n_chunks;
-                    tv = warp_min_value(lane < n_chunks ? pv_s[lane * k + jth - 1] : CUDART_INF_F);
-                }
-                int total = 0;
-#pragma unroll 4
-                for (int e0 = 0; e0 < per_row; e0 += 32) {
-                    const int e = e0 + lane;
-                    const float v = e < per_row ? pv_s[e] : 0.f;
-                    const bool keep = e < per_row && v >= tv;
-                    const unsigned m = __ballot_sync(kFull, keep);
-                    const int at = total + __popc(m & ((1u << lane) - 1u));
-                    if (keep && at < kSurvCap) lk[at] = order_key(v, pi_s[e]);
-                    total += __popc(m);
-                }
-                if (total <= kSurvCap) {
-                    if (lane == 0 && (total & 1)) lk[total] = 0ull;   // read in pairs: a key that precedes nothing
-                    __syncwarp();
-                    for (int e = lane; e < total; e += 32) {
-                        const unsigned long long ck = lk[e];
-                        int rank = 0;
-#pragma unroll 4
-                        for (int j = 0; j < total; j += 2) {
-                            const ulonglong2 kk = *reinterpret_cast<const ulonglong2*>(lk + j);
-                            rank += (kk.x > ck ? 1 : 0) + (kk.y > ck ? 1 : 0);
-                        }
-                        if (rank < k) put(rank, key_value(ck), key_index(ck));
-                    }
-                    for (int e = total + lane; e < k; e += 32) put(e, -CUDART_INF_F, 0x7fffffff);   // (only with NaN logits)
-                    merged = true;
-                }
-                __syncwarp();
-            }
-            if (!merged) {
-                // serial merge (records too large to stage, or a survivor list that overflowed)
-                const float* pv = P.staged ? pv_s : gv;
-                const int* pi = P.staged ? pi_s : gi;
-                WarpTopList<float> top;
-                top.reset();
-                float thr = -CUDART_INF_F;
-                int thr_i = 0x7fffffff;
-                for (int c = 0; c < n_chunks; ++c) {
-                    for (int e = 0; e < k; ++e) {
-                        const float cv = pv[c * k + e];
-                        const int ci = pi[c * k + e];
-                        if (!precedes(cv, ci, thr, thr_i)) break;          // each chunk's list is sorted
-                        top.insert(cv, ci);
-                        thr = top.value_at(k - 1);
-                        thr_i = top.index_at(k - 1);
-                    }
-                }
-                if (lane < k) put(lane, top.v, top.i);
-            }
+            });
         }
     } else if (run_gate) {
         // ---- 1b. the part of the prediction model that only needs the previous state ----

@@ -63,27 +63,6 @@ struct TrainParams {
 __device__ __forceinline__ float sigmoidf(float v) { return 1.f / (1.f + __expf(-v)); }
 __device__ __forceinline__ float softplusf(float v) { return v > 0.f ? v + log1pf(expf(-v)) : log1pf(expf(v)); }
 
-// Sums of N values over the warp's 32 lanes, N a power of two: lane l returns the sum of value l / (32 / N).  Halving the
-// values with every exchange costs N - 1 + log2(32 / N) shuffles; N butterflies would cost 5 N, and an SM passes one
-// warp's shuffle a clock.
-template <int N>
-__device__ __forceinline__ float transposed_sum(float (&v)[N]) {
-    const int lane = threadIdx.x & 31;
-    int o = 16;
-#pragma unroll
-    for (int m = N / 2; m > 0; m >>= 1, o >>= 1) {
-        const bool up = (lane & o) != 0;
-#pragma unroll
-        for (int i = 0; i < m; ++i) {
-            const float give = up ? v[i] : v[i + m], keep = up ? v[i + m] : v[i];
-            v[i] = keep + __shfl_xor_sync(kFull, give, o);
-        }
-    }
-    float t = v[0];
-    for (; o > 0; o >>= 1) t += __shfl_xor_sync(kFull, t, o);
-    return t;
-}
-
 // A block takes kP data points side by side.  What bounds it is the way of the weights from L2 into the SM (256 KB of W_hh
 // and 70 KB of W_1 for every decision, forwards and backwards, 64 B a clock) and the latency of that way: the points of
 // a block share every weight that is loaded, and a thread has eight or more loads of a product in flight.  With one point

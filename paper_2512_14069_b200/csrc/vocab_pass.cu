@@ -276,10 +276,10 @@ __global__ void __launch_bounds__(kThreads, WANT_LSE ? (EPT == 32 ? 5 : 6) : 5) 
         float S = 0.f;
         if (M > -CUDART_INF_F)
             for (int w = 0; w < kWarps; ++w) S += sh_s[w] * __expf(sh_m[w] - M);
-        p.part_m[rec] = M;
+        p.part_m[rec] = sh_nan && p.status == nullptr ? CUDART_NAN_F : M;
         p.part_s[rec] = S;
     }
-    if (tid == 0 && sh_nan) set_status(p.status, RADAR_ERR_NUMERIC);
+    if (tid == 0 && sh_nan && p.status != nullptr) set_status(p.status, RADAR_ERR_NUMERIC);
 }
 
 template <typename T, bool WANT_LSE>

@@ -63,10 +63,12 @@ class SpecStep:
         wb = max(rb.radar_expand_workspace_bytes(ctx, B, 1, V, k), rb.radar_expand_workspace_bytes(ctx, B, k, V, k))
         self.ws_expand = z((wb + 255,), u8)
         self.ws_expand2 = z((wb + 255,), u8)          # consecutive calls alternate, so a pass can run ahead of the select
+        cb = rb.radar_expand_calls_workspace_bytes(ctx, B, V, k, t_max)
+        self.ws_calls = z((cb + 255,), u8) if cb else None      # None: the calls are issued one by one
         self.ws_attn = z((rb.radar_attn_workspace_bytes(ctx, B, Hq, Hkv, d, rb.dtype_code(self.O), max_prefix_len) + 255,), u8)
         self.ws_accept = z((rb.radar_accept_workspace_bytes(ctx, B, V, mode) + 255,), u8)
         self.side = torch.cuda.Stream(dev)            # the vocabulary passes of the pipelined expansion
-        for n in ("ws_expand", "ws_expand2", "ws_attn", "ws_accept"):
+        for n in ("ws_expand", "ws_expand2", "ws_attn", "ws_accept") + (("ws_calls",) if cb else ()):
             t = getattr(self, n)
             off = (-t.data_ptr()) % 256
             setattr(self, n, t[off:off + t.numel() - 255])
@@ -109,6 +111,9 @@ class SpecStep:
 
     def run_expansion(self, draft_logits, gate, force_calls=None, policy=rb.RADAR_POLICY_LSTM_SCORES, features=None,
                       pipelined=True):
+        if pipelined and self.ws_calls is not None and policy != rb.RADAR_POLICY_LSTM_HIDDEN:
+            self._expand_calls(draft_logits, gate, force_calls, policy)
+            return
         slots = self._slots()
         if not pipelined:
             for t in range(1, self.t_max + 1):      # call 1 restarts the state on the device
@@ -135,6 +140,19 @@ class SpecStep:
             sel_done[t] = torch.cuda.Event()
             sel_done[t].record(main)
         main.wait_stream(side)                      # join (the last pass has been waited for already)
+
+    def _expand_calls(self, draft_logits, gate, force_calls, policy):
+        more = self.t_max > 1
+        rb.radar_expand_calls(
+            self.ctx, B=self.B, V=self.V, k=self.k, t_max=self.t_max, logits=draft_logits, logits_row_stride=self.V,
+            logits_seq_stride=self.R * self.V, parent_score=self.root_score, parent_pool_idx=self.root_pool_idx, active=self.active,
+            force_calls=force_calls, gate=gate, h=self.h, c=self.c, pool_capacity=self.C, pool_tok=self.pool_tok,
+            pool_parent=self.pool_parent, pool_depth=self.pool_depth, pool_draft_row=self.pool_draft_row, pool_score=self.pool_score,
+            pool_len=self.pool_len, frontier_tok=self.frontier_tok, frontier_score=self.frontier_score,
+            frontier_pool_idx=self.frontier_pool_idx, frontier_src_row=self.frontier_src_row, topk_tok=self.topk_tok1,
+            topk_logp=self.topk_logp1, topk_tok_next=self.topk_tok[1:] if more else None,
+            topk_logp_next=self.topk_logp[1:] if more else None, gate_logits=self.gate_logits, cont=self.cont_hist, policy=policy,
+            workspace=self.ws_calls)
 
     # ---- tree, attention, acceptance ------------------------------------------------------
     def build_tree(self, root_tok, prefix_len, n_keep=None):
