@@ -6,6 +6,7 @@
 // block of 32 query rows, KV split); all G query heads that share a KV head are rows of the
 // same block so that a K/V tile staged in shared memory is reused G * rows times.
 #include <algorithm>
+#include <cmath>
 
 #include "common.cuh"
 
@@ -17,6 +18,7 @@ constexpr int kWarps = kThreads / 32;
 constexpr int kRowsPerWarp = 4;
 constexpr int kRowsPerBlock = kWarps * kRowsPerWarp;     // 32
 constexpr int kTile = 32;                                // keys per shared-memory tile
+constexpr int kMaxSplits = 32;                           // pieces of a sequence's keys
 
 struct AttnParams {
     radar_attn_args a;
@@ -247,19 +249,29 @@ __global__ void __launch_bounds__(128) tree_attn_combine_kernel(const AttnParams
     if (node >= M || Pb < 0 || Pb > a.max_prefix_len || kv0 < 0 || kv0 + Pb > a.cache_rows) return;   // skipped by the main kernel
     const int n_valid = (Pb + M + P.split_len - 1) / P.split_len;
     const int64_t rec0 = (((int64_t)b * a.Hq + hq) * kMaxNodes + node) * P.n_splits;
-    float mx = -CUDART_INF_F;
-    for (int s = 0; s < n_valid; ++s) mx = fmaxf(mx, P.part_ml[rec0 + s].x);
-    float den = 0.f, o[D / 32];
+    // a lane per split (kMaxSplits of them at most): its weight, and the splits' rows then four at a time in flight
+    static_assert(kMaxSplits <= 32, "a lane per split");
+    const float2 ml = lane < n_valid ? P.part_ml[rec0 + lane] : make_float2(-CUDART_INF_F, 0.f);
+    const float mx = warp_max(ml.x);
+    const float w = ml.x == -CUDART_INF_F ? 0.f : __expf(ml.x - mx);
+    const float den = warp_sum(ml.y * w);
+    float o[D / 32];
 #pragma unroll
     for (int c = 0; c < D / 32; ++c) o[c] = 0.f;
+#pragma unroll 4
     for (int s = 0; s < n_valid; ++s) {
-        const float2 ml = P.part_ml[rec0 + s];
-        if (ml.x == -CUDART_INF_F) continue;
-        const float w = __expf(ml.x - mx);
-        den += ml.y * w;
+        const float ws = __shfl_sync(kFull, w, s);
         const float* src = P.part_o + (rec0 + s) * D + lane * (D / 32);
+        float v[D / 32];
+        if constexpr (D == 128) {
+            const float4 t = *reinterpret_cast<const float4*>(src);
+            v[0] = t.x; v[1] = t.y; v[2] = t.z; v[3] = t.w;
+        } else {
+            const float2 t = *reinterpret_cast<const float2*>(src);
+            v[0] = t.x; v[1] = t.y;
+        }
 #pragma unroll
-        for (int c = 0; c < D / 32; ++c) o[c] = fmaf(src[c], w, o[c]);
+        for (int c = 0; c < D / 32; ++c) o[c] = fmaf(v[c], ws, o[c]);
     }
     const float inv = 1.f / den;
     T* dst = reinterpret_cast<T*>(a.O) + (((int64_t)b * kMaxNodes + node) * a.Hq + hq) * D + lane * (D / 32);
@@ -271,18 +283,29 @@ __global__ void __launch_bounds__(128) tree_attn_combine_kernel(const AttnParams
     if (a.lse != nullptr && lane == 0) a.lse[((int64_t)b * a.Hq + hq) * kMaxNodes + node] = mx + logf(den);
 }
 
-void plan(const radar_ctx* ctx, int B, int Hq, int Hkv, int max_prefix_len, int* split_len, int* n_splits) {
+// Splits of a sequence's keys, by a model of the time: a block goes through its tiles one after the other, and an SM with c
+// blocks takes about max(1.7, c) times as long for a tile of each (one or two blocks are bound by latency, more share the
+// FMA pipes, with d = 64 for three quarters of the time; four fit, and further ones follow as those leave); a block's start
+// and end count as one tile, as two where there are more blocks than fit, whose partial results are many.  us with the
+// combine, before (256 keys a split at least) and with this rule, fp32: 192 keys of 4 heads 22.8 -> 9.1; 364 keys, 32 / 8
+// heads 44.8 -> 32.2; 1064 keys, 40 / 40 heads 134 -> 93; 564 keys, two sequences of them 137 -> 109; 2112 keys, 32 / 8
+// heads 145 both.
+void plan(const radar_ctx* ctx, int B, int Hq, int Hkv, int d, int max_prefix_len, int* split_len, int* n_splits) {
     const int G = Hq / Hkv;
     const int rblocks = (kMaxNodes * G + kRowsPerBlock - 1) / kRowsPerBlock;
-    const int Lmax = max_prefix_len + kMaxNodes;
-    long long base = (long long)B * Hkv * rblocks;
-    int want = (int)((4LL * ctx->sm_count + base - 1) / base);
-    if (want < 1) want = 1;
-    int len = (Lmax + want - 1) / want;
-    if (len < 256) len = 256;
-    len = (len + kTile - 1) / kTile * kTile;
-    *split_len = len;
-    *n_splits = (Lmax + len - 1) / len;
+    const int tiles = (max_prefix_len + kMaxNodes + kTile - 1) / kTile;
+    const double base = (double)B * Hkv * rblocks, sms = ctx->sm_count;
+    double best = 0.0;
+    for (int s = 1; s <= std::min(tiles, kMaxSplits); ++s) {
+        const int len = (tiles + s - 1) / s, n = (tiles + len - 1) / len;
+        const double blocks = base * n, c = (blocks <= 4 * sms ? std::ceil(blocks / sms) : blocks / sms) * (d == 64 ? 0.75 : 1.0);
+        const double cost = (len + (blocks <= 4 * sms ? 1 : 2)) * std::max(1.7, c);
+        if (s == 1 || cost <= best) {
+            best = cost;
+            *split_len = len * kTile;
+            *n_splits = n;
+        }
+    }
 }
 
 template <typename T, int D>
@@ -315,7 +338,7 @@ extern "C" size_t radar_attn_workspace_bytes(const radar_ctx* ctx, int B, int Hq
                                              int max_prefix_len) {
     if (!ctx || B <= 0 || Hq <= 0 || Hkv <= 0 || Hq % Hkv != 0 || max_prefix_len < 0) return 0;
     int split_len, n_splits;
-    plan(ctx, B, Hq, Hkv, max_prefix_len, &split_len, &n_splits);
+    plan(ctx, B, Hq, Hkv, d, max_prefix_len, &split_len, &n_splits);
     const size_t rec = (size_t)B * Hq * kMaxNodes * n_splits;
     size_t need = align_up(rec * sizeof(float2), 256) + align_up(rec * d * sizeof(float), 256);
     // the same buffer serves whichever kernel the call dispatches to
@@ -380,7 +403,7 @@ extern "C" int radar_tree_attention(radar_ctx* ctx, const radar_attn_args* a, vo
     P.G = a->Hq / a->Hkv;
     P.scale = a->scale > 0.f ? a->scale : 1.f / sqrtf((float)a->d);
     P.status = ctx->d_status;
-    plan(ctx, a->B, a->Hq, a->Hkv, a->max_prefix_len, &P.split_len, &P.n_splits);
+    plan(ctx, a->B, a->Hq, a->Hkv, a->d, a->max_prefix_len, &P.split_len, &P.n_splits);
     const size_t rec = (size_t)a->B * a->Hq * kMaxNodes * P.n_splits;
     const size_t need = align_up(rec * sizeof(float2), 256) + align_up(rec * a->d * sizeof(float), 256);
     if (need > a->workspace_bytes) return RADAR_ERR_WORKSPACE;
