@@ -522,7 +522,8 @@ extern "C" int radar_expand_calls(radar_ctx* ctx, const radar_expand_calls_args*
         cfg.attrs = attr;
         cfg.numAttrs = blocks > 1 ? 2 : 1;
         if (blocks > 1) {
-            RADAR_CUDA_CHECK(radar_opt_in_smem(ctx, RADAR_SMEM_EXPAND_CALLS, expand_calls_kernel<true>, smem));
+            // (with the block's 23 KB of static shared memory the limit without an opt-in lies at 25 KB)
+            RADAR_CUDA_CHECK(radar_opt_in_smem(ctx, RADAR_SMEM_EXPAND_CALLS, expand_calls_kernel<true>, std::max(smem, (size_t)96 * 1024)));
             RADAR_CUDA_CHECK(cudaLaunchKernelEx(&cfg, expand_calls_kernel<true>, cp));
         } else {
             RADAR_CUDA_CHECK(radar_opt_in_smem(ctx, RADAR_SMEM_EXPAND_CALLS_PLAIN, expand_calls_kernel<false>, smem));

@@ -57,7 +57,7 @@ def _both(ctx, draft, k, t_max, gate, force, policy, check=True):
 
 
 @pytest.mark.parametrize("B,V,k,t_max,policy", [(1, 40, 1, 1, 0), (3, 5000, 4, 2, 0), (5, 9000, 10, 3, 0), (9, 9000, 10, 8, 0),
-                                                (17, 2000, 7, 16, 0), (2, 33000, 32, 16, 0), (6, 9000, 10, 8, 1), (3, 3000, 1, 5, 0)])
+                                                (17, 2000, 7, 16, 0), (2, 9000, 12, 6, 0), (4, 3000, 16, 4, 0), (2, 33000, 32, 16, 0), (6, 9000, 10, 8, 1), (3, 3000, 1, 5, 0)])
 def test_calls_together_match_one_by_one(ctx, B, V, k, t_max, policy):
     import torch
     g = torch.Generator(device="cuda").manual_seed(B * V + k)
