@@ -315,6 +315,12 @@ def radar_expand_step(ctx: Context, *, logits, gate, workspace, logits_offset_el
     pool_depth, pool_draft_row, pool_score, pool_len, frontier_tok, frontier_score, frontier_pool_idx, frontier_src_row,
     topk_tok, topk_logp, gate_logits, cont, and, with defaults, force_calls (None), policy (RADAR_POLICY_LSTM_SCORES) and
     phase (RADAR_EXPAND_ALL)."""
+    expand_fields(ctx, kw, logits, gate, workspace, logits_offset_elems, features, stream)
+
+
+def expand_fields(ctx, kw, logits, gate, workspace, logits_offset_elems=0, features=None, stream=None):
+    """radar_expand_step with its other arguments in the dictionary `kw`, which is completed in place: a call that passes
+    forty keywords through two functions spends more on them than on its launches."""
     kw["logits"] = _ptr(logits) + logits_offset_elems * logits.element_size()
     kw["logits_dtype"] = dtype_code(logits)
     for n in _GATE:

@@ -96,18 +96,18 @@ class SpecStep:
         s = t - 1
         slots = self._slots() if slots is None else slots
         frontier_tok, frontier_score, frontier_pool_idx, frontier_src_row, topk_tok, topk_logp, gate_logits, cont = slots[s]
-        rb.radar_expand_step(
-            self.ctx, B=B, F=F, V=V, k=k, t=t, t_max=self.t_max, logits=draft_logits,
-            logits_row_stride=V, logits_seq_stride=self.R * V, logits_offset_elems=row0 * V,
-            parent_score=self.root_score if t == 1 else slots[s - 1][1],
-            parent_pool_idx=self.root_pool_idx if t == 1 else slots[s - 1][2],
-            active=vocab_mask if phase == rb.RADAR_EXPAND_VOCAB else self.active, force_calls=force_calls, gate=gate, h=self.h, c=self.c,
-            pool_capacity=self.C, pool_tok=self.pool_tok, pool_parent=self.pool_parent, pool_depth=self.pool_depth,
-            pool_draft_row=self.pool_draft_row, pool_score=self.pool_score, pool_len=self.pool_len,
-            frontier_tok=frontier_tok, frontier_score=frontier_score, frontier_pool_idx=frontier_pool_idx,
-            frontier_src_row=frontier_src_row, topk_tok=self.topk_tok1 if t == 1 else topk_tok,
-            topk_logp=self.topk_logp1 if t == 1 else topk_logp, gate_logits=gate_logits, cont=cont, workspace=self.ws_expand if workspace is None else workspace,
-            policy=policy, features=None if features is None or t >= self.t_max else features[s], phase=phase, stream=stream)
+        kw = {
+            "B": B, "F": F, "V": V, "k": k, "t": t, "t_max": self.t_max, "logits_row_stride": V, "logits_seq_stride": self.R * V,
+            "parent_score": self.root_score if t == 1 else slots[s - 1][1],
+            "parent_pool_idx": self.root_pool_idx if t == 1 else slots[s - 1][2],
+            "active": vocab_mask if phase == rb.RADAR_EXPAND_VOCAB else self.active, "force_calls": force_calls, "h": self.h, "c": self.c,
+            "pool_capacity": self.C, "pool_tok": self.pool_tok, "pool_parent": self.pool_parent, "pool_depth": self.pool_depth,
+            "pool_draft_row": self.pool_draft_row, "pool_score": self.pool_score, "pool_len": self.pool_len,
+            "frontier_tok": frontier_tok, "frontier_score": frontier_score, "frontier_pool_idx": frontier_pool_idx,
+            "frontier_src_row": frontier_src_row, "topk_tok": self.topk_tok1 if t == 1 else topk_tok,
+            "topk_logp": self.topk_logp1 if t == 1 else topk_logp, "gate_logits": gate_logits, "cont": cont, "policy": policy, "phase": phase}
+        rb.expand_fields(self.ctx, kw, draft_logits, gate, self.ws_expand if workspace is None else workspace, row0 * V,
+                         None if features is None or t >= self.t_max else features[s], stream)
 
     def run_expansion(self, draft_logits, gate, force_calls=None, policy=rb.RADAR_POLICY_LSTM_SCORES, features=None,
                       pipelined=True):
