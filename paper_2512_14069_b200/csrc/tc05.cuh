@@ -231,6 +231,23 @@ __device__ __forceinline__ void mma_ts_x4_full(uint32_t pred, uint32_t d_tmem, u
         : "memory");
 #undef RADAR_TS_STEP
 }
+//   TS, two steps of each half of a 128-key tile (64 columns of A, 64 rows of B apart).
+__device__ __forceinline__ void mma_ts_x2x2_full(uint32_t pred, uint32_t d_tmem, uint32_t a_tmem, uint32_t b_lo, uint32_t hi,
+                                                 uint32_t idesc, bool acc_first) {
+#define RADAR_TS_STEP(A, B, P)                                                                         \
+        "add.u32 a, %2, " #A ";\n\tadd.u32 b, %3, " #B ";\n\tmov.b64 db, {b, %4};\n\t"                 \
+        "@q tcgen05.mma.cta_group::1.kind::f16 [%1], [a], db, %5, " #P ";\n\t"
+    asm volatile(
+        "{\n\t.reg .pred q, p0, p1;\n\t.reg .b32 a, b;\n\t.reg .b64 db;\n\t"
+        "setp.ne.b32 q, %0, 0;\n\t"
+        "setp.ne.b32 p0, %6, 0;\n\t"
+        "setp.eq.b32 p1, 0, 0;\n\t"
+        RADAR_TS_STEP(0, 0, p0) RADAR_TS_STEP(8, 128, p1) RADAR_TS_STEP(64, 512, p1) RADAR_TS_STEP(72, 640, p1)
+        "}"
+        ::"r"(pred), "r"(d_tmem), "r"(a_tmem), "r"(b_lo), "r"(hi), "r"(idesc), "r"((uint32_t)acc_first)
+        : "memory");
+#undef RADAR_TS_STEP
+}
 // The barrier receives one arrival once every MMA issued so far by this thread has completed.
 __device__ __forceinline__ void mma_commit(uint64_t* bar) {
     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar))

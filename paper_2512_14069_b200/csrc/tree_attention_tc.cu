@@ -212,7 +212,7 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
     // swizzled tiles need a 1024-byte boundary and there is no room left for alignment slack.
     struct __align__(1024) Static {
         uint64_t bar_qfull, bar_qempty, bar_kfull[3], bar_kempty[3], bar_vfull[3], bar_vempty[3];
-        uint64_t bar_sfull[2], bar_pready[2], bar_odone[2], bar_ofree[2];
+        uint64_t bar_sfull[2], bar_pfirst[2], bar_pready[2], bar_odone[2], bar_ofree[2];
         long long range[4];      // this CTA's range [lo, hi), size of the class's space (all layers), start of its first unit
         int start[3];            // sequence, KV head and layer of the unit that contains lo
         int start_pad;
@@ -220,7 +220,7 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
         int abort;
         float xm[128];           // group 1's running max at the end of a segment (one live row block)
         float mx[2][2][128];     // per group and column half: row maxima of a tile; row sums at the end of a segment
-        unsigned char pad[kStaticSmem - (22 * 8 + 4 * 8 + 4 * 4 + 4 + 4 + 128 * 4 + 2 * 2 * 128 * 4)];
+        unsigned char pad[kStaticSmem - (24 * 8 + 4 * 8 + 4 * 4 + 4 + 4 + 128 * 4 + 2 * 2 * 128 * 4)];
     };
     static_assert(sizeof(Static) == kStaticSmem, "static shared-memory block");
     __shared__ Static st;
@@ -236,7 +236,8 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
     uint64_t (&bar_vfull)[3] = st.bar_vfull;
     uint64_t (&bar_vempty)[3] = st.bar_vempty;
     uint64_t (&bar_sfull)[2] = st.bar_sfull;
-    uint64_t (&bar_pready)[2] = st.bar_pready;
+    uint64_t (&bar_pfirst)[2] = st.bar_pfirst;       // the first chunk of every thread's P is there
+    uint64_t (&bar_pready)[2] = st.bar_pready;       // ... all of it
     uint64_t (&bar_odone)[2] = st.bar_odone;
     uint64_t (&bar_ofree)[2] = st.bar_ofree;
     uint32_t& s_tmem_base = st.tmem_base;
@@ -306,7 +307,7 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
                 mbar_init(&bar_vfull[i], 1); mbar_init(&bar_vempty[i], 1);
             }
             for (int i = 0; i < 2; ++i) {
-                mbar_init(&bar_sfull[i], 1); mbar_init(&bar_pready[i], 8);
+                mbar_init(&bar_sfull[i], 1); mbar_init(&bar_pfirst[i], 8); mbar_init(&bar_pready[i], 8);
                 mbar_init(&bar_odone[i], 1); mbar_init(&bar_ofree[i], 8);
             }
             fence_barrier_init();
@@ -489,6 +490,7 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
                 const int nk = tree ? kTreeKeys : kTileKeys;
                 const int valid = tree ? M : min(kTileKeys, Pb - (seg_t0 + i) * kTileKeys);
                 const int ksteps = (valid + 15) >> 4;
+                ok = ok && mbar_wait(&bar_pfirst[q], p_par[q], ab);
                 ok = ok && mbar_wait(&bar_pready[q], p_par[q], ab);
                 p_par[q] ^= 1;
                 if (fresh_v) {
@@ -556,18 +558,20 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
             const uint32_t a_q0 = q_lo, a_q1 = q_lo + (SM::kQBlock >> 4);
             auto wait_all = [&](uint64_t* bar, uint32_t parity) { ok = mbar_wait(bar, parity, ab) && ok; };
             auto pv_full = [&](const int q, const bool fresh_v, const bool release_v) {
-                wait_all(&bar_pready[q], p_par[q]);
-                p_par[q] ^= 1;
+                wait_all(&bar_pfirst[q], p_par[q]);
                 if (fresh_v) {
                     v_slot = v_next;
                     wait_all(&bar_vfull[v_slot], v_par);
                     if (++v_next == RV) { v_next = 0; v_par ^= 1; }
                 }
                 tc_fence_after_sync();
-                const uint32_t go = ok ? elected : 0u;
                 const uint32_t b_lo = (v_lo + v_slot * (SM::kTileBytes >> 4)) | ((uint32_t)(kTileKeys * 128 >> 4) << 16);
-                mma_ts_x4_full(go, tmem + 256 + q * 128, tmem + q * 128, b_lo, kDescHi, idesc_pv, acc[q]);
-                mma_ts_x4_full(go, tmem + 256 + q * 128, tmem + q * 128 + 64, b_lo + 4 * 128, kDescHi, idesc_pv, true);
+                mma_ts_x2x2_full(ok ? elected : 0u, tmem + 256 + q * 128, tmem + q * 128, b_lo, kDescHi, idesc_pv, acc[q]);
+                wait_all(&bar_pready[q], p_par[q]);
+                p_par[q] ^= 1;
+                tc_fence_after_sync();
+                const uint32_t go = ok ? elected : 0u;
+                mma_ts_x2x2_full(go, tmem + 256 + q * 128, tmem + q * 128 + 16, b_lo + 2 * 128, kDescHi, idesc_pv, true);
                 acc[q] = true;
                 if (release_v) mma_commit_if(go, &bar_vempty[v_slot]);
             };
@@ -624,8 +628,13 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
         // Two threads per query row: warp w of a group's eight serves tensor-memory lanes 32 (w & 3) .. + 31
         // and the column half (w >> 2) & 1, so a row's 128 scores are exponentiated by two threads at once
         // and the chain S -> softmax -> P V of a group is about half as long.
+        // That chain is what a tile costs (about 4000 cycles, of which the tensor pipe works 2048).  So the products of a
+        // thread's first 32 columns start while the second 32 are exponentiated, and only the two warps that share
+        // rows wait for each other's maxima: 32 layers, 8 sequences of 6000 to 8192 tokens, 64 / 8 heads 4457 -> 4347 us
+        // (the early products alone 4369); launches bound by memory are unchanged.
         const int grp = warp >> 3;
         const int half = (warp >> 2) & 1;
+        const int pair_bar = 1 + grp * 4 + (warp & 3);          // barriers 1 .. 8: the two warps that share 32 rows
         const int row = (warp & 3) * 32 + lane;                 // row of the block == tensor-memory lane
         const uint32_t lane_addr = (uint32_t)((warp & 3) * 32) << 16;
         const uint32_t tS = tmem + grp * 128 + lane_addr;
@@ -696,7 +705,7 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
                 }
                 // the two halves of a row exchange their maxima
                 s_mx[grp][half][row] = mx;
-                if (grp == 0) asm volatile("bar.sync 1, 256;" ::: "memory"); else asm volatile("bar.sync 2, 256;" ::: "memory");
+                asm volatile("bar.sync %0, 64;" ::"r"(pair_bar) : "memory");
                 if (ok && warp_live) {
                     mx = fmaxf(mx, s_mx[grp][half ^ 1][row]);
                     // ---- running max (log2 units), lazy rescale decision: the same in both halves of a row ----
@@ -709,6 +718,19 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
                         m_run = m_tile;
                     }
                     const float m_use = m_run == -CUDART_INF_F ? 0.f : m_run;
+                    // ---- rescale this thread's half of the accumulator when some row of the warp moved its max
+                    // (the products of the first chunk start before the second is there) ----
+                    if (j > 0 && __any_sync(kFull, factor != 1.f)) {
+#pragma unroll 1
+                        for (int c = 0; c < DH / 32; ++c) {
+                            uint32_t o[32];
+                            tmem_ld32(tO + half * DH + c * 32, o);
+                            tmem_wait_ld();
+#pragma unroll
+                            for (int e = 0; e < 32; ++e) o[e] = __float_as_uint(__uint_as_float(o[e]) * factor);
+                            tmem_st32(tO + half * DH + c * 32, o);
+                        }
+                    }
                     // ---- P = exp2(s * scale - m), row sum, bf16 pairs back to tensor memory ----
                     // (the scaling and the row sum work on pairs: one packed fp32x2 instruction per two values)
                     float2 ls[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
@@ -734,25 +756,22 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
                             pk[e] = *reinterpret_cast<const uint32_t*>(&v);
                         }
                         tmem_st16(tS + half * 64 + cc * 16, pk);
-                    }
-                    l_run = l_run * factor + ((ls[0].x + ls[0].y) + (ls[1].x + ls[1].y));
-                    // ---- rescale this thread's half of the accumulator when some row of the warp moved its max ----
-                    if (j > 0 && __any_sync(kFull, factor != 1.f)) {
-#pragma unroll 1
-                        for (int c = 0; c < DH / 32; ++c) {
-                            uint32_t o[32];
-                            tmem_ld32(tO + half * DH + c * 32, o);
-                            tmem_wait_ld();
-#pragma unroll
-                            for (int e = 0; e < 32; ++e) o[e] = __float_as_uint(__uint_as_float(o[e]) * factor);
-                            tmem_st32(tO + half * DH + c * 32, o);
+                        if (cc == 0) {
+                            tmem_wait_st();
+                            tc_fence_before_sync();
+                            __syncwarp();
+                            if (lane == 0) mbar_arrive(&bar_pfirst[grp]);
                         }
                     }
+                    l_run = l_run * factor + ((ls[0].x + ls[0].y) + (ls[1].x + ls[1].y));
                     tmem_wait_st();
                 }
                 tc_fence_before_sync();
                 __syncwarp();
-                if (lane == 0) mbar_arrive(&bar_pready[grp]);
+                if (lane == 0) {
+                    if (!(ok && warp_live)) mbar_arrive(&bar_pfirst[grp]);
+                    mbar_arrive(&bar_pready[grp]);
+                }
             }
 
             // ---- epilogue of the segment ----
@@ -767,7 +786,7 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
             // the row sum is the two halves' sums; with one live row block group 1 also hands its (m, l) to group 0
             s_xl[grp][half][row] = l_run;
             if (grp == 1 && half == 0) s_xm[row] = n_my > 0 ? m_run : -CUDART_INF_F;
-            asm volatile("bar.sync 3, 512;" ::: "memory");
+            asm volatile("bar.sync 9, 512;" ::: "memory");
             float l_out = s_xl[grp][0][row] + s_xl[grp][1][row];
             float m_out = m_run, w0 = 1.f, w1 = 0.f;
             bool writer = true, merge_any = false;
@@ -845,7 +864,7 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
                     }
                 }
             }
-            asm volatile("bar.sync 4, 512;" ::: "memory");       // the exchanged (m, l) and group 1's accumulator have been read
+            asm volatile("bar.sync 10, 512;" ::: "memory");       // the exchanged (m, l) and group 1's accumulator have been read
             tc_fence_before_sync();
             __syncwarp();
             if (lane == 0) mbar_arrive(&bar_ofree[grp]);
