@@ -212,7 +212,8 @@ __global__ void __launch_bounds__(kSelThreads, 1) expand_select_gate_kernel(cons
         for (int f = warp; f < F; f += kMergeWarps) {
             const size_t row = row0 + f;
             const float parent_sc = a.parent_score[row];
-            merge_row(P.vp, row, P.staged != 0, pv_s, pi_s, lk, [&](int rank, float v, int tok, double lse) {     // candidate `rank` of the row
+            double lse = 0.0;
+            merge_row(P.vp, row, P.staged != 0, pv_s, pi_s, lk, [&] { lse = row_normaliser(P.vp, row); }, [&](int rank, float v, int tok) {
                 const double logp = (double)v - lse;
                 a.topk_tok[row * k + rank] = tok;
                 a.topk_logp[row * k + rank] = (float)logp;

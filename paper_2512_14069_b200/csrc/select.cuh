@@ -65,15 +65,32 @@ __device__ __forceinline__ float warp_min_value(float v) {
     return __uint_as_float((u & 0x80000000u) ? (u ^ 0x80000000u) : ~u);
 }
 
-// One warp merges a row's chunk records into its top-k and log-normaliser and hands candidate `rank` to
-// put(rank, logit, token, log-normaliser).  pv_s / pi_s: the warp's copy of the records (staged), lk: kSurvCap keys.
+// Log-sum-exp over a row's chunks in fp64, by one warp.
+__device__ __forceinline__ double row_normaliser(const VocabPassParams& vp, size_t row) {
+    const int lane = threadIdx.x & 31, n_chunks = vp.n_chunks;
+    const float pm0 = lane < n_chunks ? vp.part_m[row * n_chunks + lane] : -CUDART_INF_F;
+    const float ps0 = lane < n_chunks ? vp.part_s[row * n_chunks + lane] : 0.f;
+    float mloc = pm0;
+    for (int c = lane + 32; c < n_chunks; c += 32) mloc = fmaxf(mloc, vp.part_m[row * n_chunks + c]);
+    const float M = warp_max(mloc);
+    double sloc = pm0 > -CUDART_INF_F ? (double)ps0 * exp((double)pm0 - (double)M) : 0.0;
+    for (int c = lane + 32; c < n_chunks; c += 32) {
+        const float mc = vp.part_m[row * n_chunks + c];
+        if (mc > -CUDART_INF_F) sloc += (double)vp.part_s[row * n_chunks + c] * exp((double)mc - (double)M);
+    }
+    const double S = warp_sum(sloc);
+    return (double)M + log(S);
+}
+
+// One warp merges a row's chunk records into its top-k and hands candidate `rank` to put(rank, logit, token); meanwhile() runs
+// while the records are on their way.  pv_s / pi_s: the warp's copy of the records (staged), lk: kSurvCap keys.
 // A warp works on its row alone, and on its own its time is the number of instructions it
 // issues one after the other plus what its shuffles wait for the ones of the other rows (an SM passes one
 // warp's shuffle a clock).  So the chunk heads and the survivors are ranked from shared memory, four and two
 // to a broadcast load, the records are filtered flat (a lane takes every 32nd entry, whatever its chunk), and
 // the only shuffles left are those of the log-normaliser.
-template <typename Put>
-__device__ __forceinline__ void merge_row(const VocabPassParams& vp, size_t row, bool staged, float* pv_s, int* pi_s, unsigned long long* lk, Put put) {
+template <typename Meanwhile, typename Put>
+__device__ __forceinline__ void merge_row(const VocabPassParams& vp, size_t row, bool staged, float* pv_s, int* pi_s, unsigned long long* lk, Meanwhile meanwhile, Put put) {
     const int lane = threadIdx.x & 31, k = vp.k, n_chunks = vp.n_chunks, per_row = n_chunks * k;
     const float* gv = vp.part_v + row * per_row;
     const int* gi = vp.part_i + row * per_row;
@@ -86,19 +103,7 @@ __device__ __forceinline__ void merge_row(const VocabPassParams& vp, size_t row,
             for (int e = lane; e < per_row; e += 32) { cp_async4(pv_s + e, gv + e); cp_async4(pi_s + e, gi + e); }
         }
     }
-    // log-sum-exp over the chunks in fp64
-    const float pm0 = lane < n_chunks ? vp.part_m[row * n_chunks + lane] : -CUDART_INF_F;
-    const float ps0 = lane < n_chunks ? vp.part_s[row * n_chunks + lane] : 0.f;
-    float mloc = pm0;
-    for (int c = lane + 32; c < n_chunks; c += 32) mloc = fmaxf(mloc, vp.part_m[row * n_chunks + c]);
-    const float M = warp_max(mloc);
-    double sloc = pm0 > -CUDART_INF_F ? (double)ps0 * exp((double)pm0 - (double)M) : 0.0;
-    for (int c = lane + 32; c < n_chunks; c += 32) {
-        const float mc = vp.part_m[row * n_chunks + c];
-        if (mc > -CUDART_INF_F) sloc += (double)vp.part_s[row * n_chunks + c] * exp((double)mc - (double)M);
-    }
-    const double S = warp_sum(sloc);
-    const double lse = (double)M + log(S);
+    meanwhile();
     bool merged = false;
     if (staged) {
         cp_async_wait_all();
@@ -146,9 +151,9 @@ __device__ __forceinline__ void merge_row(const VocabPassParams& vp, size_t row,
                     const ulonglong2 kk = *reinterpret_cast<const ulonglong2*>(lk + j);
                     rank += (kk.x > ck ? 1 : 0) + (kk.y > ck ? 1 : 0);
                 }
-                if (rank < k) put(rank, key_value(ck), key_index(ck), lse);
+                if (rank < k) put(rank, key_value(ck), key_index(ck));
             }
-            for (int e = total + lane; e < k; e += 32) put(e, -CUDART_INF_F, 0x7fffffff, lse);   // (only with NaN logits)
+            for (int e = total + lane; e < k; e += 32) put(e, -CUDART_INF_F, 0x7fffffff);   // (only with NaN logits)
             merged = true;
         }
         __syncwarp();
@@ -171,7 +176,7 @@ __device__ __forceinline__ void merge_row(const VocabPassParams& vp, size_t row,
                 thr_i = top.index_at(k - 1);
             }
         }
-        if (lane < k) put(lane, top.v, top.i, lse);
+        if (lane < k) put(lane, top.v, top.i);
     }
 }
 
