@@ -103,32 +103,27 @@ __device__ __forceinline__ void merge_row(const VocabPassParams& vp, size_t row,
             for (int e = lane; e < per_row; e += 32) { cp_async4(pv_s + e, gv + e); cp_async4(pi_s + e, gi + e); }
         }
     }
+    const int lists = min(n_chunks, 32), depth = lane / lists, first = (lane - depth * lists) * k + depth;
     meanwhile();
     bool merged = false;
     if (staged) {
         cp_async_wait_all();
         __syncwarp();
-        // The k-th best chunk head (best head of every 32nd chunk, if there are more than 32) bounds the row's
-        // k-th best value from below; without that many chunks, the worst of all lists' j-th entries does,
-        // where the lists' first j entries are at least k.
-        float tv;
-        if (n_chunks >= k) {
-            float hv = lane < n_chunks ? pv_s[lane * k] : -CUDART_INF_F;
-            for (int c = lane + 32; c < n_chunks; c += 32) hv = fmaxf(hv, pv_s[c * k]);
-            s_heads[lane] = hv;
-            __syncwarp();
-            int above = 0;
+        // The k-th best of 32 entries bounds the row's k-th best value from below: the first 32 / n_chunks entries of every list,
+        // or the chunk heads (the best head of every 32nd chunk, if there are more than 32).  A bound from the lists'
+        // j-th entries let twice as many through where there are fewer lists than k (41 rows of 70000 in 9 lists: 59.2 -> 55.5 us a step).
+        float hv = depth < k ? pv_s[first] : -CUDART_INF_F;
+        for (int c = lane + 32; c < n_chunks; c += 32) hv = fmaxf(hv, pv_s[c * k]);
+        s_heads[lane] = hv;
+        __syncwarp();
+        int above = 0;
 #pragma unroll
-            for (int o = 0; o < 32; o += 4) {
-                const float4 h4 = *reinterpret_cast<const float4*>(s_heads + o);
-                above += (h4.x > hv ? 1 : 0) + (h4.y > hv ? 1 : 0) + (h4.z > hv ? 1 : 0) + (h4.w > hv ? 1 : 0);
-            }
-            tv = warp_min_value(lane < n_chunks && above < k ? hv : CUDART_INF_F);
-            __syncwarp();
-        } else {
-            const int jth = (k + n_chunks - 1) / n_chunks;
-            tv = warp_min_value(lane < n_chunks ? pv_s[lane * k + jth - 1] : CUDART_INF_F);
+        for (int o = 0; o < 32; o += 4) {
+            const float4 h4 = *reinterpret_cast<const float4*>(s_heads + o);
+            above += (h4.x > hv ? 1 : 0) + (h4.y > hv ? 1 : 0) + (h4.z > hv ? 1 : 0) + (h4.w > hv ? 1 : 0);
         }
+        const float tv = warp_min_value(depth < k && above < k ? hv : CUDART_INF_F);
+        __syncwarp();
         int total = 0;
 #pragma unroll 4
         for (int e0 = 0; e0 < per_row; e0 += 32) {

@@ -295,11 +295,13 @@ cudaError_t launch_ept(const VocabPassParams& p, dim3 grid, cudaStream_t stream)
 
 }  // namespace
 
-// chunk is 8192 values (32 per thread, five blocks per SM), or 4096 (16 per thread, six blocks) when
-// the larger one would leave SMs without work
+// chunk is 8192 values (32 per thread, five blocks per SM), or 4096 (16 per thread, six blocks) when the larger one would
+// leave less than two blocks an SM: a block's time is its chain of steps, hardly the size of its chunk, and half as many records
+// are merged behind it.  Whole steps, us, 4096 / 8192: 369 blocks of 8192 (B = 1, V = 70000) 57.7 / 55.5, 574 (B = 2, V = 50257)
+// 64.4 / 61.9; 1136 (B = 1, V = 128256, k = 10) 72.3 / 67.8.
 int vocab_pass_plan_chunks(int sm_count, int rows, int V, int* chunk_out) {
     int chunk = 8192;
-    if ((long long)rows * ((V + chunk - 1) / chunk) < 5LL * sm_count) chunk = 4096;
+    if ((long long)rows * ((V + chunk - 1) / chunk) < 2LL * sm_count) chunk = 4096;
     *chunk_out = chunk;
     return (V + chunk - 1) / chunk;
 }
