@@ -11,6 +11,7 @@
 //                W_{j+1} = sum_v max(0, p(v) - a(v) q(v)).  This is the rectify / remove / renormalise
 //                recursion of Eq. 2 unrolled, so each rejection costs one read-only pass.
 #include <algorithm>
+#include <cfloat>
 #include <cmath>
 
 #include "common.cuh"
@@ -190,8 +191,17 @@ __device__ __forceinline__ double exp64(double x, const double* tab) {
 // exponential costs the pipe that bounds this, and a branch behind each keeps the chains from overlapping)
 struct ExpRange {
     double invT, shift;
-    float lo, hi;                        // logits between which |z / T + shift| stays below 700
+    float lo, hi;                        // finite logits between which |z / T + shift| stays below 700
+    // Around the logit `ref`.  Both bounds are rounded towards it: with a small T an ulp of the logits is many units of z / T,
+    // and a bound rounded away from it would let such a logit through.
+    __device__ __forceinline__ ExpRange(double invT_, float ref) : invT(invT_), shift(-((double)ref * invT_)) {
+        const double reach = 690.0 / invT_;
+        lo = fmaxf(__double2float_ru((double)ref - reach), -FLT_MAX);
+        hi = fminf(__double2float_rd((double)ref + reach), FLT_MAX);
+    }
     __device__ __forceinline__ double arg(float z) const { return fma((double)z, invT, shift); }
+    // of any logit (-inf: 0, also where 1 / T has become 0)
+    __device__ __forceinline__ double exp_of(float z, const double* tab) const { return z == -CUDART_INF_F ? 0.0 : exp64(arg(z), tab); }
 };
 template <int Q>
 __device__ __forceinline__ void exp64_quads(const float (&z)[Q][4], const ExpRange& X, const double* tab, double (&e)[Q][4]) {
@@ -210,7 +220,7 @@ __device__ __forceinline__ void exp64_quads(const float (&z)[Q][4], const ExpRan
 #pragma unroll
         for (int q = 0; q < Q; ++q)
 #pragma unroll
-            for (int i = 0; i < 4; ++i) e[q][i] = exp64(X.arg(z[q][i]), tab);
+            for (int i = 0; i < 4; ++i) e[q][i] = X.exp_of(z[q][i], tab);
     }
 }
 
@@ -450,15 +460,13 @@ __device__ double2 softmax_rows(NodeShared& S, ClusterRed& red, const T* target,
     rt = warp_max(rt);
     rd = warp_max(rd);
     const double* tab = S.exps.mine();
-    // logits within 690 T of the reference are in range
-    const float reach = (float)(690.0 / invT);
     for (int pass = 0;; ++pass) {
-        const double nt = -((double)rt * invT), nd = -((double)rd * invT);
-        const double st = slice_exp(target, v0, v1, ExpRange{invT, nt, rt - reach, rt + reach}, tab, C, 0, ft);
-        const double sd = two ? slice_exp(draft, v0, v1, ExpRange{invT, nd, rd - reach, rd + reach}, tab, C, 1, fd) : 1.0 / (kMaxCluster * kSThreads);
+        const ExpRange Xt(invT, rt), Xd(invT, rd);
+        const double st = slice_exp(target, v0, v1, Xt, tab, C, 0, ft);
+        const double sd = two ? slice_exp(draft, v0, v1, Xd, tab, C, 1, fd) : 1.0 / (kMaxCluster * kSThreads);
         if (child) {
-            S.pe[tid] = exp64(fma((double)xt, invT, nt), tab);
-            S.qe[tid] = two ? exp64(fma((double)xd, invT, nd), tab) : 0.0;
+            S.pe[tid] = Xt.exp_of(xt, tab);
+            S.qe[tid] = two ? Xd.exp_of(xd, tab) : 0.0;
         }
         red.send(warp_sum(st), warp_sum(sd));
         if (pass == 0) meanwhile();
