@@ -214,29 +214,52 @@ __device__ __forceinline__ void mma_ts_x4(uint32_t pred, uint32_t nsteps, uint32
         : "memory");
 #undef RADAR_TS_STEP
 }
-//   TS, all four steps, no per-step predicate.
-__device__ __forceinline__ void mma_ts_x4_full(uint32_t pred, uint32_t d_tmem, uint32_t a_tmem, uint32_t b_lo, uint32_t hi,
-                                               uint32_t idesc, bool acc_first) {
-#define RADAR_TS_STEP(K, P)                                                                            \
-        "add.u32 a, %2, " #K " * 8;\n\tadd.u32 b, %3, " #K " * 128;\n\tmov.b64 db, {b, %4};\n\t"         \
-        "@q tcgen05.mma.cta_group::1.kind::f16 [%1], [a], db, %5, " #P ";\n\t"
-    asm volatile(
-        "{\n\t.reg .pred q, p0, p1;\n\t.reg .b32 a, b;\n\t.reg .b64 db;\n\t"
-        "setp.ne.b32 q, %0, 0;\n\t"
-        "setp.ne.b32 p0, %6, 0;\n\t"
-        "setp.eq.b32 p1, 0, 0;\n\t"
-        RADAR_TS_STEP(0, p0) RADAR_TS_STEP(1, p1) RADAR_TS_STEP(2, p1) RADAR_TS_STEP(3, p1)
-        "}"
-        ::"r"(pred), "r"(d_tmem), "r"(a_tmem), "r"(b_lo), "r"(hi), "r"(idesc), "r"((uint32_t)acc_first)
-        : "memory");
-#undef RADAR_TS_STEP
-}
 //   TS, two steps of each half of a 128-key tile (64 columns of A, 64 rows of B apart).
 __device__ __forceinline__ void mma_ts_x2x2_full(uint32_t pred, uint32_t d_tmem, uint32_t a_tmem, uint32_t b_lo, uint32_t hi,
                                                  uint32_t idesc, bool acc_first) {
 #define RADAR_TS_STEP(A, B, P)                                                                         \
         "add.u32 a, %2, " #A ";\n\tadd.u32 b, %3, " #B ";\n\tmov.b64 db, {b, %4};\n\t"                 \
         "@q tcgen05.mma.cta_group::1.kind::f16 [%1], [a], db, %5, " #P ";\n\t"
+    asm volatile(
+        "{\n\t.reg .pred q, p0, p1;\n\t.reg .b32 a, b;\n\t.reg .b64 db;\n\t"
+        "setp.ne.b32 q, %0, 0;\n\t"
+        "setp.ne.b32 p0, %6, 0;\n\t"
+        "setp.eq.b32 p1, 0, 0;\n\t"
+        RADAR_TS_STEP(0, 0, p0) RADAR_TS_STEP(8, 128, p1) RADAR_TS_STEP(64, 512, p1) RADAR_TS_STEP(72, 640, p1)
+        "}"
+        ::"r"(pred), "r"(d_tmem), "r"(a_tmem), "r"(b_lo), "r"(hi), "r"(idesc), "r"((uint32_t)acc_first)
+        : "memory");
+#undef RADAR_TS_STEP
+}
+//   TS with A = hi + lo, two bf16 matrices side by side: 32 keys are 16 columns of hi, then 16 of lo.  A 64-key half, `nsteps`
+//   of its four steps.
+__device__ __forceinline__ void mma_ts_two_x4(uint32_t pred, uint32_t nsteps, uint32_t d_tmem, uint32_t a_tmem, uint32_t b_lo,
+                                              uint32_t hi, uint32_t idesc, bool acc_first) {
+#define RADAR_TS_STEP(K, A, P)                                                                         \
+        "setp.gt.and.u32 qk, %1, " #K ", q;\n\t"                                                        \
+        "add.u32 a, %3, " #A ";\n\tadd.u32 b, %4, " #K " * 128;\n\tmov.b64 db, {b, %5};\n\t"         \
+        "@qk tcgen05.mma.cta_group::1.kind::f16 [%2], [a], db, %6, " #P ";\n\t"                         \
+        "add.u32 a, a, 16;\n\t"                                                                         \
+        "@qk tcgen05.mma.cta_group::1.kind::f16 [%2], [a], db, %6, p1;\n\t"
+    asm volatile(
+        "{\n\t.reg .pred q, qk, p0, p1;\n\t.reg .b32 a, b;\n\t.reg .b64 db;\n\t"
+        "setp.ne.b32 q, %0, 0;\n\t"
+        "setp.ne.b32 p0, %7, 0;\n\t"
+        "setp.eq.b32 p1, 0, 0;\n\t"
+        RADAR_TS_STEP(0, 0, p0) RADAR_TS_STEP(1, 8, p1) RADAR_TS_STEP(2, 32, p1) RADAR_TS_STEP(3, 40, p1)
+        "}"
+        ::"r"(pred), "r"(nsteps), "r"(d_tmem), "r"(a_tmem), "r"(b_lo), "r"(hi), "r"(idesc), "r"((uint32_t)acc_first)
+        : "memory");
+#undef RADAR_TS_STEP
+}
+//   ... two steps of each half of a 128-key tile.
+__device__ __forceinline__ void mma_ts_two_x2x2_full(uint32_t pred, uint32_t d_tmem, uint32_t a_tmem, uint32_t b_lo, uint32_t hi,
+                                                     uint32_t idesc, bool acc_first) {
+#define RADAR_TS_STEP(A, B, P)                                                                         \
+        "add.u32 a, %2, " #A ";\n\tadd.u32 b, %3, " #B ";\n\tmov.b64 db, {b, %4};\n\t"                 \
+        "@q tcgen05.mma.cta_group::1.kind::f16 [%1], [a], db, %5, " #P ";\n\t"                          \
+        "add.u32 a, a, 16;\n\t"                                                                         \
+        "@q tcgen05.mma.cta_group::1.kind::f16 [%1], [a], db, %5, p1;\n\t"
     asm volatile(
         "{\n\t.reg .pred q, p0, p1;\n\t.reg .b32 a, b;\n\t.reg .b64 db;\n\t"
         "setp.ne.b32 q, %0, 0;\n\t"

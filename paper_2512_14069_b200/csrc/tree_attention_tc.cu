@@ -31,6 +31,8 @@
 #include <cuda.h>
 
 #include <algorithm>
+#include <cmath>
+#include <type_traits>
 
 #include "common.cuh"
 #include "tc05.cuh"
@@ -74,8 +76,9 @@ struct TcParams {
     int ncc;             // CTAs per class; grid = n_cls * ncc
     int cost_one, cost_two, unit_cost;   // tile_costs(n_cls)
     float scale_log2;
+    float scale_log2_lo; // FINE: what scale_log2 is below the scale itself (positive)
     long long cache_rows;
-    float2* part_ml;     // [grid][2][256]     (m in natural-log units, l)
+    float2* part_ml;     // [grid][2][256]     (m in natural-log units, with FINE in log2 units; l)
     float* part_o;       // [grid][2][256][D]
     CutUnit* cut;        // [grid]
     int* status;
@@ -97,6 +100,11 @@ __device__ __forceinline__ float ex2(float x) {
     float y;
     asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
     return y;
+}
+// m ln 2 + ln l, m in log2 units
+__device__ __forceinline__ float lse_of(float m, float l) {
+    constexpr float kHi = 0.693147182f, kLo = (float)(0.6931471805599453 - (double)kHi);
+    return fmaf(m, kHi, fmaf(m, kLo, logf(l)));
 }
 
 // ---- the tile space of one class (unit index pp within a KV head) ---------------------------------
@@ -192,7 +200,11 @@ struct Smem {
 // TWO: the launch may contain units with two live row blocks; decides the shared-memory layout
 // PAGED: the prefix cache is read through a block table (a separate instantiation, so that the contiguous
 // layout's code is not touched by it)
-template <int D, bool TWO, bool PAGED>
+// FINE: P goes to the tensor cores as the sum of two bf16 numbers (its value to 2^-18) in place of one (2^-9), and the scores'
+// scale is applied in two parts.  For the head ratios that do not divide 128: they came from the FMA kernel, whose
+// probabilities are fp32, and keep its precision here (error against fp64, 2-norm, of 24 / 8 heads, 2048 tokens: FMA 1.6545e-3,
+// one bf16 2.1607e-3, two 1.6545e-3, all of it the rounding of O to bf16).
+template <int D, bool TWO, bool PAGED, bool FINE>
 __global__ void __launch_bounds__(kTcThreads, 1)      // 18 warps are allocated as 20: 96 registers per thread
 tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmKc,
                     const __grid_constant__ CUtensorMap tmVc, const __grid_constant__ CUtensorMap tmKt,
@@ -522,8 +534,13 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
                 // at column 64 (each softmax thread writes inside its own column range)
                 const int hs = tree ? 2 : 4;
                 const uint32_t n1 = (uint32_t)min(ksteps, hs), n2 = (uint32_t)ksteps - n1;
-                mma_ts_x4(go, n1, tmem + 256 + q * 128, tmem + q * 128, b_lo, kDescHi, idesc_pv, acc[q]);
-                mma_ts_x4(go, n2, tmem + 256 + q * 128, tmem + q * 128 + 64, b_lo + hs * 128, kDescHi, idesc_pv, true);
+                if (FINE) {
+                    mma_ts_two_x4(go, n1, tmem + 256 + q * 128, tmem + q * 128, b_lo, kDescHi, idesc_pv, acc[q]);
+                    mma_ts_two_x4(go, n2, tmem + 256 + q * 128, tmem + q * 128 + 64, b_lo + hs * 128, kDescHi, idesc_pv, true);
+                } else {
+                    mma_ts_x4(go, n1, tmem + 256 + q * 128, tmem + q * 128, b_lo, kDescHi, idesc_pv, acc[q]);
+                    mma_ts_x4(go, n2, tmem + 256 + q * 128, tmem + q * 128 + 64, b_lo + hs * 128, kDescHi, idesc_pv, true);
+                }
                 acc[q] = true;
                 if (release_v) mma_commit_if(go, &bar_vempty[v_slot]);
                 if (two ? i == n - 1 : i + 2 >= n) mma_commit_if(go, &bar_odone[q]);
@@ -566,12 +583,14 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
                 }
                 tc_fence_after_sync();
                 const uint32_t b_lo = (v_lo + v_slot * (SM::kTileBytes >> 4)) | ((uint32_t)(kTileKeys * 128 >> 4) << 16);
-                mma_ts_x2x2_full(ok ? elected : 0u, tmem + 256 + q * 128, tmem + q * 128, b_lo, kDescHi, idesc_pv, acc[q]);
+                if (FINE) mma_ts_two_x2x2_full(ok ? elected : 0u, tmem + 256 + q * 128, tmem + q * 128, b_lo, kDescHi, idesc_pv, acc[q]);
+                else mma_ts_x2x2_full(ok ? elected : 0u, tmem + 256 + q * 128, tmem + q * 128, b_lo, kDescHi, idesc_pv, acc[q]);
                 wait_all(&bar_pready[q], p_par[q]);
                 p_par[q] ^= 1;
                 tc_fence_after_sync();
                 const uint32_t go = ok ? elected : 0u;
-                mma_ts_x2x2_full(go, tmem + 256 + q * 128, tmem + q * 128 + 16, b_lo + 2 * 128, kDescHi, idesc_pv, true);
+                if (FINE) mma_ts_two_x2x2_full(go, tmem + 256 + q * 128, tmem + q * 128 + 32, b_lo + 2 * 128, kDescHi, idesc_pv, true);
+                else mma_ts_x2x2_full(go, tmem + 256 + q * 128, tmem + q * 128 + 16, b_lo + 2 * 128, kDescHi, idesc_pv, true);
                 acc[q] = true;
                 if (release_v) mma_commit_if(go, &bar_vempty[v_slot]);
             };
@@ -671,8 +690,8 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
                 // This thread's chunks of 32 score columns: a prefix tile has four (two per thread), the tree tile
                 // two (one per thread).  Half h of a row works in columns 64 h .. 64 h + 63 of the buffer only: its
                 // scores sit there (the tree tile's second chunk is read from columns 32 .. 63 but belongs to
-                // half 1 alone) and its P goes to columns 64 h + 16 cc, so the halves never touch each other's
-                // columns and a thread overwrites only scores it has already taken into registers.
+                // half 1 alone) and its P goes to columns 64 h + 16 cc (FINE: 64 h + 32 cc, 16 of each part), so the halves
+                // never touch each other's columns and a thread overwrites only scores it has already taken into registers.
                 const bool tree = t == nt_unit - 1;
                 const int nch = tree ? 1 : 2;
                 const int c0 = tree ? half : 2 * half;
@@ -746,16 +765,23 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
                             for (int e = 0; e < 32; ++e)
                                 if (!((al >> e) & 1u)) sv[e] = 0xff800000u;
                         }
-                        uint32_t pk[16];
+                        uint32_t pk[16], pl[FINE ? 16 : 1];
 #pragma unroll
                         for (int e = 0; e < 16; ++e) {
-                            const float2 t = __ffma2_rn(make_float2(__uint_as_float(sv[2 * e]), __uint_as_float(sv[2 * e + 1])), sc2, nm2);
+                            const float2 s2 = make_float2(__uint_as_float(sv[2 * e]), __uint_as_float(sv[2 * e + 1]));
+                            float2 t = __ffma2_rn(s2, sc2, nm2);
+                            if (FINE) t = __ffma2_rn(s2, make_float2(P.scale_log2_lo, P.scale_log2_lo), t);
                             const float p0 = ex2(t.x), p1 = ex2(t.y);
                             ls[e & 1] = __fadd2_rn(ls[e & 1], make_float2(p0, p1));
                             const __nv_bfloat162 v = __floats2bfloat162_rn(p0, p1);
                             pk[e] = *reinterpret_cast<const uint32_t*>(&v);
+                            if (FINE) {
+                                const __nv_bfloat162 r = __floats2bfloat162_rn(p0 - __uint_as_float(pk[e] << 16), p1 - __uint_as_float(pk[e] & 0xffff0000u));
+                                pl[FINE ? e : 0] = *reinterpret_cast<const uint32_t*>(&r);
+                            }
                         }
-                        tmem_st16(tS + half * 64 + cc * 16, pk);
+                        tmem_st16(tS + half * 64 + cc * (FINE ? 32 : 16), pk);
+                        if constexpr (FINE) tmem_st16(tS + half * 64 + cc * 32 + 16, pl);
                         if (cc == 0) {
                             tmem_wait_st();
                             tc_fence_before_sync();
@@ -858,9 +884,9 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
                 if (row_live && half == 0) {
                     const float m_nat = m_safe * 0.6931471805599453f;
                     if (final_rows) {
-                        if (a.lse != nullptr) a.lse[cur.layer * P.lse_ls + ((int64_t)b * a.Hq + hq) * kMaxNodes + node] = m_nat + logf(l_out);
+                        if (a.lse != nullptr) a.lse[cur.layer * P.lse_ls + ((int64_t)b * a.Hq + hq) * kMaxNodes + node] = FINE ? lse_of(m_safe, l_out) : m_nat + logf(l_out);
                     } else {
-                        P.part_ml[rec] = make_float2(m_out == -CUDART_INF_F ? -CUDART_INF_F : m_nat, l_out);
+                        P.part_ml[rec] = make_float2(FINE || m_out == -CUDART_INF_F ? m_out : m_nat, l_out);
                     }
                 }
             }
@@ -896,9 +922,10 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
 // segment.  A warp merges one query row, every piece of it in flight together: the work is a chain of three trips to L2,
 // and many warps hide it better than many rows a warp do (148 cut units of 256 rows: 17.1 us event-timed with one row a
 // warp, 18.4 with two, 20.6 with four; 72 cut units of 128 rows: 10.0, 10.8, 14.7).
-template <int D>
+template <int D, bool FINE>
 __global__ void __launch_bounds__(256) tree_attn_tc_combine_kernel(const TcParams P) {
     chain_wait();
+    auto weight = [](float d) { return FINE ? ex2(d) : __expf(d); };      // of two pieces' maxima that differ by d
     const radar_attn_args& a = P.a;
     const CutUnit& cu = P.cut[blockIdx.x];
     const int valid = cu.valid, b = cu.b, g = cu.g, layer = cu.layer, slot = cu.slot, rows = cu.rows, n_pieces = cu.n_pieces;
@@ -924,7 +951,7 @@ __global__ void __launch_bounds__(256) tree_attn_tc_combine_kernel(const TcParam
         for (int q = 0; q < E; q += 2) w[q / 2] = __floats2bfloat162_rn(o[q] * inv, o[q + 1] * inv);
         if (E == 4) *reinterpret_cast<uint2*>(dst) = *reinterpret_cast<const uint2*>(w);
         else *reinterpret_cast<uint32_t*>(dst) = *reinterpret_cast<const uint32_t*>(w);
-        if (a.lse != nullptr && lane == 0) a.lse[layer * P.lse_ls + ((int64_t)b * a.Hq + hq) * kMaxNodes + node] = mx + logf(den);
+        if (a.lse != nullptr && lane == 0) a.lse[layer * P.lse_ls + ((int64_t)b * a.Hq + hq) * kMaxNodes + node] = FINE ? lse_of(mx, den) : mx + logf(den);
     };
     auto load_row = [&](const float* src, float (&v)[E]) {
         if (E == 4) {
@@ -955,7 +982,7 @@ __global__ void __launch_bounds__(256) tree_attn_tc_combine_kernel(const TcParam
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
             if (ml[j].x == -CUDART_INF_F) continue;
-            const float w = __expf(ml[j].x - mx);
+            const float w = weight(ml[j].x - mx);
             den = fmaf(ml[j].y, w, den);
 #pragma unroll
             for (int q = 0; q < E; ++q) o[q] = fmaf(v[j][q], w, o[q]);
@@ -975,12 +1002,12 @@ __global__ void __launch_bounds__(256) tree_attn_tc_combine_kernel(const TcParam
         if (jl < n_pieces && ((live >> lane) & 1u)) ml = P.part_ml[rec_of(jl)];
         const float mnew = fmaxf(mx, warp_max(ml.x));
         if (mnew == -CUDART_INF_F) continue;
-        const float rescale = __expf(mx - mnew);             // 0 on the first live batch
+        const float rescale = weight(mx - mnew);             // 0 on the first live batch
         den *= rescale;
 #pragma unroll
         for (int q = 0; q < E; ++q) o[q] *= rescale;
         mx = mnew;
-        const float wl = ml.x == -CUDART_INF_F ? 0.f : __expf(ml.x - mx);
+        const float wl = ml.x == -CUDART_INF_F ? 0.f : weight(ml.x - mx);
         den += warp_sum(ml.y * wl);
         const int nb = min(32, n_pieces - j0);
         for (int u0 = 0; u0 < nb; u0 += 4) {
@@ -1105,7 +1132,7 @@ size_t tree_attn_tc_workspace_bytes(const radar_ctx* ctx, int B, int Hq, int Hkv
     return partial_bytes((size_t)std::max(n_cls * ncc, ctx->sm_count), d);
 }
 
-template <int D, bool TWO, bool PAGED>
+template <int D, bool TWO, bool PAGED, bool FINE>
 static int launch_tc(radar_ctx* ctx, TcParams& P, cudaStream_t stream) {
     const radar_attn_args& a = P.a;
     CUtensorMap tmQ, tmKc, tmVc, tmKt, tmVt;
@@ -1121,17 +1148,17 @@ static int launch_tc(radar_ctx* ctx, TcParams& P, cudaStream_t stream) {
         !make_map(&tmVc, have_prefix ? a.Vc : a.Vt, D, a.Hkv, have_prefix ? a.cache_rows : tree_rows, 1, cache_box, L,
                   have_prefix ? a.cache_layer_stride : a.tree_kv_layer_stride))
         return RADAR_ERR_CUDA;
-    RADAR_CUDA_CHECK(radar_opt_in_smem(ctx, RADAR_SMEM_ATTN_TC + 4 * (D == 128) + 2 * TWO + PAGED, tree_attn_tc_kernel<D, TWO, PAGED>,
+    RADAR_CUDA_CHECK(radar_opt_in_smem(ctx, RADAR_SMEM_ATTN_TC + 8 * FINE + 4 * (D == 128) + 2 * TWO + PAGED, tree_attn_tc_kernel<D, TWO, PAGED, FINE>,
                                        (size_t)Smem<D, TWO>::kDynamic));
     {
         radar_launch_scope scope(ctx, RADAR_K_ATTN, stream);
-        RADAR_CUDA_CHECK(launch_chained(tree_attn_tc_kernel<D, TWO, PAGED>, dim3((unsigned)(P.n_cls * P.ncc)), dim3(kTcThreads),
+        RADAR_CUDA_CHECK(launch_chained(tree_attn_tc_kernel<D, TWO, PAGED, FINE>, dim3((unsigned)(P.n_cls * P.ncc)), dim3(kTcThreads),
                                         (size_t)Smem<D, TWO>::kDynamic, stream, tmQ, tmKc, tmVc, tmKt, tmVt, P));
     }
     RADAR_CUDA_CHECK(cudaGetLastError());
     {
         radar_launch_scope scope(ctx, RADAR_K_ATTN_COMBINE, stream);
-        RADAR_CUDA_CHECK(launch_chained(tree_attn_tc_combine_kernel<D>, dim3((unsigned)(P.n_cls * P.ncc), kPairRows / 8), dim3(256), 0, stream, P));
+        RADAR_CUDA_CHECK(launch_chained(tree_attn_tc_combine_kernel<D, FINE>, dim3((unsigned)(P.n_cls * P.ncc), kPairRows / 8), dim3(256), 0, stream, P));
     }
     RADAR_CUDA_CHECK(cudaGetLastError());
     return RADAR_OK;
@@ -1145,7 +1172,14 @@ int tree_attn_tc_launch(radar_ctx* ctx, const radar_attn_args* a, cudaStream_t s
     P.nodes_per_rb = 128 / P.G;
     P.rb_rows = P.nodes_per_rb * P.G;
     const float scale = a->scale > 0.f ? a->scale : 1.f / sqrtf((float)a->d);
+    const bool fine = 128 % P.G != 0;
     P.scale_log2 = scale * 1.4426950408889634f;
+    P.scale_log2_lo = 0.f;
+    if (fine) {                          // the second part positive: a score of -inf (a masked one) stays -inf
+        const double exact = (a->scale > 0.f ? (double)a->scale : 1.0 / std::sqrt((double)a->d)) * 1.4426950408889634;
+        if ((double)P.scale_log2 >= exact) P.scale_log2 = std::nextafterf(P.scale_log2, 0.f);
+        P.scale_log2_lo = (float)(exact - (double)P.scale_log2);
+    }
     P.cache_rows = a->cache_rows;
     P.status = ctx->d_status;
     P.n_layers = a->n_layers > 1 ? a->n_layers : 1;
@@ -1163,12 +1197,16 @@ int tree_attn_tc_launch(radar_ctx* ctx, const radar_attn_args* a, cudaStream_t s
     P.part_o = reinterpret_cast<float*>(reinterpret_cast<char*>(a->workspace) + align_up(rec * sizeof(float2), 256));
     P.cut = reinterpret_cast<CutUnit*>(reinterpret_cast<char*>(P.part_o) + align_up(rec * a->d * sizeof(float), 256));
     const bool two = P.n_blk > 1 && P.nodes_per_rb < kMaxNodes;       // some unit can have two live row blocks
-    if (a->block_table != nullptr) {
-        if (a->d == 128) return two ? launch_tc<128, true, true>(ctx, P, stream) : launch_tc<128, false, true>(ctx, P, stream);
-        return two ? launch_tc<64, true, true>(ctx, P, stream) : launch_tc<64, false, true>(ctx, P, stream);
-    }
-    if (a->d == 128) return two ? launch_tc<128, true, false>(ctx, P, stream) : launch_tc<128, false, false>(ctx, P, stream);
-    return two ? launch_tc<64, true, false>(ctx, P, stream) : launch_tc<64, false, false>(ctx, P, stream);
+    auto launch = [&](auto d, auto fine_c) {
+        constexpr int D = decltype(d)::value;
+        constexpr bool F = decltype(fine_c)::value;
+        if (a->block_table != nullptr) return two ? launch_tc<D, true, true, F>(ctx, P, stream) : launch_tc<D, false, true, F>(ctx, P, stream);
+        return two ? launch_tc<D, true, false, F>(ctx, P, stream) : launch_tc<D, false, false, F>(ctx, P, stream);
+    };
+    using d64 = std::integral_constant<int, 64>;
+    using d128 = std::integral_constant<int, 128>;
+    if (a->d == 128) return fine ? launch(d128{}, std::true_type{}) : launch(d128{}, std::false_type{});
+    return fine ? launch(d64{}, std::true_type{}) : launch(d64{}, std::false_type{});
 }
 
 }  // namespace radar
