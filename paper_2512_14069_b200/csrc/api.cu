@@ -24,7 +24,7 @@ extern "C" int radar_create(radar_ctx** out, int device) {
     c->ev_kernel = nullptr;
     c->ev_cap = c->ev_used = 0;
     for (int i = 0; i < RADAR_K_COUNT; ++i) { c->launches[i] = 0; c->prof_ms[i] = 0.0; c->prof_n[i] = 0; }
-    for (int i = 0; i < RADAR_SMEM_COUNT; ++i) c->smem_opt_in[i] = 0;
+    for (int i = 0; i < RADAR_SMEM_COUNT; ++i) c->smem_room[i] = 0;
     for (int i = 0; i < 16; ++i) c->acclen_clusters[i / 4][i % 4] = 0;
     if (cudaDeviceGetAttribute(&c->sm_count, cudaDevAttrMultiProcessorCount, device) != cudaSuccess ||
         cudaMalloc(&c->d_status, 2 * sizeof(int)) != cudaSuccess ||

@@ -30,7 +30,7 @@ enum radar_kernel_id {
     RADAR_K_COUNT
 };
 
-// kernels that opt in to more than 48 KB of dynamic shared memory: one slot per instantiation
+// kernels whose blocks may take more than 48 KB of shared memory: one slot per instantiation
 enum radar_smem_slot {
     RADAR_SMEM_SELECT_GATE = 0,
     RADAR_SMEM_SELECT_GATE_CLUSTER,   // the instantiation with helper blocks
@@ -48,9 +48,9 @@ enum radar_smem_slot {
 struct radar_ctx {
     int device;
     int sm_count;
-    // largest dynamic shared-memory size opted in to so far, per kernel, ON THIS CONTEXT'S DEVICE (the attribute
-    // is per device: a second device in the same process needs its own opt-in)
-    size_t smem_opt_in[RADAR_SMEM_COUNT];
+    // dynamic shared memory opted in to, per kernel, ON THIS CONTEXT'S DEVICE (the attribute is per device: a second device
+    // in the same process needs its own opt-in); 0: not yet
+    size_t smem_room[RADAR_SMEM_COUNT];
     int* d_status;          // sticky device status word
     int acclen_clusters[4][4];   // clusters of 1, 2, 4, 8 of each per-row kernel of Eq. 11-13 that are resident at once (0: not asked yet)
     // launch accounting (host side)
@@ -114,19 +114,27 @@ __device__ __forceinline__ void chain_wait() {
 __device__ __forceinline__ void chain_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void chain_sync() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
-// A failing runtime call becomes RADAR_ERR_CUDA; with RADAR_DEBUG set in the environment the call and the
-// runtime's message are also written to stderr.
-// Raises a kernel's dynamic shared-memory limit on the context's device when `bytes` exceeds what has been
-// set there before (48 KB need no opt-in).  Not a stream operation.
+// Raises a kernel's dynamic shared-memory limit on the context's device, once, to all that its static arrays leave of a
+// block's shared memory.  (The 48 KB that need no opt-in count the static arrays too, so a limit that looks at the dynamic
+// bytes alone refuses launches; and the limit belongs to the kernel, not to the context: every context has to set the
+// same one, or a small launch of one would take the room from another.)  Not a stream operation.
 template <typename K>
 inline cudaError_t radar_opt_in_smem(radar_ctx* ctx, int slot, K kernel, size_t bytes) {
-    const size_t have = ctx->smem_opt_in[slot] > 48 * 1024 ? ctx->smem_opt_in[slot] : 48 * 1024;
-    if (bytes <= have) return cudaSuccess;
-    const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-    if (e == cudaSuccess) ctx->smem_opt_in[slot] = bytes;
-    return e;
+    size_t& room = ctx->smem_room[slot];
+    if (room == 0) {
+        cudaFuncAttributes fa;
+        int block = 0;
+        cudaError_t e = cudaFuncGetAttributes(&fa, kernel);
+        if (e == cudaSuccess) e = cudaDeviceGetAttribute(&block, cudaDevAttrMaxSharedMemoryPerBlockOptin, ctx->device);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, block - (int)fa.sharedSizeBytes);
+        if (e != cudaSuccess) return e;
+        room = (size_t)block - fa.sharedSizeBytes;
+    }
+    return bytes <= room ? cudaSuccess : cudaErrorInvalidValue;
 }
 
+// A failing runtime call becomes RADAR_ERR_CUDA; with RADAR_DEBUG set in the environment the call and the
+// runtime's message are also written to stderr.
 #define RADAR_CUDA_CHECK(expr)                                                                     \
     do {                                                                                           \
         cudaError_t _e = (expr);                                                                   \

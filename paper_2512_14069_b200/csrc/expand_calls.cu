@@ -516,7 +516,7 @@ extern "C" int radar_expand_calls(radar_ctx* ctx, const radar_expand_calls_args*
         cp.status = ctx->d_status;
         radar_launch_scope scope(ctx, RADAR_K_EXPAND_CALLS, stream);
         const int blocks = recurrent && gate_runs ? kSelCluster : 1;
-        const size_t smem = sizeof(float) * (size_t)((recurrent ? 4 : 1) * kHidden) * (a->k | 1);
+        const size_t smem = gate_runs ? sizeof(float) * (size_t)((recurrent ? 4 : 1) * kHidden) * (a->k | 1) : 0;
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3((unsigned)(a->B * blocks));
         cfg.blockDim = dim3(kSelThreads);
@@ -532,8 +532,7 @@ extern "C" int radar_expand_calls(radar_ctx* ctx, const radar_expand_calls_args*
         cfg.attrs = attr;
         cfg.numAttrs = blocks > 1 ? 2 : 1;
         if (blocks > 1) {
-            // (with the block's 23 KB of static shared memory the limit without an opt-in lies at 25 KB)
-            RADAR_CUDA_CHECK(radar_opt_in_smem(ctx, RADAR_SMEM_EXPAND_CALLS, expand_calls_kernel<true>, std::max(smem, (size_t)96 * 1024)));
+            RADAR_CUDA_CHECK(radar_opt_in_smem(ctx, RADAR_SMEM_EXPAND_CALLS, expand_calls_kernel<true>, smem));
             RADAR_CUDA_CHECK(cudaLaunchKernelEx(&cfg, expand_calls_kernel<true>, cp));
         } else {
             RADAR_CUDA_CHECK(radar_opt_in_smem(ctx, RADAR_SMEM_EXPAND_CALLS_PLAIN, expand_calls_kernel<false>, smem));
