@@ -257,6 +257,7 @@ cudaError_t vocab_pass_preload_argbest();
 int noalloc_prepare_device(int device);
 
 // --- tensor-core tree attention (tree_attention_tc.cu) --------------------------------------
+constexpr int kTcMaxRatio = 128;         // query heads per KV head: a row block holds whole nodes
 bool tree_attn_tc_supported(const radar_attn_args* a);
 size_t tree_attn_tc_workspace_bytes(const radar_ctx* ctx, int B, int Hq, int Hkv, int d, int max_prefix_len);
 int tree_attn_tc_launch(radar_ctx* ctx, const radar_attn_args* a, cudaStream_t stream);

@@ -342,7 +342,7 @@ extern "C" size_t radar_attn_workspace_bytes(const radar_ctx* ctx, int B, int Hq
     const size_t rec = (size_t)B * Hq * kMaxNodes * n_splits;
     size_t need = align_up(rec * sizeof(float2), 256) + align_up(rec * d * sizeof(float), 256);
     // the same buffer serves whichever kernel the call dispatches to
-    if (dtype == RADAR_BF16) need = std::max(need, tree_attn_tc_workspace_bytes(ctx, B, Hq, Hkv, d, max_prefix_len));
+    if (dtype == RADAR_BF16 && Hq / Hkv <= kTcMaxRatio) need = std::max(need, tree_attn_tc_workspace_bytes(ctx, B, Hq, Hkv, d, max_prefix_len));
     return need;
 }
 

@@ -1102,7 +1102,7 @@ void plan_grid(const radar_ctx* ctx, int B, int Hq, int Hkv, int max_prefix_len,
 bool tree_attn_tc_supported(const radar_attn_args* a) {
     if (a->dtype != RADAR_BF16 || (a->d != 64 && a->d != 128)) return false;
     const int G = a->Hq / a->Hkv;
-    if (G < 1 || G > 128) return false;
+    if (G < 1 || G > kTcMaxRatio) return false;
     // Ratios that do not divide 128 leave the last 128 % G rows of a row block idle (2 of 128 at G = 3 and 7) and are
     // still far ahead of the FMA kernel (one layer, 61 tree rows, d = 128, us FMA / this kernel: 24 / 8 heads, B = 1,
     // 2048 tokens 118 / 20; B = 8 761 / 45; 28 / 4 heads, B = 8 884 / 45; d = 64, 300 tokens 28 / 13).  The FMA kernel

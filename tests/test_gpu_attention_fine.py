@@ -54,3 +54,29 @@ def test_probabilities_keep_32_bits(B, Hq, Hkv, d, P, page, M):
             assert float((lse[b, h, :M].double() - sc.logsumexp(-1)).abs().max()) < 4e-6
     assert err ** 0.5 <= 1.001 * rounding ** 0.5
     ctx.close()
+
+
+@pytest.mark.parametrize("Hq,Hkv,d", [(129, 1, 64), (260, 2, 128)])
+def test_ratios_above_128_run_on_the_fma_kernel(Hq, Hkv, d):
+    import torch
+    from paper_2512_14069_b200 import binding as rb
+    ctx, B, P, M = rb.Context(0), 2, 300, 40
+    g = torch.Generator(device="cuda").manual_seed(Hq)
+    rand = lambda *s: torch.randn(*s, device="cuda", generator=g).to(torch.bfloat16)
+    Q, Kt, Vt, Kc, Vc = rand(B, 64, Hq, d), rand(B, 64, Hkv, d), rand(B, 64, Hkv, d), rand(B * P, Hkv, d), rand(B * P, Hkv, d)
+    O = torch.zeros_like(Q)
+    ws = torch.zeros(rb.radar_attn_workspace_bytes(ctx, B, Hq, Hkv, d, rb.RADAR_BF16, P), dtype=torch.uint8, device="cuda")
+    bits = ((torch.ones(64, dtype=torch.int64) << torch.arange(1, 65)) - 1).cuda().repeat(B, 1)          # a chain: rows 0 .. i
+    kw = dict(B=B, Hq=Hq, Hkv=Hkv, d=d, Q=Q, Kc=Kc, Vc=Vc, kv_start=torch.tensor([0, P], device="cuda"), max_prefix_len=P, Kt=Kt, Vt=Vt, mask=bits,
+              prefix_len=torch.full((B,), P, dtype=torch.int32, device="cuda"), n_nodes=torch.full((B,), M, dtype=torch.int32, device="cuda"),
+              O=O, workspace=ws)
+    assert rb.radar_tree_attention_path(**kw) == rb.RADAR_ATTN_PATH_FMA
+    rb.radar_tree_attention(ctx, **kw)
+    ctx.check_device_status()
+    for b in range(B):
+        K, V = (torch.cat([c[b * P:(b + 1) * P], t[b, :M]]).double().repeat_interleave(Hq // Hkv, 1) for c, t in ((Kc, Kt), (Vc, Vt)))
+        sc = torch.einsum("mhd,khd->hmk", Q[b, :M].double(), K) * d ** -0.5
+        sc[:, :, P:] = sc[:, :, P:].masked_fill(torch.ones(M, M, device="cuda").triu(1).bool(), float("-inf"))
+        ref = torch.einsum("hmk,khd->mhd", sc.softmax(-1), V)
+        assert float((O[b, :M].double() - ref).abs().max()) < 2.0 ** -8 * float(ref.abs().max())       # half an ulp of bf16, and then some
+    ctx.close()
