@@ -18,7 +18,7 @@ constexpr int kWarps = kThreads / 32;
 constexpr int kRowsPerWarp = 4;
 constexpr int kRowsPerBlock = kWarps * kRowsPerWarp;     // 32
 constexpr int kTile = 32;                                // keys per shared-memory tile
-constexpr int kMaxSplits = 32;                           // pieces of a sequence's keys
+constexpr int kMaxSplits = 128;                          // pieces of a sequence's keys
 
 struct AttnParams {
     radar_attn_args a;
@@ -249,30 +249,51 @@ __global__ void __launch_bounds__(128) tree_attn_combine_kernel(const AttnParams
     if (node >= M || Pb < 0 || Pb > a.max_prefix_len || kv0 < 0 || kv0 + Pb > a.cache_rows) return;   // skipped by the main kernel
     const int n_valid = (Pb + M + P.split_len - 1) / P.split_len;
     const int64_t rec0 = (((int64_t)b * a.Hq + hq) * kMaxNodes + node) * P.n_splits;
-    // a lane per split (kMaxSplits of them at most): its weight, and the splits' rows then four at a time in flight
-    static_assert(kMaxSplits <= 32, "a lane per split");
-    const float2 ml = lane < n_valid ? P.part_ml[rec0 + lane] : make_float2(-CUDART_INF_F, 0.f);
-    const float mx = warp_max(ml.x);
-    const float w = ml.x == -CUDART_INF_F ? 0.f : __expf(ml.x - mx);
-    const float den = warp_sum(ml.y * w);
-    float o[D / 32];
+    // a lane per split, four batches of them at most: their weights, against the maximum over all of them, and the splits'
+    // rows then eight at a time in flight
+    constexpr int kBatches = kMaxSplits / 32;
+    float2 ml[kBatches];
+    float mx = -CUDART_INF_F;
+#pragma unroll
+    for (int i = 0; i < kBatches; ++i) {
+        ml[i] = i * 32 + lane < n_valid ? P.part_ml[rec0 + i * 32 + lane] : make_float2(-CUDART_INF_F, 0.f);
+        mx = fmaxf(mx, ml[i].x);
+    }
+    mx = warp_max(mx);
+    float den = 0.f, o[D / 32];
 #pragma unroll
     for (int c = 0; c < D / 32; ++c) o[c] = 0.f;
-#pragma unroll 4
-    for (int s = 0; s < n_valid; ++s) {
-        const float ws = __shfl_sync(kFull, w, s);
-        const float* src = P.part_o + (rec0 + s) * D + lane * (D / 32);
-        float v[D / 32];
-        if constexpr (D == 128) {
-            const float4 t = *reinterpret_cast<const float4*>(src);
-            v[0] = t.x; v[1] = t.y; v[2] = t.z; v[3] = t.w;
-        } else {
-            const float2 t = *reinterpret_cast<const float2*>(src);
-            v[0] = t.x; v[1] = t.y;
-        }
 #pragma unroll
-        for (int c = 0; c < D / 32; ++c) o[c] = fmaf(v[c], ws, o[c]);
+    for (int i = 0; i < kBatches; ++i) {
+        if (i * 32 >= n_valid) break;
+        const float w = ml[i].x == -CUDART_INF_F ? 0.f : __expf(ml[i].x - mx);
+        den += ml[i].y * w;
+        const int n = min(32, n_valid - i * 32);
+        for (int s0 = 0; s0 < n; s0 += 8) {
+            float v[8][D / 32];
+#pragma unroll
+            for (int u = 0; u < 8; ++u) {
+#pragma unroll
+                for (int c = 0; c < D / 32; ++c) v[u][c] = 0.f;
+                if (s0 + u >= n) continue;
+                const float* src = P.part_o + (rec0 + i * 32 + s0 + u) * D + lane * (D / 32);
+                if constexpr (D == 128) {
+                    const float4 t = *reinterpret_cast<const float4*>(src);
+                    v[u][0] = t.x; v[u][1] = t.y; v[u][2] = t.z; v[u][3] = t.w;
+                } else {
+                    const float2 t = *reinterpret_cast<const float2*>(src);
+                    v[u][0] = t.x; v[u][1] = t.y;
+                }
+            }
+#pragma unroll
+            for (int u = 0; u < 8; ++u) {
+                const float ws = __shfl_sync(kFull, w, s0 + u);      // (0 past the last split)
+#pragma unroll
+                for (int c = 0; c < D / 32; ++c) o[c] = fmaf(v[u][c], ws, o[c]);
+            }
+        }
     }
+    den = warp_sum(den);
     const float inv = 1.f / den;
     T* dst = reinterpret_cast<T*>(a.O) + (((int64_t)b * kMaxNodes + node) * a.Hq + hq) * D + lane * (D / 32);
 #pragma unroll
@@ -290,6 +311,11 @@ __global__ void __launch_bounds__(128) tree_attn_combine_kernel(const AttnParams
 // combine, before (256 keys a split at least) and with this rule, fp32: 192 keys of 4 heads 22.8 -> 9.1; 364 keys, 32 / 8
 // heads 44.8 -> 32.2; 1064 keys, 40 / 40 heads 134 -> 93; 564 keys, two sequences of them 137 -> 109; 2112 keys, 32 / 8
 // heads 145 both.
+// More than 32 splits, which the combine takes in further batches (its share: kMergeCost a split), where that leaves at most
+// three blocks an SM: few heads and long prefixes.  (256 keys a split at least / 32 splits at most / this rule: 1 head of
+// d = 64, 32768 keys 68 / 109 / 57; 4 heads 169 / 178 / 150; d = 128, 1 head, 8192 keys 55 / 55 / 31.  Four blocks an SM:
+// 8 heads, d = 64, 20000 keys 207 where 32 splits take 188.)
+constexpr double kMergeCost = 0.08;
 void plan(const radar_ctx* ctx, int B, int Hq, int Hkv, int d, int max_prefix_len, int* split_len, int* n_splits) {
     const int G = Hq / Hkv;
     const int rblocks = (kMaxNodes * G + kRowsPerBlock - 1) / kRowsPerBlock;
@@ -299,7 +325,8 @@ void plan(const radar_ctx* ctx, int B, int Hq, int Hkv, int d, int max_prefix_le
     for (int s = 1; s <= std::min(tiles, kMaxSplits); ++s) {
         const int len = (tiles + s - 1) / s, n = (tiles + len - 1) / len;
         const double blocks = base * n, c = (blocks <= 4 * sms ? std::ceil(blocks / sms) : blocks / sms) * (d == 64 ? 0.75 : 1.0);
-        const double cost = (len + (blocks <= 4 * sms ? 1 : 2)) * std::max(1.7, c);
+        const double cost = (len + (blocks <= 4 * sms ? 1 : 2)) * std::max(1.7, c) + kMergeCost * std::max(0, n - 32);
+        if (n > 32 && blocks > 3 * sms) continue;
         if (s == 1 || cost <= best) {
             best = cost;
             *split_len = len * kTile;

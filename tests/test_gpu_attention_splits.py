@@ -10,12 +10,24 @@ pytestmark = pytest.mark.gpu
                                             (1, 2, 1, 128, 2048, 33), (1, 16, 16, 128, 500, 60), (3, 32, 8, 64, 200, 50), (6, 16, 2, 128, 97, 20)])
 @pytest.mark.parametrize("ragged", [False, True])
 def test_key_splits(B, Hq, Hkv, d, P, M, ragged):
+    _compare(B, Hq, Hkv, d, [P // (b + 1) if ragged else P for b in range(B)], P, M)
+
+
+@pytest.mark.parametrize("Hq,Hkv,d,P,plens", [(1, 1, 64, 32768, [32768]), (1, 1, 64, 4096, [4096, 33, 2000]), (1, 1, 128, 8192, [8000]),
+                                              (4, 4, 64, 16384, [16384]), (2, 1, 64, 9000, [9000, 0, 1500, 8999]), (8, 8, 64, 8192, [8192])])
+def test_more_splits_than_lanes(Hq, Hkv, d, P, plens):
+    """Long prefixes of few heads: the combine takes the splits in batches of 32, sequences end in each of them.  The sums are over
+    up to 32768 keys, in up to 128 pieces that are summed in fp32 themselves: the same 1e-5."""
+    _compare(len(plens), Hq, Hkv, d, plens, P, 60)
+
+
+def _compare(B, Hq, Hkv, d, plens, P, M):
     import torch
     from paper_2512_14069_b200 import binding as rb
     ctx = rb.Context(0)
     g = torch.Generator(device="cuda").manual_seed(B * P + M)
     rand = lambda *s: torch.randn(*s, device="cuda", generator=g)
-    plen = torch.tensor([P // (b + 1) if ragged else P for b in range(B)], dtype=torch.int32)
+    plen = torch.tensor(plens, dtype=torch.int32)
     start = torch.cumsum(plen.long(), 0) - plen
     Q, Kt, Vt = rand(B, 64, Hq, d), rand(B, 64, Hkv, d), rand(B, 64, Hkv, d)
     Kc, Vc = rand(max(int(plen.sum()), 1), Hkv, d), rand(max(int(plen.sum()), 1), Hkv, d)
