@@ -284,6 +284,7 @@ typedef struct {
 
 enum { RADAR_ATTN_PATH_FMA = 0, RADAR_ATTN_PATH_TENSOR_CORE = 1 };
 
+/* Enough for max_prefix_len and for every shorter one. */
 size_t radar_attn_workspace_bytes(const radar_ctx* ctx, int B, int Hq, int Hkv, int d, int dtype, int max_prefix_len);
 int radar_tree_attention(radar_ctx* ctx, const radar_attn_args* args, void* stream);
 /* Which kernel radar_tree_attention runs for these arguments (host pointer): RADAR_ATTN_PATH_TENSOR_CORE or

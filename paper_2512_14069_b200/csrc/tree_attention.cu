@@ -364,8 +364,15 @@ using namespace radar;
 extern "C" size_t radar_attn_workspace_bytes(const radar_ctx* ctx, int B, int Hq, int Hkv, int d, int dtype,
                                              int max_prefix_len) {
     if (!ctx || B <= 0 || Hq <= 0 || Hkv <= 0 || Hq % Hkv != 0 || max_prefix_len < 0) return 0;
-    int split_len, n_splits;
-    plan(ctx, B, Hq, Hkv, d, max_prefix_len, &split_len, &n_splits);
+    // enough for every shorter prefix too: the splits of the plan do not grow evenly with it (4 / 4 heads of d = 64: 960
+    // tokens 32 splits, 976 tokens 17)
+    int n_splits = 1;
+    for (int p = max_prefix_len;; p = std::max(p - kTile, 0)) {
+        int split_len, n;
+        plan(ctx, B, Hq, Hkv, d, p, &split_len, &n);
+        n_splits = std::max(n_splits, n);
+        if (p == 0) break;
+    }
     const size_t rec = (size_t)B * Hq * kMaxNodes * n_splits;
     size_t need = align_up(rec * sizeof(float2), 256) + align_up(rec * d * sizeof(float), 256);
     // the same buffer serves whichever kernel the call dispatches to
