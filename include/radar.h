@@ -157,6 +157,7 @@ typedef struct {
     int phase;                          /* RADAR_EXPAND_*                                    */
 } radar_expand_args;
 
+/* Enough for B sequences of F rows and for fewer (as are the sizes of the calls below that take B). */
 size_t radar_expand_workspace_bytes(const radar_ctx* ctx, int B, int F, int V, int k);
 int radar_expand_step(radar_ctx* ctx, const radar_expand_args* args, void* stream);
 

@@ -247,6 +247,7 @@ struct VocabPassParams {
 };
 int vocab_pass_plan_chunks(int sm_count, int rows, int V, int* chunk_out);   // returns n_chunks
 size_t vocab_pass_partial_bytes(int rows, int n_chunks, int k);
+size_t vocab_pass_workspace_bytes(int sm_count, int rows, int V, int k);       // for up to `rows` rows
 void vocab_pass_carve(void* ws, int rows, int n_chunks, int k, VocabPassParams* p);
 cudaError_t vocab_pass_launch(radar_ctx* ctx, int kernel_id, const VocabPassParams& p, cudaStream_t stream);
 cudaError_t vocab_pass_preload_argbest();

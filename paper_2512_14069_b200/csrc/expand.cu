@@ -404,9 +404,7 @@ using namespace radar;
 
 extern "C" size_t radar_expand_workspace_bytes(const radar_ctx* ctx, int B, int F, int V, int k) {
     if (!ctx || B <= 0 || F <= 0 || V <= 0 || k <= 0) return 0;
-    int chunk;
-    const int n_chunks = vocab_pass_plan_chunks(ctx->sm_count, B * F, V, &chunk);
-    return align_up(vocab_pass_partial_bytes(B * F, n_chunks, k), 256) + (size_t)B * 5 * kHidden * sizeof(float);
+    return align_up(vocab_pass_workspace_bytes(ctx->sm_count, B * F, V, k), 256) + (size_t)B * 5 * kHidden * sizeof(float);
 }
 
 extern "C" int radar_expand_step(radar_ctx* ctx, const radar_expand_args* a, void* stream_) {

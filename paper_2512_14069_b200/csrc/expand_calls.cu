@@ -446,11 +446,15 @@ constexpr long long kCallsLogits = 5 << 20;
 
 using namespace radar;
 
+static bool calls_together(const radar_ctx* ctx, int B, int V, int k, int t_max) {
+    return B > 0 && k > 0 && t_max > 0 && k <= RADAR_MAX_K && V >= k && (long long)B * k * V <= kCallsLogits &&
+           B * kSelCluster <= ctx->sm_count && 1 + (long long)(t_max - 1) * k <= 65535;
+}
+
 extern "C" size_t radar_expand_calls_workspace_bytes(const radar_ctx* ctx, int B, int V, int k, int t_max) {
-    if (!ctx || B <= 0 || V <= 0 || k <= 0 || t_max <= 0 || k > RADAR_MAX_K || V < k) return 0;
-    if ((long long)B * k * V > kCallsLogits || B * kSelCluster > ctx->sm_count || 1 + (long long)(t_max - 1) * k > 65535) return 0;
+    if (!ctx || !calls_together(ctx, B, V, k, t_max)) return 0;
     const CallsPlan p = plan_calls(ctx, B, V, k, t_max);
-    return p.part_bytes + p.merged_bytes;
+    return align_up(vocab_pass_workspace_bytes(ctx->sm_count, p.rows, V, k), 256) + p.merged_bytes;
 }
 
 extern "C" int radar_expand_calls(radar_ctx* ctx, const radar_expand_calls_args* args, void* stream_) {
@@ -461,8 +465,7 @@ extern "C" int radar_expand_calls(radar_ctx* ctx, const radar_expand_calls_args*
     if (a->k > RADAR_MAX_K || a->V < a->k) return RADAR_ERR_UNSUPPORTED;
     if (a->logits_dtype != RADAR_F32 && a->logits_dtype != RADAR_BF16) return RADAR_ERR_UNSUPPORTED;
     if (a->policy != RADAR_POLICY_LSTM_SCORES && a->policy != RADAR_POLICY_MLP_SCORES) return RADAR_ERR_UNSUPPORTED;
-    const size_t need = radar_expand_calls_workspace_bytes(ctx, a->B, a->V, a->k, a->t_max);
-    if (need == 0) return RADAR_ERR_UNSUPPORTED;
+    if (!calls_together(ctx, a->B, a->V, a->k, a->t_max)) return RADAR_ERR_UNSUPPORTED;
     if (a->logits_row_stride < a->V) return RADAR_ERR_INVALID_ARG;
     if (!a->logits || !a->parent_score || !a->parent_pool_idx || !a->active || !a->h || !a->c || !a->pool_tok || !a->pool_parent ||
         !a->pool_depth || !a->pool_draft_row || !a->pool_score || !a->pool_len || !a->frontier_tok || !a->frontier_score ||
@@ -476,9 +479,9 @@ extern "C" int radar_expand_calls(radar_ctx* ctx, const radar_expand_calls_args*
         (!a->w_ih || !a->w_hh || !a->b_ih || !a->b_hh || ((reinterpret_cast<uintptr_t>(a->w_hh) | reinterpret_cast<uintptr_t>(a->w_ih)) & 15) != 0))
         return RADAR_ERR_INVALID_ARG;
     if (a->pool_capacity < a->k) return RADAR_ERR_INVALID_ARG;
-    if ((reinterpret_cast<uintptr_t>(a->workspace) & 255) != 0 || need > a->workspace_bytes) return RADAR_ERR_WORKSPACE;
-
     const CallsPlan plan = plan_calls(ctx, a->B, a->V, a->k, a->t_max);
+    if ((reinterpret_cast<uintptr_t>(a->workspace) & 255) != 0 || plan.part_bytes + plan.merged_bytes > a->workspace_bytes) return RADAR_ERR_WORKSPACE;
+
     VocabPassParams vp;
     vp.logits = a->logits;
     vp.dtype = a->logits_dtype;

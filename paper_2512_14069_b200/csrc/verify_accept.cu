@@ -972,11 +972,7 @@ static cudaError_t launch_walk(radar_ctx* ctx, StochParams& sp, int cs, cudaStre
 
 extern "C" size_t radar_accept_workspace_bytes(const radar_ctx* ctx, int B, int V, int mode) {
     if (!ctx || B <= 0 || V <= 0) return 0;
-    if (mode == RADAR_GREEDY) {
-        int chunk;
-        const int n_chunks = vocab_pass_plan_chunks(ctx->sm_count, B * kMaxNodes, V, &chunk);
-        return vocab_pass_partial_bytes(B * kMaxNodes, n_chunks, 1);
-    }
+    if (mode == RADAR_GREEDY) return vocab_pass_workspace_bytes(ctx->sm_count, B * kMaxNodes, V, 1);
     return align_up((size_t)B * cache_stride(V) * sizeof(double), 256) * 2;
 }
 
@@ -991,7 +987,7 @@ extern "C" int radar_verify_accept(radar_ctx* ctx, const radar_accept_args* a, v
         !a->workspace)
         return RADAR_ERR_INVALID_ARG;
     if ((reinterpret_cast<uintptr_t>(a->workspace) & 255) != 0) return RADAR_ERR_WORKSPACE;
-    if (radar_accept_workspace_bytes(ctx, a->B, a->V, a->mode) > a->workspace_bytes) return RADAR_ERR_WORKSPACE;
+    if (a->mode == RADAR_STOCHASTIC && radar_accept_workspace_bytes(ctx, a->B, a->V, a->mode) > a->workspace_bytes) return RADAR_ERR_WORKSPACE;
 
     if (a->mode == RADAR_GREEDY) {
         GreedyParams gp;
@@ -1010,6 +1006,7 @@ extern "C" int radar_verify_accept(radar_ctx* ctx, const radar_accept_args* a, v
         vp.seq_active = nullptr;
         vp.seq_rows = a->n_nodes;
         vp.status = ctx->d_status;
+        if (vocab_pass_partial_bytes(a->B * kMaxNodes, vp.n_chunks, 1) > a->workspace_bytes) return RADAR_ERR_WORKSPACE;
         vocab_pass_carve(a->workspace, a->B * kMaxNodes, vp.n_chunks, 1, &vp);
         RADAR_CUDA_CHECK(vocab_pass_launch(ctx, RADAR_K_VOCAB_ACCEPT, vp, stream));
         {

@@ -9,6 +9,8 @@
 // values that reach it go to a shared-memory candidate list, and their exact ranks by
 // (logit desc, token asc) are counted there.  If an adversarial chunk overflows the list, k rounds
 // of a block-wide arg-best over the registers give the same result.
+#include <algorithm>
+
 #include "common.cuh"
 
 namespace radar {
@@ -309,6 +311,17 @@ int vocab_pass_plan_chunks(int sm_count, int rows, int V, int* chunk_out) {
 size_t vocab_pass_partial_bytes(int rows, int n_chunks, int k) {
     const size_t rec = (size_t)rows * n_chunks;
     return align_up(rec * k * 4, 256) * 2 + align_up(rec * 4, 256) * 2;
+}
+
+// The records of `rows` rows or fewer: below the line of vocab_pass_plan_chunks a row has twice the chunks, so a smaller
+// launch may need more than a larger one.
+size_t vocab_pass_workspace_bytes(int sm_count, int rows, int V, int k) {
+    int chunk;
+    const int n = vocab_pass_plan_chunks(sm_count, rows, V, &chunk);
+    size_t need = vocab_pass_partial_bytes(rows, n, k);
+    const int c8 = (V + 8191) / 8192, below = std::min(rows, (2 * sm_count - 1) / c8);      // most rows below the line
+    if (below > 0) need = std::max(need, vocab_pass_partial_bytes(below, vocab_pass_plan_chunks(sm_count, below, V, &chunk), k));
+    return need;
 }
 
 void vocab_pass_carve(void* ws, int rows, int n_chunks, int k, VocabPassParams* p) {
