@@ -12,7 +12,6 @@ namespace {
 
 constexpr int kMergeWarps = 16;                      // warps 0..15 merge chunk records, warps 16..31 prepare the gate
 constexpr size_t kStageLimit = 96 * 1024;            // chunk records are staged in shared memory up to this size
-constexpr long long kShortPassLogits = 4 << 20;      // ... which is done while a vocabulary pass reads at most this many logits
 
 struct SelectParams {
     radar_expand_args a;

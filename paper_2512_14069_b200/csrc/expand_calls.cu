@@ -9,8 +9,10 @@
 // Call by call, a step is a chain of a dozen launches whose blocks each reload the gate's weights, merge a row's records and
 // hand the state on through global memory: 7 to 12 us a call, whatever the size.  Here the passes and merges, which depend on
 // nothing the calls decide, run once over all rows, and the calls themselves are a loop whose weights and state stay in
-// shared memory, 2 us a call (B = 1, V = 128256, 8 calls: 77 us call by call, 39 together).  What it costs: rows of calls that a sequence never makes are read too, so long passes go call by call
-// (radar_expand_calls_workspace_bytes has the line).
+// shared memory, 2 us a call (B = 1, V = 128256, 8 calls: 77 us call by call, 39 together).  What it costs: rows of calls that
+// a sequence never makes are read too, so long passes go call by call (calls_logits).  It takes draft logits that exist before
+// the first call (recorded ones, or a draft model that does not look at the frontier); where the draft model runs between the
+// calls, radar_expand_step is the form.
 #include <algorithm>
 #include <cstdint>
 
@@ -436,10 +438,20 @@ CallsPlan plan_calls(const radar_ctx* ctx, int B, int V, int k, int t_max) {
     return p;
 }
 
-// Logits of one call (B k V) up to which the calls are made together.  Expansion of k = 10, t_max = 8, fp32, us together /
-// one by one, where every sequence makes 3 calls and where they make 2 to 8: V = 128256, B = 1 29 / 48 and 34 / 60, B = 4
-// 53 / 52 and 63 / 90, B = 6 69 / 56 and 79 / 95, B = 16 148 / 97 and 158 / 147; V = 32000, B = 16 52 / 55 and 62 / 92.
-constexpr long long kCallsLogits = 5 << 20;
+// The line: calls whose passes are short (B k V logits at most), where each also costs a cluster of blocks when it is made one by
+// one, whether a sequence is still active or not.  Together, the rows of all calls are read, one by one those of a call more
+// than is made.  Expansion in us, together / one by one, fp32, where every sequence makes 1, 2, 3 and all calls:
+//   1.2M logits  V = 128256, B = 1, k = 10  t_max  4: 21 / 21, 23 / 27, 25 / 33, 26 / 39     8: 25 / 35, 27 / 41, 30 / 45, 39 / 73
+//   2.4M         V = 32000, B = 8, k = 10   t_max  4: 23 / 23, 25 / 27, 28 / 35, 29 / 39    16: 49 / 66, 53 / 72, 55 / 76, 85 / 150
+//   3.7M         V = 128256, B = 3, k = 10  t_max  3: 25 / 19, 27 / 27, 27 / 31              8: 41 / 37, 45 / 42, -, 57 / 82
+//   3.9M         V = 128256, B = 8, k = 4   t_max  4: 25 / 23, 28 / 27, 29 / 35, 29 / 39    16: 63 / 68, 66 / 72, 68 / 78, 94 / 154
+//   4.9M         V = 128256, B = 4, k = 10  t_max  4: 31 / 21, 33 / 27, 35 / 36, 35 / 41     8: 49 / 27, 51 / 35, 53 / 43, 64 / 89
+// Up to the line together is the faster form from two calls on (but for 3 us at 3.7M), and at one call at most 8 us the
+// slower one; above it, one by one drops the clusters, a call that is not made costs 2 us, and it takes five made calls out of
+// eight for the rows to pay.  From k = 16 on, where a call by itself merges and ranks more than twice the candidates, three do
+// (t_max = 8; 4.6M logits, V = 152000, k = 16, B = 2: 50 / 31, 53 / 43, 55 / 55, 68 / 123; k = 32, B = 1: 80 / 47, 85 / 150, 91 / 252,
+// 111 / 767), and the line lies a little higher.
+inline long long calls_logits(int k) { return k < 16 ? kShortPassLogits : 5LL << 20; }
 
 }  // namespace
 }  // namespace radar
@@ -447,7 +459,7 @@ constexpr long long kCallsLogits = 5 << 20;
 using namespace radar;
 
 static bool calls_together(const radar_ctx* ctx, int B, int V, int k, int t_max) {
-    return B > 0 && k > 0 && t_max > 0 && k <= RADAR_MAX_K && V >= k && (long long)B * k * V <= kCallsLogits &&
+    return B > 0 && k > 0 && t_max > 0 && k <= RADAR_MAX_K && V >= k && (long long)B * k * V <= calls_logits(k) &&
            B * kSelCluster <= ctx->sm_count && 1 + (long long)(t_max - 1) * k <= 65535;
 }
 

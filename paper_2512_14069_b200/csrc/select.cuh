@@ -10,7 +10,8 @@ constexpr int kSelThreads = 1024;
 constexpr int kSelWarps = kSelThreads / 32;
 constexpr int kMaxF = 32;
 constexpr int kSurvCap = 256;                        // per-row survivor list of the parallel merge (even: read in pairs)
-constexpr int kSelCluster = 4;                       // blocks per sequence when the recurrent product is shared out
+constexpr int kSelCluster = 4;                       // blocks per sequence when the recurrent product is shared out,
+constexpr long long kShortPassLogits = 4 << 20;      // ... which is done while a call's vocabulary pass reads at most this many logits
 
 __device__ __forceinline__ float sigmoidf_(float x) { return 1.f / (1.f + expf(-x)); }
 

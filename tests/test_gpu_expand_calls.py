@@ -112,4 +112,5 @@ def test_long_passes_go_call_by_call(ctx):
     from paper_2512_14069_b200 import binding as rb
     assert rb.radar_expand_calls_workspace_bytes(ctx, 1, 128256, 10, 8) > 0
     assert rb.radar_expand_calls_workspace_bytes(ctx, 32, 128256, 10, 8) == 0
+    assert rb.radar_expand_calls_workspace_bytes(ctx, 1, 1 << 19, 8, 2) > 0 and rb.radar_expand_calls_workspace_bytes(ctx, 1, (1 << 19) + 1, 8, 2) == 0
     assert rb.radar_expand_calls_workspace_bytes(ctx, 1, 1000, 33, 8) == 0
