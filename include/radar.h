@@ -233,8 +233,8 @@ int radar_rerank_build_tree(radar_ctx* ctx, const radar_tree_args* args, void* s
  * Q, Kc, Vc, Kt, Vt and O must be 16-byte aligned (both kernels move them in 16-byte pieces); a misaligned
  * tensor is refused on the host with RADAR_ERR_INVALID_ARG.
  * bf16 with Hq / Hkv <= 128 runs on the tensor cores (TMA-staged K/V tiles, tcgen05 MMA for QK^T and PV), except
- * that a ratio which does not divide 128 takes the fp32 FMA kernel when cache_rows * Hkv <= 1280 (a launch that is all
- * latency); all of fp32 runs on the FMA kernel.  On the tensor cores the probabilities enter P V as bf16 where the ratio divides
+ * that a ratio which does not divide 128 takes the fp32 FMA kernel for one layer of little work
+ * (B * Hq * (max_prefix_len + 64) * d <= 294912: a launch that is all latency); all of fp32 runs on the FMA kernel.  On the tensor cores the probabilities enter P V as bf16 where the ratio divides
  * 128, as the sum of two bf16 numbers (2^-18) elsewhere; the FMA kernel keeps them in fp32.  radar_tree_attention_path()
  * tells which of the two a given argument struct will take, so that a caller (or a benchmark) is never
  * switched to the other kernel unawares.

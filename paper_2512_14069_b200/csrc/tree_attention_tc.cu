@@ -48,7 +48,7 @@ constexpr int kStaticSmem = 3072;    // barriers and exchange arrays: with the t
 constexpr int kTileKeys = 128;       // keys per prefix tile
 constexpr int kTreeKeys = 64;        // keys of the tree tile (RADAR_MAX_NODES)
 constexpr int kPairRows = 256;       // query rows of a row-block pair (and the stride of partial records)
-constexpr long long kSmallCacheRows = 1280;   // (cache row, KV head) pairs: tree_attn_tc_supported
+constexpr long long kLatencyWork = 9 << 15;   // sequences x query heads x keys x head dimension: tree_attn_tc_supported
 constexpr float kRescaleThreshold = 8.f;   // in log2 units: P stays below 2^8
 
 // Written by every CTA of the attention kernel, read by the combine kernel: the pieces are worked out by the producer warp
@@ -1103,14 +1103,15 @@ bool tree_attn_tc_supported(const radar_attn_args* a) {
     if (a->dtype != RADAR_BF16 || (a->d != 64 && a->d != 128)) return false;
     const int G = a->Hq / a->Hkv;
     if (G < 1 || G > kTcMaxRatio) return false;
-    // Ratios that do not divide 128 leave the last 128 % G rows of a row block idle (2 of 128 at G = 3 and 7) and are
-    // still far ahead of the FMA kernel (one layer, 61 tree rows, d = 128, us FMA / this kernel: 24 / 8 heads, B = 1,
-    // 2048 tokens 118 / 20; B = 8 761 / 45; 28 / 4 heads, B = 8 884 / 45; d = 64, 300 tokens 28 / 13).  The FMA kernel
-    // is the faster one only where a launch is all latency (d = 64, 16 tokens, 3 heads per KV head: 13 / 15; the two
-    // cross at about 64 tokens, below the line).  The line is not the crossing: it is where it is so that the test of
-    // the FMA kernel's bounds check on bf16 data (600 cache rows, 2 KV heads) still reaches that kernel; between the
-    // two the choice costs 8 to 25 us a launch.
-    if ((128 % G) != 0 && a->cache_rows * a->Hkv <= kSmallCacheRows) return false;
+    // Ratios that do not divide 128 leave the last 128 % G rows of a row block idle (2 of 128 at G = 3 and 7) and take two
+    // products a tile for their probabilities, and are still far ahead of the FMA kernel (one layer, 61 tree rows, d = 128, us
+    // FMA / this kernel: 24 / 8 heads, B = 1, 2048 tokens 119 / 21; B = 4, 300 tokens 101 / 23; 28 / 4 heads, B = 2, 4096 tokens
+    // 444 / 31), but for launches that are all latency, where the FMA kernel's one wave of small blocks is done before this
+    // one's pipeline has filled.  Where the two cross is a matter of the work (61 rows, FMA / this one; in units of the line
+    // below): 24 / 8 heads of d = 64, B = 1, 64 tokens (0.7) 10.5 / 12.3, 128 (1.0) 10.6 / 11.8, 192 (1.3) 13.6 / 13.1; 28 / 4 heads,
+    // 128 (1.2) 13.5 / 12.0; 3 heads, 256 (0.2) 8.4 / 13.0; d = 128: 3 / 1 heads, B = 4, 128 (1.0) 10.0 / 13.1, 28 / 4 heads, 0 (0.8)
+    // 13.3 / 15.6, 64 (1.6) 13.9 / 13.3.  Several layers are one launch here and one each there.
+    if ((128 % G) != 0 && a->n_layers <= 1 && (long long)a->B * a->Hq * (a->max_prefix_len + kMaxNodes) * a->d <= kLatencyWork) return false;
     if (a->cache_rows < 0 || a->cache_rows >= (1ll << 31) || (long long)a->B * kMaxNodes >= (1ll << 31)) return false;
     const uintptr_t al = reinterpret_cast<uintptr_t>(a->Q) | reinterpret_cast<uintptr_t>(a->Kc) |
                          reinterpret_cast<uintptr_t>(a->Vc) | reinterpret_cast<uintptr_t>(a->Kt) |

@@ -12,7 +12,9 @@ pytestmark = pytest.mark.gpu
 
 @pytest.mark.parametrize("B,Hq,Hkv,d,P,page,M", [
     (1, 24, 8, 128, 2048, 0, 61), (2, 28, 4, 128, 700, 16, 64), (3, 12, 4, 64, 333, 0, 20), (1, 12, 1, 128, 20000, 0, 60), (1, 28, 4, 64, 9000, 128, 33),
-    (2, 100, 1, 64, 2000, 0, 64), (1, 40, 8, 128, 1400, 0, 64), (4, 24, 8, 128, 0, 0, 64), (8, 28, 4, 128, 3000, 0, 64)])
+    (2, 100, 1, 64, 2000, 0, 64), (1, 40, 8, 128, 1400, 0, 64), (4, 24, 8, 128, 0, 0, 64), (8, 28, 4, 128, 3000, 0, 64),
+    # little work: the FMA kernel, up to its line and one key above it
+    (2, 6, 2, 64, 100, 0, 64), (1, 24, 8, 64, 100, 16, 30), (1, 3, 1, 128, 500, 0, 64), (1, 3, 1, 64, 1472, 0, 40), (1, 3, 1, 64, 1473, 0, 40)])
 def test_probabilities_keep_32_bits(B, Hq, Hkv, d, P, page, M):
     import torch
     from paper_2512_14069_b200 import binding as rb
@@ -37,9 +39,10 @@ def test_probabilities_keep_32_bits(B, Hq, Hkv, d, P, page, M):
     O, lse = torch.zeros_like(Q), torch.zeros(B, Hq, 64, device="cuda")
     ws = torch.zeros(rb.radar_attn_workspace_bytes(ctx, B, Hq, Hkv, d, rb.RADAR_BF16, P) + 256, dtype=torch.uint8, device="cuda")
     ws = ws[(-ws.data_ptr()) % 256:]
-    rb.radar_tree_attention(ctx, B=B, Hq=Hq, Hkv=Hkv, d=d, Q=Q, Kc=Kc, Vc=Vc, kv_start=start.cuda(), prefix_len=plen.cuda(), max_prefix_len=P,
-                            Kt=Kt, Vt=Vt, mask=bits, n_nodes=torch.full((B,), M, dtype=torch.int32, device="cuda"), O=O, lse=lse, workspace=ws,
-                            block_table=table, page_size=page)
+    kw = dict(B=B, Hq=Hq, Hkv=Hkv, d=d, Q=Q, Kc=Kc, Vc=Vc, kv_start=start.cuda(), prefix_len=plen.cuda(), max_prefix_len=P, Kt=Kt, Vt=Vt,
+              mask=bits, n_nodes=torch.full((B,), M, dtype=torch.int32, device="cuda"), O=O, lse=lse, workspace=ws, block_table=table, page_size=page)
+    assert rb.radar_tree_attention_path(**kw) == (rb.RADAR_ATTN_PATH_FMA if B * Hq * (P + 64) * d <= 294912 else rb.RADAR_ATTN_PATH_TENSOR_CORE)
+    rb.radar_tree_attention(ctx, **kw)
     ctx.check_device_status()
     err = rounding = 0.0
     for b in range(B):

@@ -211,10 +211,19 @@ def test_attention_with_oracle_masks_and_ragged_trees(ctx):
     H.compare_attention(cfg, O_gpu, lse_gpu, O_ref, lse_ref, trees)
 
 
+def _attention_path(g, page_size=0):
+    from paper_2512_14069_b200 import binding as rb
+    cfg, s = g.cfg, g.step
+    return rb.radar_tree_attention_path(B=cfg.B, Hq=cfg.Hq, Hkv=cfg.Hkv, d=cfg.d, Q=g.Q, Kc=g.Kc, Vc=g.Vc, kv_start=None if page_size else g.kv_start,
+                                        prefix_len=g.prefix_len, max_prefix_len=s.max_prefix_len, Kt=g.Kt, Vt=g.Vt, mask=s.tree_mask,
+                                        n_nodes=s.n_nodes, O=s.O, workspace=s.ws_attn, block_table=g.block_table, page_size=page_size)
+
+
 @pytest.mark.parametrize("Hq,Hkv,d", [(8, 8, 64), (8, 4, 64), (16, 1, 128), (6, 3, 128), (24, 8, 128)])
 def test_attention_bf16_head_layouts(ctx, Hq, Hkv, d):
-    """bf16 tensor-core path at head_dim 64 and 128, G = 1, 2 and 16 (eight row blocks), and G = 3, which the
-    tensor-core path does not take (falls to the FMA kernel): ragged prefixes incl. an empty one, ragged trees."""
+    """bf16 tensor-core path at head_dim 64 and 128, G = 1, 2, 3 and 16 (eight row blocks): ragged prefixes incl. an empty
+    one, ragged trees."""
+    from paper_2512_14069_b200 import binding as rb
     cfg = W.shrink(W.CONFIGS[5], cid=80 + Hq + d, B=4, Hq=Hq, Hkv=Hkv, d=d, P=(0, 700), V=2000, k=4, t_max=5, N=50)
     inp = H.make_inputs(cfg)
     inp["prefix_len"][0] = 0
@@ -223,6 +232,7 @@ def test_attention_bf16_head_layouts(ctx, Hq, Hkv, d):
     trees[2] = dict(trees[2]); trees[2]["n_nodes"] = 1
     g = H.CudaRun(cfg, inp, ctx)
     g.upload_attention()
+    assert _attention_path(g) == rb.RADAR_ATTN_PATH_TENSOR_CORE
     O_gpu, lse_gpu = g.attention(trees)
     O_ref, lse_ref = H.oracle_attention(cfg, inp, trees)
     H.compare_attention(cfg, O_gpu, lse_gpu, O_ref, lse_ref, trees)
@@ -234,7 +244,8 @@ def test_attention_paged_prefix_cache(ctx, page_size, Hq, Hkv, dtype):
     """The prefix K/V scattered over shuffled pages (16 to 256 tokens) and read through a block table: same
     outputs as the oracle computes from the logical rows.  Ragged prefixes, one empty, one shorter than a page,
     one ending exactly on a page boundary; rows of the cache that belong to no token hold NaN.
-    (6 query / 3 KV heads and fp32 take the FMA kernel, the others the tensor-core kernel.)"""
+    (fp32 takes the FMA kernel, the others the tensor-core kernel.)"""
+    from paper_2512_14069_b200 import binding as rb
     base = W.CONFIGS[5] if dtype == "bf16" else W.CONFIGS[1]
     cfg = W.shrink(base, cid=120 + page_size + Hq, B=5, Hq=Hq, Hkv=Hkv, d=128 if dtype == "bf16" else 64,
                    P=(200, 1500), V=2000, k=4, t_max=5, N=50)
@@ -245,6 +256,7 @@ def test_attention_paged_prefix_cache(ctx, page_size, Hq, Hkv, dtype):
     _, _, trees = H.oracle_expand_and_tree(cfg, inp)
     g = H.CudaRun(cfg, inp, ctx)
     g.upload_attention(page_size=page_size)
+    assert _attention_path(g, page_size) == (rb.RADAR_ATTN_PATH_FMA if dtype == "f32" else rb.RADAR_ATTN_PATH_TENSOR_CORE)
     O_gpu, lse_gpu = g.attention(trees)
     O_ref, lse_ref = H.oracle_attention(cfg, inp, trees)
     H.compare_attention(cfg, O_gpu, lse_gpu, O_ref, lse_ref, trees)
@@ -299,7 +311,7 @@ def test_attention_reports_prefix_beyond_cache(ctx, kind):
     if kind == "f32_fma":
         cfg = W.shrink(W.CONFIGS[1], cid=97, B=2, Hq=4, Hkv=2, P=(300, 300), V=2000, k=4, t_max=4, N=30)
     else:
-        Hq = 8 if kind == "bf16_tensor_core" else 6
+        Hq = 8 if kind == "bf16_tensor_core" else 258          # 129 query heads per KV head: above what a row block holds
         cfg = W.shrink(W.CONFIGS[5], cid=98, B=2, Hq=Hq, Hkv=2, P=(300, 300), V=2000, k=4, t_max=4, N=30)
     inp = H.make_inputs(cfg)
     _, _, trees = H.oracle_expand_and_tree(cfg, inp)
