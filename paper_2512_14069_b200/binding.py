@@ -206,10 +206,11 @@ def _raw_stream(stream) -> int:
 class _Call:
     """One entry point of the library whose argument struct is filled natively from a dictionary {field: value}.
     `dtypes` gives the dtype a tensor must have for a pointer field (absent: any); `optional` the fields that may be
-    left out (0 / NULL then)."""
+    left out (0 / NULL then); `addresses` the pointer fields that may be given as a plain address (the others take a
+    tensor or None, so that a number in the wrong place is refused and never read from)."""
 
-    def __init__(self, name, struct, dtypes, optional):
-        self.name, self.struct, self.dtypes, self.optional = name, struct, dtypes, frozenset(optional)
+    def __init__(self, name, struct, dtypes, optional, addresses=()):
+        self.name, self.struct, self.dtypes, self.optional, self.addresses = name, struct, dtypes, frozenset(optional), frozenset(addresses)
         self.address = self.fill = None
 
     def _load(self):
@@ -224,7 +225,7 @@ class _Call:
                     yield from flat(t, at)
                 else:
                     yield f, at, kinds[t]
-        fields = [(f, at, kind, like.get(self.dtypes.get(f)), f not in self.optional) for f, at, kind in flat(self.struct, 0)]
+        fields = [(f, at, kind, like.get(self.dtypes.get(f)), f not in self.optional, f in self.addresses) for f, at, kind in flat(self.struct, 0)]
         self.address = ctypes.cast(getattr(lib(), self.name), _vp).value
         self.fill = _marshal.Filler(ctypes.sizeof(self.struct), fields)        # last: another thread may test it
 
@@ -303,7 +304,12 @@ _expand = _Call(
     dict({n: _f32 for n in _GATE}, parent_score=_f32, parent_pool_idx=_i32, active=_u8, force_calls=_i32, h=_f32, c=_f32, pool_tok=_i32,
          pool_parent=_i32, pool_depth=_i32, pool_draft_row=_i32, pool_score=_f32, pool_len=_i32, frontier_tok=_i32, frontier_score=_f32,
          frontier_pool_idx=_i32, frontier_src_row=_i32, topk_tok=_i32, topk_logp=_f32, gate_logits=_f32, cont=_u8, features=_f32),
-    _GATE + ("force_calls", "policy", "feat_dim", "features", "phase"))
+    _GATE + ("force_calls", "policy", "feat_dim", "features", "phase"), ("logits",))         # (an offset into the caller's tensor)
+# the same call from the pipeline, whose per-call buffers are slices of its own
+_expand_slots = _Call(
+    _expand.name, ExpandArgs, _expand.dtypes, _expand.optional,
+    ("logits", "parent_score", "parent_pool_idx", "active", "frontier_tok", "frontier_score", "frontier_pool_idx", "frontier_src_row", "topk_tok",
+     "topk_logp", "gate_logits", "cont"))
 
 
 def radar_expand_step(ctx: Context, *, logits, gate, workspace, logits_offset_elems=0, features=None, stream=None, **kw):
@@ -315,12 +321,13 @@ def radar_expand_step(ctx: Context, *, logits, gate, workspace, logits_offset_el
     pool_depth, pool_draft_row, pool_score, pool_len, frontier_tok, frontier_score, frontier_pool_idx, frontier_src_row,
     topk_tok, topk_logp, gate_logits, cont, and, with defaults, force_calls (None), policy (RADAR_POLICY_LSTM_SCORES) and
     phase (RADAR_EXPAND_ALL)."""
-    expand_fields(ctx, kw, logits, gate, workspace, logits_offset_elems, features, stream)
+    expand_fields(ctx, kw, logits, gate, workspace, logits_offset_elems, features, stream, _expand)
 
 
-def expand_fields(ctx, kw, logits, gate, workspace, logits_offset_elems=0, features=None, stream=None):
-    """radar_expand_step with its other arguments in the dictionary `kw`, which is completed in place: a call that passes
-    forty keywords through two functions spends more on them than on its launches."""
+def expand_fields(ctx, kw, logits, gate, workspace, logits_offset_elems=0, features=None, stream=None, call=_expand_slots):
+    """radar_expand_step for the pipeline: its other arguments in the dictionary `kw`, which is completed in place (a call that
+    passes forty keywords through two functions spends more on them than on its launches), the per-call buffers as
+    addresses."""
     kw["logits"] = _ptr(logits) + logits_offset_elems * logits.element_size()
     kw["logits_dtype"] = dtype_code(logits)
     for n in _GATE:
@@ -328,7 +335,7 @@ def expand_fields(ctx, kw, logits, gate, workspace, logits_offset_elems=0, featu
     if features is not None:
         kw["features"], kw["feat_dim"] = features, features.shape[-1]
     kw["workspace"], kw["workspace_bytes"] = workspace, workspace.numel() * workspace.element_size()
-    _expand(ctx, stream, kw)
+    call(ctx, stream, kw)
 
 
 _expand_calls = _Call(

@@ -20,6 +20,7 @@ struct Field {
     int kind;
     int dtype;          // c10::ScalarType a tensor must have, -1: any
     bool required;
+    bool address;       // a pointer field that may also be given as a plain address
 };
 
 struct Filler {
@@ -74,9 +75,12 @@ bool fill(const Field& f, PyObject* name, PyObject* v, unsigned char* out) {
                     PyErr_SetString(PyExc_RuntimeError, e.what());
                     return false;
                 }
-            } else {
+            } else if (f.address) {
                 p = PyLong_AsVoidPtr(v);
                 if (p == nullptr && PyErr_Occurred()) return false;
+            } else {
+                PyErr_Format(PyExc_TypeError, "%U: expected a tensor or None, got %s", name, Py_TYPE(v)->tp_name);
+                return false;
             }
             std::memcpy(to, &p, sizeof p);
             return true;
@@ -126,7 +130,7 @@ PyObject* filler_call(PyObject* self_, PyObject* args, PyObject* kwargs) {
     return PyLong_FromLong(status);
 }
 
-// Filler(struct size, [(name, offset, kind, dtype, required), ...]); dtype: a tensor of the type, or None
+// Filler(struct size, [(name, offset, kind, dtype, required, address), ...]); dtype: a tensor of the type, or None
 PyObject* filler_new(PyTypeObject* type, PyObject* args, PyObject*) {
     Py_ssize_t size;
     PyObject* list;
@@ -141,11 +145,11 @@ PyObject* filler_new(PyTypeObject* type, PyObject* args, PyObject*) {
     for (Py_ssize_t i = 0; i < PyList_GET_SIZE(list); ++i) {
         PyObject *name, *dtype;
         Py_ssize_t offset;
-        int kind, required;
-        if (!PyArg_ParseTuple(PyList_GET_ITEM(list, i), "O!niOp", &PyUnicode_Type, &name, &offset, &kind, &dtype, &required)) { Py_DECREF(self); return nullptr; }
+        int kind, required, address;
+        if (!PyArg_ParseTuple(PyList_GET_ITEM(list, i), "O!niOpp", &PyUnicode_Type, &name, &offset, &kind, &dtype, &required, &address)) { Py_DECREF(self); return nullptr; }
         const Py_ssize_t bytes = kind == kInt || kind == kFloat ? 4 : 8;
         if (kind < kInt || kind > kPointer || offset < 0 || offset + bytes > size) { Py_DECREF(self); PyErr_SetString(PyExc_ValueError, "bad field"); return nullptr; }
-        Field f{offset, kind, -1, required != 0};
+        Field f{offset, kind, -1, required != 0, address != 0};
         if (dtype != Py_None) {
             if (!THPVariable_Check(dtype)) { Py_DECREF(self); PyErr_SetString(PyExc_TypeError, "dtype: a tensor of the type, or None"); return nullptr; }
             f.dtype = static_cast<int>(THPVariable_Unpack(dtype).scalar_type());

@@ -14,10 +14,10 @@ def built():
     rbuild.build()
 
 
-def _filler(struct, optional=(), like=None):
+def _filler(struct, optional=(), like=None, addresses=True):
     from paper_2512_14069_b200 import _marshal
     kinds = {ctypes.c_int: 0, ctypes.c_int64: 1, ctypes.c_size_t: 1, ctypes.c_float: 2, ctypes.c_void_p: 3}
-    return _marshal.Filler(ctypes.sizeof(struct), [(f, getattr(struct, f).offset, kinds[t], like, f not in optional) for f, t in struct._fields_])
+    return _marshal.Filler(ctypes.sizeof(struct), [(f, getattr(struct, f).offset, kinds[t], like, f not in optional, addresses) for f, t in struct._fields_])
 
 
 @pytest.mark.parametrize("struct", [rb.ExpandArgs, rb.TreeArgs, rb.AttnArgs, rb.AcceptArgs])
@@ -51,3 +51,24 @@ def test_what_does_not_fit_is_refused():
         fill(1, 0, 0, dict(good, pool_tok=torch.zeros(3)))
     with pytest.raises(TypeError):
         fill(1, 0, 0, dict(good, pool_tok="x"))
+
+
+def test_a_number_is_no_tensor():
+    """Only fields that are declared to take an address do; for the public calls that is the logits' own offset."""
+    fill = _filler(rb.TreeArgs, addresses=False)
+    numbers = {f: 1 if t is ctypes.c_int else None for f, t in rb.TreeArgs._fields_}
+    for name in ("pool_tok", "tree_mask", "n_keep"):
+        for value in (0, 4096, True):
+            with pytest.raises(TypeError, match="%s: expected a tensor or None, got" % name):
+                fill(1, 0, 0, dict(numbers, **{name: value}))
+    for call in (rb._expand, rb._expand_calls, rb._tree, rb._attention, rb._accept):
+        assert call.addresses <= {"logits"}
+
+
+def test_public_calls_refuse_numbers():
+    class Ctx:
+        handle = None
+    tree = {f: 1 if t is ctypes.c_int else None for f, t in rb.TreeArgs._fields_}
+    stream = type("S", (), {"cuda_stream": 0})()
+    with pytest.raises(TypeError, match="retrieve: expected a tensor"):
+        rb.radar_rerank_build_tree(Ctx, stream=stream, **dict(tree, retrieve=12345))
