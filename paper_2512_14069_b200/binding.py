@@ -1,7 +1,7 @@
-"""Thin binding of libradar_b200.so: same names as include/radar.h, argument marshalling only.  The four calls
-of a step fill their argument structs natively (csrc/marshal.cpp), the others through ctypes.  torch
-tensors are used for device memory and streams; every step of the path runs in the library's CUDA kernels.  There is no CPU fallback: if the library
-is missing or a call fails, an exception is raised.
+"""Thin binding of libradar_b200.so: same names as include/radar.h, argument marshalling only.  The calls of a step fill
+their argument structs natively (csrc/marshal.cpp, built against the installed torch), the others through ctypes.  torch
+tensors are used for device memory and streams; every step of the path runs in the library's CUDA kernels.  There is no
+CPU fallback: if the library is missing or a call fails, an exception is raised.
 """
 from __future__ import annotations
 
@@ -104,16 +104,29 @@ class TrainArgs(ctypes.Structure):
 
 
 _lib = None
+_BUILD_HINT = "build it with `python -m paper_2512_14069_b200.build` (there is no CPU fallback)"
+
+
+def _check_marshal():
+    """Raises unless the argument marshaller is there and built for the torch and Python that are running."""
+    from . import build
+    tag = build.marshal_tag()
+    try:
+        from . import _marshal
+    except ImportError as e:
+        raise RuntimeError("the argument marshaller (_marshal.so) cannot be loaded (%s): %s" % (e, _BUILD_HINT)) from e
+    if getattr(_marshal, "BUILT_FOR", None) != tag:
+        raise RuntimeError("the argument marshaller (_marshal.so) was %s and this is another one (%s): %s"
+                           % (getattr(_marshal, "BUILT_FOR", "built for another torch"), tag, _BUILD_HINT))
 
 
 def lib() -> ctypes.CDLL:
-    """The loaded library; raises if it has not been built (there is no fallback path)."""
+    """The loaded library; raises if it, or the marshaller next to it, has not been built (there is no fallback path)."""
     global _lib
     if _lib is None:
         if not os.path.exists(LIB_PATH):
-            raise RuntimeError(
-                "libradar_b200.so is missing: build it with `python -m paper_2512_14069_b200.build` "
-                "(there is no CPU fallback)")
+            raise RuntimeError("libradar_b200.so is missing: " + _BUILD_HINT)
+        _check_marshal()
         L = ctypes.CDLL(LIB_PATH)
         L.radar_create.restype = _c_int
         L.radar_create.argtypes = [ctypes.POINTER(_vp), _c_int]

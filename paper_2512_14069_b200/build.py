@@ -18,15 +18,35 @@ MARSHAL_SRC = os.path.join(CSRC, "marshal.cpp")
 MARSHAL = os.path.join(HERE, "_marshal.so")
 
 
+def _torch_dir() -> str:
+    from importlib.util import find_spec
+    return os.path.dirname(find_spec("torch").origin)
+
+
+def marshal_tag() -> str:
+    """What the marshaller is compiled against: it reads tensors by torch's C++ layout and objects by Python's."""
+    import re
+    import sysconfig
+    with open(os.path.join(_torch_dir(), "version.py")) as f:
+        version = re.search(r"__version__ = ['\"](.*?)['\"]", f.read()).group(1)
+    return "built for torch %s, %s" % (version, sysconfig.get_config_var("SOABI"))
+
+
+def _marshal_is_current() -> bool:
+    if not os.path.exists(MARSHAL) or os.path.getmtime(MARSHAL) < os.path.getmtime(MARSHAL_SRC):
+        return False
+    with open(MARSHAL, "rb") as f:                   # the module carries its tag as a string
+        return marshal_tag().encode() + b"\0" in f.read()
+
+
 def _start_marshal(force: bool):
     """Starts the compiler for the marshaller if it is out of date; (process, temporary file) or None."""
-    if not force and os.path.exists(MARSHAL) and os.path.getmtime(MARSHAL) >= os.path.getmtime(MARSHAL_SRC):
+    if not force and _marshal_is_current():
         return None
     import sysconfig
-    from importlib.util import find_spec
-    tdir = os.path.dirname(find_spec("torch").origin)
+    tdir = _torch_dir()
     tmp = MARSHAL + ".%d.tmp" % os.getpid()
-    cmd = [os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-shared", "-fPIC", "-I" + os.path.join(tdir, "include"),
+    cmd = [os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-shared", "-fPIC", '-DRADAR_BUILT_FOR="%s"' % marshal_tag(), "-I" + os.path.join(tdir, "include"),
            "-I" + os.path.join(tdir, "include", "torch", "csrc", "api", "include"), "-I" + sysconfig.get_paths()["include"], MARSHAL_SRC,
            "-o", tmp, "-L" + os.path.join(tdir, "lib"), "-lc10", "-ltorch_cpu", "-ltorch", "-ltorch_python"]
     return subprocess.Popen(cmd, stdout=subprocess.PIPE, stderr=subprocess.STDOUT, text=True), tmp

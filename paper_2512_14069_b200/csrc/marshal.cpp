@@ -1,7 +1,7 @@
 // Argument marshalling of the ctypes-free call path: fills an argument struct of radar.h from a dictionary of Python
 // objects and calls the library.  A step makes a dozen calls of thirty arguments each, and where the draft model runs
 // between them nothing hides their host time: filled field by field from Python a call took 25 us, of which the library
-// and its launches are 5.  Nothing is kept between calls: every tensor is checked and its address taken each time.
+// and its launches are 5.  RADAR_BUILT_FOR names the torch and Python it is compiled against.  Nothing is kept between calls: every tensor is checked and its address taken each time.
 #include <Python.h>
 
 #include <torch/csrc/autograd/python_variable.h>
@@ -186,7 +186,7 @@ PyMODINIT_FUNC PyInit__marshal() {
     PyObject* m = PyModule_Create(&module_def);
     if (m == nullptr) return nullptr;
     PyObject* type = PyType_FromSpec(&filler_spec);
-    if (type == nullptr || PyModule_AddObject(m, "Filler", type) != 0) {
+    if (type == nullptr || PyModule_AddStringConstant(m, "BUILT_FOR", RADAR_BUILT_FOR) != 0 || PyModule_AddObject(m, "Filler", type) != 0) {
         Py_XDECREF(type);
         Py_DECREF(m);
         return nullptr;

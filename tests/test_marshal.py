@@ -72,3 +72,23 @@ def test_public_calls_refuse_numbers():
     stream = type("S", (), {"cuda_stream": 0})()
     with pytest.raises(TypeError, match="retrieve: expected a tensor"):
         rb.radar_rerank_build_tree(Ctx, stream=stream, **dict(tree, retrieve=12345))
+
+
+def test_a_marshaller_of_another_torch_is_rebuilt_and_not_used(monkeypatch):
+    from paper_2512_14069_b200 import _marshal
+    assert _marshal.BUILT_FOR == rbuild.marshal_tag() and torch.__version__ in _marshal.BUILT_FOR and rbuild._marshal_is_current()
+    rb._check_marshal()
+    monkeypatch.setattr(rbuild, "marshal_tag", lambda: "built for torch 0.0, none")
+    assert not rbuild._marshal_is_current()
+    with pytest.raises(RuntimeError, match="another one .*build it with"):
+        rb._check_marshal()
+
+
+def test_a_missing_marshaller_is_named_when_the_library_is_loaded(monkeypatch):
+    import sys
+    import paper_2512_14069_b200 as pkg
+    monkeypatch.setattr(rb, "_lib", None)
+    monkeypatch.delattr(pkg, "_marshal", raising=False)
+    monkeypatch.setitem(sys.modules, "paper_2512_14069_b200._marshal", None)
+    with pytest.raises(RuntimeError, match="_marshal.so.*build it with"):
+        rb.lib()
