@@ -121,8 +121,9 @@ constexpr int kAccMinSlice = 4096;       // ... where there are rows enough to f
 constexpr int kTileTokens = 128;
 constexpr int kTileDoubles = 2 * kTileTokens;
 constexpr size_t kTileBytes = kTileDoubles * sizeof(double);
-// shared memory left for cached tiles when `per_sm` CTAs share an SM's 228 KB (1 KB of each is the system's, 20 KB static)
-constexpr size_t cache_room(int per_sm) { return ((228 * 1024 / per_sm - 1024 - 20 * 1024 - 512) / kTileBytes) * kTileBytes; }
+// shared memory left for cached tiles when `per_sm` CTAs with `fixed` bytes of static arrays share an SM's 228 KB (1 KB of each
+// is the system's)
+constexpr size_t cache_room(int per_sm, size_t fixed) { return ((228 * 1024 / per_sm - 1024 - fixed) / kTileBytes) * kTileBytes; }
 __host__ __device__ inline size_t cache_stride(int V) { return (((size_t)V + 3) & ~(size_t)3) + kTileTokens * 8; }
 extern __shared__ __align__(16) double s_cache[];
 struct Cache {
@@ -537,6 +538,11 @@ struct Residual {
     }
 };
 
+struct WalkShared {                      // all static shared memory of the kernel: cache_room counts on it
+    NodeShared node;
+    float ua[kMaxNodes];
+};
+
 template <typename T, int kPerSm>
 __global__ void __launch_bounds__(kSThreads, kPerSm) stochastic_walk_kernel(const __grid_constant__ StochParams P) {
     const radar_accept_args& a = P.a;
@@ -545,8 +551,9 @@ __global__ void __launch_bounds__(kSThreads, kPerSm) stochastic_walk_kernel(cons
     asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(csize));
     const int b = blockIdx.x / csize, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int V = a.V, W = a.t_max + 1;
-    __shared__ NodeShared S;
-    __shared__ float s_ua[kMaxNodes];
+    __shared__ WalkShared sh;
+    NodeShared& S = sh.node;
+    float (&s_ua)[kMaxNodes] = sh.ua;
     S.exps.fill(P.tab);
     ClusterRed red{S.red, P.status, crank, csize, 0};
     red.start();
@@ -732,6 +739,15 @@ struct AccLenParams {
     ExpTable tab;
 };
 
+constexpr int kAccBatch = 8, kAccRows = kAccBatch * kMaxNodes;     // sequences whose trees are looked at together, their rows
+struct AccLenShared {                    // all static shared memory of the kernel
+    NodeShared node;
+    __align__(16) int count[kAccRows + 4];      // children of each of their rows, then the order's keys
+    int group[kAccRows / 32];
+    int tok[kAccRows], par[kAccRows], drow[kAccRows];      // the batch's trees
+    short order[kAccRows];
+};
+
 // One item = one tree row with children of one sequence, evaluated by a cluster of CTAs (slices of the vocabulary, as in
 // the walk above).  The resident clusters take the items in turn; a row's children are tried in order with the same
 // closed-form residual recursion, but every rejection branch is followed: child j gets reach_j a_j with
@@ -744,12 +760,13 @@ __global__ void __launch_bounds__(kSThreads, kPerSm) accept_length_nodes_kernel(
     asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(crank));
     asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(csize));
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, V = a.V;
-    __shared__ NodeShared S;
-    constexpr int kBatch = 8, kRows = kBatch * kMaxNodes, kEach = kRows / kSThreads;      // sequences whose trees are looked at together
-    __shared__ __align__(16) int s_count[kRows + 4];         // children of each of their rows, then the order's keys
-    __shared__ int s_group[kRows / 32];
-    __shared__ short s_order[kRows];
-    __shared__ int s_tok[kRows], s_par[kRows], s_drow[kRows];      // the batch's trees
+    constexpr int kBatch = kAccBatch, kRows = kAccRows, kEach = kRows / kSThreads;
+    __shared__ AccLenShared sh;
+    NodeShared& S = sh.node;
+    int (&s_count)[kRows + 4] = sh.count;
+    int (&s_group)[kRows / 32] = sh.group;
+    short (&s_order)[kRows] = sh.order;
+    int (&s_tok)[kRows] = sh.tok, (&s_par)[kRows] = sh.par, (&s_drow)[kRows] = sh.drow;
     S.exps.fill(P.tab);
     ClusterRed red{S.red, P.status, crank, csize, 0};
     red.start();
@@ -935,9 +952,9 @@ ExpTable exp_table() {
 using namespace radar;
 
 // shared memory for the cached tiles of a slice, all of them or as many as fit
-static size_t cache_smem(int V, int cs, int per_sm) {
+static size_t cache_smem(int V, int cs, size_t room) {
     const int slice = 4 * (((V + 3) / 4 + cs - 1) / cs);
-    return std::min(cache_room(per_sm), (size_t)(slice + kTileTokens - 1) / kTileTokens * kTileBytes);
+    return std::min(room, (size_t)(slice + kTileTokens - 1) / kTileTokens * kTileBytes);
 }
 
 // launch configuration of the cluster kernels (attr: two attributes that outlive it)
@@ -960,9 +977,10 @@ static cudaLaunchConfig_t cluster_config(int ctas, int cs, size_t smem, cudaStre
 
 template <typename T, int kPerSm>
 static cudaError_t launch_walk(radar_ctx* ctx, StochParams& sp, int cs, cudaStream_t stream) {
-    const size_t smem = cache_smem(sp.a.V, cs, kPerSm);
+    constexpr size_t kRoom = cache_room(kPerSm, sizeof(WalkShared));
+    const size_t smem = cache_smem(sp.a.V, cs, kRoom);
     sp.smem_tiles = (int)(smem / kTileBytes);
-    cudaError_t e = radar_opt_in_smem(ctx, RADAR_SMEM_WALK + 2 * (sizeof(T) == 2) + kPerSm - 1, stochastic_walk_kernel<T, kPerSm>, cache_room(kPerSm));
+    cudaError_t e = radar_opt_in_smem(ctx, RADAR_SMEM_WALK + 2 * (sizeof(T) == 2) + kPerSm - 1, stochastic_walk_kernel<T, kPerSm>, kRoom);
     if (e != cudaSuccess) return e;
     cudaLaunchAttribute attr[2];
     const cudaLaunchConfig_t cfg = cluster_config(sp.a.B * cs, cs, smem, stream, attr);
@@ -1053,7 +1071,8 @@ extern "C" size_t radar_acclen_workspace_bytes(const radar_ctx* ctx, int B, int 
 template <typename T, int kPerSm>
 static cudaError_t launch_acclen(radar_ctx* ctx, AccLenParams& P, int cs, int max_clusters, cudaStream_t stream) {
     constexpr int kind = 2 * (sizeof(T) == 2) + kPerSm - 1;
-    cudaError_t e = radar_opt_in_smem(ctx, RADAR_SMEM_ACCLEN + kind, accept_length_nodes_kernel<T, kPerSm>, cache_room(kPerSm));
+    constexpr size_t kRoom = cache_room(kPerSm, sizeof(AccLenShared));
+    cudaError_t e = radar_opt_in_smem(ctx, RADAR_SMEM_ACCLEN + kind, accept_length_nodes_kernel<T, kPerSm>, kRoom);
     if (e != cudaSuccess) return e;
     // As many clusters as are resident at once: the rows are dealt out over them in advance.  How many that is, is a
     // property of the kernel and the device, asked for once per cluster size (with the most shared memory it may get).
@@ -1062,14 +1081,14 @@ static cudaError_t launch_acclen(radar_ctx* ctx, AccLenParams& P, int cs, int ma
     cudaLaunchAttribute attr[2];
     int& resident = ctx->acclen_clusters[kind][log_cs];
     if (resident == 0) {
-        cudaLaunchConfig_t q = cluster_config(2 * ctx->sm_count / cs * cs, cs, cache_room(kPerSm), stream, attr);
+        cudaLaunchConfig_t q = cluster_config(2 * ctx->sm_count / cs * cs, cs, kRoom, stream, attr);
         q.numAttrs = 1;
         int n = 0;
         e = cudaOccupancyMaxActiveClusters(&n, accept_length_nodes_kernel<T, kPerSm>, &q);
         if (e != cudaSuccess) return e;
         resident = n > 0 ? n : 1;
     }
-    const size_t smem = cache_smem(P.a.V, cs, kPerSm);
+    const size_t smem = cache_smem(P.a.V, cs, kRoom);
     P.smem_tiles = (int)(smem / kTileBytes);
     const cudaLaunchConfig_t cfg = cluster_config(std::min(max_clusters, resident) * cs, cs, smem, stream, attr);
     radar_launch_scope scope(ctx, RADAR_K_ACCLEN_NODES, stream);
