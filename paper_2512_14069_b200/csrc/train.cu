@@ -481,11 +481,15 @@ extern "C" int radar_policy_train_step(radar_ctx* ctx, const radar_train_args* a
     {
         radar_launch_scope scope(ctx, RADAR_K_TRAIN_ROLLOUT, stream);
         const unsigned n = (unsigned)a->n, sms = (unsigned)ctx->sm_count;
-        // Points per block: one wave of blocks, four points at most.  A block lasts as long as its longest trajectory, so
-        // where trajectories of 1 to 8 calls are mixed (an untrained gate) blocks of one point in several waves do as well
-        // (rollout alone, 1 / 2 / 4 points a block: n = 148 65 / 73 / 96 us, 290 77 / 75 / 95, 420 84 / 83 / 97, 592
-        // 112 / 104 / 99, 4000 484 / 410 / 373); where a trained gate makes them alike the wave decides (n = 256, whole
-        // step: 38 us with one point, 31 with two).
+        // Points per block: one wave of blocks, four points at most.  Whole step in us with 1 / 2 / 4 points a block, where the
+        // trajectories are 2, 3.1 and 6.8 calls long on average (a gate that has been trained makes 5 to 7):
+        //   n = 200   91 / 95 / 117    105 / 99 / 123    165 / 115 / 139
+        //   n = 290   106 / 99 / 121   132 / 114 / 137   184 / 135 / 160
+        //   n = 310   97 / 99 / 121    137 / 126 / 139   188 / 183 / 160
+        //   n = 420   122 / 117 / 131  158 / 149 / 144   255 / 220 / 180
+        //   n = 592   146 / 137 / 140  200 / 192 / 159   351 / 258 / 214
+        //   n = 1024  220 / 207 / 212  308 / 281 / 275   552 / 450 / 370
+        // A block lasts as long as its longest trajectory, so with short, mixed ones two points would do a little longer.
         const int kp = n <= sms ? 1 : n <= 2 * sms ? 2 : 4;
         const size_t smem = (size_t)kp * kGroups * H * sizeof(float);
         if (kp == 1) {

@@ -1116,8 +1116,9 @@ extern "C" int radar_accept_length_distribution(radar_ctx* ctx, const radar_accl
     P.status = ctx->d_status;
     P.tab = exp_table();
     // One CTA per SM while the rows (about twenty with children to a tree) are few waves, two when their passes are what
-    // takes the time: 4 trees, V = 32000 (16 CTAs times rows) 31 / 36 us for one / two; 4 trees, V = 70000 (32) 52 / 44;
-    // 16 trees, V = 32000 (64) 88 / 72; 8 trees, V = 128256 (64) 191 / 135.
+    // takes the time.  us for one / two, by trees times CTAs a row: 8 (1 tree, V = 128256) 42 / 47; 16 (4, 32000) 29 / 36, (8, 16000)
+    // 29 / 37, (2, 128256) 43 / 50; 20 (5, 32000) 33 / 37; 24 (6, 32000) 39 / 37, (3, 70000) 41 / 39, (3, 128256) 66 / 55; 32 (4, 70000)
+    // 47 / 41; 64 (16, 32000) 88 / 72, (8, 128256) 191 / 135.  (Short vocabularies cross later: 16 trees, V = 16000 47 / 65.)
     const bool one = a->B * cs <= 16;
     if (a->logits_dtype == RADAR_F32) RADAR_CUDA_CHECK((one ? launch_acclen<float, 1>(ctx, P, cs, max_clusters, stream) : launch_acclen<float, 2>(ctx, P, cs, max_clusters, stream)));
     else RADAR_CUDA_CHECK((one ? launch_acclen<__nv_bfloat16, 1>(ctx, P, cs, max_clusters, stream) : launch_acclen<__nv_bfloat16, 2>(ctx, P, cs, max_clusters, stream)));
