@@ -111,3 +111,27 @@ def test_temperature_range(T, ref, steps, masked, V):
         assert nodes.cpu().tolist()[0] == path + [-1] * (t_max + 1 - len(path)) and int(alen) == len(path) - 1
         assert int(nxt) == int(np.searchsorted(cdf, float(us) * cdf[-1], side="right"))
     ctx.close()
+
+
+def test_exponentials_to_the_last_places():
+    """Two tokens that matter, q = 1/2 each: P_acc of the one d below the other is 2 e^-d / (1 + e^-d), to the 1.1 ulp of the
+    exponential and half an ulp for each of the sum, two products and the quotient: below 4 units of 2^-53 x 2."""
+    import torch
+    from paper_2512_14069_b200 import binding as rb
+    ctx, B, V = rb.Context(0), 2048, 5
+    rng = np.random.default_rng(3)
+    d = np.concatenate([rng.uniform(0, 2, B // 4), rng.uniform(0, 40, B // 4), rng.uniform(0, 700, B // 2)]).astype(np.float32)
+    target, draft = np.full((B, 64, V), -np.inf, np.float32), np.full((B, 1, V), -np.inf, np.float32)
+    target[:, 0, 1], target[:, 0, 3], draft[:, 0, 1], draft[:, 0, 3] = 0.0, -d, 0.5, 0.5
+    dev = lambda x: torch.from_numpy(np.ascontiguousarray(x)).cuda()
+    rows = lambda a, b, fill: dev(np.tile(np.array([[a, b] + [fill] * 62], np.int32), (B, 1)))
+    dist, pacc = (torch.zeros(B, n, dtype=torch.float64, device="cuda") for n in (2, 64))
+    ws = torch.zeros(rb.radar_acclen_workspace_bytes(ctx, B, V), dtype=torch.uint8, device="cuda")
+    rb.radar_accept_length_distribution(ctx, B=B, V=V, t_max=1, temperature=1.0, target_logits=dev(target), tree_tok=rows(-1, 3, -1),
+                                        tree_parent=rows(-1, 0, -1), tree_depth=rows(0, 1, 0), tree_draft_row=rows(0, -1, -1),
+                                        n_nodes=dev(np.full(B, 2, np.int32)), draft_logits=dev(draft), R=1, dist=dist, p_acc_node=pacc, workspace=ws)
+    ctx.check_device_status()
+    e = np.exp(-d.astype(np.longdouble))
+    want = np.minimum(2 * e / (1 + e), 1)
+    assert np.max(np.abs(pacc[:, 1].cpu().numpy() / want - 1)) < 8 * 2.0 ** -53
+    ctx.close()

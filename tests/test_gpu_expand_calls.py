@@ -114,3 +114,24 @@ def test_long_passes_go_call_by_call(ctx):
     assert rb.radar_expand_calls_workspace_bytes(ctx, 32, 128256, 10, 8) == 0
     assert rb.radar_expand_calls_workspace_bytes(ctx, 1, 1 << 19, 8, 2) > 0 and rb.radar_expand_calls_workspace_bytes(ctx, 1, (1 << 19) + 1, 8, 2) == 0
     assert rb.radar_expand_calls_workspace_bytes(ctx, 1, 1000, 33, 8) == 0
+
+
+def test_a_workspace_full_of_other_sizes(ctx):
+    """Nothing of the workspace is read before it has been written: one that other sizes, and NaN patterns, have left behind."""
+    import torch
+    V, k, t_max = 9000, 10, 5
+    big = _step(ctx, 6, 30000, 12, 6)
+    big.run_expansion(torch.randn(6, big.R, 30000, device="cuda"), _gate(12, 6, 0))
+    draft = torch.randn(3, 1 + (t_max - 1) * k, V, device="cuda") * 3
+    gate, got = _gate(k, t_max, 0), []
+    for fill in (None, 0xff, 0):
+        s = _step(ctx, 3, V, k, t_max)
+        if fill is None:
+            s.ws_calls = big.ws_calls
+        else:
+            s.ws_calls.fill_(fill)
+        s.run_expansion(draft, gate)
+        ctx.check_device_status()
+        got.append([getattr(s, n).cpu() for n in NAMES])
+    for other in got[:2]:
+        assert all(torch.equal(x, y) for x, y in zip(got[2], other))
