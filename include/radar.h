@@ -161,16 +161,18 @@ typedef struct {
 size_t radar_expand_workspace_bytes(const radar_ctx* ctx, int B, int F, int V, int k);
 int radar_expand_step(radar_ctx* ctx, const radar_expand_args* args, void* stream);
 
-/* radar_expand_calls - all t_max draft calls of a step at once, for draft logits that are there already: the results of
- * radar_expand_step for t = 1 .. t_max, in three launches.  `call` holds the arguments of call 1 (t = 1, F = 1), with these
+/* radar_expand_calls - all t_max draft calls of a step at once, for draft logits that are there already (recorded ones, or a
+ * draft model that does not look at the frontier; where the draft model has to run on the frontier that a call selects
+ * before the next call's logits exist, radar_expand_step is the form): the results of radar_expand_step for
+ * t = 1 .. t_max, in three launches.  `call` holds the arguments of call 1 (t = 1, F = 1), with these
  * differences: logits is [B][1+(t_max-1)*k][V], call 1's row first, then the k rows of every further call in turn;
  * frontier_tok / _score / _pool_idx / _src_row [t_max][B][k], gate_logits [t_max][B][2] and cont [t_max][B] have a slice
  * per call (as with radar_expand_step only the calls a sequence makes write theirs, cont excepted); topk_tok and
  * topk_logp receive call 1's lists, topk_tok_next and topk_logp_next [t_max-1][B][k][k] those of the calls behind it;
  * phase is ignored.  Rows of calls a sequence does not make are read but reach no result.
  * Policies: RADAR_POLICY_LSTM_SCORES and RADAR_POLICY_MLP_SCORES.
- * Workspace: radar_expand_calls_workspace_bytes, 256-byte aligned; 0 where call by call is the better form (long rows, many
- * sequences) or the sizes are out of range: radar_expand_calls returns RADAR_ERR_UNSUPPORTED there. */
+ * Workspace: radar_expand_calls_workspace_bytes, 256-byte aligned; 0 where call by call is the better form (more than 4 Mi
+ * logits a call, B k V, or 5 Mi from k = 16 on; many sequences) or the sizes are out of range: radar_expand_calls returns RADAR_ERR_UNSUPPORTED there. */
 typedef struct {
     radar_expand_args call;
     int32_t* topk_tok_next;
@@ -341,7 +343,7 @@ int radar_verify_accept(radar_ctx* ctx, const radar_accept_args* args, void* str
  * plus tree_depth; no uniforms: every internal row is evaluated, not only one sampled path.
  * Outputs, fp64: dist[b][0..t_max] = p_0..p_tmax (sums to 1); p_acc_node[b][row] = P_acc(row)
  * (rows >= n_nodes[b]: 0).  Probabilities are evaluated in fp64.
- * Workspace: radar_acclen_workspace_bytes (two fp64 vocabulary rows per resident block).
+ * Workspace: radar_acclen_workspace_bytes (two fp64 vocabulary rows per resident cluster of blocks).
  */
 typedef struct {
     int B, V, t_max;

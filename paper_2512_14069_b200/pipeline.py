@@ -4,10 +4,17 @@
 acceptance output, workspaces) and issues the library calls in order on the current
 stream: t_max expansion calls (sequences the prediction model has stopped are skipped on
 the device, so no decision ever returns to the host), rerank + tree build, tree
-attention, acceptance.  The expansion calls are issued as two overlapping chains: the
-bandwidth-bound vocabulary passes run ahead on a side stream while the latency-bound
-select + gate blocks follow on the main stream (the pass of call t+1 skips the sequences
-that had stopped before call t; one that stops at call t is read once in vain).
+attention, acceptance.  Which form the expansion calls take is a matter of when their draft logits exist:
+
+  `expand(t, ...)`, or `run_expansion(pipelined=False)`: one call behind the other.  The form of a decoding loop, whose
+      draft model runs on the frontier of call t before the logits of call t + 1 are there.
+  `run_expansion(pipelined=True)`: for logits that are all there before call 1 (recorded ones, gathering training data for
+      the gate, a draft model that does not look at the frontier).  With short passes all calls go in one go
+      (`radar_expand_calls`); with long ones, and for the hidden-state policy, as two overlapping chains: the
+      bandwidth-bound vocabulary passes run ahead on a side stream while the latency-bound select + gate blocks follow
+      on the main stream (the pass of call t+1 skips the sequences that had stopped before call t; one that stops at
+      call t is read once in vain).
+
 It contains no arithmetic of the method.
 """
 from __future__ import annotations
@@ -111,6 +118,8 @@ class SpecStep:
 
     def run_expansion(self, draft_logits, gate, force_calls=None, policy=rb.RADAR_POLICY_LSTM_SCORES, features=None,
                       pipelined=True):
+        """All draft calls of a step on draft_logits [B,R,V].  `pipelined` needs the rows of all calls before the first one
+        (see the top of this file); without it call t reads its own rows only."""
         if pipelined and self.ws_calls is not None and policy != rb.RADAR_POLICY_LSTM_HIDDEN:
             self._expand_calls(draft_logits, gate, force_calls, policy)
             return
