@@ -34,6 +34,38 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
         : "memory");
     return ok != 0;
 }
+// Bounded wait: false once `limit` polls (each sleeps for up to a millisecond; polling warps take issue
+// slots from the others) have not seen the phase.  After a wait
+// that ran out (`ok` false) one poll is all that is spent, so that loops over waits run dry.  In one block of instructions: a
+// loop in C++ is unrolled at every one of its many sites, and a kernel's size is instruction-cache misses.
+__device__ __forceinline__ bool mbar_wait_while(bool ok, uint64_t* bar, uint32_t parity, uint32_t limit = 1u << 12) {
+    uint32_t r;
+    asm volatile(
+        "{\n\t.reg .pred p, q;\n\t.reg .u32 n;\n\t"
+        "mov.u32 n, %3;\n\t"
+        "WAIT:\n\t"
+        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, 1000000;\n\t"
+        "@p bra DONE;\n\t"
+        "sub.u32 n, n, 1;\n\t"
+        "setp.ne.u32 q, n, 0;\n\t"
+        "@q bra WAIT;\n\t"
+        "DONE:\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(r)
+        : "r"(smem_u32(bar)), "r"(parity), "r"(ok ? limit : 1u)
+        : "memory");
+    return ok && r != 0;
+}
+// For a wait that is long and whose end nothing hurries after: naps between the polls.
+__device__ __forceinline__ bool mbar_wait_lazy(bool ok, uint64_t* bar, uint32_t parity, uint32_t limit = 1u << 22) {
+#pragma unroll 1
+    for (uint32_t it = ok ? limit : 1u; it > 0; --it) {
+        if (mbar_try_wait(bar, parity)) return ok;
+        __nanosleep(200);
+    }
+    return false;
+}
+
 // Bounded wait: gives up after `limit` polls (each poll itself blocks for a hardware-defined short
 // time) or once *abort_flag has been set by another thread.  Returns false on give-up and sets the
 // flag.  A wait that is satisfied at once costs one try_wait and nothing else: the flag is looked at
@@ -50,13 +82,6 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volati
     }
     *abort_flag = 1;
     return false;
-}
-// The same for a whole (converged) warp: one lane polls, the others learn the outcome from it, so that
-// the barrier word is not hit by 32 polls at a time.  `ok` chains earlier outcomes (false: do not wait).
-__device__ __forceinline__ bool mbar_wait_warp(bool ok, uint64_t* bar, uint32_t parity, volatile int* abort_flag) {
-    int r = 0;
-    if ((threadIdx.x & 31) == 0) r = ok && mbar_wait(bar, parity, abort_flag);
-    return __shfl_sync(0xffffffffu, r, 0) != 0;
 }
 
 // ---- proxies and fences -------------------------------------------------------------------------
@@ -81,6 +106,11 @@ __device__ __forceinline__ void tma_load_4d(void* smem_dst, const void* tmap, ui
         "cp.async.bulk.tensor.4d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5, %6}], [%2];"
         ::"r"(smem_u32(smem_dst)), "l"(reinterpret_cast<uint64_t>(tmap)), "r"(smem_u32(bar)), "r"(c0), "r"(c1), "r"(c2), "r"(c3)
         : "memory");
+}
+
+__device__ __forceinline__ void tma_prefetch_4d(const void* tmap, int c0, int c1, int c2, int c3) {
+    asm volatile("cp.async.bulk.prefetch.tensor.4d.L2.global.tile [%0, {%1, %2, %3, %4}];"
+                 ::"l"(reinterpret_cast<uint64_t>(tmap)), "r"(c0), "r"(c1), "r"(c2), "r"(c3) : "memory");
 }
 
 // ---- tensor memory ------------------------------------------------------------------------------
@@ -197,10 +227,10 @@ __device__ __forceinline__ void mma_ss_x4(uint32_t pred, uint32_t d_tmem, uint32
 }
 //   TS: four steps; A advances by 8 tensor-memory columns (16 bf16) and B by 128 descriptor units (16 rows of
 //   an N-major tile) per step.  Steps at or beyond `nsteps` are not issued.
-__device__ __forceinline__ void mma_ts_x4(uint32_t pred, uint32_t nsteps, uint32_t d_tmem, uint32_t a_tmem, uint32_t b_lo,
+__device__ __forceinline__ void mma_ts_x4(uint32_t pred, int nsteps, uint32_t d_tmem, uint32_t a_tmem, uint32_t b_lo,
                                           uint32_t hi, uint32_t idesc, bool acc_first) {
 #define RADAR_TS_STEP(K, P)                                                                            \
-        "setp.gt.and.u32 qk, %1, " #K ", q;\n\t"                                                        \
+        "setp.gt.and.s32 qk, %1, " #K ", q;\n\t"                                                        \
         "add.u32 a, %3, " #K " * 8;\n\tadd.u32 b, %4, " #K " * 128;\n\tmov.b64 db, {b, %5};\n\t"         \
         "@qk tcgen05.mma.cta_group::1.kind::f16 [%2], [a], db, %6, " #P ";\n\t"
     asm volatile(
@@ -214,18 +244,18 @@ __device__ __forceinline__ void mma_ts_x4(uint32_t pred, uint32_t nsteps, uint32
         : "memory");
 #undef RADAR_TS_STEP
 }
-//   TS, two steps of each half of a 128-key tile (64 columns of A, 64 rows of B apart).
-__device__ __forceinline__ void mma_ts_x2x2_full(uint32_t pred, uint32_t d_tmem, uint32_t a_tmem, uint32_t b_lo, uint32_t hi,
-                                                 uint32_t idesc, bool acc_first) {
-#define RADAR_TS_STEP(A, B, P)                                                                         \
-        "add.u32 a, %2, " #A ";\n\tadd.u32 b, %3, " #B ";\n\tmov.b64 db, {b, %4};\n\t"                 \
+//   ... all four.
+__device__ __forceinline__ void mma_ts_x4(uint32_t pred, uint32_t d_tmem, uint32_t a_tmem, uint32_t b_lo,
+                                          uint32_t hi, uint32_t idesc, bool acc_first) {
+#define RADAR_TS_STEP(K, P)                                                                            \
+        "add.u32 a, %2, " #K " * 8;\n\tadd.u32 b, %3, " #K " * 128;\n\tmov.b64 db, {b, %4};\n\t"         \
         "@q tcgen05.mma.cta_group::1.kind::f16 [%1], [a], db, %5, " #P ";\n\t"
     asm volatile(
         "{\n\t.reg .pred q, p0, p1;\n\t.reg .b32 a, b;\n\t.reg .b64 db;\n\t"
         "setp.ne.b32 q, %0, 0;\n\t"
         "setp.ne.b32 p0, %6, 0;\n\t"
         "setp.eq.b32 p1, 0, 0;\n\t"
-        RADAR_TS_STEP(0, 0, p0) RADAR_TS_STEP(8, 128, p1) RADAR_TS_STEP(64, 512, p1) RADAR_TS_STEP(72, 640, p1)
+        RADAR_TS_STEP(0, p0) RADAR_TS_STEP(1, p1) RADAR_TS_STEP(2, p1) RADAR_TS_STEP(3, p1)
         "}"
         ::"r"(pred), "r"(d_tmem), "r"(a_tmem), "r"(b_lo), "r"(hi), "r"(idesc), "r"((uint32_t)acc_first)
         : "memory");
@@ -287,6 +317,15 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&r)[32]) {
           "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]), "=r"(r[16]),
           "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]),
           "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
+        : "r"(taddr)
+        : "memory");
+}
+__device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[16]) {
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
+        "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
+          "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
         : "r"(taddr)
         : "memory");
 }

@@ -13,21 +13,25 @@
 // there are several pairs per KV head, CTAs alternate between them so that they stream the same K/V
 // at the same time and all but the first read hit L2.
 //
-// Inside the CTA (10 warps):
-//   warp 8     TMA producer: per segment the Q rows, then K and V tiles into two rings (128-byte
-//              swizzle), in the order the MMA warp consumes them.
-//   warp 9     MMA issuer (one lane): S = Q K^T into one of two tensor-memory score buffers, and
-//              O (+)= P V with P read back from tensor memory (bf16, overlaying S) and V consumed
-//              N-major straight from the row-major tile.
-//   warps 0-3 / 4-7  softmax groups 0 / 1, one thread per query row: S row from tensor memory,
-//              prefix-boundary / ancestor-bit masking in registers, running max with lazy rescaling
-//              of the O accumulator, exp2, P back to tensor memory.
+// Inside the CTA (16 warps; the registers are shared out by warpgroup):
+//   warp 12    TMA producer: works out the CTA's segments for itself and, through a ring in shared memory, for the others;
+//              per segment the Q rows, then K and V tiles into two rings (128-byte swizzle), in the order the MMA warp
+//              consumes them.
+//   warp 13    MMA issuer: S = Q K^T into one of two tensor-memory score buffers, and O (+)= P V with P read back from
+//              tensor memory (bf16, overlaying S) and V consumed N-major straight from the row-major tile.
+//   warps 0-3 / 4-7  softmax groups 0 / 1, one thread per query row: the row's scores from tensor memory into registers,
+//              running max with lazy rescaling of the O accumulator, exp2, P back to tensor memory.
 //              Unit with two live row blocks: group s owns row block s and sees every tile, so each
 //              K/V tile is loaded once for 256 query rows.  Unit with one live row block: the
 //              groups take alternate tiles with separate (m, l, O) and are merged at the end.
 //              Either way one group's softmax overlaps the other's MMAs.
+//   warps 8-11 epilogue: a finished accumulator to O or to the partials, while the others are in the next segment.
+//   warps 14, 15 only fill up the producer's warpgroup.
+// What is rare (ends of segments, tiles that are not full) shares its code with what is not, or is written as loops: with every
+// wait, schedule and mask unrolled in line the kernel had 140 KB of code, a segment's end missed the instruction cache all
+// along, and 8.5 thousand cycles lay between a segment's last product and the next one's first.
 // Every mbarrier wait is bounded; a wait that runs out sets RADAR_ERR_TIMEOUT on the device status
-// word, the CTA drains without skipping any hardware barrier, frees its tensor memory and returns.
+// word, the CTA drains, frees its tensor memory and returns.
 #include <cuda.h>
 
 #include <algorithm>
@@ -42,10 +46,14 @@ namespace {
 
 using namespace tc05;
 
-constexpr int kTcThreads = 576;      // 16 softmax warps, TMA producer, MMA issuer
-constexpr int kProducerWarp = 16, kMmaWarp = 17;
+constexpr int kTcThreads = 512;
+constexpr int kEpilogueWarp = 8, kProducerWarp = 12, kMmaWarp = 13;
+// Registers a thread: 128 at launch, then shared out by warpgroup (two of softmax; what they take the other two give).
+constexpr int kSoftmaxRegs = 176, kEpilogueRegs = 88, kIssueRegs = 72;
+static_assert(2 * kSoftmaxRegs + kEpilogueRegs + kIssueRegs <= 512, "a block shares out the registers it was launched with");
 constexpr int kStaticSmem = 3072;    // barriers and exchange arrays: with the tiles exactly the 227 KB a block may have
 constexpr int kTileKeys = 128;       // keys per prefix tile
+constexpr int kFirstKeys = 64;       // keys of a tile whose products start before the rest of its probabilities is there
 constexpr int kTreeKeys = 64;        // keys of the tree tile (RADAR_MAX_NODES)
 constexpr int kPairRows = 256;       // query rows of a row-block pair (and the stride of partial records)
 constexpr long long kLatencyWork = 9 << 15;   // sequences x query heads x keys x head dimension: tree_attn_tc_supported
@@ -76,9 +84,9 @@ struct TcParams {
     int ncc;             // CTAs per class; grid = n_cls * ncc
     int cost_one, cost_two, unit_cost;   // tile_costs(n_cls)
     float scale_log2;
-    float scale_log2_lo; // FINE: what scale_log2 is below the scale itself (positive)
+    float scale_log2_lo; // two parts of P: what scale_log2 is below the scale itself (positive)
     long long cache_rows;
-    float2* part_ml;     // [grid][2][256]     (m in natural-log units, with FINE in log2 units; l)
+    float2* part_ml;     // [grid][2][256]     (m in natural-log units, with two parts of P in log2 units; l)
     float* part_o;       // [grid][2][256][D]
     CutUnit* cut;        // [grid]
     int* status;
@@ -101,6 +109,32 @@ __device__ __forceinline__ float ex2(float x) {
     asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
     return y;
 }
+// the same and the other steps of a probability, kept in the order in which they are written
+__device__ __forceinline__ float ex2_in_order(float x) {
+    float y;
+    asm volatile("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+__device__ __forceinline__ float2 fma2_in_order(float2 a, float2 b, float2 c) {
+    float2 d;
+    asm volatile("{\n\t.reg .b64 a, b, c, d;\n\tmov.b64 a, {%2, %3};\n\tmov.b64 b, {%4, %5};\n\tmov.b64 c, {%6, %7};\n\t"
+                 "fma.rn.f32x2 d, a, b, c;\n\tmov.b64 {%0, %1}, d;\n\t}"
+                 : "=f"(d.x), "=f"(d.y) : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y), "f"(c.x), "f"(c.y));
+    return d;
+}
+__device__ __forceinline__ float2 add2_in_order(float2 a, float2 b) {
+    float2 d;
+    asm volatile("{\n\t.reg .b64 a, b, d;\n\tmov.b64 a, {%2, %3};\n\tmov.b64 b, {%4, %5};\n\tadd.rn.f32x2 d, a, b;\n\tmov.b64 {%0, %1}, d;\n\t}"
+                 : "=f"(d.x), "=f"(d.y) : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+    return d;
+}
+__device__ __forceinline__ uint32_t bf16x2_in_order(float lo, float hi) {
+    uint32_t d;
+    asm volatile("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(d) : "f"(hi), "f"(lo));
+    return d;
+}
+template <int N> __device__ __forceinline__ void regs_inc() { asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(N)); }
+template <int N> __device__ __forceinline__ void regs_dec() { asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(N)); }
 // m ln 2 + ln l, m in log2 units
 __device__ __forceinline__ float lse_of(float m, float l) {
     constexpr float kHi = 0.693147182f, kLo = (float)(0.6931471805599453 - (double)kHi);
@@ -185,6 +219,75 @@ struct Cursor {
     __device__ __forceinline__ bool two_rb(const TcParams& P) const { return s.rows > P.rb_rows; }
 };
 
+// The first segment of CTA ci of a class, by a whole warp: the unit that contains the start of its range, from the unit's first
+// tile that starts at or after it.  tot_all: size of the class's space (all layers).
+template <bool PAGED>
+__device__ __forceinline__ Cursor<PAGED> first_segment(const TcParams& P, int pp, int ci, long long& tot_all) {
+    const radar_attn_args& a = P.a;
+    const int lane = threadIdx.x & 31;
+    long long tot = 0;
+#pragma unroll 1
+    for (int b0 = 0; b0 < a.B; b0 += 32) {
+        const int b = b0 + lane;
+        if (pp == 0 && ci == 0 && b < a.B) {
+            const int Pb = a.prefix_len[b];
+            const long long kv0 = PAGED ? 0 : a.kv_start[b];
+            if (Pb < 0 || Pb > a.max_prefix_len || kv0 < 0 || kv0 + Pb > P.cache_rows) set_status(P.status, RADAR_ERR_INVALID_ARG);
+        }
+        tot += warp_sum(b < a.B ? seq_cost<PAGED>(P, b, pp) : 0ll);
+    }
+    // the space of all layers: layer l occupies [l * tot, (l + 1) * tot)
+    tot_all = tot * P.n_layers;
+    const long long lo_all = tot_all * ci / P.ncc;
+    Cursor<PAGED> cur;
+    cur.hi = tot_all * (ci + 1) / P.ncc;
+    cur.unit_cost = P.unit_cost;
+    cur.layer = tot > 0 ? (int)(lo_all / tot) : 0;
+    cur.t0 = cur.t1 = 0;
+    cur.b = -1;
+    cur.g = 0;
+    cur.U = 0;
+    const long long lo = lo_all - (long long)cur.layer * tot;
+    long long cum = 0;
+#pragma unroll 1
+    for (int b0 = 0; b0 < a.B && cur.b < 0; b0 += 32) {
+        const int b = b0 + lane;
+        const long long sz = b < a.B ? seq_cost<PAGED>(P, b, pp) : 0;
+        long long incl = sz;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const long long v = __shfl_up_sync(kFull, incl, o);
+            if (lane >= o) incl += v;
+        }
+        const unsigned hit = __ballot_sync(kFull, cum + incl > lo);
+        if (hit) {
+            const int src = __ffs(hit) - 1;
+            const long long before = cum + __shfl_sync(kFull, incl - sz, src);
+            cur.b = b0 + src;
+            cur.s = seq_info<PAGED>(P, cur.b, pp);
+            const long long unit = (long long)cur.s.nt * cur.s.w + P.unit_cost;
+            cur.g = (int)((lo - before) / unit);
+            cur.U = before + cur.g * unit + (long long)cur.layer * tot;
+        }
+        cum += __shfl_sync(kFull, incl, 31);
+    }
+    if (cur.b >= 0 && cur.layer < P.n_layers) {
+        cur.t0 = tiles_before(lo_all, cur.U, cur.s.nt, cur.s.w, P.unit_cost);
+        if (cur.t0 >= cur.s.nt) cur.next_unit(P, pp);       // every tile of that unit starts before the range
+        else cur.clip();
+    }
+    return cur;
+}
+
+// What the other warps know of a segment.
+constexpr int kSegRing = 4;
+struct __align__(16) Segment {
+    int n;                               // tiles; 0: there is no further segment
+    int t0, nt, Pb, M, rows;             // first tile, tiles of the unit, prefix length, tree rows, live query rows
+    int b, g, layer;
+    int pad[3];
+};
+
 template <int D, bool TWO>
 struct Smem {
     static constexpr int kHalves = D / 64;
@@ -200,13 +303,671 @@ struct Smem {
 // TWO: the launch may contain units with two live row blocks; decides the shared-memory layout
 // PAGED: the prefix cache is read through a block table (a separate instantiation, so that the contiguous
 // layout's code is not touched by it)
-// FINE: P goes to the tensor cores as the sum of two bf16 numbers (its value to 2^-18) in place of one (2^-9), and the scores'
-// scale is applied in two parts.  For the head ratios that do not divide 128: they came from the FMA kernel, whose
-// probabilities are fp32, and keep its precision here (error against fp64, 2-norm, of 24 / 8 heads, 2048 tokens: FMA 1.6545e-3,
-// one bf16 2.1607e-3, two 1.6545e-3, all of it the rounding of O to bf16).
-template <int D, bool TWO, bool PAGED, bool FINE>
-__global__ void __launch_bounds__(kTcThreads, 1)      // 18 warps are allocated as 20: 96 registers per thread
+template <int D, bool TWO, bool PAGED>
+__global__ void __launch_bounds__(kTcThreads, 1)
 tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmKc,
+                    const __grid_constant__ CUtensorMap tmVc, const __grid_constant__ CUtensorMap tmKt,
+                    const __grid_constant__ CUtensorMap tmVt, const TcParams P) {
+    chain_trigger();                     // the producer waits for the predecessor below; the barrier, tensor-memory and
+                                         // descriptor set-up of the other warps needs nothing from global memory
+    using SM = Smem<D, TWO>;
+    constexpr int H = SM::kHalves;
+    constexpr int RK = SM::kRingK, RV = SM::kRingV;
+    const radar_attn_args& a = P.a;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int pp = blockIdx.x % P.n_cls;                    // class
+    const int ci = blockIdx.x / P.n_cls;
+    const int G = P.G;
+
+    // Static block first (padded to a multiple of 1024 bytes and aligned to it), the tiles behind it: the
+    // swizzled tiles need a 1024-byte boundary and there is no room left for alignment slack.
+    struct __align__(1024) Static {
+        uint64_t bar_qfull, bar_qempty, bar_kfull[3], bar_kempty[3], bar_vfull[3], bar_vempty[3];
+        uint64_t bar_sfull[2], bar_odone[2], bar_ofree[2], bar_mlfull, bar_mlempty;
+        uint64_t bar_pfirst[2];          // the probabilities of the tile's first kFirstKeys keys are there
+        uint64_t bar_pready[2];          // ... all of them
+        uint64_t bar_segfull[kSegRing], bar_segempty[kSegRing];
+        Segment seg[kSegRing];
+        float2 ml[2][128];               // per group: (m in log2 units, l) of the rows at the end of a segment
+        uint32_t tmem_base;
+        int abort;
+        unsigned char pad[kStaticSmem - ((26 + 2 * kSegRing) * 8 + kSegRing * (int)sizeof(Segment) + 2 * 128 * 8 + 8)];
+    };
+    static_assert(sizeof(Static) == kStaticSmem, "static shared-memory block");
+    __shared__ Static st;
+    extern __shared__ __align__(1024) unsigned char smem_raw[];
+    unsigned char* sQ = smem_raw;
+    unsigned char* sK = sQ + SM::kQBytes;
+    unsigned char* sV = sK + RK * SM::kTileBytes;
+
+    // ---- set-up ----
+    if (warp == 0) {
+        if (lane == 0) {
+            st.abort = 0;
+            mbar_init(&st.bar_qfull, 1);
+            mbar_init(&st.bar_qempty, 1);
+            for (int i = 0; i < 3; ++i) {
+                mbar_init(&st.bar_kfull[i], 1); mbar_init(&st.bar_kempty[i], 1);
+                mbar_init(&st.bar_vfull[i], 1); mbar_init(&st.bar_vempty[i], 1);
+            }
+            for (int i = 0; i < 2; ++i) {
+                mbar_init(&st.bar_sfull[i], 1); mbar_init(&st.bar_pfirst[i], 4); mbar_init(&st.bar_pready[i], 4);
+                mbar_init(&st.bar_odone[i], 1); mbar_init(&st.bar_ofree[i], 4);
+            }
+            for (int i = 0; i < kSegRing; ++i) { mbar_init(&st.bar_segfull[i], 1); mbar_init(&st.bar_segempty[i], kProducerWarp + 1); }
+            mbar_init(&st.bar_mlfull, 8);
+            mbar_init(&st.bar_mlempty, 4);
+            fence_barrier_init();
+        }
+    } else if (warp == kMmaWarp) {
+        tmem_alloc(&st.tmem_base, 512);
+        tmem_relinquish();
+        if (lane == 0) {
+            tma_prefetch_desc(&tmQ); tma_prefetch_desc(&tmKc); tma_prefetch_desc(&tmVc);
+            tma_prefetch_desc(&tmKt); tma_prefetch_desc(&tmVt);
+        }
+    }
+    tc_fence_before_sync();
+    __syncthreads();
+    tc_fence_after_sync();
+    // All of tensor memory is this CTA's, so its addresses are constants (the producer checks): S/P buffers in columns 0 and
+    // 128, O accumulators in 256 and 384.  An address that the compiler does not know to be the same in every lane costs the
+    // issuing warp a handful of instructions for every product.
+    constexpr uint32_t tmem = 0;
+    bool ok = true;                         // no wait of this thread has run out
+    // the producer's next segment; false behind the last one
+    auto take_segment = [&](uint32_t seg, Segment& s) {
+        ok = mbar_wait_while(ok, &st.bar_segfull[seg % kSegRing], (seg / kSegRing) & 1);
+        ok = __all_sync(kFull, ok);
+        s = st.seg[seg % kSegRing];
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&st.bar_segempty[seg % kSegRing]);
+        return ok && s.n > 0;
+    };
+
+    if (warp < kEpilogueWarp) {
+        regs_inc<kSoftmaxRegs>();
+        // =================================== softmax groups ===================================
+        // One thread per query row, which holds the tile's 128 scores in registers: tensor memory is read once and no two
+        // threads have to agree on a maximum.  (Two threads a row, 64 scores each read twice for want of registers, was the
+        // form before: 32 layers, 8 sequences of 6000 to 8192 tokens, 64 / 8 heads 4118 -> 3930 us; one layer of it within a
+        // step 307 -> 295; 32 layers of one sequence of 2048 tokens, 32 / 8 heads 105 -> 101.)
+        const int grp = warp >> 2;
+        const int row = (warp & 3) * 32 + lane;                 // row of the block == tensor-memory lane
+        const uint32_t lane_addr = (uint32_t)((warp & 3) * 32) << 16;
+        const uint32_t tS = tmem + grp * 128 + lane_addr;
+        const uint32_t tO = tmem + 256 + grp * 128 + lane_addr;
+        const int rb_node = (int)(((uint32_t)row * P.g_magic) >> 16);        // row / G
+        uint32_t sc = 0;                         // S tiles this group has waited for
+        Segment s;
+        for (uint32_t seg = 0; take_segment(seg, s); ++seg) {
+            const bool two = TWO && s.rows > P.rb_rows;
+            const int blk = two ? grp : 0;                       // row block within the unit
+            const int node = (pp * P.n_blk + blk) * P.nodes_per_rb + rb_node;
+            const int rows_here = min(s.rows - blk * P.rb_rows, P.rb_rows);  // live rows of this row block
+            // A warp none of whose 32 rows is live does no arithmetic (the products of its rows are never read):
+            // it only keeps the barriers going.
+            const bool warp_live = row - lane < rows_here;
+            // the row's ancestor word is needed by the tree tile only (the unit's last): it is loaded here and first
+            // touched there, so that the segment does not start with a wait for global memory
+            uint32_t mask_lo, mask_hi;
+            asm volatile("ld.global.v2.u32 {%0, %1}, [%2];" : "=r"(mask_lo), "=r"(mask_hi) : "l"(a.mask + (int64_t)s.b * kMaxNodes + min(node, kMaxNodes - 1)));
+            const int n_my = two ? s.n : (s.n - grp + 1) >> 1;
+            float m_run = -CUDART_INF_F, l_run = 0.f;
+
+#pragma unroll 1
+            for (int j = 0; j < n_my; ++j) {
+                const int t = s.t0 + (two ? j : 2 * j + grp);
+                ok = mbar_wait_while(ok, &st.bar_sfull[grp], sc & 1);
+                ok = __all_sync(kFull, ok);                      // warp-uniform: guards .aligned ops
+                ++sc;
+                tc_fence_after_sync();
+                if (ok && warp_live) {
+                    uint32_t sv[4][32];
+                    const int valid = s.Pb - t * kTileKeys;
+                    if (t == s.nt - 1 || valid < kTileKeys) {
+                        // Keys that the row may not attend to (and, of the tree tile, which has 64, the columns that are stale)
+                        // become -inf in tensor memory, 32 at a time: one tile of a unit or two need it, and an unrolled path
+                        // for them would be fetched into the instruction cache anew each time.
+#pragma unroll 1
+                        for (int c = 0; c < 4; ++c) {
+                            uint32_t al;
+                            if (t == s.nt - 1) {
+                                const int live = s.M - c * 32;
+                                al = row < rows_here && c < 2 && live > 0 ? (c == 0 ? mask_lo : mask_hi) & (live >= 32 ? 0xffffffffu : (1u << live) - 1u) : 0u;
+                            } else {
+                                const int lim = valid - c * 32;
+                                al = lim >= 32 ? 0xffffffffu : (lim <= 0 ? 0u : ((1u << lim) - 1u));
+                            }
+                            tmem_ld32(tS + c * 32, sv[0]);
+                            tmem_wait_ld();
+#pragma unroll
+                            for (int e = 0; e < 32; ++e)
+                                if (!((al >> e) & 1u)) sv[0][e] = 0xff800000u;     // -inf
+                            tmem_st32(tS + c * 32, sv[0]);
+                        }
+                        tmem_wait_st();
+                    }
+#pragma unroll
+                    for (int c = 0; c < 4; ++c) tmem_ld32(tS + c * 32, sv[c]);
+                    tmem_wait_ld();
+                    float mxa[4];
+#pragma unroll
+                    for (int c = 0; c < 4; ++c) {
+                        mxa[c] = __uint_as_float(sv[c][0]);
+#pragma unroll
+                        for (int e = 1; e < 31; e += 2)                     // three-input maxima: half the instructions
+                            mxa[c] = max3(mxa[c], __uint_as_float(sv[c][e]), __uint_as_float(sv[c][e + 1]));
+                        mxa[c] = fmaxf(mxa[c], __uint_as_float(sv[c][31]));
+                    }
+                    const float mx = fmaxf(max3(mxa[0], mxa[1], mxa[2]), mxa[3]);
+                    // ---- running max (log2 units), lazy rescale of the accumulator when some row of the warp moved its max ----
+                    const float m_tile = mx * P.scale_log2;
+                    float factor = 1.f;
+                    if (j == 0) {
+                        m_run = m_tile;
+                    } else if (m_tile > m_run + kRescaleThreshold) {
+                        factor = ex2(m_run - m_tile);           // m_run may be -inf: factor 0 clears O and l
+                        m_run = m_tile;
+                    }
+                    const float m_use = m_run == -CUDART_INF_F ? 0.f : m_run;
+                    if (j > 0 && __any_sync(kFull, factor != 1.f)) {
+#pragma unroll 1
+                        for (int c = 0; c < D; c += 16) {
+                            uint32_t o[16];
+                            tmem_ld16(tO + c, o);
+                            tmem_wait_ld();
+#pragma unroll
+                            for (int e = 0; e < 16; ++e) o[e] = __float_as_uint(__uint_as_float(o[e]) * factor);
+                            tmem_st16(tO + c, o);
+                        }
+                    }
+                    // ---- P = exp2(s * scale - m), row sum, bf16 pairs back to tensor memory ----
+                    // (the scaling and the row sum work on pairs: one packed fp32x2 instruction per two values)
+                    // The warp issues in order and an exponential takes its unit 8 cycles: what else there is to do stands between
+                    // two of them.
+                    float2 ls[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
+                    const float2 sc2 = make_float2(P.scale_log2, P.scale_log2), nm2 = make_float2(-m_use, -m_use);
+                    uint32_t pk[16];
+                    auto scale = [&](const int p) {
+                        uint32_t &x = sv[p >> 4][2 * (p & 15)], &y = sv[p >> 4][2 * (p & 15) + 1];
+                        const float2 s2 = make_float2(__uint_as_float(x), __uint_as_float(y));
+                        const float2 t2 = fma2_in_order(s2, sc2, nm2);
+                        x = __float_as_uint(t2.x);
+                        y = __float_as_uint(t2.y);
+                    };
+                    auto finish = [&](const int p) {
+                        const float p0 = __uint_as_float(sv[p >> 4][2 * (p & 15)]), p1 = __uint_as_float(sv[p >> 4][2 * (p & 15) + 1]);
+                        ls[p & 1] = add2_in_order(ls[p & 1], make_float2(p0, p1));
+                        pk[p & 15] = bf16x2_in_order(p0, p1);
+                        if ((p & 15) == 15) tmem_st16(tS + (p >> 4) * 16, pk);
+                    };
+                    // pairs that the scaling is ahead, that the rest is behind, and that the first stores are given to land in
+                    constexpr int kAhead = 2, kLag = 4, kLanding = 4;
+#pragma unroll
+                    for (int p = 0; p < kAhead; ++p) scale(p);
+#pragma unroll
+                    for (int p = 0; p < 64 + kLag; ++p) {
+                        if (p < 64) sv[p >> 4][2 * (p & 15)] = __float_as_uint(ex2_in_order(__uint_as_float(sv[p >> 4][2 * (p & 15)])));
+                        if (p + kAhead < 64) scale(p + kAhead);
+                        if (p < 64) sv[p >> 4][2 * (p & 15) + 1] = __float_as_uint(ex2_in_order(__uint_as_float(sv[p >> 4][2 * (p & 15) + 1])));
+                        if (p >= kLag) finish(p - kLag);
+                        if (p == kFirstKeys / 2 - 1 + kLag + kLanding) {
+                            tmem_wait_st();
+                            tc_fence_before_sync();
+                            __syncwarp();
+                            if (lane == 0) mbar_arrive(&st.bar_pfirst[grp]);
+                        }
+                    }
+                    l_run = l_run * factor + ((ls[0].x + ls[0].y) + (ls[1].x + ls[1].y));
+                    tmem_wait_st();
+                }
+                tc_fence_before_sync();
+                __syncwarp();
+                if (lane == 0) {
+                    if (!(ok && warp_live)) mbar_arrive(&st.bar_pfirst[grp]);
+                    mbar_arrive(&st.bar_pready[grp]);
+                }
+            }
+
+            // the rows' (m, l) go to the epilogue, which has taken those of the segment before
+            ok = mbar_wait_while(ok, &st.bar_mlempty, (seg & 1) ^ 1);
+            st.ml[grp][row] = make_float2(m_run, l_run);
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&st.bar_mlfull);
+        }
+    } else if (warp < kProducerWarp) {
+        regs_dec<kEpilogueRegs>();
+        // =================================== epilogue ===================================
+        // One thread per tensor-memory lane takes the finished accumulators to O (or to the partials) while the softmax
+        // groups and the tensor cores are already in the next segment; each accumulator is handed back as soon as it is read.
+        const int row = (warp - kEpilogueWarp) * 32 + lane;
+        const uint32_t tO = tmem + 256 + ((uint32_t)((warp - kEpilogueWarp) * 32) << 16);
+        const int rb_node = (int)(((uint32_t)row * P.g_magic) >> 16);        // row / G
+        uint32_t oc[2] = {0, 0};             // accumulators waited for
+        Segment s;
+        for (uint32_t seg = 0; take_segment(seg, s); ++seg) {
+            const bool two = TWO && s.rows > P.rb_rows;
+            const bool final_rows = s.n == s.nt;                 // the whole unit
+            const int slot = seg == 0 ? 0 : 1;                   // a CTA has at most a cut first and a cut last segment
+            ok = mbar_wait_lazy(ok, &st.bar_mlfull, seg & 1);
+            const float2 ml0 = st.ml[0][row], ml1 = st.ml[1][row];
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&st.bar_mlempty);
+#pragma unroll 1
+            for (int blk = 0; blk < 2; ++blk) {
+                // two live row blocks: accumulator blk is row block blk; one: both belong to it, merged in the first trip
+                if (blk == 1 && !two) {
+                    if (lane == 0) mbar_arrive(&st.bar_ofree[1]);
+                    break;
+                }
+                ok = mbar_wait_while(ok, &st.bar_odone[blk], oc[blk] & 1);
+                ++oc[blk];
+                const bool merge = !two && s.n > 1;
+                if (merge) {
+                    ok = mbar_wait_while(ok, &st.bar_odone[1], oc[1] & 1);
+                    ++oc[1];
+                }
+                ok = __all_sync(kFull, ok);
+                tc_fence_after_sync();
+                const int rows_here = min(s.rows - blk * P.rb_rows, P.rb_rows);  // live rows of this row block
+                const bool row_live = row < rows_here;
+                if (ok && row - lane < rows_here) {
+                    float m_out = blk == 0 ? ml0.x : ml1.x, l_out = blk == 0 ? ml0.y : ml1.y, w0 = 1.f, w1 = 0.f;
+                    if (merge) {
+                        m_out = fmaxf(ml0.x, ml1.x);
+                        const float ms = m_out == -CUDART_INF_F ? 0.f : m_out;
+                        w0 = ex2(ml0.x - ms);                        // exp2(-inf) = 0
+                        w1 = ex2(ml1.x - ms);
+                        l_out = ml0.y * w0 + ml1.y * w1;
+                    }
+                    const float m_safe = m_out == -CUDART_INF_F ? 0.f : m_out;
+                    const float inv = final_rows ? 1.f / l_out : 1.f;
+                    const int node = (pp * P.n_blk + blk) * P.nodes_per_rb + rb_node;
+                    const int hq = s.g * G + row - rb_node * G;
+                    const int64_t out_row = ((int64_t)s.b * kMaxNodes + node) * a.Hq + hq;
+                    const int64_t rec = ((int64_t)blockIdx.x * 2 + slot) * kPairRows + blk * 128 + row;
+                    __nv_bfloat16* dst_o = reinterpret_cast<__nv_bfloat16*>(a.O) + s.layer * P.o_ls + out_row * D;
+                    float* dst_p = P.part_o + rec * D;                  // 128-byte aligned (workspace carve)
+                    const bool wide = (reinterpret_cast<uintptr_t>(dst_o) & 31) == 0;
+#pragma unroll 1
+                    for (int col = 0; col < D; col += 16) {
+                        uint32_t o[16], o2[16];
+                        tmem_ld16(tO + blk * 128 + col, o);
+                        if (merge) tmem_ld16(tO + 128 + col, o2);
+                        tmem_wait_ld();
+                        float v[16];
+#pragma unroll
+                        for (int e = 0; e < 16; ++e) v[e] = __uint_as_float(o[e]) * w0;
+                        if (merge) {
+#pragma unroll
+                            for (int e = 0; e < 16; ++e) v[e] = fmaf(__uint_as_float(o2[e]), w1, v[e]);
+                        }
+                        if (row_live) {
+                            uint32_t w[8];
+                            if (final_rows) {
+#pragma unroll
+                                for (int e = 0; e < 8; ++e) {
+                                    const __nv_bfloat162 t2 = __floats2bfloat162_rn(v[2 * e] * inv, v[2 * e + 1] * inv);
+                                    w[e] = *reinterpret_cast<const uint32_t*>(&t2);
+                                }
+                                if (wide) {
+                                    st_global_32b(dst_o + col, w);
+                                } else {
+                                    *reinterpret_cast<uint4*>(dst_o + col) = make_uint4(w[0], w[1], w[2], w[3]);
+                                    *reinterpret_cast<uint4*>(dst_o + col + 8) = make_uint4(w[4], w[5], w[6], w[7]);
+                                }
+                            } else {
+#pragma unroll
+                                for (int q = 0; q < 2; ++q) {
+#pragma unroll
+                                    for (int e = 0; e < 8; ++e) w[e] = __float_as_uint(v[q * 8 + e]);
+                                    st_global_32b(dst_p + col + q * 8, w);
+                                }
+                            }
+                        }
+                    }
+                    if (row_live) {
+                        const float m_nat = m_safe * 0.6931471805599453f;
+                        if (final_rows) {
+                            if (a.lse != nullptr) a.lse[s.layer * P.lse_ls + ((int64_t)s.b * a.Hq + hq) * kMaxNodes + node] = m_nat + logf(l_out);
+                        } else {
+                            P.part_ml[rec] = make_float2(m_out == -CUDART_INF_F ? m_out : m_nat, l_out);
+                        }
+                    }
+                }
+                tc_fence_before_sync();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&st.bar_ofree[blk]);
+            }
+        }
+    } else {
+        regs_dec<kIssueRegs>();
+        if (warp == kProducerWarp) {
+            // =================================== TMA producer ===================================
+            // One lane does everything for the contiguous cache.  With a paged cache the whole warp walks the same
+            // loop and lane p looks up and fetches page p of a tile (up to eight boxes per tile), the leading lane
+            // still doing the waits, the byte counts, Q and the tree tile.
+            chain_sync();                        // every global access of the CTA comes after the first segment is there
+            const bool lead = lane == 0;
+            const bool usable = (smem_u32(smem_raw) & 1023u) == 0 && st.tmem_base == 0;     // (else the tiles would not sit on their swizzle boundary)
+            if (!usable && lead) set_status(P.status, RADAR_ERR_CUDA);
+            long long tot_all;
+            Cursor<PAGED> cur = first_segment<PAGED>(P, pp, ci, tot_all);
+            if (!usable) cur.t0 = cur.t1 = 0;
+            CutUnit cu;
+            cu.valid = 0;
+            int cut_nt = 0, cut_w = 0;
+            long long cut_u0 = 0;
+            uint32_t k_slot = 0, k_par = 1, v_slot = 0, v_par = 1;   // ring slot to fill next and the phase that frees it
+            const int n_cache_pages = PAGED ? (int)P.cache_rows / a.page_size : 0;            // (cache_rows: below 2^31)
+            const int box_shift = PAGED ? __ffs(min(a.page_size, kTileKeys)) - 1 : 0, tiles_per_page = PAGED ? max(a.page_size / kTileKeys, 1) : 1;
+            auto first_page = [&](int t) { return tiles_per_page > 1 ? t / tiles_per_page : t << (7 - box_shift); };     // of tile t
+            // asks for the lines of the block table that tiles [t0, t1) of a sequence are looked up in
+            auto fetch_pages = [&](int b, int t0, int t1) {
+                const int last = min(first_page(t1), a.max_pages - 1);
+                for (int i = first_page(t0) + lane * 32; i <= last; i += 32 * 32)
+                    asm volatile("prefetch.global.L1 [%0];" ::"l"(a.block_table + (long long)b * a.max_pages + i));
+            };
+            for (uint32_t seg = 0;; ++seg) {
+                const bool on = cur.valid();
+                const int b = cur.b, g = cur.g, n = cur.t1 - cur.t0, t0 = cur.t0, layer = cur.layer, nt = cur.s.nt, Pb = cur.s.Pb;
+                const long long kv0 = cur.s.kv0;
+                const bool two = TWO && cur.two_rb(P);
+                if (lead) {
+                    ok = mbar_wait_while(ok, &st.bar_segempty[seg % kSegRing], ((seg / kSegRing) & 1) ^ 1);
+                    Segment s;
+                    s.n = on ? n : 0; s.t0 = t0; s.nt = nt; s.Pb = Pb; s.M = cur.s.M; s.rows = cur.s.rows; s.b = b; s.g = g; s.layer = layer;
+                    st.seg[seg % kSegRing] = s;
+                    mbar_arrive(&st.bar_segfull[seg % kSegRing]);
+                }
+                if (!on) break;
+                if (t0 == 0 && n < nt) {                             // necessarily the last segment of this CTA
+                    cu.valid = 1; cu.b = b; cu.g = g; cu.slot = seg == 0 ? 0 : 1; cu.layer = layer; cu.rows = cur.s.rows;
+                    cut_nt = nt; cut_w = cur.s.w; cut_u0 = cur.U;
+                }
+                cur.next(P, pp);
+                if (!PAGED && !lead) continue;
+                // Order: the first K tile(s), Q (behind them, for its slot is free only after the last S of the segment before; the
+                // CTA's first segment finds it free), then V(i), K(i + la), the order in which the MMA warp consumes them.
+                const int la = two ? 1 : 2;
+#pragma unroll 1
+                for (int j = -2 * la; j < 2 * n; ++j) {              // even: V(j / 2), odd: K(j / 2 + la)
+                    const bool is_k = (j & 1) != 0;
+                    const int i = (j >> 1) + (is_k ? la : 0);
+                    if (i >= 0 && i < n) {
+                        const int t = t0 + i;
+                        const bool tree = t == nt - 1, boxes = PAGED && !tree;
+                        // paged cache: one box per page (or per tile when a page holds whole tiles); only pages
+                        // that hold live keys are fetched, what stays stale in the slot is masked / never read.
+                        // The pages are looked up while the slot is not free yet.
+                        int n_ld = 0, per = 0, page_row = 0;
+                        if (boxes) {
+                            per = min(a.page_size, kTileKeys);
+                            n_ld = (min(kTileKeys, Pb - t * kTileKeys) + per - 1) >> box_shift;
+                            if (lane < n_ld) {
+                                const int index = first_page(t) + lane;
+                                int page = __ldg(a.block_table + (long long)b * a.max_pages + index);
+                                if (page < 0 || page >= n_cache_pages) { set_status(P.status, RADAR_ERR_INVALID_ARG); page = 0; }
+                                page_row = page * a.page_size + (tiles_per_page > 1 ? (t - index * tiles_per_page) * kTileKeys : 0);   // (below cache_rows)
+                            }
+                        }
+                        const uint32_t slot = is_k ? k_slot : v_slot;
+                        uint64_t* full = is_k ? &st.bar_kfull[slot] : &st.bar_vfull[slot];
+                        unsigned char* dst = (is_k ? sK : sV) + slot * SM::kTileBytes;
+                        if (lead) ok = mbar_wait_while(ok, is_k ? &st.bar_kempty[slot] : &st.bar_vempty[slot], is_k ? k_par : v_par);
+                        if (PAGED) ok = __shfl_sync(kFull, ok, 0);
+                        if (is_k) { if (++k_slot == RK) { k_slot = 0; k_par ^= 1; } }
+                        else if (++v_slot == RV) { v_slot = 0; v_par ^= 1; }
+                        if (ok && !boxes) {
+                            if (lead) {
+                                const int keys = tree ? kTreeKeys : kTileKeys;
+                                const CUtensorMap* tm = tree ? (is_k ? &tmKt : &tmVt) : (is_k ? &tmKc : &tmVc);
+                                const int row = tree ? b * kMaxNodes : (int)(kv0 + (long long)t * kTileKeys);
+                                mbar_arrive_expect_tx(full, keys * D * 2);
+                                for (int h = 0; h < H; ++h) tma_load_4d(dst + h * (keys * 128), tm, full, h * 64, g, row, layer);
+                            }
+                        } else if (ok) {
+                            if (lead) mbar_arrive_expect_tx(full, n_ld * per * D * 2);
+                            __syncwarp();
+                            if (lane < n_ld)
+                                for (int h = 0; h < H; ++h)
+                                    tma_load_4d(dst + h * (kTileKeys * 128) + lane * per * 128, is_k ? &tmKc : &tmVc, full, h * 64, g, page_row, layer);
+                        }
+                    }
+                    if (j == (seg == 0 ? -2 * la : -1) && lead) {
+                        ok = mbar_wait_while(ok, &st.bar_qempty, (seg & 1) ^ 1);
+                        const int blocks = two ? 2 : 1, node0 = b * kMaxNodes + pp * P.n_blk * P.nodes_per_rb;
+                        if (ok) {
+                            mbar_arrive_expect_tx(&st.bar_qfull, blocks * P.rb_rows * D * 2);   // rows past rb_rows stay stale: never read back
+                            for (int q = 0; q < blocks; ++q)
+                                for (int h = 0; h < H; ++h)
+                                    tma_load_4d(sQ + q * SM::kQBlock + h * (128 * 128), &tmQ, &st.bar_qfull, h * 64, g * G, node0 + q * P.nodes_per_rb, layer);
+                        }
+                        // ... so the next segment's Q waits for it in L2
+                        if (cur.valid()) {
+                            const int next0 = cur.b * kMaxNodes + pp * P.n_blk * P.nodes_per_rb;
+                            for (int q = 0; q < (TWO && cur.two_rb(P) ? 2 : 1); ++q)
+                                for (int h = 0; h < H; ++h) tma_prefetch_4d(&tmQ, h * 64, cur.g * G, next0 + q * P.nodes_per_rb, cur.layer);
+                        }
+                    }
+                    if (PAGED && j == 0 && cur.valid()) fetch_pages(cur.b, cur.t0, cur.t1);
+                }
+            }
+            __syncwarp();
+            if (cu.valid) {
+                const long long u1 = cut_u0 + (long long)cut_nt * cut_w + P.unit_cost;
+                cu.n_pieces = 0;
+#pragma unroll 1
+                for (int k = 0; k < kMaxPerClass / 32; ++k) {
+                    const int c = ci + k * 32 + lane;
+                    const long long lo = tot_all * c / P.ncc, hi = tot_all * (c + 1) / P.ncc;
+                    const bool piece = c < P.ncc && lo < u1;
+                    const bool live = piece && tiles_before(hi, cut_u0, cut_nt, cut_w, P.unit_cost) > tiles_before(lo, cut_u0, cut_nt, cut_w, P.unit_cost);
+                    const uint32_t pieces = __ballot_sync(kFull, piece), bits = __ballot_sync(kFull, live);
+                    cu.n_pieces += __popc(pieces);
+                    if (lane == 0) P.cut[blockIdx.x].live[k] = bits;
+                    if (pieces != 0xffffffffu) break;
+                }
+            }
+            if (lane == 0) {
+                CutUnit* out = P.cut + blockIdx.x;
+                out->valid = cu.valid; out->b = cu.b; out->g = cu.g; out->layer = cu.layer;
+                out->slot = cu.slot; out->rows = cu.rows; out->n_pieces = cu.n_pieces;
+            }
+            __syncwarp();
+        } else if (warp == kMmaWarp) {
+            // =================================== MMA issuer ===================================
+            // The warp runs converged: every lane waits on the barriers and executes the same straight-line issue
+            // sequences with warp-uniform descriptor words, and the elected lane issues the instructions and the
+            // commits (predicated, no branch around them).  Whatever this warp executes between two MMAs costs
+            // tensor-pipe time, so no control flow depends on a wait's outcome: after a wait that ran out the
+            // predicate is off and the loops run dry.
+            constexpr uint32_t idesc_s128 = idesc_bf16_f32(128, kTileKeys, false, false);
+            constexpr uint32_t idesc_s64 = idesc_bf16_f32(128, kTreeKeys, false, false);
+            constexpr uint32_t idesc_pv = idesc_bf16_f32(128, D, false, true);
+            // high word of every shared-memory descriptor (stride between 8-row groups 1024 B, version, swizzle)
+            constexpr uint32_t kDescHi = (1024u >> 4) | (1u << 14) | (2u << 29);
+            const uint32_t q_lo = ((smem_u32(sQ) & 0x3ffff) >> 4) | (1u << 16);
+            const uint32_t k_lo = ((smem_u32(sK) & 0x3ffff) >> 4) | (1u << 16);
+            const uint32_t v_lo = (smem_u32(sV) & 0x3ffff) >> 4;
+            const uint32_t elected = elect_one();
+            uint32_t k_next = 0, k_par = 0, v_next = 0, v_par = 0;   // ring slot to take next and its phase parity
+            uint32_t p_par[2] = {0, 0};              // phase parity of the next P tile per group
+            // The segment's shape comes from memory; passing it through a broadcast from lane 0 tells the
+            // compiler that it is the same in every lane, so that the loops below and the descriptor arithmetic in
+            // them stay on the uniform datapath (this warp's own instruction stream is what bounds the issue rate).
+            auto uni = [](int v) { return __shfl_sync(kFull, v, 0); };
+            Segment s;
+            for (uint32_t seg = 0; take_segment(seg, s); ++seg) {
+                const int seg_t0 = uni(s.t0), n = uni(s.n), M = uni(s.M), Pb = uni(s.Pb), last = uni(s.nt) - 1;
+                const bool two = TWO && uni(s.rows) > P.rb_rows;
+                ok = mbar_wait_while(ok, &st.bar_qfull, seg & 1);
+                uint32_t k_slot = 0, v_slot = 0;      // ring slots of the K and V tiles in use
+                bool acc[2] = {false, false};         // accumulator holds a product of this segment
+                auto take_v = [&]() {
+                    v_slot = v_next;
+                    ok = mbar_wait_while(ok, &st.bar_vfull[v_slot], v_par);
+                    if (++v_next == RV) { v_next = 0; v_par ^= 1; }
+                };
+                auto take_k = [&]() {
+                    k_slot = k_next;
+                    ok = mbar_wait_while(ok, &st.bar_kfull[k_slot], k_par);
+                    if (++k_next == RK) { k_next = 0; k_par ^= 1; }
+                };
+                // the accumulator's first product of the segment: the epilogue of the previous one has read it
+                auto take_o = [&](const int q) {
+                    if (!acc[q]) ok = mbar_wait_while(ok, &st.bar_ofree[q], (seg & 1) ^ 1);
+                };
+
+                // ---- O[q] (+)= P[q] V for tile i (q is a literal at every call site) ----
+                auto pv = [&](const int q, const int i, const bool fresh_v, const bool release_v) {
+                    const bool tree = seg_t0 + i == last;
+                    const int nk = tree ? kTreeKeys : kTileKeys;
+                    const int valid = tree ? M : min(kTileKeys, Pb - (seg_t0 + i) * kTileKeys);
+                    const int ksteps = (valid + 15) >> 4;
+                    if (fresh_v) {
+                        take_v();
+                        if (valid < ksteps * 16) {
+                            // rows past the last live key meet P = 0; they must not hold NaN/Inf bit patterns
+                            unsigned char* vtile = sV + v_slot * SM::kTileBytes;
+                            const int nrows = ksteps * 16 - valid;
+#pragma unroll 1
+                            for (int e = lane; e < nrows * 8 * H; e += 32) {
+                                const int h = e / (nrows * 8), rem = e % (nrows * 8);
+                                const int r = valid + rem / 8, c = rem % 8;
+                                *reinterpret_cast<uint4*>(vtile + h * (nk * 128) + r * 128 + c * 16) = make_uint4(0, 0, 0, 0);
+                            }
+                            fence_proxy_async_smem();
+                            __syncwarp();
+                        }
+                    }
+                    take_o(q);
+                    ok = mbar_wait_while(ok, &st.bar_pready[q], p_par[q]);
+                    p_par[q] ^= 1;
+                    tc_fence_after_sync();
+                    const uint32_t go = ok ? elected : 0u;
+                    // V is consumed N-major: 16 keys are 2048 B; 64-column blocks are nk * 128 B apart
+                    const uint32_t b_lo = (v_lo + v_slot * (SM::kTileBytes >> 4)) | ((uint32_t)(nk * 128 >> 4) << 16);
+                    mma_ts_x4(go, ksteps, tmem + 256 + q * 128, tmem + q * 128, b_lo, kDescHi, idesc_pv, acc[q]);
+                    mma_ts_x4(go, ksteps - 4, tmem + 256 + q * 128, tmem + q * 128 + 32, b_lo + 4 * 128, kDescHi, idesc_pv, true);
+                    acc[q] = true;
+                    if (release_v) mma_commit_if(go, &st.bar_vempty[v_slot]);
+                    if (two ? i == n - 1 : i + 2 >= n) mma_commit_if(go, &st.bar_odone[q]);
+                };
+                // ---- S[q] = Q K^T for tile si.  Nothing in tensor memory changes hands here: K arrives through the
+                // async proxy, and the buffer was last read by this thread's own P V, which runs first. ----
+                auto qk = [&](const int q, const int si, const bool fresh_k, const bool release_k) {
+                    if (fresh_k) take_k();
+                    const uint32_t go = ok ? elected : 0u;
+                    const bool tree = seg_t0 + si == last;
+                    const uint32_t a0 = q_lo + (two ? q : 0) * (SM::kQBlock >> 4);
+                    const uint32_t b0 = k_lo + k_slot * (SM::kTileBytes >> 4);
+                    const uint32_t idesc = tree ? idesc_s64 : idesc_s128;
+                    mma_ss_x4(go, tmem + q * 128, a0, b0, kDescHi, idesc, false);
+                    if (D == 128)                     // second 64-column block of Q and K
+                        mma_ss_x4(go, tmem + q * 128, a0 + (128 * 128 >> 4), b0 + ((uint32_t)((tree ? kTreeKeys : kTileKeys) * 128) >> 4),
+                                  kDescHi, idesc, true);
+                    if (release_k) mma_commit_if(go, &st.bar_kempty[k_slot]);
+                    mma_commit_if(go, &st.bar_sfull[q]);
+                    // the last S of the segment: Q may be overwritten once it has run
+                    if (si == n - 1 && release_k) mma_commit_if(go, &st.bar_qempty);
+                };
+                // Schedule.  Two live row blocks: group s owns row block s; per tile PV0(i) S0(i+1) PV1(i) S1(i+1),
+                // both groups sharing K(i+1) and V(i).  One live row block: the groups take alternate tiles,
+                // PV(i) S(i+2) for group i & 1.  S of the first tile(s) comes from the iterations with i < 0.
+                // Steady state (all tiles involved are full prefix tiles): the same steps with nothing to decide,
+                // so that the issuing warp executes as few instructions per MMA as possible.  The waits for K and V, which are
+                // there most of the time, stand where the warp would wait for P.
+                auto full = [&](const int q, const uint32_t a0, const bool fresh, const bool release) {
+                    static_assert(kFirstKeys == 64 && kTileKeys == 128, "four steps before and behind the second wait");
+                    const uint32_t o_col = tmem + 256 + q * 128, p_col = tmem + q * 128;
+                    if (fresh) take_v();
+                    take_o(q);
+                    const uint32_t b_lo = (v_lo + v_slot * (SM::kTileBytes >> 4)) | ((uint32_t)(kTileKeys * 128 >> 4) << 16);
+                    ok = mbar_wait_while(ok, &st.bar_pfirst[q], p_par[q]);
+                    tc_fence_after_sync();
+                    mma_ts_x4(ok ? elected : 0u, o_col, p_col, b_lo, kDescHi, idesc_pv, acc[q]);
+                    if (fresh) take_k();
+                    const uint32_t b0 = k_lo + k_slot * (SM::kTileBytes >> 4);
+                    ok = mbar_wait_while(ok, &st.bar_pready[q], p_par[q]);
+                    p_par[q] ^= 1;
+                    acc[q] = true;
+                    tc_fence_after_sync();
+                    const uint32_t go = ok ? elected : 0u;
+                    mma_ts_x4(go, o_col, p_col + 32, b_lo + 4 * 128, kDescHi, idesc_pv, true);
+                    if (release) mma_commit_if(go, &st.bar_vempty[v_slot]);
+                    mma_ss_x4(go, p_col, a0, b0, kDescHi, idesc_s128, false);
+                    if (D == 128) mma_ss_x4(go, p_col, a0 + (128 * 128 >> 4), b0 + (kTileKeys * 128 >> 4), kDescHi, idesc_s128, true);
+                    mma_commit_if(go, &st.bar_sfull[q]);
+                    if (release) mma_commit_if(go, &st.bar_kempty[k_slot]);
+                };
+                const uint32_t a_q0 = q_lo, a_q1 = q_lo + (SM::kQBlock >> 4);
+                const int n_full = min(n, Pb / kTileKeys - seg_t0);   // tiles [0, n_full) of the segment are full prefix tiles
+                if (two) {
+#pragma unroll 1
+                    for (int i = -1; i < n; ++i) {
+                        if (i >= 0 && i + 2 < n_full) {           // tiles i and i+1 full, and S(i+1) is not the segment's last
+                            full(0, a_q0, true, false);
+                            full(1, a_q1, false, true);
+                        } else {
+                            if (i >= 0) pv(0, i, true, false);
+                            if (i + 1 < n) qk(0, i + 1, true, false);
+                            if (i >= 0) pv(1, i, false, true);
+                            if (i + 1 < n) qk(1, i + 1, false, true);
+                        }
+                    }
+                } else {
+#pragma unroll 1
+                    for (int i = -2; i < n; i += 2) {
+                        if (i >= 0 && i + 4 < n_full) {           // tiles i to i+3 full, S(i+3) not the last
+                            full(0, a_q0, true, true);
+                            full(1, a_q0, true, true);
+                        } else {
+                            if (i >= 0) pv(0, i, true, true);
+                            if (i + 2 < n) qk(0, i + 2, true, true);
+                            if (i >= 0 && i + 1 < n) pv(1, i + 1, true, true);
+                            if (i + 3 < n) qk(1, i + 3, true, true);
+                        }
+                    }
+                }
+            }
+            __syncwarp();
+        }
+    }
+
+    // ---- teardown ----
+    if (!ok) st.abort = 1;
+    tc_fence_before_sync();
+    __syncthreads();
+    if (warp == kMmaWarp) {
+        if (st.abort) {
+            // let loads that are still in flight land before the CTA's shared memory is released
+            if (lane == 0) {
+                for (int i = 0; i < 3; ++i) {
+                    mbar_wait_while(true, &st.bar_kfull[i], 0, 64);
+                    mbar_wait_while(true, &st.bar_vfull[i], 0, 64);
+                }
+                set_status(P.status, RADAR_ERR_TIMEOUT);
+            }
+            __syncwarp();
+        }
+        tmem_dealloc(st.tmem_base, 512);
+    }
+}
+
+// The form for head ratios that do not divide 128, which came from the FMA kernel, whose probabilities are fp32, and keep its
+// precision: P goes to the tensor cores as the sum of two bf16 numbers (its value to 2^-18) in place of one (2^-9), and the
+// scores' scale is applied in two parts (error against fp64, 2-norm, of 24 / 8 heads, 2048 tokens: FMA 1.6545e-3, one bf16
+// 2.1607e-3, two 1.6545e-3, all of it the rounding of O to bf16).  That doubles the instructions between two exponentials,
+// which one thread a row issues one after the other and two a row side by side: 16 softmax warps here, which also do the
+// epilogue, TMA producer and MMA issuer (this form / the one above with two parts: 24 / 8 heads, B = 6, 300 to 4500 tokens
+// 33.8 / 37.3 us, paged 39.1 / 43.6; 16 layers, B = 2, 1000 to 2000 tokens 105 / 131).
+constexpr int kFineThreads = 576;
+constexpr int kFineProducerWarp = 16, kFineMmaWarp = 17;
+template <int D, bool TWO, bool PAGED>
+__global__ void __launch_bounds__(kFineThreads, 1)      // 18 warps are allocated as 20: 96 registers per thread
+tree_attn_tc_fine_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmKc,
                     const __grid_constant__ CUtensorMap tmVc, const __grid_constant__ CUtensorMap tmKt,
                     const __grid_constant__ CUtensorMap tmVt, const TcParams P) {
     chain_trigger();                     // warp 0 waits for the predecessor below; the barrier, tensor-memory and
@@ -324,7 +1085,7 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
             }
             fence_barrier_init();
         }
-    } else if (warp == kProducerWarp) {
+    } else if (warp == kFineProducerWarp) {
         tmem_alloc(&s_tmem_base, 512);
         tmem_relinquish();
         if (lane == 0) {
@@ -358,11 +1119,11 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
         }
         tc_fence_before_sync();
         __syncthreads();
-        if (warp == kProducerWarp) tmem_dealloc(tmem, 512);
+        if (warp == kFineProducerWarp) tmem_dealloc(tmem, 512);
         return;
     }
 
-    if (warp == kProducerWarp) {
+    if (warp == kFineProducerWarp) {
         // =================================== TMA producer ===================================
         // One lane does everything for the contiguous cache.  With a paged cache the whole warp walks the same
         // loop and lane p looks up and fetches page p of a tile (up to eight boxes per tile), the leading lane
@@ -464,7 +1225,7 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
             out->slot = cu.slot; out->rows = cu.rows; out->n_pieces = cu.n_pieces;
         }
         __syncwarp();
-    } else if (warp == kMmaWarp) {
+    } else if (warp == kFineMmaWarp) {
         // =================================== MMA issuer ===================================
         // The warp runs converged: every lane waits on the barriers and executes the same straight-line issue
         // sequences with warp-uniform descriptor words, and the elected lane issues the instructions and the
@@ -534,13 +1295,8 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
                 // at column 64 (each softmax thread writes inside its own column range)
                 const int hs = tree ? 2 : 4;
                 const uint32_t n1 = (uint32_t)min(ksteps, hs), n2 = (uint32_t)ksteps - n1;
-                if (FINE) {
-                    mma_ts_two_x4(go, n1, tmem + 256 + q * 128, tmem + q * 128, b_lo, kDescHi, idesc_pv, acc[q]);
-                    mma_ts_two_x4(go, n2, tmem + 256 + q * 128, tmem + q * 128 + 64, b_lo + hs * 128, kDescHi, idesc_pv, true);
-                } else {
-                    mma_ts_x4(go, n1, tmem + 256 + q * 128, tmem + q * 128, b_lo, kDescHi, idesc_pv, acc[q]);
-                    mma_ts_x4(go, n2, tmem + 256 + q * 128, tmem + q * 128 + 64, b_lo + hs * 128, kDescHi, idesc_pv, true);
-                }
+                mma_ts_two_x4(go, n1, tmem + 256 + q * 128, tmem + q * 128, b_lo, kDescHi, idesc_pv, acc[q]);
+                mma_ts_two_x4(go, n2, tmem + 256 + q * 128, tmem + q * 128 + 64, b_lo + hs * 128, kDescHi, idesc_pv, true);
                 acc[q] = true;
                 if (release_v) mma_commit_if(go, &bar_vempty[v_slot]);
                 if (two ? i == n - 1 : i + 2 >= n) mma_commit_if(go, &bar_odone[q]);
@@ -583,14 +1339,12 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
                 }
                 tc_fence_after_sync();
                 const uint32_t b_lo = (v_lo + v_slot * (SM::kTileBytes >> 4)) | ((uint32_t)(kTileKeys * 128 >> 4) << 16);
-                if (FINE) mma_ts_two_x2x2_full(ok ? elected : 0u, tmem + 256 + q * 128, tmem + q * 128, b_lo, kDescHi, idesc_pv, acc[q]);
-                else mma_ts_x2x2_full(ok ? elected : 0u, tmem + 256 + q * 128, tmem + q * 128, b_lo, kDescHi, idesc_pv, acc[q]);
+                mma_ts_two_x2x2_full(ok ? elected : 0u, tmem + 256 + q * 128, tmem + q * 128, b_lo, kDescHi, idesc_pv, acc[q]);
                 wait_all(&bar_pready[q], p_par[q]);
                 p_par[q] ^= 1;
                 tc_fence_after_sync();
                 const uint32_t go = ok ? elected : 0u;
-                if (FINE) mma_ts_two_x2x2_full(go, tmem + 256 + q * 128, tmem + q * 128 + 32, b_lo + 2 * 128, kDescHi, idesc_pv, true);
-                else mma_ts_x2x2_full(go, tmem + 256 + q * 128, tmem + q * 128 + 16, b_lo + 2 * 128, kDescHi, idesc_pv, true);
+                mma_ts_two_x2x2_full(go, tmem + 256 + q * 128, tmem + q * 128 + 32, b_lo + 2 * 128, kDescHi, idesc_pv, true);
                 acc[q] = true;
                 if (release_v) mma_commit_if(go, &bar_vempty[v_slot]);
             };
@@ -647,10 +1401,8 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
         // Two threads per query row: warp w of a group's eight serves tensor-memory lanes 32 (w & 3) .. + 31
         // and the column half (w >> 2) & 1, so a row's 128 scores are exponentiated by two threads at once
         // and the chain S -> softmax -> P V of a group is about half as long.
-        // That chain is what a tile costs (about 4000 cycles, of which the tensor pipe works 2048).  So the products of a
-        // thread's first 32 columns start while the second 32 are exponentiated, and only the two warps that share
-        // rows wait for each other's maxima: 32 layers, 8 sequences of 6000 to 8192 tokens, 64 / 8 heads 4457 -> 4347 us
-        // (the early products alone 4369); launches bound by memory are unchanged.
+        // That chain is what a tile costs, so the products of a thread's first 32 columns start while the second 32 are
+        // exponentiated, and only the two warps that share rows wait for each other's maxima.
         const int grp = warp >> 3;
         const int half = (warp >> 2) & 1;
         const int pair_bar = 1 + grp * 4 + (warp & 3);          // barriers 1 .. 8: the two warps that share 32 rows
@@ -690,7 +1442,7 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
                 // This thread's chunks of 32 score columns: a prefix tile has four (two per thread), the tree tile
                 // two (one per thread).  Half h of a row works in columns 64 h .. 64 h + 63 of the buffer only: its
                 // scores sit there (the tree tile's second chunk is read from columns 32 .. 63 but belongs to
-                // half 1 alone) and its P goes to columns 64 h + 16 cc (FINE: 64 h + 32 cc, 16 of each part), so the halves
+                // half 1 alone) and its P goes to columns 64 h + 32 cc, 16 of each part, so the halves
                 // never touch each other's columns and a thread overwrites only scores it has already taken into registers.
                 const bool tree = t == nt_unit - 1;
                 const int nch = tree ? 1 : 2;
@@ -765,23 +1517,21 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
                             for (int e = 0; e < 32; ++e)
                                 if (!((al >> e) & 1u)) sv[e] = 0xff800000u;
                         }
-                        uint32_t pk[16], pl[FINE ? 16 : 1];
+                        uint32_t pk[16], pl[16];
 #pragma unroll
                         for (int e = 0; e < 16; ++e) {
                             const float2 s2 = make_float2(__uint_as_float(sv[2 * e]), __uint_as_float(sv[2 * e + 1]));
                             float2 t = __ffma2_rn(s2, sc2, nm2);
-                            if (FINE) t = __ffma2_rn(s2, make_float2(P.scale_log2_lo, P.scale_log2_lo), t);
+                            t = __ffma2_rn(s2, make_float2(P.scale_log2_lo, P.scale_log2_lo), t);
                             const float p0 = ex2(t.x), p1 = ex2(t.y);
                             ls[e & 1] = __fadd2_rn(ls[e & 1], make_float2(p0, p1));
                             const __nv_bfloat162 v = __floats2bfloat162_rn(p0, p1);
                             pk[e] = *reinterpret_cast<const uint32_t*>(&v);
-                            if (FINE) {
-                                const __nv_bfloat162 r = __floats2bfloat162_rn(p0 - __uint_as_float(pk[e] << 16), p1 - __uint_as_float(pk[e] & 0xffff0000u));
-                                pl[FINE ? e : 0] = *reinterpret_cast<const uint32_t*>(&r);
-                            }
+                            const __nv_bfloat162 r = __floats2bfloat162_rn(p0 - __uint_as_float(pk[e] << 16), p1 - __uint_as_float(pk[e] & 0xffff0000u));
+                            pl[e] = *reinterpret_cast<const uint32_t*>(&r);
                         }
-                        tmem_st16(tS + half * 64 + cc * (FINE ? 32 : 16), pk);
-                        if constexpr (FINE) tmem_st16(tS + half * 64 + cc * 32 + 16, pl);
+                        tmem_st16(tS + half * 64 + cc * 32, pk);
+                        tmem_st16(tS + half * 64 + cc * 32 + 16, pl);
                         if (cc == 0) {
                             tmem_wait_st();
                             tc_fence_before_sync();
@@ -882,11 +1632,10 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
                     }
                 }
                 if (row_live && half == 0) {
-                    const float m_nat = m_safe * 0.6931471805599453f;
                     if (final_rows) {
-                        if (a.lse != nullptr) a.lse[cur.layer * P.lse_ls + ((int64_t)b * a.Hq + hq) * kMaxNodes + node] = FINE ? lse_of(m_safe, l_out) : m_nat + logf(l_out);
+                        if (a.lse != nullptr) a.lse[cur.layer * P.lse_ls + ((int64_t)b * a.Hq + hq) * kMaxNodes + node] = lse_of(m_safe, l_out);
                     } else {
-                        P.part_ml[rec] = make_float2(FINE || m_out == -CUDART_INF_F ? m_out : m_nat, l_out);
+                        P.part_ml[rec] = make_float2(m_out, l_out);
                     }
                 }
             }
@@ -900,7 +1649,7 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
     // ---- teardown ----
     tc_fence_before_sync();
     __syncthreads();
-    if (warp == kProducerWarp) {
+    if (warp == kFineProducerWarp) {
         if (s_abort) {
             // let loads that are still in flight land before the CTA's shared memory is released
             if (lane == 0) {
@@ -1149,11 +1898,11 @@ static int launch_tc(radar_ctx* ctx, TcParams& P, cudaStream_t stream) {
         !make_map(&tmVc, have_prefix ? a.Vc : a.Vt, D, a.Hkv, have_prefix ? a.cache_rows : tree_rows, 1, cache_box, L,
                   have_prefix ? a.cache_layer_stride : a.tree_kv_layer_stride))
         return RADAR_ERR_CUDA;
-    RADAR_CUDA_CHECK(radar_opt_in_smem(ctx, RADAR_SMEM_ATTN_TC + 8 * FINE + 4 * (D == 128) + 2 * TWO + PAGED, tree_attn_tc_kernel<D, TWO, PAGED, FINE>,
-                                       (size_t)Smem<D, TWO>::kDynamic));
+    auto* const kernel = FINE ? tree_attn_tc_fine_kernel<D, TWO, PAGED> : tree_attn_tc_kernel<D, TWO, PAGED>;
+    RADAR_CUDA_CHECK(radar_opt_in_smem(ctx, RADAR_SMEM_ATTN_TC + 8 * FINE + 4 * (D == 128) + 2 * TWO + PAGED, kernel, (size_t)Smem<D, TWO>::kDynamic));
     {
         radar_launch_scope scope(ctx, RADAR_K_ATTN, stream);
-        RADAR_CUDA_CHECK(launch_chained(tree_attn_tc_kernel<D, TWO, PAGED, FINE>, dim3((unsigned)(P.n_cls * P.ncc)), dim3(kTcThreads),
+        RADAR_CUDA_CHECK(launch_chained(kernel, dim3((unsigned)(P.n_cls * P.ncc)), dim3(FINE ? kFineThreads : kTcThreads),
                                         (size_t)Smem<D, TWO>::kDynamic, stream, tmQ, tmKc, tmVc, tmKt, tmVt, P));
     }
     RADAR_CUDA_CHECK(cudaGetLastError());
