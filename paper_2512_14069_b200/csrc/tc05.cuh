@@ -34,11 +34,12 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
         : "memory");
     return ok != 0;
 }
-// Bounded wait: false once `limit` polls (each sleeps for up to a millisecond; polling warps take issue
-// slots from the others) have not seen the phase.  After a wait
-// that ran out (`ok` false) one poll is all that is spent, so that loops over waits run dry.  In one block of instructions: a
-// loop in C++ is unrolled at every one of its many sites, and a kernel's size is instruction-cache misses.
-__device__ __forceinline__ bool mbar_wait_while(bool ok, uint64_t* bar, uint32_t parity, uint32_t limit = 1u << 12) {
+// Bounded wait: false once `limit` polls have not seen the phase.  A poll gives up after 4.0 us on this part, whatever its
+// suspend-time hint says (none, 0, 20 us and 1 ms measured), so the limit stands for about 4 s.  (Without a hint the waits are
+// as long and launches up to 4 % slower: 16 / 1 heads, B = 8, 8192 tokens 54.4 against 56.8 us.)  After a wait that ran out
+// (`ok` false) one poll is all that is spent, so that loops over waits run dry.  In one block of instructions: a loop in C++
+// is unrolled at every one of its many sites, and a kernel's size is instruction-cache misses.
+__device__ __forceinline__ bool mbar_wait_while(bool ok, uint64_t* bar, uint32_t parity, uint32_t limit = 1u << 20) {
     uint32_t r;
     asm volatile(
         "{\n\t.reg .pred p, q;\n\t.reg .u32 n;\n\t"
@@ -56,8 +57,8 @@ __device__ __forceinline__ bool mbar_wait_while(bool ok, uint64_t* bar, uint32_t
         : "memory");
     return ok && r != 0;
 }
-// For a wait that is long and whose end nothing hurries after: naps between the polls.
-__device__ __forceinline__ bool mbar_wait_lazy(bool ok, uint64_t* bar, uint32_t parity, uint32_t limit = 1u << 22) {
+// For a wait that is long and whose end nothing hurries after: naps between the polls (limit: about 4.5 s).
+__device__ __forceinline__ bool mbar_wait_lazy(bool ok, uint64_t* bar, uint32_t parity, uint32_t limit = 1u << 20) {
 #pragma unroll 1
     for (uint32_t it = ok ? limit : 1u; it > 0; --it) {
         if (mbar_try_wait(bar, parity)) return ok;
