@@ -308,8 +308,8 @@ __global__ void __launch_bounds__(kTcThreads, 1)
 tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmKc,
                     const __grid_constant__ CUtensorMap tmVc, const __grid_constant__ CUtensorMap tmKt,
                     const __grid_constant__ CUtensorMap tmVt, const TcParams P) {
-    chain_trigger();                     // the producer waits for the predecessor below; the barrier, tensor-memory and
-                                         // descriptor set-up of the other warps needs nothing from global memory
+    chain_trigger();                     // every warp waits for the predecessor where its role begins; the barrier,
+                                         // tensor-memory and descriptor set-up needs nothing from global memory
     using SM = Smem<D, TWO>;
     constexpr int H = SM::kHalves;
     constexpr int RK = SM::kRingK, RV = SM::kRingV;
@@ -375,6 +375,8 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
     // issuing warp a handful of instructions for every product.
     constexpr uint32_t tmem = 0;
     bool ok = true;                         // no wait of this thread has run out
+    // Each role starts with chain_sync(): the bounds of the waits behind it are for this kernel's own work.  (A warp that went
+    // straight to its first wait would spend them on whatever is left of the predecessor.)
     // the producer's next segment; false behind the last one
     auto take_segment = [&](uint32_t seg, Segment& s) {
         ok = mbar_wait_while(ok, &st.bar_segfull[seg % kSegRing], (seg / kSegRing) & 1);
@@ -387,6 +389,7 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
 
     if (warp < kEpilogueWarp) {
         regs_inc<kSoftmaxRegs>();
+        chain_sync();
         // =================================== softmax groups ===================================
         // One thread per query row, which holds the tile's 128 scores in registers: tensor memory is read once and no two
         // threads have to agree on a maximum.  (Two threads a row, 64 scores each read twice for want of registers, was the
@@ -538,6 +541,7 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
         }
     } else if (warp < kProducerWarp) {
         regs_dec<kEpilogueRegs>();
+        chain_sync();
         // =================================== epilogue ===================================
         // One thread per tensor-memory lane takes the finished accumulators to O (or to the partials) while the softmax
         // groups and the tensor cores are already in the next segment; each accumulator is handed back as soon as it is read.
@@ -643,12 +647,12 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
         }
     } else {
         regs_dec<kIssueRegs>();
+        chain_sync();                            // every global access of the CTA comes behind one
         if (warp == kProducerWarp) {
             // =================================== TMA producer ===================================
             // One lane does everything for the contiguous cache.  With a paged cache the whole warp walks the same
             // loop and lane p looks up and fetches page p of a tile (up to eight boxes per tile), the leading lane
             // still doing the waits, the byte counts, Q and the tree tile.
-            chain_sync();                        // every global access of the CTA comes after the first segment is there
             const bool lead = lane == 0;
             const bool usable = (smem_u32(smem_raw) & 1023u) == 0 && st.tmem_base == 0;     // (else the tiles would not sit on their swizzle boundary)
             if (!usable && lead) set_status(P.status, RADAR_ERR_CUDA);

@@ -38,3 +38,14 @@ extern "C" int waits_that_run_out(unsigned long long* ns, int* seen) {
     waits_that_run_out_kernel<<<1, 64>>>(ns, seen);
     return (int)cudaDeviceSynchronize();
 }
+
+// A predecessor that lets its dependents start at once and then takes `ns` nanoseconds (bounded by its naps as well).
+__global__ void slow_predecessor_kernel(unsigned long long ns, int naps) {
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    const unsigned long long end = now_ns() + ns;
+    for (int i = 0; i < naps && now_ns() < end; ++i) __nanosleep(500000);
+}
+extern "C" int launch_slow_predecessor(void* stream, unsigned long long ns) {
+    slow_predecessor_kernel<<<1, 1, 0, reinterpret_cast<cudaStream_t>(stream)>>>(ns, (int)(ns / 100000));
+    return (int)cudaGetLastError();
+}

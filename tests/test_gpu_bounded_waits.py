@@ -1,4 +1,5 @@
-"""The bounded waits of the tensor-core attention: long enough for any healthy kernel, and bounded."""
+"""The bounded waits of the tensor-core attention: long enough for any healthy kernel, bounded, and for the kernel's own work
+only, whatever its predecessor takes."""
 import ctypes
 import os
 import subprocess
@@ -30,3 +31,40 @@ def test_a_wait_gives_up_after_seconds(waits):
     took = ns.tolist()
     assert all(1e9 < t < 6e10 for t in took[:2]), took
     assert took[2] < 1e8, took
+
+
+@pytest.mark.parametrize("Hq,page", [(16, 0), (32, 16), (12, 0)])
+def test_a_slow_predecessor_is_not_a_timeout(waits, Hq, page):
+    """The launch begins while its predecessor, which lets it, still runs for longer than the waits of the kernel are bounded by
+    (4 s); results are those of a launch with nothing in front, bit for bit.  A ratio of 3 runs the kernel's other form."""
+    import torch
+    from paper_2512_14069_b200 import binding as rb
+    ctx = rb.Context(0)
+    B, M, Hkv, d, P = 2, 64, 4, 128, 700
+    g = torch.Generator(device="cuda").manual_seed(Hq)
+    randn = lambda *s: torch.randn(*s, device="cuda", generator=g).bfloat16()
+    rows = B * (-(-P // 16) * 16)
+    Kc, Vc, Q, Kt, Vt = randn(rows, Hkv, d), randn(rows, Hkv, d), randn(B, M, Hq, d), randn(B, M, Hkv, d), randn(B, M, Hkv, d)
+    ints = lambda v: torch.tensor(v, dtype=torch.int32, device="cuda")
+    where = dict(kv_start=None, block_table=ints(list(range(rows // 16))).view(B, -1), page_size=page) if page else \
+        dict(kv_start=torch.tensor([0, P], device="cuda"))
+    mask = torch.full((B, M), -1, dtype=torch.int64, device="cuda")
+    ws = torch.zeros(rb.radar_attn_workspace_bytes(ctx, B, Hq, Hkv, d, rb.RADAR_BF16, P), dtype=torch.uint8, device="cuda")
+    plen, nodes = ints([P, P - 100]), ints([M, 40])
+
+    def attend():
+        O, lse = torch.zeros_like(Q), torch.zeros(B, Hq, M, device="cuda")
+        torch.cuda.synchronize()
+        return (O, lse), lambda: rb.radar_tree_attention(
+            ctx, B=B, Hq=Hq, Hkv=Hkv, d=d, Q=Q, Kc=Kc, Vc=Vc, prefix_len=plen, max_prefix_len=P, Kt=Kt, Vt=Vt, mask=mask, n_nodes=nodes,
+            O=O, lse=lse, workspace=ws, **where)
+
+    plain, run = attend()
+    run()
+    ctx.check_device_status()
+    behind, run = attend()
+    assert waits.launch_slow_predecessor(ctypes.c_void_p(torch.cuda.current_stream().cuda_stream), ctypes.c_ulonglong(6_000_000_000)) == 0
+    run()
+    ctx.check_device_status()
+    assert plain[0].any() and all(torch.equal(a, b) for a, b in zip(plain, behind))
+    ctx.close()
