@@ -67,6 +67,17 @@ __device__ __forceinline__ bool mbar_wait_lazy(bool ok, uint64_t* bar, uint32_t 
     return false;
 }
 
+// Before a block leaves: waits, up to `limit` polls (0.25 s), for what it has in flight itself.
+__device__ __forceinline__ bool mbar_drain(uint64_t* bar, uint32_t parity, uint32_t limit = 1u << 16) {
+#pragma unroll 1
+    for (; limit > 0; --limit)
+        if (mbar_try_wait(bar, parity)) return true;
+    return false;
+}
+// The phase that slot `i` of a ring of loads was last armed for, as the parity to wait with, where the next load would go to
+// slot `next` once phase parity `par` has freed it (1 in the first round).  A slot never armed gives 1, which a new barrier passes.
+__host__ __device__ constexpr uint32_t last_armed_parity(uint32_t i, uint32_t next, uint32_t par) { return i < next ? par ^ 1u : par; }
+
 // Bounded wait: gives up after `limit` polls (each poll itself blocks for a hardware-defined short
 // time) or once *abort_flag has been set by another thread.  Returns false on give-up and sets the
 // flag.  A wait that is satisfied at once costs one try_wait and nothing else: the flag is looked at

@@ -324,6 +324,8 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
     struct __align__(1024) Static {
         uint64_t bar_qfull, bar_qempty, bar_kfull[3], bar_kempty[3], bar_vfull[3], bar_vempty[3];
         uint64_t bar_sfull[2], bar_odone[2], bar_ofree[2], bar_mlfull, bar_mlempty;
+        uint64_t bar_idle;               // every product issued has run
+        uint32_t q_last, spare;          // phase parity of the last Q; the ring below starts on 16 bytes
         uint64_t bar_pfirst[2];          // the probabilities of the tile's first kFirstKeys keys are there
         uint64_t bar_pready[2];          // ... all of them
         uint64_t bar_segfull[kSegRing], bar_segempty[kSegRing];
@@ -331,7 +333,7 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
         float2 ml[2][128];               // per group: (m in log2 units, l) of the rows at the end of a segment
         uint32_t tmem_base;
         int abort;
-        unsigned char pad[kStaticSmem - ((26 + 2 * kSegRing) * 8 + kSegRing * (int)sizeof(Segment) + 2 * 128 * 8 + 8)];
+        unsigned char pad[kStaticSmem - ((28 + 2 * kSegRing) * 8 + kSegRing * (int)sizeof(Segment) + 2 * 128 * 8 + 8)];
     };
     static_assert(sizeof(Static) == kStaticSmem, "static shared-memory block");
     __shared__ Static st;
@@ -355,6 +357,8 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
                 mbar_init(&st.bar_odone[i], 1); mbar_init(&st.bar_ofree[i], 4);
             }
             for (int i = 0; i < kSegRing; ++i) { mbar_init(&st.bar_segfull[i], 1); mbar_init(&st.bar_segempty[i], kProducerWarp + 1); }
+            mbar_init(&st.bar_idle, 1);
+            st.q_last = 1;
             mbar_init(&st.bar_mlfull, 8);
             mbar_init(&st.bar_mlempty, 4);
             fence_barrier_init();
@@ -680,8 +684,8 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
                 const bool two = TWO && cur.two_rb(P);
                 if (lead) {
                     ok = mbar_wait_while(ok, &st.bar_segempty[seg % kSegRing], ((seg / kSegRing) & 1) ^ 1);
-                    Segment s;
-                    s.n = on ? n : 0; s.t0 = t0; s.nt = nt; s.Pb = Pb; s.M = cur.s.M; s.rows = cur.s.rows; s.b = b; s.g = g; s.layer = layer;
+                    Segment s;                       // (behind a wait that ran out the others are sent home)
+                    s.n = on && ok ? n : 0; s.t0 = t0; s.nt = nt; s.Pb = Pb; s.M = cur.s.M; s.rows = cur.s.rows; s.b = b; s.g = g; s.layer = layer;
                     st.seg[seg % kSegRing] = s;
                     mbar_arrive(&st.bar_segfull[seg % kSegRing]);
                 }
@@ -721,9 +725,10 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
                         unsigned char* dst = (is_k ? sK : sV) + slot * SM::kTileBytes;
                         if (lead) ok = mbar_wait_while(ok, is_k ? &st.bar_kempty[slot] : &st.bar_vempty[slot], is_k ? k_par : v_par);
                         if (PAGED) ok = __shfl_sync(kFull, ok, 0);
+                        if (!ok) break;                              // (the ring's position stays that of the last load)
                         if (is_k) { if (++k_slot == RK) { k_slot = 0; k_par ^= 1; } }
                         else if (++v_slot == RV) { v_slot = 0; v_par ^= 1; }
-                        if (ok && !boxes) {
+                        if (!boxes) {
                             if (lead) {
                                 const int keys = tree ? kTreeKeys : kTileKeys;
                                 const CUtensorMap* tm = tree ? (is_k ? &tmKt : &tmVt) : (is_k ? &tmKc : &tmVc);
@@ -731,7 +736,7 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
                                 mbar_arrive_expect_tx(full, keys * D * 2);
                                 for (int h = 0; h < H; ++h) tma_load_4d(dst + h * (keys * 128), tm, full, h * 64, g, row, layer);
                             }
-                        } else if (ok) {
+                        } else {
                             if (lead) mbar_arrive_expect_tx(full, n_ld * per * D * 2);
                             __syncwarp();
                             if (lane < n_ld)
@@ -743,6 +748,7 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
                         ok = mbar_wait_while(ok, &st.bar_qempty, (seg & 1) ^ 1);
                         const int blocks = two ? 2 : 1, node0 = b * kMaxNodes + pp * P.n_blk * P.nodes_per_rb;
                         if (ok) {
+                            st.q_last = seg & 1;
                             mbar_arrive_expect_tx(&st.bar_qfull, blocks * P.rb_rows * D * 2);   // rows past rb_rows stay stale: never read back
                             for (int q = 0; q < blocks; ++q)
                                 for (int h = 0; h < H; ++h)
@@ -778,6 +784,13 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
                 CutUnit* out = P.cut + blockIdx.x;
                 out->valid = cu.valid; out->b = cu.b; out->g = cu.g; out->layer = cu.layer;
                 out->slot = cu.slot; out->rows = cu.rows; out->n_pieces = cu.n_pieces;
+            }
+            // no load may land in shared memory that the CTA has left
+            if (lead) {
+                bool landed = mbar_drain(&st.bar_qfull, st.q_last);
+                for (int i = 0; i < RK; ++i) landed &= mbar_drain(&st.bar_kfull[i], last_armed_parity(i, k_slot, k_par));
+                for (int i = 0; i < RV; ++i) landed &= mbar_drain(&st.bar_vfull[i], last_armed_parity(i, v_slot, v_par));
+                ok &= landed;
             }
             __syncwarp();
         } else if (warp == kMmaWarp) {
@@ -936,26 +949,20 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
                     }
                 }
             }
+            // nor may a product read shared memory or write tensor memory that it has given back
+            mma_commit_if(elected, &st.bar_idle);
+            ok &= mbar_drain(&st.bar_idle, 0);
             __syncwarp();
         }
     }
 
-    // ---- teardown ----
+    // ---- teardown: producer and issuer have waited for what they had in flight ----
     if (!ok) st.abort = 1;
     tc_fence_before_sync();
     __syncthreads();
     if (warp == kMmaWarp) {
-        if (st.abort) {
-            // let loads that are still in flight land before the CTA's shared memory is released
-            if (lane == 0) {
-                for (int i = 0; i < 3; ++i) {
-                    mbar_wait_while(true, &st.bar_kfull[i], 0, 64);
-                    mbar_wait_while(true, &st.bar_vfull[i], 0, 64);
-                }
-                set_status(P.status, RADAR_ERR_TIMEOUT);
-            }
-            __syncwarp();
-        }
+        if (lane == 0 && st.abort) set_status(P.status, RADAR_ERR_TIMEOUT);
+        __syncwarp();
         tmem_dealloc(st.tmem_base, 512);
     }
 }
@@ -990,6 +997,8 @@ tree_attn_tc_fine_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_c
     struct __align__(1024) Static {
         uint64_t bar_qfull, bar_qempty, bar_kfull[3], bar_kempty[3], bar_vfull[3], bar_vempty[3];
         uint64_t bar_sfull[2], bar_pfirst[2], bar_pready[2], bar_odone[2], bar_ofree[2];
+        uint64_t bar_idle;       // every product issued has run
+        uint32_t armed[4];       // K and V loads of the producer, phase parity of its last Q
         long long range[4];      // this CTA's range [lo, hi), size of the class's space (all layers), start of its first unit
         int start[3];            // sequence, KV head and layer of the unit that contains lo
         int start_pad;
@@ -997,7 +1006,7 @@ tree_attn_tc_fine_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_c
         int abort;
         float xm[128];           // group 1's running max at the end of a segment (one live row block)
         float mx[2][2][128];     // per group and column half: row maxima of a tile; row sums at the end of a segment
-        unsigned char pad[kStaticSmem - (24 * 8 + 4 * 8 + 4 * 4 + 4 + 4 + 128 * 4 + 2 * 2 * 128 * 4)];
+        unsigned char pad[kStaticSmem - (25 * 8 + 4 * 4 + 4 * 8 + 4 * 4 + 4 + 4 + 128 * 4 + 2 * 2 * 128 * 4)];
     };
     static_assert(sizeof(Static) == kStaticSmem, "static shared-memory block");
     __shared__ Static st;
@@ -1079,6 +1088,8 @@ tree_attn_tc_fine_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_c
             s_abort = 0;
             mbar_init(&bar_qfull, 1);
             mbar_init(&bar_qempty, 1);
+            mbar_init(&st.bar_idle, 1);
+            st.armed[2] = 1;
             for (int i = 0; i < 3; ++i) {
                 mbar_init(&bar_kfull[i], 1); mbar_init(&bar_kempty[i], 1);
                 mbar_init(&bar_vfull[i], 1); mbar_init(&bar_vempty[i], 1);
@@ -1149,6 +1160,7 @@ tree_attn_tc_fine_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_c
                 }
                 if (lead) ok = ok && mbar_wait(&bar_qempty, (seg & 1) ^ 1, ab);
                 if (lead && ok) {
+                    st.armed[2] = seg & 1;
                     mbar_arrive_expect_tx(&bar_qfull, (two ? 2 : 1) * P.rb_rows * D * 2);   // rows past rb_rows stay stale: never read back
                     for (int q = 0; q < (two ? 2 : 1); ++q)
                         for (int h = 0; h < H; ++h)
@@ -1160,13 +1172,13 @@ tree_attn_tc_fine_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_c
                     const int ring = is_k ? RK : RV;
                     const int slot = cnt % ring;
                     const uint32_t use = cnt / ring;
-                    ++cnt;
                     uint64_t* full = is_k ? &bar_kfull[slot] : &bar_vfull[slot];
                     uint64_t* empty = is_k ? &bar_kempty[slot] : &bar_vempty[slot];
                     unsigned char* dst = (is_k ? sK : sV) + slot * SM::kTileBytes;
                     if (lead && (!ok || !mbar_wait(empty, (use & 1) ^ 1, ab))) ok = false;
                     if (PAGED) ok = __shfl_sync(kFull, ok, 0);
                     if (!ok) return;
+                    ++cnt;                           // loads armed
                     if (t == cur.s.nt - 1) {
                         if (lead) {
                             mbar_arrive_expect_tx(full, kTreeKeys * D * 2);
@@ -1205,6 +1217,7 @@ tree_attn_tc_fine_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_c
                     if (i + la < n) load_tile(cur.t0 + i + la, true);
                 }
             }
+            if (lead) { st.armed[0] = kc; st.armed[1] = vc; }
         }
         __syncwarp();
         if (__shfl_sync(kFull, cu.valid, 0)) {
@@ -1399,6 +1412,9 @@ tree_attn_tc_fine_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_c
                 }
             }
         }
+        // no product may read shared memory or write tensor memory that the CTA has given back
+        mma_commit_if(elected, &st.bar_idle);
+        if (!mbar_drain(&st.bar_idle, 0)) s_abort = 1;
         __syncwarp();
     } else {
         // =================================== softmax groups ===================================
@@ -1655,12 +1671,14 @@ tree_attn_tc_fine_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_c
     __syncthreads();
     if (warp == kFineProducerWarp) {
         if (s_abort) {
-            // let loads that are still in flight land before the CTA's shared memory is released
+            // no load may land in shared memory that the CTA has left
             if (lane == 0) {
                 int dummy = 0;
-                for (int i = 0; i < 3; ++i) {
-                    mbar_wait(&bar_kfull[i], 0, &dummy, 1u << 12);
-                    mbar_wait(&bar_vfull[i], 0, &dummy, 1u << 12);
+                const uint32_t nk = st.armed[0], nv = st.armed[1];
+                mbar_wait(&bar_qfull, st.armed[2], &dummy, 1u << 12);
+                for (int i = 0; i < RK; ++i) {
+                    mbar_wait(&bar_kfull[i], last_armed_parity(i, nk % RK, (nk / RK & 1) ^ 1), &dummy, 1u << 12);
+                    if (i < RV) mbar_wait(&bar_vfull[i], last_armed_parity(i, nv % RV, (nv / RV & 1) ^ 1), &dummy, 1u << 12);
                 }
                 set_status(P.status, RADAR_ERR_TIMEOUT);
             }

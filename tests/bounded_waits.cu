@@ -12,8 +12,8 @@ __device__ unsigned long long now_ns() {
     return t;
 }
 
-// A wait of each kind for an arrival that never comes, one thread each: ns[i] it took, seen[i] its outcome; then, in ns[2] and
-// seen[2], 1000 waits behind the first one that ran out.
+// Waits for an arrival that never comes, one thread each: ns[i] it took, seen[i] its outcome.  0: a wait that polls, 1: one that
+// naps, 2: 1000 waits behind the first, 3: a block's wait for what it has in flight.
 __global__ void waits_that_run_out_kernel(unsigned long long* ns, int* seen) {
     __shared__ uint64_t bar;
     if (threadIdx.x == 0) {
@@ -22,22 +22,29 @@ __global__ void waits_that_run_out_kernel(unsigned long long* ns, int* seen) {
     }
     __syncthreads();
     if ((threadIdx.x & 31) != 0) return;
-    const int i = threadIdx.x >> 5;
-    const unsigned long long t0 = now_ns();
-    bool ok = i == 0 ? mbar_wait_while(true, &bar, 0) : mbar_wait_lazy(true, &bar, 0);
-    const unsigned long long t1 = now_ns();
-    ns[i] = t1 - t0;
-    seen[i] = ok;
-    if (i == 0) {
-        for (int n = 0; n < 1000; ++n) ok = mbar_wait_while(ok, &bar, 0);
-        ns[2] = now_ns() - t1;
-        seen[2] = ok;
+    auto timed = [&](int i, auto wait) {
+        const unsigned long long t0 = now_ns();
+        seen[i] = wait();
+        ns[i] = now_ns() - t0;
+    };
+    switch (threadIdx.x >> 5) {
+        case 0:
+            timed(0, [&] { return mbar_wait_while(true, &bar, 0); });
+            timed(2, [&] {
+                bool ok = false;
+                for (int n = 0; n < 1000; ++n) ok |= mbar_wait_while(false, &bar, 0);
+                return ok;
+            });
+            break;
+        case 1: timed(1, [&] { return mbar_wait_lazy(true, &bar, 0); }); break;
+        case 2: timed(3, [&] { return mbar_drain(&bar, 0); }); break;
     }
 }
 extern "C" int waits_that_run_out(unsigned long long* ns, int* seen) {
-    waits_that_run_out_kernel<<<1, 64>>>(ns, seen);
+    waits_that_run_out_kernel<<<1, 96>>>(ns, seen);
     return (int)cudaDeviceSynchronize();
 }
+extern "C" unsigned ring_parity(unsigned slot, unsigned next, unsigned par) { return last_armed_parity(slot, next, par); }
 
 // A predecessor that lets its dependents start at once and then takes `ns` nanoseconds (bounded by its naps as well).
 __global__ void slow_predecessor_kernel(unsigned long long ns, int naps) {

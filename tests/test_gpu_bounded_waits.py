@@ -6,8 +6,6 @@ import subprocess
 
 import pytest
 
-pytestmark = pytest.mark.gpu
-
 HERE = os.path.dirname(os.path.abspath(__file__))
 
 
@@ -20,19 +18,34 @@ def waits(tmp_path_factory):
     return ctypes.CDLL(so)
 
 
-def test_a_wait_gives_up_after_seconds(waits):
+def test_the_phase_that_a_block_drains(waits):
+    """Every slot of a ring of loads is waited for in the phase it was last armed for (a slot never armed: the one that a new
+    barrier passes), after any number of loads.  No GPU needed."""
+    for ring in (2, 3):
+        for loads in range(5 * ring):
+            armed = [len(range(slot, loads, ring)) for slot in range(ring)]
+            for slot in range(ring):
+                expect = (armed[slot] - 1) & 1
+                assert waits.ring_parity(slot, loads % ring, ((loads // ring) & 1) ^ 1) == expect, (ring, loads, slot)
+
+
+@pytest.mark.gpu
+def test_waits_that_run_out(waits):
     """A wait for an arrival that never comes returns false, after more than a second (a healthy launch can be held up for tens
-    of milliseconds, by the memory system or by its neighbours) and less than a minute; those behind it cost microseconds."""
+    of milliseconds, by the memory system or by its neighbours) and less than a minute; those behind it cost microseconds.  A
+    block's wait for what it has in flight is bounded as well."""
     import torch
-    ns, seen = torch.zeros(3, dtype=torch.int64, device="cuda"), torch.ones(3, dtype=torch.int32, device="cuda")
+    ns, seen = torch.zeros(4, dtype=torch.int64, device="cuda"), torch.ones(4, dtype=torch.int32, device="cuda")
     torch.cuda.synchronize()
     assert waits.waits_that_run_out(ctypes.c_void_p(ns.data_ptr()), ctypes.c_void_p(seen.data_ptr())) == 0
     assert not seen.any()
     took = ns.tolist()
     assert all(1e9 < t < 6e10 for t in took[:2]), took
     assert took[2] < 1e8, took
+    assert 1e8 < took[3] < 1e10, took
 
 
+@pytest.mark.gpu
 @pytest.mark.parametrize("Hq,page", [(16, 0), (32, 16), (12, 0)])
 def test_a_slow_predecessor_is_not_a_timeout(waits, Hq, page):
     """The launch begins while its predecessor, which lets it, still runs for longer than the waits of the kernel are bounded by
