@@ -71,6 +71,13 @@ struct __align__(16) CutUnit {
     uint32_t live[kMaxPerClass / 32];    // bit j: piece j's range holds the start of a tile of the unit
 };
 
+// ... and what its table of pieces follows from.
+struct Cut {
+    CutUnit unit;
+    long long u0, tot;   // start of the unit, size of the class's space (all layers)
+    int nt, w;           // tiles of the unit and their cost
+};
+
 struct TcParams {
     radar_attn_args a;
     int G, nodes_per_rb; // a row block holds whole nodes: nodes_per_rb = 128 / G (rounded down) of them
@@ -330,10 +337,11 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
         uint64_t bar_pready[2];          // ... all of them
         uint64_t bar_segfull[kSegRing], bar_segempty[kSegRing];
         Segment seg[kSegRing];
+        Cut cut;                         // (paged: the producer's)
         float2 ml[2][128];               // per group: (m in log2 units, l) of the rows at the end of a segment
         uint32_t tmem_base;
         int abort;
-        unsigned char pad[kStaticSmem - ((28 + 2 * kSegRing) * 8 + kSegRing * (int)sizeof(Segment) + 2 * 128 * 8 + 8)];
+        unsigned char pad[kStaticSmem - ((28 + 2 * kSegRing) * 8 + kSegRing * (int)sizeof(Segment) + (int)sizeof(Cut) + 2 * 128 * 8 + 8)];
     };
     static_assert(sizeof(Static) == kStaticSmem, "static shared-memory block");
     __shared__ Static st;
@@ -663,10 +671,14 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
             long long tot_all;
             Cursor<PAGED> cur = first_segment<PAGED>(P, pp, ci, tot_all);
             if (!usable) cur.t0 = cur.t1 = 0;
-            CutUnit cu;
-            cu.valid = 0;
-            int cut_nt = 0, cut_w = 0;
-            long long cut_u0 = 0;
+            // Needed behind the last load only, and a dozen registers.  With a paged cache, whose producer would spill for them
+            // (132 bytes, in its loop over the tiles), in shared memory: B = 1, 32 / 8 heads, 2048 tokens in pages of 16 21.9 ->
+            // 20.2 us, of 256 19.4 -> 17.7; B = 8, 64 / 8 heads, 8192 tokens, pages of 16 198.3 -> 192.8.  Without one, where
+            // nothing is spilled, in registers (8 layers of B = 8, 64 / 8 heads 1073, in shared memory 1081).
+            Cut own;
+            Cut& cut = PAGED ? st.cut : own;
+            cut.unit.valid = 0;
+            cut.tot = tot_all;
             uint32_t k_slot = 0, k_par = 1, v_slot = 0, v_par = 1;   // ring slot to fill next and the phase that frees it
             const int n_cache_pages = PAGED ? (int)P.cache_rows / a.page_size : 0;            // (cache_rows: below 2^31)
             const int box_shift = PAGED ? __ffs(min(a.page_size, kTileKeys)) - 1 : 0, tiles_per_page = PAGED ? max(a.page_size / kTileKeys, 1) : 1;
@@ -691,8 +703,8 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
                 }
                 if (!on) break;
                 if (t0 == 0 && n < nt) {                             // necessarily the last segment of this CTA
-                    cu.valid = 1; cu.b = b; cu.g = g; cu.slot = seg == 0 ? 0 : 1; cu.layer = layer; cu.rows = cur.s.rows;
-                    cut_nt = nt; cut_w = cur.s.w; cut_u0 = cur.U;
+                    cut.unit.valid = 1; cut.unit.b = b; cut.unit.g = g; cut.unit.slot = seg == 0 ? 0 : 1; cut.unit.layer = layer; cut.unit.rows = cur.s.rows;
+                    cut.nt = nt; cut.w = cur.s.w; cut.u0 = cur.U;
                 }
                 cur.next(P, pp);
                 if (!PAGED && !lead) continue;
@@ -765,15 +777,18 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
                 }
             }
             __syncwarp();
+            CutUnit cu = cut.unit;
             if (cu.valid) {
-                const long long u1 = cut_u0 + (long long)cut_nt * cut_w + P.unit_cost;
+                const long long u0 = cut.u0, tot = cut.tot;
+                const int nt = cut.nt, w = cut.w;
+                const long long u1 = u0 + (long long)nt * w + P.unit_cost;
                 cu.n_pieces = 0;
 #pragma unroll 1
                 for (int k = 0; k < kMaxPerClass / 32; ++k) {
                     const int c = ci + k * 32 + lane;
-                    const long long lo = tot_all * c / P.ncc, hi = tot_all * (c + 1) / P.ncc;
+                    const long long lo = tot * c / P.ncc, hi = tot * (c + 1) / P.ncc;
                     const bool piece = c < P.ncc && lo < u1;
-                    const bool live = piece && tiles_before(hi, cut_u0, cut_nt, cut_w, P.unit_cost) > tiles_before(lo, cut_u0, cut_nt, cut_w, P.unit_cost);
+                    const bool live = piece && tiles_before(hi, u0, nt, w, P.unit_cost) > tiles_before(lo, u0, nt, w, P.unit_cost);
                     const uint32_t pieces = __ballot_sync(kFull, piece), bits = __ballot_sync(kFull, live);
                     cu.n_pieces += __popc(pieces);
                     if (lane == 0) P.cut[blockIdx.x].live[k] = bits;
