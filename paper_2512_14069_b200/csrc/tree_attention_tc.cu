@@ -286,6 +286,34 @@ __device__ __forceinline__ Cursor<PAGED> first_segment(const TcParams& P, int pp
     return cur;
 }
 
+// What a CTA leaves to the combine, by a whole warp that agrees on `cut`.
+__device__ __forceinline__ void write_cut_unit(const TcParams& P, int ci, const Cut& cut) {
+    const int lane = threadIdx.x & 31;
+    CutUnit* out = P.cut + blockIdx.x;
+    int n_pieces = 0;
+    if (cut.unit.valid) {
+        const long long u0 = cut.u0, tot = cut.tot;
+        const int nt = cut.nt, w = cut.w;
+        const long long u1 = u0 + (long long)nt * w + P.unit_cost;
+#pragma unroll 1
+        for (int k = 0; k < kMaxPerClass / 32; ++k) {
+            const int c = ci + k * 32 + lane;
+            const long long lo = tot * c / P.ncc, hi = tot * (c + 1) / P.ncc;
+            const bool piece = c < P.ncc && lo < u1;
+            const bool live = piece && tiles_before(hi, u0, nt, w, P.unit_cost) > tiles_before(lo, u0, nt, w, P.unit_cost);
+            const uint32_t pieces = __ballot_sync(kFull, piece), bits = __ballot_sync(kFull, live);
+            n_pieces += __popc(pieces);
+            if (lane == 0) out->live[k] = bits;
+            if (pieces != 0xffffffffu) break;
+        }
+    }
+    if (lane == 0) {
+        const CutUnit& u = cut.unit;
+        out->valid = u.valid; out->b = u.b; out->g = u.g; out->layer = u.layer;
+        out->slot = u.slot; out->rows = u.rows; out->n_pieces = n_pieces;
+    }
+}
+
 // What the other warps know of a segment.
 constexpr int kSegRing = 4;
 struct __align__(16) Segment {
@@ -777,29 +805,7 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
                 }
             }
             __syncwarp();
-            CutUnit cu = cut.unit;
-            if (cu.valid) {
-                const long long u0 = cut.u0, tot = cut.tot;
-                const int nt = cut.nt, w = cut.w;
-                const long long u1 = u0 + (long long)nt * w + P.unit_cost;
-                cu.n_pieces = 0;
-#pragma unroll 1
-                for (int k = 0; k < kMaxPerClass / 32; ++k) {
-                    const int c = ci + k * 32 + lane;
-                    const long long lo = tot * c / P.ncc, hi = tot * (c + 1) / P.ncc;
-                    const bool piece = c < P.ncc && lo < u1;
-                    const bool live = piece && tiles_before(hi, u0, nt, w, P.unit_cost) > tiles_before(lo, u0, nt, w, P.unit_cost);
-                    const uint32_t pieces = __ballot_sync(kFull, piece), bits = __ballot_sync(kFull, live);
-                    cu.n_pieces += __popc(pieces);
-                    if (lane == 0) P.cut[blockIdx.x].live[k] = bits;
-                    if (pieces != 0xffffffffu) break;
-                }
-            }
-            if (lane == 0) {
-                CutUnit* out = P.cut + blockIdx.x;
-                out->valid = cu.valid; out->b = cu.b; out->g = cu.g; out->layer = cu.layer;
-                out->slot = cu.slot; out->rows = cu.rows; out->n_pieces = cu.n_pieces;
-            }
+            write_cut_unit(P, ci, cut);
             // no load may land in shared memory that the CTA has left
             if (lead) {
                 bool landed = mbar_drain(&st.bar_qfull, st.q_last);
@@ -1158,10 +1164,10 @@ tree_attn_tc_fine_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_c
         // One lane does everything for the contiguous cache.  With a paged cache the whole warp walks the same
         // loop and lane p looks up and fetches page p of a tile (up to eight boxes per tile), the leading lane
         // still doing the waits, the byte counts, Q and the tree tile.
-        CutUnit cu;
-        cu.valid = 0;
-        int cut_nt = 0, cut_w = 0;
-        long long cut_u0 = 0;
+        Cut cut;
+        cut.unit.valid = 0;
+        cut.nt = cut.w = 0;
+        cut.u0 = 0;
         if (PAGED || lane == 0) {
             const bool lead = lane == 0;
             uint32_t kc = 0, vc = 0;
@@ -1170,8 +1176,9 @@ tree_attn_tc_fine_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_c
                 const int b = cur.b, g = cur.g, n = cur.t1 - cur.t0;
                 const bool two = TWO && cur.two_rb(P);
                 if (cur.t0 == 0 && cur.t1 < cur.s.nt) {          // necessarily the last segment of this CTA
-                    cu.valid = 1; cu.b = b; cu.g = g; cu.slot = seg == 0 ? 0 : 1; cu.layer = cur.layer; cu.rows = cur.s.rows;
-                    cut_nt = cur.s.nt; cut_w = cur.s.w; cut_u0 = cur.U;
+                    cut.unit.valid = 1; cut.unit.b = b; cut.unit.g = g; cut.unit.slot = seg == 0 ? 0 : 1;
+                    cut.unit.layer = cur.layer; cut.unit.rows = cur.s.rows;
+                    cut.nt = cur.s.nt; cut.w = cur.s.w; cut.u0 = cur.U;
                 }
                 if (lead) ok = ok && mbar_wait(&bar_qempty, (seg & 1) ^ 1, ab);
                 if (lead && ok) {
@@ -1235,27 +1242,12 @@ tree_attn_tc_fine_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_c
             if (lead) { st.armed[0] = kc; st.armed[1] = vc; }
         }
         __syncwarp();
-        if (__shfl_sync(kFull, cu.valid, 0)) {
-            const int nt = __shfl_sync(kFull, cut_nt, 0), w = __shfl_sync(kFull, cut_w, 0);
-            const long long u0 = __shfl_sync(kFull, cut_u0, 0), u1 = u0 + (long long)nt * w + P.unit_cost, tot = s_range[2];
-            cu.n_pieces = 0;
-#pragma unroll 1
-            for (int k = 0; k < kMaxPerClass / 32; ++k) {
-                const int c = ci + k * 32 + lane;
-                const long long lo = tot * c / P.ncc, hi = tot * (c + 1) / P.ncc;
-                const bool piece = c < P.ncc && lo < u1;
-                const bool on = piece && tiles_before(hi, u0, nt, w, P.unit_cost) > tiles_before(lo, u0, nt, w, P.unit_cost);
-                const uint32_t pieces = __ballot_sync(kFull, piece), live = __ballot_sync(kFull, on);
-                cu.n_pieces += __popc(pieces);
-                if (lane == 0) P.cut[blockIdx.x].live[k] = live;
-                if (pieces != 0xffffffffu) break;
-            }
+        if (!PAGED) {                    // lane 0 alone has gone through the segments
+            cut.unit.valid = __shfl_sync(kFull, cut.unit.valid, 0);
+            cut.nt = __shfl_sync(kFull, cut.nt, 0); cut.w = __shfl_sync(kFull, cut.w, 0); cut.u0 = __shfl_sync(kFull, cut.u0, 0);
         }
-        if (lane == 0) {
-            CutUnit* out = P.cut + blockIdx.x;
-            out->valid = cu.valid; out->b = cu.b; out->g = cu.g; out->layer = cu.layer;
-            out->slot = cu.slot; out->rows = cu.rows; out->n_pieces = cu.n_pieces;
-        }
+        cut.tot = s_range[2];
+        write_cut_unit(P, ci, cut);
         __syncwarp();
     } else if (warp == kFineMmaWarp) {
         // =================================== MMA issuer ===================================
