@@ -74,8 +74,9 @@ __device__ __forceinline__ bool mbar_drain(uint64_t* bar, uint32_t parity, uint3
         if (mbar_try_wait(bar, parity)) return true;
     return false;
 }
-// The phase that slot `i` of a ring of loads was last armed for, as the parity to wait with, where the next load would go to
-// slot `next` once phase parity `par` has freed it (1 in the first round).  A slot never armed gives 1, which a new barrier passes.
+// The phase that slot `i` of a ring of loads was last armed for, as the parity to wait with, where the next load would go
+// to slot `next` once phase parity `par` has freed it (1 in the first round).  A slot never armed gives 1, which a new
+// barrier passes.
 __host__ __device__ constexpr uint32_t last_armed_parity(uint32_t i, uint32_t next, uint32_t par) { return i < next ? par ^ 1u : par; }
 
 // Bounded wait: gives up after `limit` polls (each poll itself blocks for a hardware-defined short
@@ -132,8 +133,8 @@ __device__ __forceinline__ void tmem_dealloc(uint32_t taddr, uint32_t ncols) {
 }
 
 // ---- descriptors ----------------------------------------------------------------------------------
-// Shared-memory operand descriptors (their words are put together in the issue sequences below) for tiles written by TMA with the 128-byte swizzle: rows of 128
-// bytes, 8 rows per 1024-byte swizzle atom.
+// Shared-memory operand descriptors (their words are put together in the issue sequences below) for tiles written by TMA with
+// the 128-byte swizzle: rows of 128 bytes, 8 rows per 1024-byte swizzle atom.
 //   K-major operand  (rows = M or N index, the 128 bytes run along K): SBO = bytes between 8-row groups.
 //   MN-major operand (rows = K index, the 128 bytes run along M/N): SBO = bytes between 8-row (8 K) groups,
 //                     LBO = bytes between consecutive 64-element blocks along M/N.
@@ -146,8 +147,9 @@ __host__ __device__ constexpr uint32_t idesc_bf16_f32(int M, int N, bool a_mn_ma
 }
 
 // ---- MMA issue ------------------------------------------------------------------------------------
-// SS: D[tmem] (+)= A[smem] * B[smem]; TS: D[tmem] (+)= A[tmem] * B[smem].  Predicated, for a warp that runs the issue code converged: every lane executes the instruction
-// stream (so the descriptor arithmetic stays warp-uniform), the lane with `pred` != 0 issues.
+// SS: D[tmem] (+)= A[smem] * B[smem]; TS: D[tmem] (+)= A[tmem] * B[smem].  Predicated, for a warp that runs the issue code
+// converged: every lane executes the instruction stream (so the descriptor arithmetic stays warp-uniform), the lane with `pred`
+// != 0 issues.
 __device__ __forceinline__ uint32_t elect_one() {
     uint32_t pred;
     asm volatile("{\n\t.reg .pred p;\n\t.reg .b32 r;\n\telect.sync r|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(pred));

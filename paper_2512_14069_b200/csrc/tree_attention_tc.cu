@@ -28,8 +28,8 @@
 //   warps 8-11 epilogue: a finished accumulator to O or to the partials, while the others are in the next segment.
 //   warps 14, 15 only fill up the producer's warpgroup.
 // What is rare (ends of segments, tiles that are not full) shares its code with what is not, or is written as loops: with every
-// wait, schedule and mask unrolled in line the kernel had 140 KB of code, a segment's end missed the instruction cache all
-// along, and 8.5 thousand cycles lay between a segment's last product and the next one's first.
+// wait, schedule and mask unrolled in line the kernel had up to 145 KB of code (112 now), a segment's end missed the instruction
+// cache all along, and 8.5 thousand cycles lay between a segment's last product and the next one's first.
 // Every mbarrier wait is bounded; a wait that runs out sets RADAR_ERR_TIMEOUT on the device status
 // word, the CTA drains, frees its tensor memory and returns.
 #include <cuda.h>
@@ -153,10 +153,10 @@ __device__ __forceinline__ float lse_of(float m, float l) {
 // a unit with one live row block cost_one, and every unit books cost_unit in front of its first tile for what it
 // costs beside its tiles (pipeline fill, epilogue), so that a CTA whose range holds several unit starts gets fewer
 // tiles; equal position ranges are then about equal amounts of time.  A tile belongs to the CTA whose range
-// contains the tile's start position.  The weights are measured, not derived (attention kernel inside whole steps,
-// A/B on one GPU, against 3 : 5 without the unit term): with one class per KV head 2 : 4 + 12 (ragged batch of 32:
-// 605 -> 554 us; batch 1 is not of this kind), with several classes 3 : 5 + 15 (batch 1: 27.3 -> 23.3 us; batch 8 with
-// ragged trees: 167 -> 165 us, where 2 : 4 + 12 gave 175 us).
+// contains the tile's start position.  The weights are measured, not derived (us a launch with its combine, against 3 : 5 without
+// the unit term): several classes per KV head, 3 : 5 + 15: 32 / 8 heads, B = 1, 2048 tokens 18.7 -> 17.1; 64 / 8 heads, B = 8, 2000
+// to 8192 tokens, trees of two calls 114 -> 111; one class, 2 : 4 + 12: 32 / 8 heads, B = 32, 4096 to 32768 tokens 780 -> 772.
+// It is the unit term that counts; 2 : 4 + 12 everywhere gives 17.3, 103 to 108 and 764, other sets lie within 2 %.
 struct TileCosts { int one, two, unit; };
 inline TileCosts tile_costs(int n_cls) { return n_cls == 1 ? TileCosts{2, 4, 12} : TileCosts{3, 5, 15}; }
 
@@ -1844,10 +1844,11 @@ bool make_map(CUtensorMap* tm, const void* base, int d, int heads, long long row
 
 // Grid shape.  A class is one row-block pair (256 query rows: both row blocks share every K/V tile in
 // shared memory) or, when such fused units would leave most SMs without work, one row block (128 rows).
-// CTAs per class: the grid is one CTA per SM, but at least two tiles per CTA when every sequence
-// has the longest prefix (four: 16.8 us for 32 / 8 heads, 1000 tokens, two: 15.0; 4 / 4 heads, d = 64, 500 tokens: 14.1, 12.2).  Both decisions look at the tiles of the whole launch, all its layers: 32 layers of one
-// sequence with 2048 tokens (32 / 8 heads, d = 128) run as 148 CTAs of fused units, where one layer alone would
-// be split into half units on 68 CTAs.
+// CTAs per class: the grid is one CTA per SM, but at least two tiles per CTA when every sequence has the longest prefix (four
+// instead of two, us: 32 / 8 heads, 1000 tokens 16.0 / 14.6; 4 / 4 heads, d = 64, 500 tokens 13.6 / 11.5; 16 / 16 heads, 1000 tokens
+// 14.5 / 13.6; but 32 / 8 heads, 2048 tokens 16.5 / 17.1).  Both decisions look at the tiles of the whole launch, all its
+// layers: 32 layers of one sequence with 2048 tokens (32 / 8 heads, d = 128) run as 148 CTAs of fused units, where one layer
+// alone would be split into half units on 128 CTAs.
 void plan_grid(const radar_ctx* ctx, int B, int Hq, int Hkv, int max_prefix_len, int layers, int* n_blk, int* n_cls, int* ncc,
                bool* whole) {
     const int G = Hq / Hkv;
@@ -1863,7 +1864,7 @@ void plan_grid(const radar_ctx* ctx, int B, int Hq, int Hkv, int max_prefix_len,
     // All units of one sequence are alike, so where they are no more than the CTAs of a class a grid can be chosen in
     // which every CTA has one piece of one unit and pays for one segment (fill and epilogue, what tile_costs books per
     // unit) and not for two.  Not where that leaves so many CTAs unused that the pieces get longer than what it saves.
-    // (Attention + combine, d = 128: 40 / 40 heads, 2048 tokens 26.8 -> 24.8 us; 16 / 16 heads, 1000 tokens 20.6 -> 17.2.)
+    // (Attention + combine, d = 128: 40 / 40 heads, 2048 tokens 22.9 -> 19.6 us; 16 / 16 heads, 1000 tokens 14.8 -> 13.6.)
     const long long units = (long long)layers * Hkv, tiles = unit_tiles / (B * units);
     *whole = false;
     if (B == 1 && units <= per) {
