@@ -1060,6 +1060,8 @@ tree_attn_tc_fine_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_c
     const bool smem_aligned = (smem_u32(smem_raw) & 1023u) == 0;
 
     // ---- set-up: warp 0 finds this CTA's range while the barriers and tensor memory are prepared ----
+    // (The steps of first_segment, which has to give the same ranges.  That function called here: 24 / 8 heads, B = 1, 2048 tokens
+    // 19.2 -> 19.5 us, 28 / 4 heads, B = 1, 1000 tokens 16.8 -> 17.0, others within 2 % either way.)
     if (warp == 0) {
         chain_sync();                    // every global access of the CTA comes after the block barrier below
         long long tot = 0;
