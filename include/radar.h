@@ -182,6 +182,23 @@ typedef struct {
 size_t radar_expand_calls_workspace_bytes(const radar_ctx* ctx, int B, int V, int k, int t_max);
 int radar_expand_calls(radar_ctx* ctx, const radar_expand_calls_args* args, void* stream);
 
+/* radar_expand_range - calls t_first .. t_last of such a step: the ranges of a step, issued one behind the other, leave what
+ * radar_expand_calls would.  A range reads the rows of the sequences that are still active when it begins, so where the passes
+ * are long, shorter ranges read less in vain (the last ones rows of calls that no sequence makes, the first ones nothing).
+ * `call`, the buffers and the limits are those of radar_expand_calls, without its bound on the logits of a call, and with
+ * RADAR_POLICY_LSTM_HIDDEN as a third policy, whose `features` are [t_max-1][B][feat_dim], a slice per call; 1 <= t_first
+ * <= t_last <= t_max.  Workspace: radar_expand_range_workspace_bytes (0: sizes out of range, RADAR_ERR_UNSUPPORTED); ranges
+ * that are issued on one stream may share it. */
+typedef struct {
+    radar_expand_args call;
+    int32_t* topk_tok_next;
+    float* topk_logp_next;
+    int t_first, t_last;
+} radar_expand_range_args;
+
+size_t radar_expand_range_workspace_bytes(const radar_ctx* ctx, int B, int V, int k, int t_first, int t_last);
+int radar_expand_range(radar_ctx* ctx, const radar_expand_range_args* args, void* stream);
+
 /* ------------------------------------------------------------------------------------------
  * radar_rerank_build_tree - top-N rerank of the pool and serialisation for one masked pass.
  * (Sec. 1: the candidates form a tree that is serialised and verified via masked attention

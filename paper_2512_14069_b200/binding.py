@@ -47,6 +47,10 @@ class ExpandCallsArgs(ctypes.Structure):
     _fields_ = [("call", ExpandArgs), ("topk_tok_next", _vp), ("topk_logp_next", _vp)]
 
 
+class ExpandRangeArgs(ctypes.Structure):
+    _fields_ = ExpandCallsArgs._fields_ + [("t_first", _c_int), ("t_last", _c_int)]
+
+
 class TreeArgs(ctypes.Structure):
     _fields_ = [
         ("B", _c_int), ("N", _c_int), ("t_max", _c_int), ("pool_capacity", _c_int),
@@ -142,6 +146,10 @@ def lib() -> ctypes.CDLL:
         L.radar_expand_calls_workspace_bytes.argtypes = [_vp, _c_int, _c_int, _c_int, _c_int]
         L.radar_expand_calls.restype = _c_int
         L.radar_expand_calls.argtypes = [_vp, ctypes.POINTER(ExpandCallsArgs), _vp]
+        L.radar_expand_range_workspace_bytes.restype = _sz
+        L.radar_expand_range_workspace_bytes.argtypes = [_vp, _c_int, _c_int, _c_int, _c_int, _c_int]
+        L.radar_expand_range.restype = _c_int
+        L.radar_expand_range.argtypes = [_vp, ctypes.POINTER(ExpandRangeArgs), _vp]
         L.radar_expand_step.restype = _c_int
         L.radar_expand_step.argtypes = [_vp, ctypes.POINTER(ExpandArgs), _vp]
         L.radar_rerank_build_tree.restype = _c_int
@@ -369,6 +377,22 @@ def radar_expand_calls(ctx: Context, *, logits, gate, workspace, stream=None, **
     for n in _GATE:
         kw[n] = gate.get(n)
     _expand_calls(ctx, stream, kw)
+
+
+_expand_range = _Call("radar_expand_range", ExpandRangeArgs, _expand_calls.dtypes, _expand_calls.optional)
+
+
+def radar_expand_range_workspace_bytes(ctx: Context, B, V, k, t_first, t_last) -> int:
+    return int(lib().radar_expand_range_workspace_bytes(ctx.handle, B, V, k, t_first, t_last))
+
+
+def radar_expand_range(ctx: Context, *, t_first, t_last, logits, gate, workspace, stream=None, **kw):
+    """Calls t_first .. t_last of a step; the other arguments are those of radar_expand_calls."""
+    kw.update(logits=logits, logits_dtype=dtype_code(logits), F=1, t=1, t_first=t_first, t_last=t_last, workspace=workspace,
+              workspace_bytes=workspace.numel() * workspace.element_size())
+    for n in _GATE:
+        kw[n] = gate.get(n)
+    _expand_range(ctx, stream, kw)
 
 
 _tree = _Call(

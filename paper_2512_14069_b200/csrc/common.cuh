@@ -11,8 +11,8 @@
 
 // kernels the library launches (index into the profiling tables)
 enum radar_kernel_id {
-    RADAR_K_VOCAB_EXPAND = 0,   // vocabulary pass of radar_expand_step
-    RADAR_K_SELECT_GATE,        // partial merge + frontier selection + prediction model
+    RADAR_K_VOCAB_EXPAND = 0,   // expansion: top-k and log-normaliser of every row
+    RADAR_K_SELECT_GATE,        // frontier selection + prediction model
     RADAR_K_TREE_BUILD,
     RADAR_K_ATTN,               // tree attention main kernel
     RADAR_K_ATTN_COMBINE,
@@ -25,7 +25,7 @@ enum radar_kernel_id {
     RADAR_K_TRAIN_ROLLOUT,      // REINFORCE step: rollout + backpropagation through time per data point
     RADAR_K_TRAIN_OUTER,        // REINFORCE step: parameter gradients
     RADAR_K_TRAIN_ADAM,         // REINFORCE step: batch loss + Adam update
-    RADAR_K_ROW_MERGE,          // radar_expand_calls: chunk records -> top-k of every row
+    RADAR_K_ROW_MERGE,          // expansion: the merge of a long pass's rows
     RADAR_K_EXPAND_CALLS,       // radar_expand_calls: the calls of a sequence in one kernel
     RADAR_K_COUNT
 };
@@ -224,33 +224,52 @@ struct WarpTopList {
     __device__ __forceinline__ int index_at(int lane) const { return __shfl_sync(kFull, i, lane); }
 };
 
-// --- vocabulary pass (vocab_pass.cu) ------------------------------------------------------
-// One launch reduces every (row, chunk) of a [rows][V] logits matrix to a partial record:
-//   topv/topi [k] best (logit, token) of the chunk, sorted; m = max logit; s = sum exp(logit - m).
+// --- best logit of every row (vocab_pass.cu) ----------------------------------------------
+// One launch reduces every (row, chunk) of a [rows][V] logits matrix to its best (logit, token).
 // rows are addressed as base + seq * seq_stride + f * row_stride with row = seq * F + f; rows whose
-// sequence has skip[seq] == 0 (if skip != NULL) or whose index within the sequence is >= nrows[seq]
-// (if nrows != NULL) are not read.
+// index within the sequence is >= nrows[seq] are not read.
 struct VocabPassParams {
     const void* logits;
     int dtype;
     int64_t row_stride, seq_stride;
-    int n_seq, F, V, k;
+    int n_seq, F, V;
     int n_chunks, chunk;             // chunk = elements per chunk (multiple of 8)
-    int want_lse;                    // 0: top-k only (argmax pass), 1: also (m, s)
-    const uint8_t* seq_active;       // or NULL
-    const int32_t* seq_rows;         // or NULL: rows to process per sequence
-    float* part_v;                   // [rows][n_chunks][k]
-    int32_t* part_i;                 // [rows][n_chunks][k]
-    float* part_m;                   // [rows][n_chunks]
-    float* part_s;                   // [rows][n_chunks]
-    int* status;                     // NULL (with want_lse): a NaN logit is left in part_m for the merge to report
+    const int32_t* seq_rows;         // rows to process per sequence
+    float* part_v;                   // [rows][n_chunks]
+    int32_t* part_i;                 // [rows][n_chunks]
+    int* status;
 };
 int vocab_pass_plan_chunks(int sm_count, int rows, int V, int* chunk_out);   // returns n_chunks
-size_t vocab_pass_partial_bytes(int rows, int n_chunks, int k);
-size_t vocab_pass_workspace_bytes(int sm_count, int rows, int V, int k);       // for up to `rows` rows
-void vocab_pass_carve(void* ws, int rows, int n_chunks, int k, VocabPassParams* p);
-cudaError_t vocab_pass_launch(radar_ctx* ctx, int kernel_id, const VocabPassParams& p, cudaStream_t stream);
+size_t vocab_pass_partial_bytes(int rows, int n_chunks);
+size_t vocab_pass_workspace_bytes(int sm_count, int rows, int V);       // for up to `rows` rows
+void vocab_pass_carve(void* ws, int rows, int n_chunks, VocabPassParams* p);
+cudaError_t vocab_pass_launch(radar_ctx* ctx, const VocabPassParams& p, cudaStream_t stream);
 cudaError_t vocab_pass_preload_argbest();
+
+// --- top-k and log-normaliser of rows (row_topk.cu) ------------------------------------------
+// Rows as above; those of sequences with seq_active[seq] == 0 (if not NULL) are not read.
+struct RowTopkParams {
+    const void* logits;
+    int dtype;
+    int64_t row_stride, seq_stride;
+    int n_seq, F, V, k;
+    const uint8_t* seq_active;
+    int32_t* tok;                    // [rows][k] in the workspace: tokens in order (kNanRow set where the row has a NaN),
+    double* logp;                    // [rows][k] and their log-probabilities
+    int spans, n_slots, lines;       // shares of a row, warps that go through them, and how many a warp has at most
+    int live, per;                   // the merge's bound: warps that have maxima, and how many of each it looks at
+    float* gmax;                     // [rows][n_slots][32]: largest logit of every group of a warp's
+    float2* part;                    // [rows][n_slots]: (max, sum exp(logit - max)); max is NaN if there is one
+    int* status;
+};
+constexpr int32_t kNanRow = INT32_MIN;
+size_t row_topk_workspace_bytes(int rows, int V, int k);
+void row_topk_carve(RowTopkParams& p, void* ws);      // sets what follows seq_active, from the rest
+cudaError_t row_topk_launch(radar_ctx* ctx, RowTopkParams p, cudaStream_t stream);
+
+// --- hidden-state policy (expand.cu) -----------------------------------------------------------
+// Input-side products of the a.B rows of a.features: pre [B][4H] = W_ih f, and behind it [B][H] = W_1[:, H:] f.
+cudaError_t gate_features_launch(radar_ctx* ctx, const radar_expand_args& a, float* pre, cudaStream_t stream);
 
 // --- workspace-free greedy acceptance (verify_accept.cu) --------------------------------------
 // Resolves the device address of the library's scratch array on the current device and loads the two kernels of

@@ -990,7 +990,7 @@ static cudaError_t launch_walk(radar_ctx* ctx, StochParams& sp, int cs, cudaStre
 
 extern "C" size_t radar_accept_workspace_bytes(const radar_ctx* ctx, int B, int V, int mode) {
     if (!ctx || B <= 0 || V <= 0) return 0;
-    if (mode == RADAR_GREEDY) return vocab_pass_workspace_bytes(ctx->sm_count, B * kMaxNodes, V, 1);
+    if (mode == RADAR_GREEDY) return vocab_pass_workspace_bytes(ctx->sm_count, B * kMaxNodes, V);
     return align_up((size_t)B * cache_stride(V) * sizeof(double), 256) * 2;
 }
 
@@ -1018,15 +1018,12 @@ extern "C" int radar_verify_accept(radar_ctx* ctx, const radar_accept_args* a, v
         vp.n_seq = a->B;
         vp.F = kMaxNodes;
         vp.V = a->V;
-        vp.k = 1;
         vp.n_chunks = vocab_pass_plan_chunks(ctx->sm_count, a->B * kMaxNodes, a->V, &vp.chunk);
-        vp.want_lse = 0;
-        vp.seq_active = nullptr;
         vp.seq_rows = a->n_nodes;
         vp.status = ctx->d_status;
-        if (vocab_pass_partial_bytes(a->B * kMaxNodes, vp.n_chunks, 1) > a->workspace_bytes) return RADAR_ERR_WORKSPACE;
-        vocab_pass_carve(a->workspace, a->B * kMaxNodes, vp.n_chunks, 1, &vp);
-        RADAR_CUDA_CHECK(vocab_pass_launch(ctx, RADAR_K_VOCAB_ACCEPT, vp, stream));
+        if (vocab_pass_partial_bytes(a->B * kMaxNodes, vp.n_chunks) > a->workspace_bytes) return RADAR_ERR_WORKSPACE;
+        vocab_pass_carve(a->workspace, a->B * kMaxNodes, vp.n_chunks, &vp);
+        RADAR_CUDA_CHECK(vocab_pass_launch(ctx, vp, stream));
         {
             radar_launch_scope scope(ctx, RADAR_K_GREEDY_WALK, stream);
             RADAR_CUDA_CHECK(launch_chained(greedy_walk_kernel, dim3(a->B), dim3(kGreedyThreads), 0, stream, gp));
@@ -1197,7 +1194,7 @@ extern "C" int radar_verify_accept_greedy_noalloc(radar_ctx* ctx, const radar_ac
     int chunk = 0;
     const int n_chunks = vocab_pass_plan_chunks(ctx->sm_count, a->B * kMaxNodes, a->V, &chunk);
     if ((long long)a->B * kMaxNodes > 0x7fffffff / (n_chunks > 0 ? n_chunks : 1)) return RADAR_ERR_UNSUPPORTED;
-    if (vocab_pass_partial_bytes(a->B * kMaxNodes, n_chunks, 1) > kNoAllocScratchBytes) return RADAR_ERR_UNSUPPORTED;
+    if (2 * vocab_pass_partial_bytes(a->B * kMaxNodes, n_chunks) > kNoAllocScratchBytes) return RADAR_ERR_UNSUPPORTED;     // 16 bytes a record: the documented limit
     if (!a->target_logits || !a->tree_tok || !a->tree_parent || !a->n_nodes || !a->retrieve || !a->n_leaves ||
         !a->accept_len || !a->path_nodes || !a->path_tokens || !a->next_token || !a->best_retrieve_row)
         return RADAR_ERR_INVALID_ARG;
@@ -1228,15 +1225,12 @@ extern "C" int radar_verify_accept_greedy_noalloc(radar_ctx* ctx, const radar_ac
     vp.n_seq = a->B;
     vp.F = kMaxNodes;
     vp.V = a->V;
-    vp.k = 1;
     vp.n_chunks = n_chunks;
     vp.chunk = chunk;
-    vp.want_lse = 0;
-    vp.seq_active = nullptr;
     vp.seq_rows = a->n_nodes;
     vp.status = ctx->d_status;
-    vocab_pass_carve(scratch, a->B * kMaxNodes, n_chunks, 1, &vp);
-    RADAR_CUDA_CHECK(vocab_pass_launch(ctx, RADAR_K_VOCAB_ACCEPT, vp, stream));
+    vocab_pass_carve(scratch, a->B * kMaxNodes, n_chunks, &vp);
+    RADAR_CUDA_CHECK(vocab_pass_launch(ctx, vp, stream));
     {
         radar_launch_scope scope(ctx, RADAR_K_GREEDY_WALK, stream);
         RADAR_CUDA_CHECK(launch_chained(greedy_walk_kernel, dim3(a->B), dim3(kGreedyThreads), 0, stream, gp));

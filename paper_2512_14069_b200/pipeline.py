@@ -9,11 +9,11 @@ attention, acceptance.  Which form the expansion calls take is a matter of when 
   `expand(t, ...)`, or `run_expansion(pipelined=False)`: one call behind the other.  The form of a decoding loop, whose
       draft model runs on the frontier of call t before the logits of call t + 1 are there.
   `run_expansion(pipelined=True)`: for logits that are all there before call 1 (recorded ones, gathering training data for
-      the gate, a draft model that does not look at the frontier).  With short passes all calls go in one go
-      (`radar_expand_calls`); with long ones, and for the hidden-state policy, as two overlapping chains: the
-      bandwidth-bound vocabulary passes run ahead on a side stream while the latency-bound select + gate blocks follow
-      on the main stream (the pass of call t+1 skips the sequences that had stopped before call t; one that stops at
-      call t is read once in vain).
+      the gate, a draft model that does not look at the frontier).  Several calls go in one go (`radar_expand_range`): all
+      of them with short passes, a few at a time with long ones.  Batches too large for that, and features that do not lie
+      in one piece, run as two overlapping chains: the bandwidth-bound vocabulary passes ahead on a side stream, the
+      merge + select + gate kernels behind them on the main stream (the pass of call t+1 skips the sequences that had
+      stopped before call t; one that stops at call t is read once in vain).
 
 It contains no arithmetic of the method.
 """
@@ -22,6 +22,23 @@ from __future__ import annotations
 import torch
 
 from . import binding as rb
+
+
+def _ranges(t_max, call_bytes):
+    """The draft calls that are made in one go.  A range costs three launches, some 12 us; a call that is read and not
+    made, its logits.  So with short passes (a call's rows of 24 MB take 4 us) up to eight calls go together, then up to
+    four, and beyond 48 MB two and then about three at a time.  us for 1, 4, 5 to 7 and 8 calls, t_max = 8, V = 128256, k = 10:
+        B = 4   two chains 29 / 58 / 83 / 89     8: 35 / 44 / 51 / 52     4, 4: 28 / 35 / 65 / 66     2, 3, 3: 24 / 52 / 74 / 77
+        B = 8              38 / 74 / 101 / 114      55 / 64 / 71 / 73           41 / 48 / 85 / 87              32 / 67 / 86 / 99
+        B = 32             91 / 200 / 278 / 318     195 / 204 / 212 / 212      117 / 124 / 221 / 220           79 / 155 / 210 / 231
+    (two chains: the calls one by one, the passes ahead on a second stream, as they were before there were ranges)."""
+    first = 0 if call_bytes <= 48 << 20 else 2
+    most = 8 if call_bytes <= 24 << 20 else 4
+    left = t_max - min(first, t_max)
+    n = -(-left // most) if not first else max(round(left / 3), 1) if left else 0
+    sizes = ([min(first, t_max)] if first else []) + [left // n + (i < left % n) for i in range(n)]
+    ends = [sum(sizes[:i + 1]) for i in range(len(sizes))]
+    return [(e - x + 1, e) for x, e in zip(sizes, ends)]
 
 
 class SpecStep:
@@ -71,6 +88,9 @@ class SpecStep:
         self.ws_expand = z((wb + 255,), u8)
         self.ws_expand2 = z((wb + 255,), u8)          # consecutive calls alternate, so a pass can run ahead of the select
         cb = rb.radar_expand_calls_workspace_bytes(ctx, B, V, k, t_max)
+        self.ranges = [(1, t_max)] if cb else _ranges(t_max, B * k * V * logits_dtype.itemsize)
+        sizes = [rb.radar_expand_range_workspace_bytes(ctx, B, V, k, *r) for r in self.ranges]
+        cb = max(sizes) if min(sizes) else 0
         self.ws_calls = z((cb + 255,), u8) if cb else None      # None: the calls are issued one by one
         self.ws_attn = z((rb.radar_attn_workspace_bytes(ctx, B, Hq, Hkv, d, rb.dtype_code(self.O), max_prefix_len) + 255,), u8)
         self.ws_accept = z((rb.radar_accept_workspace_bytes(ctx, B, V, mode) + 255,), u8)
@@ -120,8 +140,12 @@ class SpecStep:
                       pipelined=True):
         """All draft calls of a step on draft_logits [B,R,V].  `pipelined` needs the rows of all calls before the first one
         (see the top of this file); without it call t reads its own rows only."""
-        if pipelined and self.ws_calls is not None and policy != rb.RADAR_POLICY_LSTM_HIDDEN:
-            self._expand_calls(draft_logits, gate, force_calls, policy)
+        together = self.ws_calls is not None
+        if policy == rb.RADAR_POLICY_LSTM_HIDDEN and self.t_max > 1:          # all calls' features in one piece
+            together = together and torch.is_tensor(features) and features.is_contiguous() and features.dim() == 3 and \
+                features.shape[0] >= self.t_max - 1 and features.shape[1] == self.B
+        if pipelined and together:
+            self._expand_calls(draft_logits, gate, force_calls, policy, features)
             return
         slots = self._slots()
         if not pipelined:
@@ -150,10 +174,10 @@ class SpecStep:
             sel_done[t].record(main)
         main.wait_stream(side)                      # join (the last pass has been waited for already)
 
-    def _expand_calls(self, draft_logits, gate, force_calls, policy):
+    def _expand_calls(self, draft_logits, gate, force_calls, policy, features):
         more = self.t_max > 1
-        rb.radar_expand_calls(
-            self.ctx, B=self.B, V=self.V, k=self.k, t_max=self.t_max, logits=draft_logits, logits_row_stride=self.V,
+        kw = dict(
+            B=self.B, V=self.V, k=self.k, t_max=self.t_max, logits=draft_logits, logits_row_stride=self.V,
             logits_seq_stride=self.R * self.V, parent_score=self.root_score, parent_pool_idx=self.root_pool_idx, active=self.active,
             force_calls=force_calls, gate=gate, h=self.h, c=self.c, pool_capacity=self.C, pool_tok=self.pool_tok,
             pool_parent=self.pool_parent, pool_depth=self.pool_depth, pool_draft_row=self.pool_draft_row, pool_score=self.pool_score,
@@ -162,6 +186,10 @@ class SpecStep:
             topk_logp=self.topk_logp1, topk_tok_next=self.topk_tok[1:] if more else None,
             topk_logp_next=self.topk_logp[1:] if more else None, gate_logits=self.gate_logits, cont=self.cont_hist, policy=policy,
             workspace=self.ws_calls)
+        if policy == rb.RADAR_POLICY_LSTM_HIDDEN and more:
+            kw.update(features=features, feat_dim=features.shape[-1])
+        for first, last in self.ranges:
+            rb.radar_expand_range(self.ctx, t_first=first, t_last=last, **kw)
 
     # ---- tree, attention, acceptance ------------------------------------------------------
     def build_tree(self, root_tok, prefix_len, n_keep=None):
