@@ -61,12 +61,24 @@ struct TrainParams {
 };
 
 __device__ __forceinline__ float sigmoidf(float v) { return 1.f / (1.f + __expf(-v)); }
+__device__ __forceinline__ void copy4(float* smem, const float* gmem) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"((uint32_t)__cvta_generic_to_shared(smem)), "l"(gmem) : "memory");
+}
+__device__ __forceinline__ void copy16(float* smem, const float* gmem) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(smem)), "l"(gmem) : "memory");
+}
+__device__ __forceinline__ void copies_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int kLeft>
+__device__ __forceinline__ void copies_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(kLeft) : "memory"); }
 __device__ __forceinline__ float softplusf(float v) { return v > 0.f ? v + log1pf(expf(-v)) : log1pf(expf(v)); }
 
 // A block takes kP data points side by side.  What bounds it is the way of the weights from L2 into the SM (256 KB of W_hh
 // and 70 KB of W_1 for every decision, forwards and backwards, 64 B a clock) and the latency of that way: the points of
 // a block share every weight that is loaded, and a thread has eight or more loads of a product in flight.  With one point
 // a block, a row at a time and five shuffles a row, n = 148 took 134 us and n = 1024 332; now 65 and 139.
+// W_1, W_ih, the states and the uniform numbers are in shared memory before the first decision, so that W_hh is all that is
+// read again for every one (and not for the first: its h is zero).  Whole step, us, before / after: 256 points that
+// make one call 31.2 / 27.0, 64 points of two calls on average 76.9 / 68.5, 1024 of them 211 / 205.
 template <int kP>
 __global__ void __launch_bounds__(kTrainThreads, 1) train_rollout_kernel(const TrainParams P) {
     chain_wait();
@@ -77,10 +89,29 @@ __global__ void __launch_bounds__(kTrainThreads, 1) train_rollout_kernel(const T
     __shared__ __align__(16) float sh[kP][H], sc[kP][H], sx[kP][kXPad], sg[kP][4 * H], shid[kP][H], sd1[kP][H], sdp[kP][4 * H], sdh[kP][H], sdc[kP][H];
     extern __shared__ __align__(16) float train_smem[];
     float (*spart)[kGroups][H] = reinterpret_cast<float (*)[kGroups][H]>(train_smem);      // [kP]
-    __shared__ float sy[kP][2], spi1[kP][kMaxSteps], sG[kP][kMaxSteps];
+    float* s_w1 = train_smem + kP * kGroups * H;         // [H][H + k]
+    float* s_wih = s_w1 + H * (H + k);                   // [4H][k]
+    float* s_state = s_wih + 4 * H * k;                  // [kP][t_max - 1][k] log states
+    __shared__ float sy[kP][2], spi1[kP][kMaxSteps], sG[kP][kMaxSteps], s_u[kP][kMaxSteps];
+    __shared__ double s_dist[kP][kMaxSteps + 1];
     __shared__ int sact[kP][kMaxSteps], sT[kP], sndec[kP], s_going[kP];
+    // What every decision needs, once: the head's and the input's weights, all states, the uniform numbers.  (Fetched where they are
+    // used, each is a wait of a microsecond in the chain of every decision.)
+    for (int e = tid; e < 4 * H * k / 4; e += kTrainThreads) copy16(s_wih + 4 * e, W.w_ih + 4 * e);
+    for (int e = tid; e < kP * (t_max - 1) * k; e += kTrainThreads) {
+        const int p = e / ((t_max - 1) * k), r = e % ((t_max - 1) * k);
+        if (j0 + p < n) copy4(s_state + e, a.log_states + ((size_t)(r / k) * n + j0 + p) * k + r % k);
+    }
+    for (int e = tid; e < kP * (t_max - 1); e += kTrainThreads) {
+        const int p = e / (t_max - 1), r = e % (t_max - 1);
+        if (j0 + p < n) copy4(&s_u[p][r], a.u_action + (size_t)(j0 + p) * t_max + r);
+    }
+    copies_commit();
+    for (int e = tid; e < H * (H + k) / 4; e += kTrainThreads) copy16(s_w1 + 4 * e, W.w1 + 4 * e);
+    copies_commit();
     for (int e = tid; e < kP * H; e += kTrainThreads) { (&sh[0][0])[e] = 0.f; (&sc[0][0])[e] = 0.f; }
     if (tid < kP) { s_going[tid] = j0 + tid < n; sT[tid] = t_max; sndec[tid] = 0; }
+    copies_wait<1>();                                    // all but the head's weights
     __syncthreads();
     auto record = [&](int p, int s) { return P.rec + ((size_t)(j0 + p) * (t_max - 1) + s) * R_STRIDE; };
 
@@ -92,7 +123,7 @@ __global__ void __launch_bounds__(kTrainThreads, 1) train_rollout_kernel(const T
         if (!any) break;
         for (int e = tid; e < kP * kXPad; e += kTrainThreads) {
             const int p = e / kXPad, c = e % kXPad;
-            sx[p][c] = c < k && going[p] ? __expf(a.log_states[((size_t)(t - 1) * n + j0 + p) * k + c]) : 0.f;
+            sx[p][c] = c < k && going[p] ? __expf(s_state[(p * (t_max - 1) + t - 1) * k + c]) : 0.f;
         }
         for (int e = tid; e < kP * H; e += kTrainThreads) {
             const int p = e / H, c = e % H;
@@ -109,19 +140,32 @@ __global__ void __launch_bounds__(kTrainThreads, 1) train_rollout_kernel(const T
 #pragma unroll
         for (int half = 0; half < 2; ++half) {
             const int r0 = warp * 32 + half * 16;
+            const float* wx = s_wih + r0 * k + lane;
+            if (t == 1) {                                     // the state before the first call is zero
+#pragma unroll
+                for (int p = 0; p < kP; ++p) {
+                    const float x = sx[p][lane];
+                    float v[16];
+#pragma unroll
+                    for (int i = 0; i < 16; ++i) v[i] = lane < k ? wx[i * k] * x : 0.f;
+                    const float sum = transposed_sum<16>(v);
+                    if ((lane & 1) == half) mine[p] = sum;
+                }
+                continue;
+            }
             float4 w[16];
-            float wx[16];
 #pragma unroll
             for (int i = 0; i < 16; ++i) w[i] = *reinterpret_cast<const float4*>(W.w_hh + (size_t)(r0 + i) * H + 4 * lane);
+            float wr[16];
 #pragma unroll
-            for (int i = 0; i < 16; ++i) wx[i] = lane < k ? W.w_ih[(size_t)(r0 + i) * k + lane] : 0.f;
+            for (int i = 0; i < 16; ++i) wr[i] = lane < k ? wx[i * k] : 0.f;
 #pragma unroll
             for (int p = 0; p < kP; ++p) {
                 const float4 h4 = *reinterpret_cast<const float4*>(&sh[p][4 * lane]);
                 const float x = sx[p][lane];
                 float v[16];
 #pragma unroll
-                for (int i = 0; i < 16; ++i) v[i] = fmaf(wx[i], x, w[i].x * h4.x + w[i].y * h4.y + w[i].z * h4.z + w[i].w * h4.w);
+                for (int i = 0; i < 16; ++i) v[i] = fmaf(wr[i], x, w[i].x * h4.x + w[i].y * h4.y + w[i].z * h4.z + w[i].w * h4.w);
                 const float sum = transposed_sum<16>(v);
                 if ((lane & 1) == half) mine[p] = sum;
             }
@@ -153,13 +197,14 @@ __global__ void __launch_bounds__(kTrainThreads, 1) train_rollout_kernel(const T
                 rec[R_CAT + c] = sx[p][c - H];
             }
         }
+        if (t == 1) copies_wait<0>();
         __syncthreads();
         // head: warp w owns hidden rows 8 w .. 8 w + 7
         {
             float w[8][4], wx[8];
 #pragma unroll
             for (int i = 0; i < 8; ++i) {
-                const float* wr = W.w1 + (size_t)(warp * 8 + i) * (H + k);
+                const float* wr = s_w1 + (warp * 8 + i) * (H + k);
 #pragma unroll
                 for (int c = 0; c < 4; ++c) w[i][c] = wr[lane + 32 * c];
                 wx[i] = lane < k ? wr[H + lane] : 0.f;
@@ -195,7 +240,7 @@ __global__ void __launch_bounds__(kTrainThreads, 1) train_rollout_kernel(const T
             const int p = tid;
             const float d = sy[p][1] - sy[p][0];
             const float pi1 = 1.f / (1.f + expf(-d));
-            const int act = a.u_action[(size_t)(j0 + p) * t_max + (t - 1)] < pi1 ? 1 : 0;
+            const int act = s_u[p][t - 1] < pi1 ? 1 : 0;
             spi1[p][t - 1] = pi1;
             sact[p][t - 1] = act;
             sG[p][t - 1] = act ? -softplusf(-d) : -softplusf(d);       // log pi(a_t) for now
@@ -205,11 +250,13 @@ __global__ void __launch_bounds__(kTrainThreads, 1) train_rollout_kernel(const T
         __syncthreads();
     }
     __syncthreads();
+    if (warp < kP && j0 + warp < n && lane <= t_max) s_dist[warp][lane] = a.dists[((size_t)(sT[warp] - 1) * n + j0 + warp) * (t_max + 1) + lane];
+    __syncthreads();
 
     // ---- acceptance length, reward, returns, loss (one thread per point, fp64) ----
     if (tid < kP && j0 + tid < n) {
         const int p = tid, j = j0 + p, T = sT[p], ndec = sndec[p];
-        const double* drow = a.dists + ((size_t)(T - 1) * n + j) * (t_max + 1);
+        const double* drow = s_dist[p];
         double total = 0.0;
         for (int i = 0; i <= t_max; ++i) total += drow[i];
         const double target = (double)a.u_length[j] * total;
@@ -246,7 +293,17 @@ __global__ void __launch_bounds__(kTrainThreads, 1) train_rollout_kernel(const T
 
     // ---- backpropagation through time (a point joins at its own last decision) ----
     const int q = tid >> 7, col = tid & (H - 1);
+    static_assert(kP * H <= kTrainThreads, "one unit of one point to a thread");
     for (int s = steps - 1; s >= 0; --s) {
+        // what the cell's derivative takes from the record, on its way while the head's is worked out
+        const int up = tid / H, uc = tid % H;
+        const bool mine = up < kP && s < sndec[up < kP ? up : 0];
+        float gi = 0.f, gf = 0.f, gg = 0.f, go = 0.f, cell = 0.f, cell_before = 0.f;
+        if (mine) {
+            const float* rec = record(up, s);
+            gi = rec[R_GATES + uc]; gf = rec[R_GATES + H + uc]; gg = rec[R_GATES + 2 * H + uc]; go = rec[R_GATES + 3 * H + uc];
+            cell = rec[R_C + uc]; cell_before = rec[R_CPREV + uc];
+        }
         for (int e = tid; e < kP * H; e += kTrainThreads) {
             const int p = e / H, c = e % H;
             float v = 0.f;
@@ -269,7 +326,7 @@ __global__ void __launch_bounds__(kTrainThreads, 1) train_rollout_kernel(const T
             for (int p = 0; p < kP; ++p) acc[p] = 0.f;
 #pragma unroll 16
             for (int r = q * 32; r < q * 32 + 32; ++r) {
-                const float w = W.w1[(size_t)r * (H + k) + col];
+                const float w = s_w1[r * (H + k) + col];
 #pragma unroll
                 for (int p = 0; p < kP; ++p) acc[p] += w * sd1[p][r];
             }
@@ -277,16 +334,15 @@ __global__ void __launch_bounds__(kTrainThreads, 1) train_rollout_kernel(const T
             for (int p = 0; p < kP; ++p) spart[p][q][col] = acc[p];
         }
         __syncthreads();
-        for (int e = tid; e < kP * H; e += kTrainThreads) {
-            const int p = e / H, c = e % H;
+        if (up < kP) {
+            const int p = up, c = uc;
             float di = 0.f, df = 0.f, dg = 0.f, dob = 0.f;
-            if (s < sndec[p]) {
+            if (mine) {
                 float* rec = record(p, s);
                 const float dh = spart[p][0][c] + spart[p][1][c] + spart[p][2][c] + spart[p][3][c] + sdh[p][c];
-                const float gi = rec[R_GATES + c], gf = rec[R_GATES + H + c], gg = rec[R_GATES + 2 * H + c], go = rec[R_GATES + 3 * H + c];
-                const float tc = tanhf(rec[R_C + c]);
+                const float tc = tanhf(cell);
                 const float dc = dh * go * (1.f - tc * tc) + sdc[p][c];
-                di = dc * gg * gi * (1.f - gi); df = dc * rec[R_CPREV + c] * gf * (1.f - gf);
+                di = dc * gg * gi * (1.f - gi); df = dc * cell_before * gf * (1.f - gf);
                 dg = dc * gi * (1.f - gg * gg); dob = dh * tc * go * (1.f - go);
                 rec[R_DPRE + c] = di; rec[R_DPRE + H + c] = df; rec[R_DPRE + 2 * H + c] = dg; rec[R_DPRE + 3 * H + c] = dob;
                 sdc[p][c] = dc * gf;
@@ -327,6 +383,7 @@ __global__ void __launch_bounds__(kTrainThreads, 1) train_rollout_kernel(const T
 // out[m][c] = scale * sum over valid records of A[rec][m] * B[rec][c]   (B absent: a column of ones)
 struct OuterJob {
     int a_off, M, b_off, N;     // offsets into a record; b_off < 0: ones
+    int first;                  // first decision whose record counts (1: B is zero before the first call)
     int ld_out;                 // row stride of the output (N for matrices, 1 for vectors)
     long long out_off, out_off2;   // offsets into grad (out_off2 >= 0: a second copy, for the two LSTM biases)
 };
@@ -360,7 +417,7 @@ __global__ void __launch_bounds__(256) train_outer_kernel(const OuterParams P) {
     for (int p0 = (int)((long long)P.n * blockIdx.y / kSlices); p0 < p_end; p0 += 256) {
         // list of the records of points p0 .. p0 + 255
         const int pt = p0 + threadIdx.x;
-        const int mine = pt < p_end ? P.ndec[pt] : 0;
+        const int mine = pt < p_end ? max(P.ndec[pt] - J.first, 0) : 0;
         int incl = mine;
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
@@ -376,7 +433,7 @@ __global__ void __launch_bounds__(256) train_outer_kernel(const OuterParams P) {
             if (w < ty) at += s_sum[w];
             total += s_sum[w];
         }
-        for (int s = 0; s < mine; ++s) s_rec[at + s] = pt * P.steps + s;
+        for (int s = 0; s < mine; ++s) s_rec[at + s] = pt * P.steps + J.first + s;
         __syncthreads();
         for (int r0 = 0; r0 < total; r0 += 32) {
             // stage 32 records x 32 columns of each operand (past the list and past the edge: zero)
@@ -414,8 +471,8 @@ __global__ void __launch_bounds__(256) train_outer_kernel(const OuterParams P) {
 __global__ void __launch_bounds__(256) train_adam_kernel(const TrainParams P, size_t count) {
     chain_wait();
     const radar_train_args& a = P.a;
-    if (blockIdx.x == 0) {
-        // batch loss: fixed-order sum
+    if (blockIdx.x == gridDim.x - 1) {
+        // the last block: batch loss, a fixed-order sum
         __shared__ double part[256];
         double s = 0.0;
         for (int j = threadIdx.x; j < a.n; j += 256) s += (double)P.point_loss[j];
@@ -426,22 +483,28 @@ __global__ void __launch_bounds__(256) train_adam_kernel(const TrainParams P, si
             __syncthreads();
         }
         if (threadIdx.x == 0) a.loss[0] = (float)(part[0] / a.n);
+        return;
     }
     const float c1 = 1.f - powf(a.beta1, (float)max(a.step, 1)), c2 = 1.f - powf(a.beta2, (float)max(a.step, 1));
     const float scale = 1.f / (float)a.n;
-    for (size_t i = (size_t)blockIdx.x * 256 + threadIdx.x; i < count; i += (size_t)gridDim.x * 256) {
-        float g = 0.f;
+    const size_t i = (size_t)blockIdx.x * 256 + threadIdx.x;            // one parameter a thread: every load in flight at once
+    if (i >= count) return;
+    const bool update = a.step >= 1;
+    float part_sum[kSlices];
 #pragma unroll
-        for (int sl = 0; sl < kSlices; ++sl) g += P.part[(size_t)sl * count + i];
-        g *= scale;
-        a.grad[i] = g;
-        if (a.step < 1) continue;
-        const float m = a.beta1 * a.adam_m[i] + (1.f - a.beta1) * g;
-        const float v = a.beta2 * a.adam_v[i] + (1.f - a.beta2) * g * g;
-        a.adam_m[i] = m;
-        a.adam_v[i] = v;
-        a.theta[i] -= a.lr * (m / c1) / (sqrtf(v / c2) + a.eps);
-    }
+    for (int sl = 0; sl < kSlices; ++sl) part_sum[sl] = P.part[(size_t)sl * count + i];
+    const float m0 = update ? a.adam_m[i] : 0.f, v0 = update ? a.adam_v[i] : 0.f, theta = update ? a.theta[i] : 0.f;
+    float g = 0.f;
+#pragma unroll
+    for (int sl = 0; sl < kSlices; ++sl) g += part_sum[sl];
+    g *= scale;
+    a.grad[i] = g;
+    if (!update) return;
+    const float m = a.beta1 * m0 + (1.f - a.beta1) * g;
+    const float v = a.beta2 * v0 + (1.f - a.beta2) * g * g;
+    a.adam_m[i] = m;
+    a.adam_v[i] = v;
+    a.theta[i] = theta - a.lr * (m / c1) / (sqrtf(v / c2) + a.eps);
 }
 
 }  // namespace
@@ -491,15 +554,14 @@ extern "C" int radar_policy_train_step(radar_ctx* ctx, const radar_train_args* a
         //   n = 1024  220 / 207 / 212  308 / 281 / 275   552 / 450 / 370
         // A block lasts as long as its longest trajectory, so with short, mixed ones two points would do a little longer.
         const int kp = n <= sms ? 1 : n <= 2 * sms ? 2 : 4;
-        const size_t smem = (size_t)kp * kGroups * H * sizeof(float);
-        if (kp == 1) {
-            RADAR_CUDA_CHECK(launch_chained(train_rollout_kernel<1>, dim3(n), dim3(kTrainThreads), smem, stream, P));
-        } else if (kp == 2) {
-            RADAR_CUDA_CHECK(launch_chained(train_rollout_kernel<2>, dim3((n + 1) / 2), dim3(kTrainThreads), smem, stream, P));
-        } else {                                              // 30 KB static and 32 KB dynamic
-            RADAR_CUDA_CHECK(radar_opt_in_smem(ctx, RADAR_SMEM_TRAIN_ROLLOUT, train_rollout_kernel<4>, 64 * 1024));
-            RADAR_CUDA_CHECK(launch_chained(train_rollout_kernel<4>, dim3((n + 3) / 4), dim3(kTrainThreads), smem, stream, P));
-        }
+        const size_t smem = ((size_t)kp * kGroups * H + (size_t)H * (H + k) + (size_t)4 * H * k + (size_t)kp * (a->t_max - 1) * k) * sizeof(float);
+        auto launch = [&](int slot, auto kernel) {
+            const cudaError_t e = radar_opt_in_smem(ctx, RADAR_SMEM_TRAIN_ROLLOUT + slot, kernel, smem);
+            return e != cudaSuccess ? e : launch_chained(kernel, dim3((n + kp - 1) / kp), dim3(kTrainThreads), smem, stream, P);
+        };
+        if (kp == 1) RADAR_CUDA_CHECK(launch(0, train_rollout_kernel<1>));
+        else if (kp == 2) RADAR_CUDA_CHECK(launch(1, train_rollout_kernel<2>));
+        else RADAR_CUDA_CHECK(launch(2, train_rollout_kernel<4>));
     }
     {
         // offsets of the tensors inside theta / grad
@@ -507,13 +569,13 @@ extern "C" int radar_policy_train_step(radar_ctx* ctx, const radar_train_args* a
         const long long o_w1 = o_b_hh + 4 * H, o_b1 = o_w1 + (long long)H * (H + k), o_w2 = o_b1 + H, o_b2 = o_w2 + 2 * H;
         OuterParams O = {};
         O.rec = P.rec; O.ndec = P.ndec; O.part = P.part; O.count = (long long)param_count(k); O.n = a->n; O.steps = a->t_max - 1;
-        O.job[0] = {R_DPRE, 4 * H, R_CAT + H, k, k, o_w_ih, -1};            // w_ih: dpre (x) x
-        O.job[1] = {R_DPRE, 4 * H, R_HPREV, H, H, o_w_hh, -1};              // w_hh: dpre (x) h before the step
-        O.job[2] = {R_DPRE, 4 * H, -1, 1, 1, o_b_ih, o_b_hh};         // both LSTM biases
-        O.job[3] = {R_DPRE1, H, R_CAT, H + k, H + k, o_w1, -1};             // w1: dpre1 (x) [h; x]
-        O.job[4] = {R_DPRE1, H, -1, 1, 1, o_b1, -1};
-        O.job[5] = {R_DY, 2, R_HID, H, H, o_w2, -1};                        // w2: dy (x) relu output
-        O.job[6] = {R_DY, 2, -1, 1, 1, o_b2, -1};
+        O.job[0] = {R_DPRE, 4 * H, R_CAT + H, k, 0, k, o_w_ih, -1};            // w_ih: dpre (x) x
+        O.job[1] = {R_DPRE, 4 * H, R_HPREV, H, 1, H, o_w_hh, -1};              // w_hh: dpre (x) h before the step
+        O.job[2] = {R_DPRE, 4 * H, -1, 1, 0, 1, o_b_ih, o_b_hh};         // both LSTM biases
+        O.job[3] = {R_DPRE1, H, R_CAT, H + k, 0, H + k, o_w1, -1};             // w1: dpre1 (x) [h; x]
+        O.job[4] = {R_DPRE1, H, -1, 1, 0, 1, o_b1, -1};
+        O.job[5] = {R_DY, 2, R_HID, H, 0, H, o_w2, -1};                        // w2: dy (x) relu output
+        O.job[6] = {R_DY, 2, -1, 1, 0, 1, o_b2, -1};
         O.first[0] = 0;
         for (int x = 0; x < kJobs; ++x) O.first[x + 1] = O.first[x] + (O.job[x].M + 31) / 32 * ((O.job[x].N + 31) / 32);
         radar_launch_scope scope(ctx, RADAR_K_TRAIN_OUTER, stream);
@@ -522,7 +584,7 @@ extern "C" int radar_policy_train_step(radar_ctx* ctx, const radar_train_args* a
     {
         const size_t count = param_count(k);
         radar_launch_scope scope(ctx, RADAR_K_TRAIN_ADAM, stream);
-        RADAR_CUDA_CHECK(launch_chained(train_adam_kernel, dim3((unsigned)ctx->sm_count), dim3(256), 0, stream, P, count));
+        RADAR_CUDA_CHECK(launch_chained(train_adam_kernel, dim3((unsigned)((count + 255) / 256 + 1)), dim3(256), 0, stream, P, count));
     }
     return RADAR_OK;
 }
