@@ -380,14 +380,15 @@ __global__ void __launch_bounds__(kTrainThreads, 1) train_rollout_kernel(const T
     }
 }
 
-// out[m][c] = scale * sum over valid records of A[rec][m] * B[rec][c]   (B absent: a column of ones)
+// out[m][c] = sum over valid records of A[rec][m] * B[rec][c], c < N; column N of B is ones, and its sums are the biases'
 struct OuterJob {
-    int a_off, M, b_off, N;     // offsets into a record; b_off < 0: ones
+    int a_off, M, b_off, N;     // offsets into a record
     int first;                  // first decision whose record counts (1: B is zero before the first call)
-    int ld_out;                 // row stride of the output (N for matrices, 1 for vectors)
-    long long out_off, out_off2;   // offsets into grad (out_off2 >= 0: a second copy, for the two LSTM biases)
+    long long out_off;          // [M][N] in grad
+    long long bias_off[2];      // [M] each, or -1
 };
-constexpr int kJobs = 7;
+constexpr int kJobs = 4;
+constexpr int kTile = 64, kBatchRecs = 32;
 struct OuterParams {
     OuterJob job[kJobs];
     int first[kJobs + 1];       // first output tile of each job (and their number)
@@ -398,71 +399,91 @@ struct OuterParams {
     int n, steps;               // records per data point = t_max - 1
 };
 
-// Block (tile, slice): a 32 x 32 tile of one output, summed over the records of the slice's data points.  Only decisions that
-// were taken have a record, on average two of a point's t_max - 1: the block lists them first, 256 points at a time, and
-// goes through the list in batches of 32 (in the order of the points, so the sum does not depend on scheduling).  Visiting
-// every possible record cost 60 us at 256 points and 205 at 1024; the list 23 and 57.
+// Block (tile, slice): a 64 x 64 tile of one output, four by four to a thread, summed over the records of the slice's data points.
+// Only decisions that were taken have a record, on average two of a point's t_max - 1: the block lists them first, 256 points at a
+// time, and goes through the list in batches of 32 (in the order of the points, so the sum does not depend on
+// scheduling).  Visiting every possible record cost 60 us at 256 points and 205 at 1024; the list 23 and 57.  What bounds it is the
+// issue of instructions: with four products a thread, nine instructions for them, 32 x 32 tiles and the biases as
+// tiles of their own, 256 points of one / two calls took 12.8 / 21.0 us, now 10.7 / 13.5; 1024 points 31.3 / 50.5, now 19.8 / 29.2.
 __global__ void __launch_bounds__(256) train_outer_kernel(const OuterParams P) {
     chain_wait();
     int job = 0;
     while ((int)blockIdx.x >= P.first[job + 1]) ++job;
     const OuterJob J = P.job[job];
-    const int tile = blockIdx.x - P.first[job], tiles_x = (J.N + 31) / 32;
-    const int m0 = tile / tiles_x * 32, c0 = tile % tiles_x * 32;
-    __shared__ float As[32][33], Bs[32][33];
+    const int tile = blockIdx.x - P.first[job], columns = J.bias_off[0] >= 0 ? J.N + 1 : J.N, tiles_x = (columns + kTile - 1) / kTile;
+    const int m0 = tile / tiles_x * kTile, c0 = tile % tiles_x * kTile;
+    __shared__ __align__(16) float As[kBatchRecs][kTile], Bs[kBatchRecs][kTile];
     __shared__ int s_rec[256 * (kMaxSteps - 1)], s_sum[8];
-    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;     // 32 x 8
-    float acc[4] = {0.f, 0.f, 0.f, 0.f};
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, tx = tid & 15, ty = tid >> 4;
+    float acc[4][4] = {};
     const int p_end = (int)((long long)P.n * (blockIdx.y + 1) / kSlices);
     for (int p0 = (int)((long long)P.n * blockIdx.y / kSlices); p0 < p_end; p0 += 256) {
         // list of the records of points p0 .. p0 + 255
-        const int pt = p0 + threadIdx.x;
+        const int pt = p0 + tid;
         const int mine = pt < p_end ? max(P.ndec[pt] - J.first, 0) : 0;
         int incl = mine;
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
             const int v = __shfl_up_sync(kFull, incl, o);
-            if (tx >= o) incl += v;
+            if (lane >= o) incl += v;
         }
         __syncthreads();                                        // the previous list has been read
-        if (tx == 31) s_sum[ty] = incl;
+        if (lane == 31) s_sum[warp] = incl;
         __syncthreads();
         int at = incl - mine, total = 0;
 #pragma unroll
         for (int w = 0; w < 8; ++w) {
-            if (w < ty) at += s_sum[w];
+            if (w < warp) at += s_sum[w];
             total += s_sum[w];
         }
         for (int s = 0; s < mine; ++s) s_rec[at + s] = pt * P.steps + J.first + s;
         __syncthreads();
-        for (int r0 = 0; r0 < total; r0 += 32) {
-            // stage 32 records x 32 columns of each operand (past the list and past the edge: zero)
+        for (int r0 = 0; r0 < total; r0 += kBatchRecs) {
+            // 32 records x 64 columns of each operand; past the list zero, past the edges whatever the record holds there
+            // (those sums are not kept)
 #pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                const int e = ty + 8 * i;
-                const bool live = r0 + e < total;
-                const float* rec = P.rec + (size_t)(live ? s_rec[r0 + e] : 0) * R_STRIDE;
-                As[e][tx] = live && m0 + tx < J.M ? rec[J.a_off + m0 + tx] : 0.f;
-                Bs[e][tx] = live && c0 + tx < J.N ? (J.b_off < 0 ? 1.f : rec[J.b_off + c0 + tx]) : 0.f;
+            for (int i = 0; i < 2; ++i) {
+                const int e = ty + 16 * i;
+                float4 av = make_float4(0.f, 0.f, 0.f, 0.f), bv = av;
+                if (r0 + e < total) {
+                    const float* rec = P.rec + (size_t)s_rec[r0 + e] * R_STRIDE + 4 * tx;
+                    av = *reinterpret_cast<const float4*>(rec + J.a_off + m0);
+                    bv = *reinterpret_cast<const float4*>(rec + J.b_off + c0);
+                    const int one = J.N - c0 - 4 * tx;
+                    if (one == 0) bv.x = 1.f;
+                    if (one == 1) bv.y = 1.f;
+                    if (one == 2) bv.z = 1.f;
+                    if (one == 3) bv.w = 1.f;
+                }
+                *reinterpret_cast<float4*>(&As[e][4 * tx]) = av;
+                *reinterpret_cast<float4*>(&Bs[e][4 * tx]) = bv;
             }
             __syncthreads();
-#pragma unroll 8
-            for (int e = 0; e < 32; ++e) {
-                const float b = Bs[e][tx];
+            const int live = min(kBatchRecs, total - r0);
+#pragma unroll 4
+            for (int e = 0; e < live; ++e) {
+                const float4 av = *reinterpret_cast<const float4*>(&As[e][4 * ty]), bv = *reinterpret_cast<const float4*>(&Bs[e][4 * tx]);
+                const float x[4] = {av.x, av.y, av.z, av.w}, y[4] = {bv.x, bv.y, bv.z, bv.w};
 #pragma unroll
-                for (int i = 0; i < 4; ++i) acc[i] += As[e][ty + 8 * i] * b;
+                for (int i = 0; i < 4; ++i)
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) acc[i][j] += x[i] * y[j];
             }
             __syncthreads();
         }
     }
-    if (c0 + tx < J.N) {
+    float* out = P.part + (long long)blockIdx.y * P.count;
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            const int m = m0 + ty + 8 * i;
-            if (m < J.M) {
-                float* out = P.part + (long long)blockIdx.y * P.count;
-                out[J.out_off + (long long)m * J.ld_out + c0 + tx] = acc[i];
-                if (J.out_off2 >= 0) out[J.out_off2 + (long long)m * J.ld_out + c0 + tx] = acc[i];
+    for (int i = 0; i < 4; ++i) {
+        const int m = m0 + 4 * ty + i;
+        if (m >= J.M) break;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const int c = c0 + 4 * tx + j;
+            if (c < J.N) out[J.out_off + (long long)m * J.N + c] = acc[i][j];
+            if (c == J.N) {
+                if (J.bias_off[0] >= 0) out[J.bias_off[0] + m] = acc[i][j];
+                if (J.bias_off[1] >= 0) out[J.bias_off[1] + m] = acc[i][j];
             }
         }
     }
@@ -569,15 +590,16 @@ extern "C" int radar_policy_train_step(radar_ctx* ctx, const radar_train_args* a
         const long long o_w1 = o_b_hh + 4 * H, o_b1 = o_w1 + (long long)H * (H + k), o_w2 = o_b1 + H, o_b2 = o_w2 + 2 * H;
         OuterParams O = {};
         O.rec = P.rec; O.ndec = P.ndec; O.part = P.part; O.count = (long long)param_count(k); O.n = a->n; O.steps = a->t_max - 1;
-        O.job[0] = {R_DPRE, 4 * H, R_CAT + H, k, 0, k, o_w_ih, -1};            // w_ih: dpre (x) x
-        O.job[1] = {R_DPRE, 4 * H, R_HPREV, H, 1, H, o_w_hh, -1};              // w_hh: dpre (x) h before the step
-        O.job[2] = {R_DPRE, 4 * H, -1, 1, 0, 1, o_b_ih, o_b_hh};         // both LSTM biases
-        O.job[3] = {R_DPRE1, H, R_CAT, H + k, 0, H + k, o_w1, -1};             // w1: dpre1 (x) [h; x]
-        O.job[4] = {R_DPRE1, H, -1, 1, 0, 1, o_b1, -1};
-        O.job[5] = {R_DY, 2, R_HID, H, 0, H, o_w2, -1};                        // w2: dy (x) relu output
-        O.job[6] = {R_DY, 2, -1, 1, 0, 1, o_b2, -1};
+        O.job[0] = {R_DPRE, 4 * H, R_CAT + H, k, 0, o_w_ih, {o_b_ih, o_b_hh}};        // w_ih and both LSTM biases: dpre (x) [x; 1]
+        O.job[1] = {R_DPRE, 4 * H, R_HPREV, H, 1, o_w_hh, {-1, -1}};                  // w_hh: dpre (x) h before the step
+        O.job[2] = {R_DPRE1, H, R_CAT, H + k, 0, o_w1, {o_b1, -1}};                   // w1 and b1: dpre1 (x) [h; x; 1]
+        O.job[3] = {R_DY, 2, R_HID, H, 0, o_w2, {o_b2, -1}};                          // w2 and b2: dy (x) [relu output; 1]
         O.first[0] = 0;
-        for (int x = 0; x < kJobs; ++x) O.first[x + 1] = O.first[x] + (O.job[x].M + 31) / 32 * ((O.job[x].N + 31) / 32);
+        for (int x = 0; x < kJobs; ++x) {
+            const OuterJob& J = O.job[x];
+            const int columns = J.bias_off[0] >= 0 ? J.N + 1 : J.N;
+            O.first[x + 1] = O.first[x] + (J.M + kTile - 1) / kTile * ((columns + kTile - 1) / kTile);
+        }
         radar_launch_scope scope(ctx, RADAR_K_TRAIN_OUTER, stream);
         RADAR_CUDA_CHECK(launch_chained(train_outer_kernel, dim3((unsigned)O.first[kJobs], kSlices), dim3(256), 0, stream, O));
     }
