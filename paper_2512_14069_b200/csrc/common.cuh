@@ -40,8 +40,8 @@ enum radar_smem_slot {
     RADAR_SMEM_TRAIN_ROLLOUT,   // + log2 of the points a block
     RADAR_SMEM_WALK = RADAR_SMEM_TRAIN_ROLLOUT + 3,            // + 2 * (bf16) + CTAs per SM - 1
     RADAR_SMEM_ACCLEN = RADAR_SMEM_WALK + 4,        // the same
-    RADAR_SMEM_ATTN_FMA = RADAR_SMEM_ACCLEN + 4,        // + 2 * (bf16) + (d == 128)
-    RADAR_SMEM_ATTN_TC = RADAR_SMEM_ATTN_FMA + 4,   // + 8 * fine + 4 * (d == 128) + 2 * two + paged
+    RADAR_SMEM_ATTN_FMA = RADAR_SMEM_ACCLEN + 4,        // + 4 * (bf16) + 2 * (d == 128) + (clusters)
+    RADAR_SMEM_ATTN_TC = RADAR_SMEM_ATTN_FMA + 8,   // + 8 * fine + 4 * (d == 128) + 2 * two + paged
     RADAR_SMEM_COUNT = RADAR_SMEM_ATTN_TC + 16
 };
 

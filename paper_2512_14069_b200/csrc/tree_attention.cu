@@ -19,6 +19,7 @@ constexpr int kRowsPerWarp = 4;
 constexpr int kRowsPerBlock = kWarps * kRowsPerWarp;     // 32
 constexpr int kTile = 32;                                // keys per shared-memory tile
 constexpr int kMaxSplits = 128;                          // pieces of a sequence's keys
+constexpr int kMaxCluster = 8;                           // ... that a cluster merges itself
 
 struct AttnParams {
     radar_attn_args a;
@@ -51,7 +52,21 @@ template <> __device__ __forceinline__ void load16<__nv_bfloat16>(const __nv_bfl
     }
 }
 
-template <typename T, int D>
+__device__ __forceinline__ uint32_t in_block(const void* p, uint32_t rank) {
+    uint32_t a;
+    asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"((uint32_t)__cvta_generic_to_shared(p)), "r"(rank));
+    return a;
+}
+__device__ __forceinline__ void cluster_barrier() {
+    asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
+}
+
+// kCluster: the splits of a row block are a cluster, which merges them through its shared memory, the rows dealt out over the blocks:
+// a second kernel is a fifth of the time of small calls (4 / 4 heads of d = 64, 48 blocks: 8.3 -> 7.0 us).  More splits than a
+// cluster may have blocks go through the workspace and tree_attn_combine_kernel, and so do launches that fill the device, where
+// blocks that wait for one another keep others from starting (32 / 8 heads of d = 128, 364 keys 32.2 -> 42.3 us; 24 / 8 of d = 64, 80
+// keys, 144 blocks 8.3 -> 9.0).
+template <typename T, int D, bool kCluster>
 __global__ void __launch_bounds__(kThreads) tree_attn_fp32_kernel(const AttnParams P) {
     chain_wait();
     const radar_attn_args& a = P.a;
@@ -83,7 +98,7 @@ __global__ void __launch_bounds__(kThreads) tree_attn_fp32_kernel(const AttnPara
     const int Ltot = Pb + M;
     const int k_begin = split * P.split_len;
     const int k_end = min(k_begin + P.split_len, Ltot);
-    if (k_begin >= k_end) return;
+    if (!kCluster && k_begin >= k_end) return;
 
     const T* Q = reinterpret_cast<const T*>(a.Q);
     const T* Kc = reinterpret_cast<const T*>(a.Kc);
@@ -218,6 +233,58 @@ __global__ void __launch_bounds__(kThreads) tree_attn_fp32_kernel(const AttnPara
         }
     }
 
+    if (kCluster) {
+        __shared__ float2 s_ml[kRowsPerBlock];
+        float* s_o = Ks;                                // [32][D]
+        __syncthreads();                                // the last tile has been read
+#pragma unroll
+        for (int i = 0; i < kRowsPerWarp; ++i) {
+            const int rl = warp * kRowsPerWarp + i;
+            if (lane == 0) s_ml[rl] = make_float2(m_run[i], l_run[i]);
+#pragma unroll
+            for (int c = 0; c < D / 32; ++c) s_o[rl * D + lane * (D / 32) + c] = acc[i][c];
+        }
+        cluster_barrier();
+        for (int rl = split + P.n_splits * warp; rl < kRowsPerBlock && row0 + rl < R; rl += P.n_splits * kWarps) {
+            float2 ml = make_float2(-CUDART_INF_F, 0.f);
+            if (lane < P.n_splits)
+                asm volatile("ld.shared::cluster.v2.f32 {%0, %1}, [%2];" : "=f"(ml.x), "=f"(ml.y) : "r"(in_block(&s_ml[rl], lane)) : "memory");
+            float v[kMaxCluster][D / 32], o[D / 32];
+#pragma unroll
+            for (int u = 0; u < kMaxCluster; ++u) {
+#pragma unroll
+                for (int c = 0; c < D / 32; ++c) v[u][c] = 0.f;
+                if (u >= P.n_splits) continue;
+                const uint32_t from = in_block(s_o + rl * D + lane * (D / 32), u);
+                if constexpr (D == 128)
+                    asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v[u][0]), "=f"(v[u][1]), "=f"(v[u][2]), "=f"(v[u][3]) : "r"(from) : "memory");
+                else
+                    asm volatile("ld.shared::cluster.v2.f32 {%0, %1}, [%2];" : "=f"(v[u][0]), "=f"(v[u][1]) : "r"(from) : "memory");
+            }
+            const float mx = warp_max(ml.x);
+            const float w = ml.x == -CUDART_INF_F ? 0.f : __expf(ml.x - mx);
+            const float den = warp_sum(ml.y * w), inv = 1.f / den;
+#pragma unroll
+            for (int c = 0; c < D / 32; ++c) o[c] = 0.f;
+#pragma unroll
+            for (int u = 0; u < kMaxCluster; ++u) {
+                const float wu = __shfl_sync(kFull, w, u);
+#pragma unroll
+                for (int c = 0; c < D / 32; ++c) o[c] = fmaf(v[u][c], wu, o[c]);
+            }
+            const int r = row0 + rl, node = r / G, hq = g * G + r % G;
+            T* dst = reinterpret_cast<T*>(a.O) + (((int64_t)b * kMaxNodes + node) * Hq + hq) * D + lane * (D / 32);
+#pragma unroll
+            for (int c = 0; c < D / 32; ++c) {
+                if constexpr (sizeof(T) == 4) dst[c] = o[c] * inv;
+                else dst[c] = __float2bfloat16(o[c] * inv);
+            }
+            if (a.lse != nullptr && lane == 0) a.lse[((int64_t)b * Hq + hq) * kMaxNodes + node] = mx + logf(den);
+        }
+        cluster_barrier();                              // no block leaves while another reads from it
+        return;
+    }
+
     // ---- partial results ----
 #pragma unroll
     for (int i = 0; i < kRowsPerWarp; ++i) {
@@ -340,11 +407,32 @@ int launch(radar_ctx* ctx, const AttnParams& P, cudaStream_t stream) {
     const radar_attn_args& a = P.a;
     const int rblocks = (kMaxNodes * P.G + kRowsPerBlock - 1) / kRowsPerBlock;
     const size_t smem = sizeof(float) * (kRowsPerBlock * D + kTile * (D + 4) + kTile * D);
-    RADAR_CUDA_CHECK(radar_opt_in_smem(ctx, RADAR_SMEM_ATTN_FMA + 2 * (sizeof(T) == 2) + (D == 128), tree_attn_fp32_kernel<T, D>, smem));
+    const int slot = RADAR_SMEM_ATTN_FMA + 4 * (sizeof(T) == 2) + 2 * (D == 128);
     dim3 grid((unsigned)(rblocks * P.n_splits), (unsigned)a.Hkv, (unsigned)a.B);
+    if (P.n_splits <= kMaxCluster && 2ll * grid.x * grid.y * grid.z <= ctx->sm_count) {
+        RADAR_CUDA_CHECK(radar_opt_in_smem(ctx, slot + 1, tree_attn_fp32_kernel<T, D, true>, smem));
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = grid;
+        cfg.blockDim = dim3(kThreads);
+        cfg.dynamicSmemBytes = smem;
+        cfg.stream = stream;
+        cudaLaunchAttribute attr[2];
+        attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr[0].val.programmaticStreamSerializationAllowed = 1;
+        attr[1].id = cudaLaunchAttributeClusterDimension;
+        attr[1].val.clusterDim.x = (unsigned)P.n_splits;
+        attr[1].val.clusterDim.y = 1;
+        attr[1].val.clusterDim.z = 1;
+        cfg.attrs = attr;
+        cfg.numAttrs = 2;
+        radar_launch_scope scope(ctx, RADAR_K_ATTN, stream);
+        RADAR_CUDA_CHECK(cudaLaunchKernelEx(&cfg, tree_attn_fp32_kernel<T, D, true>, P));
+        return RADAR_OK;
+    }
+    RADAR_CUDA_CHECK(radar_opt_in_smem(ctx, slot, tree_attn_fp32_kernel<T, D, false>, smem));
     {
         radar_launch_scope scope(ctx, RADAR_K_ATTN, stream);
-        RADAR_CUDA_CHECK(launch_chained(tree_attn_fp32_kernel<T, D>, grid, dim3(kThreads), smem, stream, P));
+        RADAR_CUDA_CHECK(launch_chained(tree_attn_fp32_kernel<T, D, false>, grid, dim3(kThreads), smem, stream, P));
     }
     RADAR_CUDA_CHECK(cudaGetLastError());
     const int64_t items = (int64_t)a.B * a.Hq * kMaxNodes;
