@@ -117,8 +117,7 @@ __global__ void __launch_bounds__(kSelThreads, 1) expand_select_gate_kernel(cons
     float w1r[4][4], w1x[4];                           // a warp's four rows of the head's hidden layer
     static_assert(H == 4 * kSelWarps, "four rows of the hidden layer per warp");
     if (run_gate) {
-        if (!hidden)
-            for (int e = tid; e < (lstm ? 4 * H : H) * k; e += kSelThreads) cp_async4(s_w + e / k * ws + e % k, (lstm ? a.w_ih : a.w1) + e);
+        if (!hidden) copy_rows(s_w, lstm ? a.w_ih : a.w1, lstm ? 4 * H : H, k);
         if (lstm) {
 #pragma unroll
             for (int i = 0; i < 4; ++i) {

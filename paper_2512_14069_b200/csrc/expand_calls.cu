@@ -101,7 +101,7 @@ __global__ void __launch_bounds__(kSelThreads, 1) expand_calls_kernel(const Call
     float w1r[4][4], w1x[4];
     const bool hidden = kRecurrent && a.policy == RADAR_POLICY_LSTM_HIDDEN;
     if (t_max > 1) {
-        for (int e = tid; e < (hidden ? 0 : kRecurrent ? 4 * H : H) * k; e += kSelThreads) cp_async4(s_w + e / k * ws + e % k, (kRecurrent ? a.w_ih : a.w1) + e);
+        if (!hidden) copy_rows(s_w, kRecurrent ? a.w_ih : a.w1, kRecurrent ? 4 * H : H, k);
         if (kRecurrent) {
 #pragma unroll
             for (int i = 0; i < 4; ++i) {

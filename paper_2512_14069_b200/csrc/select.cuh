@@ -17,6 +17,12 @@ __device__ __forceinline__ float sigmoidf_(float x) { return 1.f / (1.f + expf(-
 __device__ __forceinline__ void cp_async4(void* smem, const void* gmem) {
     asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"((uint32_t)__cvta_generic_to_shared(smem)), "l"(gmem) : "memory");
 }
+// [rows][k] into shared memory at the odd stride k | 1, by the block; kSelThreads a multiple of rows.  Several threads to a row: an
+// index over all elements would be divided by k for each, 2400 cycles of a block's instructions in front of every call.
+__device__ __forceinline__ void copy_rows(float* smem, const float* gmem, int rows, int k) {
+    const int per = kSelThreads / rows, r = (int)threadIdx.x / per;
+    for (int j = (int)threadIdx.x % per; j < k; j += per) cp_async4(smem + r * (k | 1) + j, gmem + r * k + j);
+}
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
 __device__ __forceinline__ uint32_t smem_addr(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
