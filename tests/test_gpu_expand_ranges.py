@@ -107,3 +107,29 @@ def test_rows_top_k(ctx, dtype, V, k):     # noqa: F811
     assert torch.equal(got == float("-inf"), lp == float("-inf"))
     fin = torch.isfinite(lp)
     assert float((got - lp)[fin].abs().max()) < 2e-6 + 16 * 2 ** -24
+
+
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("V,k", [(32, 32), (263, 10), (1028, 1), (8200, 10), (40000, 32), (131073, 4), (170001, 10), (270001, 32)])
+def test_many_rows_top_k(ctx, dtype, V, k):     # noqa: F811
+    """The same kinds of rows where there are too many of them for a cluster each (301 > 2 * 148): pass and merge kernels,
+    longer rows than 128 spans, and every row of an odd V at another distance from a 16-byte boundary."""
+    import torch
+    dt = torch.float32 if dtype == "f32" else torch.bfloat16
+    g = torch.Generator(device="cuda").manual_seed(V + k)
+    x = torch.randn(7, V, device="cuda", generator=g)
+    x[1, :] = float("-inf"); x[1, V // 2::max(V // 4, 1)] = 1.0
+    x[2, :] = float("-inf"); x[2, V - min(V, 200):] = torch.randn(min(V, 200), device="cuda", generator=g)
+    x[3, :] = float("-inf"); x[3, 5::1024] = torch.randn(len(x[3, 5::1024]), device="cuda", generator=g)
+    x[4, :] = 0.5
+    x[5, ::3] = 7.0
+    x = x.to(dt)
+    s, status = _run(ctx, x.repeat(43, 1).view(301, 1, V), k, 1, None, 0, None)
+    assert status == 0
+    order = torch.sort(x.double(), dim=-1, descending=True, stable=True).indices[:, :k]
+    assert torch.equal(s.topk_tok1[:, 0].long().view(43, 7, k), order.expand(43, 7, k))
+    lp = torch.log_softmax(x.double(), -1).gather(1, order).expand(43, 7, k)
+    got = s.topk_logp1[:, 0].double().view(43, 7, k)
+    assert torch.equal(got == float("-inf"), lp == float("-inf"))
+    fin = torch.isfinite(lp)
+    assert float((got - lp)[fin].abs().max()) < 2e-6 + 16 * 2 ** -24
