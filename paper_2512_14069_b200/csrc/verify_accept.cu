@@ -113,8 +113,10 @@ constexpr int kAccMinSlice = 4096;       // ... where there are rows enough to f
 // A CTA's slice of the vocabulary is worked on in tiles of 128 tokens, a contiguous run of tiles to each warp, a quad of
 // tokens to a lane: a warp's partial sum is the mass of a run of tokens, and the partial sums of the pass that settles the
 // last weights are all that the final draw needs to find the warp that owns the sampled point.
-// The exponentials of both rows are cached tile by tile (128 of the target row, 128 of the draft row): a slice's first tiles
-// in shared memory, what has no room there in the workspace.  Inside a tile come the first pairs of its
+// The exponentials of both rows are cached tile by tile (128 of the target row, 128 of the draft row): the first tiles of every
+// warp's run in shared memory, what has no room there in the workspace (all warps wait for L2 then, a third as long; with the
+// slice's first tiles on chip, the last warps' runs lay in the workspace as a whole: walk, one sequence of 128256 tokens 43.5 -> 37.4 us,
+// 32 of them 99 -> 95; acceptance lengths, one tree of 151001 51 -> 44).  Inside a tile come the first pairs of its
 // quads, then their second pairs, so that a warp's two 16-byte accesses each cover 512 bytes without gaps.  A slice's
 // last tile may be only partly real (its padding holds zeros); in the workspace CTA r's tiles start 128 r tokens
 // behind its first one's index, which keeps the slices apart.
@@ -126,19 +128,27 @@ constexpr size_t kTileBytes = kTileDoubles * sizeof(double);
 constexpr size_t cache_room(int per_sm, size_t fixed) { return ((228 * 1024 / per_sm - 1024 - fixed) / kTileBytes) * kTileBytes; }
 __host__ __device__ inline size_t cache_stride(int V) { return (((size_t)V + 3) & ~(size_t)3) + kTileTokens * 8; }
 extern __shared__ __align__(16) double s_cache[];
-struct Cache {
-    double* g;                           // this CTA's tiles in the workspace
-    int st;                              // tiles [0, st) are in shared memory
-    __device__ __forceinline__ double* tile(int t) const { return (t < st ? s_cache : g) + (size_t)t * kTileDoubles; }
-    __device__ __forceinline__ double& token(int o, int which) const {       // o: offset in the slice
-        return tile(o / kTileTokens)[which * kTileTokens + 2 * ((o >> 2) & 31) + 32 * (o & 2) + (o & 1)];
-    }
-};
 struct Tiles { int t0, t1; };            // a warp's run
 __device__ __forceinline__ Tiles warp_tiles(int n, int warp) {       // n: tokens of the slice
     const int T = (n + kTileTokens - 1) / kTileTokens;
     return {T * warp / kSWarps, T * (warp + 1) / kSWarps};
 }
+// A warp's tiles (no other warp touches them): the first of its run, as many as are its share, in shared memory.
+struct Cache {
+    double* g;                           // this CTA's tiles in the workspace
+    double* s;                           // where its first tile would lie in shared memory, if this warp's run went on to it
+    int end;                             // tiles [t0, end) are there
+    __device__ __forceinline__ Cache(double* g_, int smem_tiles, int n) : g(g_) {
+        const int warp = threadIdx.x >> 5, first = smem_tiles * warp / kSWarps;
+        const Tiles w = warp_tiles(n, warp);
+        end = w.t0 + smem_tiles * (warp + 1) / kSWarps - first;
+        s = s_cache + (first - w.t0) * kTileDoubles;
+    }
+    __device__ __forceinline__ double* tile(int t) const { return (t < end ? s : g) + (ptrdiff_t)t * kTileDoubles; }
+    __device__ __forceinline__ double& token(int o, int which) const {       // o: offset in the slice
+        return tile(o / kTileTokens)[which * kTileTokens + 2 * ((o >> 2) & 31) + 32 * (o & 2) + (o & 1)];
+    }
+};
 
 struct ExpTable { double t[64]; };       // 2^(j/64)
 // 64 / ln 2; ln 2 / 64 and what its rounding left; 1/5!, 1/4!, 1/3!: instructions take them from the constant bank
@@ -481,10 +491,12 @@ __device__ double2 softmax_rows(NodeShared& S, ClusterRed& red, const T* target,
     }
 }
 
-// this thread's share of the sum over the slice (n tokens) of max(0, e_p - rho e_q), the exponentials from the caches
+// this thread's share of the sum over the slice (n tokens) of max(0, e_p - rho e_q), the exponentials from the caches (U tiles'
+// loads side by side: four in the workspace; with more, or with the first of them ahead of the tiles on chip, kernels<2> spill: 3 to 13 % slower)
+template <int U>
 __device__ __forceinline__ double residual_of_tiles(const double* base, int t0, int t1, double rho) {
     double g0 = 0.0, g1 = 0.0;
-#pragma unroll 2
+#pragma unroll U
     for (int t = t0; t < t1; ++t) {
         double p[4], q[4];
         load_quad(base + (size_t)t * kTileDoubles, p);
@@ -499,8 +511,8 @@ __device__ __forceinline__ double residual_of_tiles(const double* base, int t0, 
 }
 __device__ __forceinline__ double slice_residual(const Cache C, int n, double rho) {
     const Tiles w = warp_tiles(n, threadIdx.x >> 5);
-    const int mid = min(max(C.st, w.t0), w.t1);
-    return residual_of_tiles(s_cache, w.t0, mid, rho) + residual_of_tiles(C.g, mid, w.t1, rho);
+    const int mid = min(C.end, w.t1);
+    return residual_of_tiles<2>(C.s, w.t0, mid, rho) + residual_of_tiles<4>(C.g, mid, w.t1, rho);
 }
 
 // The residual pair of a node while its children are tried in order (file header), in units of the target row's sum:
@@ -576,7 +588,7 @@ __global__ void __launch_bounds__(kSThreads, kPerSm) stochastic_walk_kernel(cons
     }
     const T* target = reinterpret_cast<const T*>(a.target_logits) + (size_t)b * kMaxNodes * V;
     const T* draft = reinterpret_cast<const T*>(a.draft_logits) + (size_t)b * a.R * V;
-    const Cache C{P.cache + 2 * ((size_t)b * cache_stride(V) + v0 + kTileTokens * crank), P.smem_tiles};
+    const Cache C(P.cache + 2 * ((size_t)b * cache_stride(V) + v0 + kTileTokens * crank), P.smem_tiles, v1 - v0);
     if (tid == 0) prefetch_slice(target, v0, v1);                 // the root's rows
     if (tid == 0) prefetch_slice(draft, v0, v1);
     __syncthreads();
@@ -774,7 +786,7 @@ __global__ void __launch_bounds__(kSThreads, kPerSm) accept_length_nodes_kernel(
     const int cluster = blockIdx.x / csize, n_clusters = gridDim.x / csize;
     const int nq = (V + 3) / 4;
     const int v0 = 4 * (int)((long long)nq * crank / csize), v1 = min(V, 4 * (int)((long long)nq * (crank + 1) / csize));
-    const Cache C{P.cache + 2 * ((size_t)cluster * cache_stride(V) + v0 + kTileTokens * crank), P.smem_tiles};
+    const Cache C(P.cache + 2 * ((size_t)cluster * cache_stride(V) + v0 + kTileTokens * crank), P.smem_tiles, v1 - v0);
     const double invT = 1.0 / (double)a.temperature;
     bool nan_seen = false, bad_tree = false;
 
