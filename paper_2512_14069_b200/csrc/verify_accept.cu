@@ -198,23 +198,42 @@ __device__ __forceinline__ double exp64(double x, const double* tab) {
     if (fabs(x) > 700.0) return x > 0.0 ? CUDART_INF : x < -760.0 ? 0.0 : times_2_to(y, m + 512) * 7.458340731200207e-155;   // 2^-512
     return times_2_to(y, m);
 }
-// exp(z[i] / T + shift) for 4 Q logits, with one fp32 test and one branch for the rare ranges (an fp64 comparison behind each
+__device__ __forceinline__ float max_nan(float a, float b) {
+    float y;
+    asm("max.NaN.f32 %0, %1, %2;" : "=f"(y) : "f"(a), "f"(b));
+    return y;
+}
+__device__ __forceinline__ float min_nan(float a, float b) {
+    float y;
+    asm("min.NaN.f32 %0, %1, %2;" : "=f"(y) : "f"(a), "f"(b));
+    return y;
+}
+// exp(z[i] / T + shift) for 4 Q logits, with one fp32 test and one branch for the rare ranges and NaN (an fp64 comparison behind each
 // exponential costs the pipe that bounds this, and a branch behind each keeps the chains from overlapping)
+// kBits: the logit becomes a double by integer operations.  A conversion is an fp64 instruction at a fraction of the others' rate,
+// which two blocks per SM are bound by (walk, 32 sequences of 50256 tokens 41.6 -> 37.0 us, 16 33.7 -> 30.6; lengths, eight trees 67.4 ->
+// 64.4); a block by itself waits for its chains, which the three operations lengthen (4 of 32000 22.4 -> 24.0: not there).
 struct ExpRange {
-    double invT, shift;
+    double invT, scaled, shift;          // scaled: 2^896 / T
     float lo, hi;                        // finite logits between which |z / T + shift| stays below 700
     // Around the logit `ref`.  Both bounds are rounded towards it: with a small T an ulp of the logits is many units of z / T,
     // and a bound rounded away from it would let such a logit through.
-    __device__ __forceinline__ ExpRange(double invT_, float ref) : invT(invT_), shift(-((double)ref * invT_)) {
+    __device__ __forceinline__ ExpRange(double invT_, float ref) : invT(invT_), scaled(invT_ * 0x1p896), shift(-((double)ref * invT_)) {
         const double reach = 690.0 / invT_;
-        lo = fmaxf(__double2float_ru((double)ref - reach), -FLT_MAX);
+        // (2^896 / T overflows for T up to 2^-128: no logit is in the range then)
+        lo = scaled < CUDART_INF ? fmaxf(__double2float_ru((double)ref - reach), -FLT_MAX) : CUDART_INF_F;
         hi = fminf(__double2float_rd((double)ref + reach), FLT_MAX);
     }
     __device__ __forceinline__ double arg(float z) const { return fma((double)z, invT, shift); }
+    // ... of a finite one: its fields moved to where a double has them are z 2^-896, also for zeros and below fp32's normal range
+    __device__ __forceinline__ double arg_by_bits(float z) const {
+        const int u = __float_as_int(z);
+        return fma(__hiloint2double((u >> 3) & 0x8fffffff, u << 29), scaled, shift);
+    }
     // of any logit (-inf: 0, also where 1 / T has become 0)
     __device__ __forceinline__ double exp_of(float z, const double* tab) const { return z == -CUDART_INF_F ? 0.0 : exp64(arg(z), tab); }
 };
-template <int Q>
+template <int Q, bool kBits>
 __device__ __forceinline__ void exp64_quads(const float (&z)[Q][4], const ExpRange& X, const double* tab, double (&e)[Q][4]) {
     float lo = z[0][0], hi = z[0][0];
 #pragma unroll
@@ -222,10 +241,10 @@ __device__ __forceinline__ void exp64_quads(const float (&z)[Q][4], const ExpRan
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
             int m;
-            const double y = exp_split(X.arg(z[q][i]), tab, m);
+            const double y = exp_split(kBits ? X.arg_by_bits(z[q][i]) : X.arg(z[q][i]), tab, m);
             e[q][i] = times_2_to(y, m);
-            lo = fminf(lo, z[q][i]);
-            hi = fmaxf(hi, z[q][i]);
+            lo = min_nan(lo, z[q][i]);
+            hi = max_nan(hi, z[q][i]);
         }
     if (!(lo >= X.lo && hi <= X.hi)) {
 #pragma unroll
@@ -235,11 +254,6 @@ __device__ __forceinline__ void exp64_quads(const float (&z)[Q][4], const ExpRan
     }
 }
 
-__device__ __forceinline__ float max_nan(float a, float b) {
-    float y;
-    asm("max.NaN.f32 %0, %1, %2;" : "=f"(y) : "f"(a), "f"(b));
-    return y;
-}
 // logits v .. v + 3 of a row; -inf from v1 on.  `wide`: the row starts on a boundary of four
 __device__ __forceinline__ void load_quad(const float* row, int v, int v1, bool wide, float (&o)[4]) {
     if (wide && v + 4 <= v1) {
@@ -403,8 +417,8 @@ __device__ __forceinline__ float slice_max(const T* row, int v0, int v1) {
 
 // This CTA's slice of one row into the cache (which: 0 target, 1 draft): exp(z / T + shift); returns this thread's sum.
 // Two tiles at a time, eight chains of exponentials side by side, the next two tiles' quads on their way meanwhile.
-// z: the thread's first quad.  Not inlined: with the caller's state in the same registers the loop would spill.
-template <typename T>
+// first: the thread's first quad.
+template <typename T, bool kBits>
 __device__ __forceinline__ double slice_exp(const T* row, int v0, int v1, const ExpRange X, const double* tab, const Cache C, int which, float4 first) {
     const bool wide = row_is_wide(row);
     const Tiles w = warp_tiles(v1 - v0, threadIdx.x >> 5);
@@ -418,7 +432,7 @@ __device__ __forceinline__ double slice_exp(const T* row, int v0, int v1, const 
         load_quad(row, t + 2 < w.t1 ? mine + (t + 2) * kTileTokens : v1, v1, wide, zn[0]);
         load_quad(row, t + 3 < w.t1 ? mine + (t + 3) * kTileTokens : v1, v1, wide, zn[1]);
         double e[2][4];
-        exp64_quads<2>(z, X, tab, e);
+        exp64_quads<2, kBits>(z, X, tab, e);
         store_quad(C.tile(t) + which * kTileTokens, e[0]);
         store_quad(C.tile(t + 1) + which * kTileTokens, e[1]);
         s0 += (e[0][0] + e[0][1]) + (e[0][2] + e[0][3]);
@@ -429,7 +443,7 @@ __device__ __forceinline__ double slice_exp(const T* row, int v0, int v1, const 
     if (t < w.t1) {
         const float zl[1][4] = {{z[0][0], z[0][1], z[0][2], z[0][3]}};
         double e[1][4];
-        exp64_quads<1>(zl, X, tab, e);
+        exp64_quads<1, kBits>(zl, X, tab, e);
         store_quad(C.tile(t) + which * kTileTokens, e[0]);
         s0 += (e[0][0] + e[0][1]) + (e[0][2] + e[0][3]);
     }
@@ -456,7 +470,7 @@ __device__ __forceinline__ float2 slice_maxima(const T* target, const T* draft, 
 // the scale.  It is the largest of 32 of the row's logits, the same ones in every warp, so a row is read once
 // and its two rows take one exchange.  Only if a sum shows that some logit lies so far above (or that the sample held
 // nothing finite) the pass is repeated from the exact maxima.
-template <typename T, typename F>
+template <typename T, bool kBits, typename F>
 __device__ double2 softmax_rows(NodeShared& S, ClusterRed& red, const T* target, const T* draft, int V, int v0, int v1,
                                 double invT, const Cache C, unsigned long long children, bool* nan_seen,
                                 F&& meanwhile) {
@@ -473,8 +487,8 @@ __device__ double2 softmax_rows(NodeShared& S, ClusterRed& red, const T* target,
     const double* tab = S.exps.mine();
     for (int pass = 0;; ++pass) {
         const ExpRange Xt(invT, rt), Xd(invT, rd);
-        const double st = slice_exp(target, v0, v1, Xt, tab, C, 0, ft);
-        const double sd = two ? slice_exp(draft, v0, v1, Xd, tab, C, 1, fd) : 1.0 / (kMaxCluster * kSThreads);
+        const double st = slice_exp<T, kBits>(target, v0, v1, Xt, tab, C, 0, ft);
+        const double sd = two ? slice_exp<T, kBits>(draft, v0, v1, Xd, tab, C, 1, fd) : 1.0 / (kMaxCluster * kSThreads);
         if (child) {
             S.pe[tid] = Xt.exp_of(xt, tab);
             S.qe[tid] = two ? Xd.exp_of(xd, tab) : 0.0;
@@ -614,7 +628,7 @@ __global__ void __launch_bounds__(kSThreads, kPerSm) stochastic_walk_kernel(cons
                 if (dr >= 0 && dr < a.R) prefetch_slice(draft + (size_t)dr * V, v0, v1);
             }
         };
-        const double2 sums = softmax_rows<T>(S, red, target + (size_t)cur * V, kids != 0 ? draft + (size_t)drow * V : nullptr, V, v0, v1, invT,
+        const double2 sums = softmax_rows<T, kPerSm == 2>(S, red, target + (size_t)cur * V, kids != 0 ? draft + (size_t)drow * V : nullptr, V, v0, v1, invT,
                                              C, kids, &nan_seen, [&] { fetch_ahead(kids); });
         res = Residual(sums.x, sums.y);
         int accepted = -1;
@@ -873,7 +887,7 @@ __global__ void __launch_bounds__(kSThreads, kPerSm) accept_length_nodes_kernel(
                 const T* draft = reinterpret_cast<const T*>(a.draft_logits) + ((size_t)b * a.R + drow) * V;
                 // the rows of this cluster's next item are asked for while this one's are worked on
                 const int next = (round + 1) * n_clusters + ((round & 1) ? cluster : n_clusters - 1 - cluster);
-                const double2 sums = softmax_rows<T>(S, red, target, draft, V, v0, v1, invT, C, kids, &nan_seen, [&] {
+                const double2 sums = softmax_rows<T, kPerSm == 2>(S, red, target, draft, V, v0, v1, invT, C, kids, &nan_seen, [&] {
                     if (tid == 0 && next < n_items) {
                         const size_t bn = b0 + s_order[next] / kMaxNodes, cn = s_order[next] % kMaxNodes;
                         const int dn = s_drow[s_order[next]];
