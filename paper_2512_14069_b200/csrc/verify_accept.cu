@@ -233,11 +233,14 @@ struct ExpRange {
     // of any logit (-inf: 0, also where 1 / T has become 0)
     __device__ __forceinline__ double exp_of(float z, const double* tab) const { return z == -CUDART_INF_F ? 0.0 : exp64(arg(z), tab); }
 };
-template <int Q, bool kBits>
-__device__ __forceinline__ void exp64_quads(const float (&z)[Q][4], const ExpRange& X, const double* tab, double (&e)[Q][4]) {
-    float lo = z[0][0], hi = z[0][0];
+// quad q: of range range(q)
+template <int Q, bool kBits, typename F>
+__device__ __forceinline__ void exp64_quads(const float (&z)[Q][4], F&& range, const double* tab, double (&e)[Q][4]) {
+    bool usual = true;
 #pragma unroll
-    for (int q = 0; q < Q; ++q)
+    for (int q = 0; q < Q; ++q) {
+        const ExpRange& X = range(q);
+        float lo = z[q][0], hi = z[q][0];
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
             int m;
@@ -246,11 +249,13 @@ __device__ __forceinline__ void exp64_quads(const float (&z)[Q][4], const ExpRan
             lo = min_nan(lo, z[q][i]);
             hi = max_nan(hi, z[q][i]);
         }
-    if (!(lo >= X.lo && hi <= X.hi)) {
+        usual = usual && lo >= X.lo && hi <= X.hi;
+    }
+    if (!usual) {
 #pragma unroll
         for (int q = 0; q < Q; ++q)
 #pragma unroll
-            for (int i = 0; i < 4; ++i) e[q][i] = X.exp_of(z[q][i], tab);
+            for (int i = 0; i < 4; ++i) e[q][i] = range(q).exp_of(z[q][i], tab);
     }
 }
 
@@ -432,7 +437,7 @@ __device__ __forceinline__ double slice_exp(const T* row, int v0, int v1, const 
         load_quad(row, t + 2 < w.t1 ? mine + (t + 2) * kTileTokens : v1, v1, wide, zn[0]);
         load_quad(row, t + 3 < w.t1 ? mine + (t + 3) * kTileTokens : v1, v1, wide, zn[1]);
         double e[2][4];
-        exp64_quads<2, kBits>(z, X, tab, e);
+        exp64_quads<2, kBits>(z, [&](int) -> const ExpRange& { return X; }, tab, e);
         store_quad(C.tile(t) + which * kTileTokens, e[0]);
         store_quad(C.tile(t + 1) + which * kTileTokens, e[1]);
         s0 += (e[0][0] + e[0][1]) + (e[0][2] + e[0][3]);
@@ -443,11 +448,42 @@ __device__ __forceinline__ double slice_exp(const T* row, int v0, int v1, const 
     if (t < w.t1) {
         const float zl[1][4] = {{z[0][0], z[0][1], z[0][2], z[0][3]}};
         double e[1][4];
-        exp64_quads<1, kBits>(zl, X, tab, e);
+        exp64_quads<1, kBits>(zl, [&](int) -> const ExpRange& { return X; }, tab, e);
         store_quad(C.tile(t) + which * kTileTokens, e[0]);
         s0 += (e[0][0] + e[0][1]) + (e[0][2] + e[0][3]);
     }
     return s0 + s1;
+}
+// ... of both rows in one loop, a tile of each at a time; both sums.  Eight chains as well, and half the code: a warp goes through a
+// few tiles of a row only, and its first pass over a loop waits for the instructions.  us in one loop / two: acceptance lengths of
+// eight trees 124 / 133 (V = 128256), 62.7 / 64.3 (50256), of four of 32000 23.9 / 25.2, of one of 151001 43.5 / 43.7.  (In the
+// walk, whose last node has no draft row, 94 / 90.5 for 32 sequences of 128256, 33.5 / 31.6 for 6 of 50257: not there.)
+template <typename T, bool kBits>
+__device__ __forceinline__ double2 slice_exp_both(const T* target, const T* draft, int v0, int v1, const ExpRange (&X)[2], const double* tab,
+                                                  const Cache C, float4 first_t, float4 first_d) {
+    const T* const row[2] = {target, draft};
+    const bool wide[2] = {row_is_wide(target), row_is_wide(draft)};
+    const Tiles w = warp_tiles(v1 - v0, threadIdx.x >> 5);
+    const int mine = v0 + 4 * (threadIdx.x & 31);
+    double s[2] = {0.0, 0.0};
+    float z[2][4] = {{first_t.x, first_t.y, first_t.z, first_t.w}, {first_d.x, first_d.y, first_d.z, first_d.w}};
+#pragma unroll 1
+    for (int t = w.t0; t < w.t1; ++t) {
+        float zn[2][4];
+#pragma unroll
+        for (int q = 0; q < 2; ++q) load_quad(row[q], t + 1 < w.t1 ? mine + (t + 1) * kTileTokens : v1, v1, wide[q], zn[q]);
+        double e[2][4];
+        exp64_quads<2, kBits>(z, [&](int q) -> const ExpRange& { return X[q]; }, tab, e);
+        double* const tile = C.tile(t);
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+            store_quad(tile + q * kTileTokens, e[q]);
+            s[q] += (e[q][0] + e[q][1]) + (e[q][2] + e[q][3]);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) z[q][i] = zn[q][i];
+        }
+    }
+    return make_double2(s[0], s[1]);
 }
 template <typename T>
 __device__ __forceinline__ float4 first_quad(const T* row, int v0, int v1) {
@@ -469,13 +505,13 @@ __device__ __forceinline__ float2 slice_maxima(const T* target, const T* draft, 
 // The reference of a row need not be its maximum: fp64 has room for exp(700), and relative precision does not depend on
 // the scale.  It is the largest of 32 of the row's logits, the same ones in every warp, so a row is read once
 // and its two rows take one exchange.  Only if a sum shows that some logit lies so far above (or that the sample held
-// nothing finite) the pass is repeated from the exact maxima.
-template <typename T, bool kBits, typename F>
+// nothing finite) the pass is repeated from the exact maxima.  kBoth: `draft` is not NULL.
+template <typename T, bool kBits, bool kBoth, typename F>
 __device__ double2 softmax_rows(NodeShared& S, ClusterRed& red, const T* target, const T* draft, int V, int v0, int v1,
                                 double invT, const Cache C, unsigned long long children, bool* nan_seen,
                                 F&& meanwhile) {
     const int tid = threadIdx.x;
-    const bool two = draft != nullptr;
+    const bool two = kBoth || draft != nullptr;
     const int x = tid < kMaxNodes && ((children >> tid) & 1) ? S.tok[tid] : -1;
     const bool child = x >= 0 && x < V;
     const float xt = child ? to_float(target[x]) : 0.f, xd = child && two ? to_float(draft[x]) : 0.f;
@@ -486,14 +522,19 @@ __device__ double2 softmax_rows(NodeShared& S, ClusterRed& red, const T* target,
     rd = warp_max(rd);
     const double* tab = S.exps.mine();
     for (int pass = 0;; ++pass) {
-        const ExpRange Xt(invT, rt), Xd(invT, rd);
-        const double st = slice_exp<T, kBits>(target, v0, v1, Xt, tab, C, 0, ft);
-        const double sd = two ? slice_exp<T, kBits>(draft, v0, v1, Xd, tab, C, 1, fd) : 1.0 / (kMaxCluster * kSThreads);
-        if (child) {
-            S.pe[tid] = Xt.exp_of(xt, tab);
-            S.qe[tid] = two ? Xd.exp_of(xd, tab) : 0.0;
+        const ExpRange X[2] = {ExpRange(invT, rt), ExpRange(invT, rd)};
+        double2 sum;
+        if constexpr (kBoth) {
+            sum = slice_exp_both<T, kBits>(target, draft, v0, v1, X, tab, C, ft, fd);
+        } else {
+            sum.x = slice_exp<T, kBits>(target, v0, v1, X[0], tab, C, 0, ft);
+            sum.y = two ? slice_exp<T, kBits>(draft, v0, v1, X[1], tab, C, 1, fd) : 1.0 / (kMaxCluster * kSThreads);
         }
-        red.send(warp_sum(st), warp_sum(sd));
+        if (child) {
+            S.pe[tid] = X[0].exp_of(xt, tab);
+            S.qe[tid] = two ? X[1].exp_of(xd, tab) : 0.0;
+        }
+        red.send(warp_sum(sum.x), warp_sum(sum.y));
         if (pass == 0) meanwhile();
         const double2 s = red.receive_sum2();                      // ... and S.pe and S.qe
         if ((s.x > 0.0 && s.x < 1e250 && s.y > 0.0 && s.y < 1e250) || pass == 1) return make_double2(s.x, two ? s.y : 1.0);
@@ -628,7 +669,7 @@ __global__ void __launch_bounds__(kSThreads, kPerSm) stochastic_walk_kernel(cons
                 if (dr >= 0 && dr < a.R) prefetch_slice(draft + (size_t)dr * V, v0, v1);
             }
         };
-        const double2 sums = softmax_rows<T, kPerSm == 2>(S, red, target + (size_t)cur * V, kids != 0 ? draft + (size_t)drow * V : nullptr, V, v0, v1, invT,
+        const double2 sums = softmax_rows<T, kPerSm == 2, false>(S, red, target + (size_t)cur * V, kids != 0 ? draft + (size_t)drow * V : nullptr, V, v0, v1, invT,
                                              C, kids, &nan_seen, [&] { fetch_ahead(kids); });
         res = Residual(sums.x, sums.y);
         int accepted = -1;
@@ -887,7 +928,7 @@ __global__ void __launch_bounds__(kSThreads, kPerSm) accept_length_nodes_kernel(
                 const T* draft = reinterpret_cast<const T*>(a.draft_logits) + ((size_t)b * a.R + drow) * V;
                 // the rows of this cluster's next item are asked for while this one's are worked on
                 const int next = (round + 1) * n_clusters + ((round & 1) ? cluster : n_clusters - 1 - cluster);
-                const double2 sums = softmax_rows<T, kPerSm == 2>(S, red, target, draft, V, v0, v1, invT, C, kids, &nan_seen, [&] {
+                const double2 sums = softmax_rows<T, kPerSm == 2, true>(S, red, target, draft, V, v0, v1, invT, C, kids, &nan_seen, [&] {
                     if (tid == 0 && next < n_items) {
                         const size_t bn = b0 + s_order[next] / kMaxNodes, cn = s_order[next] % kMaxNodes;
                         const int dn = s_drow[s_order[next]];
