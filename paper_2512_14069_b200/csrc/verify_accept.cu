@@ -421,38 +421,44 @@ __device__ __forceinline__ float slice_max(const T* row, int v0, int v1) {
 }
 
 // This CTA's slice of one row into the cache (which: 0 target, 1 draft): exp(z / T + shift); returns this thread's sum.
-// Two tiles at a time, eight chains of exponentials side by side, the next two tiles' quads on their way meanwhile.
-// first: the thread's first quad.
+// Q tiles at a time, four chains of exponentials each, the next quads on their way meanwhile.  Two where the SM is full (walk of
+// 32 sequences of 128256 tokens 88 us, one at a time 94), one in a block by itself, which goes through few tiles and waits for the
+// loop's instructions (four of 32000 21.0, two at a time 22.4, four 26.2).  first: the thread's first quad.
 template <typename T, bool kBits>
-__device__ __forceinline__ double slice_exp(const T* row, int v0, int v1, const ExpRange X, const double* tab, const Cache C, int which, float4 first) {
+__device__ __forceinline__ double slice_exp(const T* row, int v0, int v1, const ExpRange& X, const double* tab, const Cache C, int which, float4 first) {
+    constexpr int Q = kBits ? 2 : 1;
+    const auto range = [&](int) -> const ExpRange& { return X; };
     const bool wide = row_is_wide(row);
     const Tiles w = warp_tiles(v1 - v0, threadIdx.x >> 5);
     const int mine = v0 + 4 * (threadIdx.x & 31);
-    double s0 = 0.0, s1 = 0.0;
-    float z[2][4] = {{first.x, first.y, first.z, first.w}, {-CUDART_INF_F, -CUDART_INF_F, -CUDART_INF_F, -CUDART_INF_F}};
-    if (w.t0 + 1 < w.t1) load_quad(row, mine + (w.t0 + 1) * kTileTokens, v1, wide, z[1]);
+    double s[Q] = {};
+    float z[Q][4] = {{first.x, first.y, first.z, first.w}};
+    auto load = [&](int t, float (&o)[4]) { load_quad(row, t < w.t1 ? mine + t * kTileTokens : v1, v1, wide, o); };
+    if (Q == 2) load(w.t0 + 1, z[Q - 1]);
     int t = w.t0;
-    for (; t + 1 < w.t1; t += 2) {
-        float zn[2][4];
-        load_quad(row, t + 2 < w.t1 ? mine + (t + 2) * kTileTokens : v1, v1, wide, zn[0]);
-        load_quad(row, t + 3 < w.t1 ? mine + (t + 3) * kTileTokens : v1, v1, wide, zn[1]);
-        double e[2][4];
-        exp64_quads<2, kBits>(z, [&](int) -> const ExpRange& { return X; }, tab, e);
-        store_quad(C.tile(t) + which * kTileTokens, e[0]);
-        store_quad(C.tile(t + 1) + which * kTileTokens, e[1]);
-        s0 += (e[0][0] + e[0][1]) + (e[0][2] + e[0][3]);
-        s1 += (e[1][0] + e[1][1]) + (e[1][2] + e[1][3]);
+#pragma unroll 1
+    for (; t + Q <= w.t1; t += Q) {
+        float zn[Q][4];
 #pragma unroll
-        for (int i = 0; i < 4; ++i) { z[0][i] = zn[0][i]; z[1][i] = zn[1][i]; }
+        for (int q = 0; q < Q; ++q) load(t + Q + q, zn[q]);
+        double e[Q][4];
+        exp64_quads<Q, kBits>(z, range, tab, e);
+#pragma unroll
+        for (int q = 0; q < Q; ++q) {
+            store_quad(C.tile(t + q) + which * kTileTokens, e[q]);
+            s[q] += (e[q][0] + e[q][1]) + (e[q][2] + e[q][3]);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) z[q][i] = zn[q][i];
+        }
     }
-    if (t < w.t1) {
+    if (Q == 2 && t < w.t1) {
         const float zl[1][4] = {{z[0][0], z[0][1], z[0][2], z[0][3]}};
         double e[1][4];
-        exp64_quads<1, kBits>(zl, [&](int) -> const ExpRange& { return X; }, tab, e);
+        exp64_quads<1, kBits>(zl, range, tab, e);
         store_quad(C.tile(t) + which * kTileTokens, e[0]);
-        s0 += (e[0][0] + e[0][1]) + (e[0][2] + e[0][3]);
+        s[0] += (e[0][0] + e[0][1]) + (e[0][2] + e[0][3]);
     }
-    return s0 + s1;
+    return Q == 2 ? s[0] + s[Q - 1] : s[0];
 }
 // ... of both rows in one loop, a tile of each at a time; both sums.  Eight chains as well, and half the code: a warp goes through a
 // few tiles of a row only, and its first pass over a loop waits for the instructions.  us in one loop / two: acceptance lengths of
