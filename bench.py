@@ -40,7 +40,7 @@ NCU_TRAFFIC_RATIO = {
     ("tree_attention", 5): 395.99 / 388.08,      # captured on the first four sequences of the configuration (--batch 4)
     ("tree_attention", 4): 453.40 / 284.58,
     ("tree_attention", 3): 351.81 / 343.57,
-    ("vocab_pass(expand)", 4): 41.142 / 41.042,
+    ("vocab_pass(expand)", 4): 130.663 / 127.230,
     ("vocab_pass(accept)", 4): 228.67 / 224.70,
 }
 

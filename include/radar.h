@@ -116,7 +116,7 @@ enum { RADAR_POLICY_LSTM_SCORES = 0, RADAR_POLICY_MLP_SCORES = 1, RADAR_POLICY_L
  *                        `workspace`.  `active` is only READ here, as the mask of sequences whose rows are worth
  *                        reading: it may be an older mask than the one the select half will see (a sequence that has
  *                        stopped since is read in vain, nothing else), or NULL for "all";
- *   RADAR_EXPAND_SELECT  only the select + gate half, on the records a RADAR_EXPAND_VOCAB call with the same
+ *   RADAR_EXPAND_SELECT  only the select + gate half, on the rows' results that a RADAR_EXPAND_VOCAB call with the same
  *                        arguments left in the same `workspace`.  The caller orders it after that call and after the
  *                        previous draft call's select half.
  * Results are identical in the three forms. */
@@ -164,7 +164,7 @@ int radar_expand_step(radar_ctx* ctx, const radar_expand_args* args, void* strea
 /* radar_expand_calls - all t_max draft calls of a step at once, for draft logits that are there already (recorded ones, or a
  * draft model that does not look at the frontier; where the draft model has to run on the frontier that a call selects
  * before the next call's logits exist, radar_expand_step is the form): the results of radar_expand_step for
- * t = 1 .. t_max, in three launches.  `call` holds the arguments of call 1 (t = 1, F = 1), with these
+ * t = 1 .. t_max, in two or three launches.  `call` holds the arguments of call 1 (t = 1, F = 1), with these
  * differences: logits is [B][1+(t_max-1)*k][V], call 1's row first, then the k rows of every further call in turn;
  * frontier_tok / _score / _pool_idx / _src_row [t_max][B][k], gate_logits [t_max][B][2] and cont [t_max][B] have a slice
  * per call (as with radar_expand_step only the calls a sequence makes write theirs, cont excepted); topk_tok and
