@@ -285,7 +285,8 @@ __device__ __forceinline__ void select_row(const RowTopkParams& p, const Row<T>&
 
     // The bound: the k-th largest of 64 maxima, the best ones of every warp that has groups.  Where that is -inf (the finite
     // values sit in few spans), the best of the warps' k-th largest.  Maxima are ranked as integers, made distinct by
-    // their lowest bits, which can only lower the bound.
+    // their lowest bits; either bound is the integer it was ranked by without those bits (not the maximum itself, which
+    // may lie above some that were ranked ahead of it), so that the k ranked first are all at or above it.
     const int live = p.live, per = p.per;
     {
         const uint32_t key = (order_bits(mine) & ~31u) | (31u - lane);
@@ -299,7 +300,7 @@ __device__ __forceinline__ void select_row(const RowTopkParams& p, const Row<T>&
         }
         const int slot = warp * per + rank;
         if (warp < live && rank < per) S.slots[slot] = (order_bits(mine) & ~63u) | (63u - slot);
-        if (rank == k - 1) S.kth[warp] = mine;
+        if (rank == k - 1) S.kth[warp] = fmaxf(bits_value(key & ~31u), -FLT_MAX);      // (of -inf: NaN, which loses)
         if (tid >= live * per && tid < kBoundSlots) S.slots[tid] = 63u - tid;
     }
     selection_barrier();
