@@ -441,22 +441,34 @@ __device__ __forceinline__ void merge_row(const RowTopkParams& p, const Row<T>& 
     }
 }
 
+// The mask may be written while this runs (a sequence that stops meanwhile is read in vain): the first CTA's look at it decides
+// for the cluster, whose blocks would else wait for messages of blocks that have left, or send to one.  Each thread's own look
+// only decides whether its span is asked for ahead of that.
 template <typename T>
 __global__ void __launch_bounds__(kThreads, 2) row_topk_kernel(const RowTopkParams p) {
     __shared__ MergeShared S;
     __shared__ __align__(16) float s_gmax[kMaxSlots * 32];           // the first CTA's: what all warps of the cluster leave
     __shared__ __align__(16) float2 s_part[kMaxSlots];
     __shared__ __align__(8) uint64_t s_bar;                          // completes when they have sent it
+    __shared__ uint32_t s_live;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, n = gridDim.x, rank = blockIdx.x, f = blockIdx.y, seq = blockIdx.z;
     if (rank == 0 && threadIdx.x == 0) init_message_barrier(&s_bar, (uint32_t)(n * kWarps * (32 * sizeof(float) + sizeof(float2))));
     chain_wait();
-    if (p.seq_active != nullptr && p.seq_active[seq] == 0) return;
+    const bool ahead = p.seq_active == nullptr || p.seq_active[seq] != 0;
+    if (threadIdx.x == 0) s_live = ahead;
     const Row<T> r(p, seq, f);
     const int slot = rank * kWarps + warp;
     Span<T> x;
-    x.load(r, slot);                                  // (past the row's end: -inf, nothing is read)
+    if (ahead) x.load(r, slot);                       // (past the row's end: -inf, nothing is read)
     if (n > 1) cluster_barrier();                     // the first CTA has started and its barrier word is initialised
     else __syncthreads();
+    if (p.seq_active != nullptr) {
+        if (load_u32(cluster_addr(&s_live, 0)) == 0) {
+            if (n > 1) cluster_barrier();             // the first CTA stays until all have looked
+            return;
+        }
+        if (!ahead) x.load(r, slot);
+    }
     float gmax, m, s;
     pass_row<T>(p, r, slot, x, gmax, m, s);
     const uint32_t bar = cluster_addr(&s_bar, 0);
