@@ -35,7 +35,8 @@ constexpr int kSelThreadsRow = 256;                  // of the merge's selection
 constexpr int kSelWarpsRow = kSelThreadsRow / 32, kMergeThreads = kSelThreadsRow + 32;
 constexpr int kHeld = kMaxSlots * 32 / kSelThreadsRow;       // maxima a thread of the merge holds
 constexpr int kBoundSlots = 64;                      // maxima that the bound is chosen from
-constexpr int kGroupCap = 512, kCandCap = 1024;      // groups and values that the merge ranks; beyond, it scans the row
+constexpr int kGroupCap = 512, kCandCap = 2048;      // groups and values that the merge lists; beyond, it scans the row
+constexpr int kRankAll = 128;                        // values that it ranks as they are; more are thinned out first
 constexpr float kLog2e = 1.4426950408889634f;
 
 __device__ __forceinline__ float fast_exp2(float x) {
@@ -160,13 +161,14 @@ __device__ __forceinline__ void merge_barrier() { asm volatile("bar.sync 2, 288;
 
 struct __align__(16) MergeShared {
     unsigned long long key[kCandCap];
+    unsigned long long best[kSelWarpsRow][32], best_slots[kBoundSlots], best_bound[2];       // (two: 16-byte boundaries)
     int group[kGroupCap];
     uint32_t lanes[kSelWarpsRow][32], slots[kBoundSlots];
     uint32_t bound;
     float kth[kSelWarpsRow];
     float best_v[kSelWarpsRow];
     int best_i[kSelWarpsRow];
-    int n_groups, n_cand;
+    int n_groups, n_cand, n_kept;
     float v[RADAR_MAX_K];
     int t[RADAR_MAX_K];
     double lse;
@@ -235,6 +237,49 @@ __device__ __noinline__ void select_by_scan(const T* x, int V, int k, MergeShare
     }
 }
 
+// Many values are listed where fewer than about 2 k groups have any (short rows with a large k, masked rows).  A better bound, the
+// k-th largest of 64 of them, the eight best of every warp's, thins out more than kRankAll: ranks take n^2 comparisons.  Us for the
+// calls of a step without this / with it, bf16: t_max = 5, V = 1000, k = 32, one sequence that makes the first call 153 / 35, eight
+// that make all 550 / 84; V = 600, k = 16 135 / 33.  Returns how many are left.
+__device__ __forceinline__ int thin_out(MergeShared& S, int n, int k) {
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    constexpr int kEach = kCandCap / kSelThreadsRow, kPer = kBoundSlots / kSelWarpsRow;
+    unsigned long long key[kEach], best = 31 - lane;   // (of none: distinct, and less than any listed value's)
+#pragma unroll
+    for (int i = 0; i < kEach; ++i) {
+        const int at = tid + kSelThreadsRow * i;
+        key[i] = at < n ? S.key[at] : 0ull;
+        best = max(best, key[i]);
+    }
+    S.best[warp][lane] = best;
+    __syncwarp();
+    int rank = 0;
+#pragma unroll 4
+    for (int o = 0; o < 32; o += 2) {
+        const ulonglong2 q = *reinterpret_cast<const ulonglong2*>(&S.best[warp][o]);
+        rank += (q.x > best ? 1 : 0) + (q.y > best ? 1 : 0);
+    }
+    if (rank < kPer) S.best_slots[warp * kPer + rank] = best;
+    selection_barrier();
+    const unsigned long long mine = S.best_slots[tid >> 2];
+    rank = 0;
+#pragma unroll 4
+    for (int o = 0; o < kBoundSlots / 4; o += 2) {
+        const ulonglong2 q = *reinterpret_cast<const ulonglong2*>(&S.best_slots[(tid & 3) * (kBoundSlots / 4) + o]);
+        rank += (q.x > mine ? 1 : 0) + (q.y > mine ? 1 : 0);
+    }
+    rank += __shfl_xor_sync(kFull, rank, 1);
+    rank += __shfl_xor_sync(kFull, rank, 2);
+    if (rank == k - 1) S.best_bound[0] = mine;
+    selection_barrier();
+    const unsigned long long bound = S.best_bound[0];
+#pragma unroll
+    for (int i = 0; i < kEach; ++i)
+        if (key[i] >= bound) S.key[atomicAdd(&S.n_kept, 1)] = key[i];
+    selection_barrier();
+    return S.n_kept;
+}
+
 // What the warps of a row have left, where it is.
 struct InShared {
     const float* gmax;                                // [n_slots][32]
@@ -262,7 +307,7 @@ template <typename T, typename Left>
 __device__ __forceinline__ void select_row(const RowTopkParams& p, const Row<T>& r, const Left& left, MergeShared& S) {
     constexpr int N = Unpack<T>::N;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, k = p.k, n_slots = p.n_slots;
-    if (tid == 0) { S.n_groups = 0; S.n_cand = 0; }
+    if (tid == 0) { S.n_groups = 0; S.n_cand = 0; S.n_kept = 0; }
     // Thread tid holds 16 groups: four in a row of every 1024 (a request for 512 bytes takes the SM hardly longer than one for
     // 128: 16 KB in fours 0.6 us, one by one 1.3), or, where there are at most 1024, every 256th, so that every
     // warp has some.
@@ -363,8 +408,9 @@ __device__ __forceinline__ void select_row(const RowTopkParams& p, const Row<T>&
     selection_barrier();
 
     // ---- ranks: a warp to a value ----
-    const int nc = S.n_cand;
+    int nc = S.n_cand;
     if (S.n_groups <= kGroupCap && nc <= kCandCap) {
+        if (nc > kRankAll) nc = thin_out(S, nc, k);
         const unsigned long long k0 = lane < nc ? S.key[lane] : 0ull;
         for (int c = warp; c < nc; c += kSelWarpsRow) {
             const unsigned long long key = S.key[c];
