@@ -30,6 +30,24 @@ struct CallsParams {
     int* status;
 };
 
+// Rank of candidate c among n (key desc, index asc), by the 16 threads of a half-warp.  For more than 64 of them, where two to a
+// warp with ballots (ranks_of) takes longer: five calls of two sequences, V = 32000, k = 32, 70.6 -> 55.0 us, k = 16, eight 35.2 -> 33.0.
+// Not inlined: in the calls' loop its instructions cost the others 0.8 us a step.
+__device__ __noinline__ int rank_among_many(const unsigned long long* keys, const short* index, int n, int c) {
+    const unsigned long long mine = keys[c];
+    const int idx = index[c];
+    int rank = 0;
+#pragma unroll 2
+    for (int j = threadIdx.x & 15; j < n; j += 16) {
+        const unsigned long long kj = keys[j];
+        const int ij = index[j];
+        rank += (int)(kj > mine) | ((int)(kj == mine) & (int)(ij < idx));
+    }
+#pragma unroll
+    for (int o = 8; o > 0; o >>= 1) rank += __shfl_xor_sync(kFull, rank, o);
+    return rank;
+}
+
 // Block 0 of a cluster goes through the calls of its sequence; with the recurrent policy the other blocks hold W_hh (256 KB) in
 // their registers: they receive h as soon as the cell has produced it and deliver W_hh h + biases while block 0 finishes
 // the call and ranks the next one's candidates.  What bounds a call is block 0's chain of steps, each a few dozen dependent
@@ -332,12 +350,20 @@ __global__ void __launch_bounds__(kSelThreads, 1) expand_calls_kernel(const Call
             if ((lane & 7) == 0) s_hid[t & 1][head_row] = fmaxf(sum + s_b1[head_row] + feat_h, 0.f);
         }
         fetch_features(t + 1);
-        // the k best survivors (score desc, flat index asc): a warp to two candidates
-        for (int c = warp, n = more ? s_count : 0; c < n; c += 2 * kSelWarps) {
-            const int c1 = min(c + kSelWarps, n - 1), idx0 = s_cand[c], idx1 = s_cand[c1];
-            const int2 rank = ranks_of(s_key, s_cand, n, s_key[c], idx0, s_key[c1], idx1);
-            if (lane == 0 && rank.x < k) frontier(rank.x, s_score[c], idx0, base, (t + 1) & 1);
-            if (lane == 1 && rank.y < k && c + kSelWarps < n) frontier(rank.y, s_score[c1], idx1, base, (t + 1) & 1);
+        // the k best survivors (score desc, flat index asc): up to 64, a warp to two of them, else a half-warp to each
+        const int n = more ? s_count : 0;
+        if (n <= 2 * kSelWarps) {
+            if (warp < n) {
+                const int c1 = min(warp + kSelWarps, n - 1), idx0 = s_cand[warp], idx1 = s_cand[c1];
+                const int2 rank = ranks_of(s_key, s_cand, n, s_key[warp], idx0, s_key[c1], idx1);
+                if (lane == 0 && rank.x < k) frontier(rank.x, s_score[warp], idx0, base, (t + 1) & 1);
+                if (lane == 1 && rank.y < k && warp + kSelWarps < n) frontier(rank.y, s_score[c1], idx1, base, (t + 1) & 1);
+            }
+        } else {
+            for (int c0 = 0; c0 + warp * 2 < n; c0 += kSelThreads / 16) {
+                const int c = min(c0 + (tid >> 4), n - 1), rank = rank_among_many(s_key, s_cand, n, c);
+                if ((tid & 15) == 0 && rank < k && c0 + (tid >> 4) < n) frontier(rank, s_score[c], s_cand[c], base, (t + 1) & 1);
+            }
         }
         if (kRecurrent) {
             if (run_gate && tid >= kSelThreads - H) {

@@ -241,7 +241,7 @@ __device__ __noinline__ void select_by_scan(const T* x, int V, int k, MergeShare
 // k-th largest of 64 of them, the eight best of every warp's, thins out more than kRankAll: ranks take n^2 comparisons.  Us for the
 // calls of a step without this / with it, bf16: t_max = 5, V = 1000, k = 32, one sequence that makes the first call 153 / 35, eight
 // that make all 550 / 84; V = 600, k = 16 135 / 33.  Returns how many are left.
-__device__ __forceinline__ int thin_out(MergeShared& S, int n, int k) {
+__device__ __noinline__ int thin_out(MergeShared& S, int n, int k) {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     constexpr int kEach = kCandCap / kSelThreadsRow, kPer = kBoundSlots / kSelWarpsRow;
     unsigned long long key[kEach], best = 31 - lane;   // (of none: distinct, and less than any listed value's)
