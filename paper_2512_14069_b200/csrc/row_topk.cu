@@ -38,12 +38,18 @@ constexpr int kBoundSlots = 64;                      // maxima that the bound is
 constexpr int kGroupCap = 512, kCandCap = 2048;      // groups and values that the merge lists; beyond, it scans the row
 constexpr int kRankAll = 128;                        // values that it ranks as they are; more are thinned out first
 constexpr float kLog2e = 1.4426950408889634f;
+constexpr float kNear = 128.f;                       // span maxima up to which the second product of 2^(x log2 e - max log2 e) is
+                                                     // rounded by less than 8e-6
 
 __device__ __forceinline__ float fast_exp2(float x) {
     float y;
     asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
     return y;
-    chain_trigger();
+}
+// e^(x - top), mb = top * kLog2e
+template <bool kFar>
+__device__ __forceinline__ float power(float x, float top, float mb) {
+    return fast_exp2(kFar ? (x - top) * kLog2e : fmaf(x, kLog2e, -mb));
 }
 // largest of the warp's values, in every lane (NaN loses)
 __device__ __forceinline__ float warp_max_value(float v) {
@@ -128,12 +134,16 @@ struct Span {
         }
         return g[0];
     }
-    __device__ __forceinline__ float exp_sum(float mb) const {       // of this lane, relative to 2^mb
+    // of this lane, relative to e^top.  kFar: for maxima so far from zero that the rounding of top log2 e counts (a span that is
+    // masked as a whole; at -1e10 the rounding alone is up to 512, and such a span's infinite sum would make its row NaN).
+    template <bool kFar>
+    __device__ __forceinline__ float exp_sum(float top) const {
         float s[4] = {0.f, 0.f, 0.f, 0.f};
+        const float mb = top * kLog2e;
 #pragma unroll
         for (int u = 0; u < kLaneVecs; ++u)
 #pragma unroll
-            for (int e = 0; e < U::N; ++e) s[e & 3] += fast_exp2(fmaf(U::at(w[u], e), kLog2e, -mb));
+            for (int e = 0; e < U::N; ++e) s[e & 3] += power<kFar>(U::at(w[u], e), top, mb);
         return (s[0] + s[1]) + (s[2] + s[3]);
     }
     __device__ __forceinline__ bool has_nan() const {
@@ -449,10 +459,8 @@ __device__ __forceinline__ void pass_row(const RowTopkParams& p, const Row<T>& r
         if (span == p.spans - 1 && lane < r.head + r.ntail) xs = to_float(r.x[r.scalar(lane)]);
         const float g = x.group_max(), top = warp_max_value(fmaxf(g, xs));
         float sum = 0.f;
-        if (top > -CUDART_INF_F) {
-            const float mb = top * kLog2e;
-            sum = warp_sum(x.exp_sum(mb) + fast_exp2(fmaf(xs, kLog2e, -mb)));
-        }
+        if (fabsf(top) <= kNear) sum = warp_sum(x.template exp_sum<false>(top) + power<false>(xs, top, top * kLog2e));
+        else if (top > -CUDART_INF_F) sum = warp_sum(x.template exp_sum<true>(top) + power<true>(xs, top, 0.f));
         float seen = top;
         if (sum != sum || top == -CUDART_INF_F) {     // +inf, or a NaN (the maxima pass it by): the merge reports it
             if (__any_sync(kFull, xs != xs || x.has_nan())) seen = CUDART_NAN_F;
