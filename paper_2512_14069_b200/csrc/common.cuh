@@ -160,9 +160,6 @@ __device__ __forceinline__ float to_float(__nv_bfloat16 x) { return __bfloat162f
 __device__ __forceinline__ bool precedes(float va, int ia, float vb, int ib) {
     return va > vb || (va == vb && ia < ib);
 }
-__device__ __forceinline__ bool precedes(double va, int ia, double vb, int ib) {
-    return va > vb || (va == vb && ia < ib);
-}
 
 template <typename T>
 __device__ __forceinline__ T warp_max(T v) {
@@ -198,31 +195,26 @@ __device__ __forceinline__ float transposed_sum(float (&v)[N]) {
     return t;
 }
 
-// Sorted list of the 32 best (value, index) pairs seen by a warp, one per lane (lane 0 = best).
-// V is float or double.  Empty slots hold (-inf, INT_MAX).
-template <typename V>
-struct WarpTopList {
-    V v;
-    int i;
-    __device__ __forceinline__ void reset() {
-        v = -CUDART_INF_F;
-        i = 0x7fffffff;
+// best (value desc, index asc) pair over the warp, in every lane
+__device__ __forceinline__ void warp_best(float& v, int& i) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        const float ov = __shfl_xor_sync(kFull, v, o);
+        const int oi = __shfl_xor_sync(kFull, i, o);
+        if (precedes(ov, oi, v, i)) { v = ov; i = oi; }
     }
-    // all lanes call with the same candidate
-    __device__ __forceinline__ void insert(V cv, int ci) {
-        const bool worse = precedes(cv, ci, v, i);               // this lane's entry comes after the candidate
-        const unsigned w = __ballot_sync(kFull, worse);
-        if (w == 0) return;
-        const int pos = __ffs(w) - 1;                             // entries are sorted: worse lanes are a suffix
-        const V uv = __shfl_up_sync(kFull, v, 1);
-        const int ui = __shfl_up_sync(kFull, i, 1);
-        const int lane = threadIdx.x & 31;
-        if (lane == pos) { v = cv; i = ci; }
-        else if (lane > pos) { v = uv; i = ui; }
-    }
-    __device__ __forceinline__ V value_at(int lane) const { return __shfl_sync(kFull, v, lane); }
-    __device__ __forceinline__ int index_at(int lane) const { return __shfl_sync(kFull, i, lane); }
-};
+}
+
+__device__ __forceinline__ uint32_t smem_addr(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
+__device__ __forceinline__ void cluster_barrier() {
+    asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
+}
+// where another block of the cluster has this block's shared variable *p
+__device__ __forceinline__ uint32_t cluster_addr(const void* p, uint32_t rank) {
+    uint32_t a;
+    asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(smem_addr(p)), "r"(rank));
+    return a;
+}
 
 // --- best logit of every row (vocab_pass.cu) ----------------------------------------------
 // One launch reduces every (row, chunk) of a [rows][V] logits matrix to its best (logit, token).

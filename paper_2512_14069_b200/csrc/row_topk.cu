@@ -156,15 +156,6 @@ struct Span {
     }
 };
 
-// best (value desc, index asc) pair over the warp, in every lane
-__device__ __forceinline__ void warp_best(float& v, int& i) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        const float ov = __shfl_xor_sync(kFull, v, o);
-        const int oi = __shfl_xor_sync(kFull, i, o);
-        if (precedes(ov, oi, v, i)) { v = ov; i = oi; }
-    }
-}
 // barriers of the merge: its 256 selecting threads, and with the normaliser's warp
 __device__ __forceinline__ void selection_barrier() { asm volatile("bar.sync 1, 256;" ::: "memory"); }
 __device__ __forceinline__ void merge_barrier() { asm volatile("bar.sync 2, 288;" ::: "memory"); }

@@ -52,15 +52,6 @@ template <> __device__ __forceinline__ void load16<__nv_bfloat16>(const __nv_bfl
     }
 }
 
-__device__ __forceinline__ uint32_t in_block(const void* p, uint32_t rank) {
-    uint32_t a;
-    asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"((uint32_t)__cvta_generic_to_shared(p)), "r"(rank));
-    return a;
-}
-__device__ __forceinline__ void cluster_barrier() {
-    asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
-}
-
 // kCluster: the splits of a row block are a cluster, which merges them through its shared memory, the rows dealt out over the blocks:
 // a second kernel is a fifth of the time of small calls (4 / 4 heads of d = 64, 48 blocks: 8.3 -> 7.0 us).  More splits than a
 // cluster may have blocks go through the workspace and tree_attn_combine_kernel, and so do launches that fill the device, where
@@ -233,7 +224,7 @@ __global__ void __launch_bounds__(kThreads) tree_attn_fp32_kernel(const AttnPara
         }
     }
 
-    if (kCluster) {
+    if constexpr (kCluster) {
         __shared__ float2 s_ml[kRowsPerBlock];
         float* s_o = Ks;                                // [32][D]
         __syncthreads();                                // the last tile has been read
@@ -248,14 +239,14 @@ __global__ void __launch_bounds__(kThreads) tree_attn_fp32_kernel(const AttnPara
         for (int rl = split + P.n_splits * warp; rl < kRowsPerBlock && row0 + rl < R; rl += P.n_splits * kWarps) {
             float2 ml = make_float2(-CUDART_INF_F, 0.f);
             if (lane < P.n_splits)
-                asm volatile("ld.shared::cluster.v2.f32 {%0, %1}, [%2];" : "=f"(ml.x), "=f"(ml.y) : "r"(in_block(&s_ml[rl], lane)) : "memory");
+                asm volatile("ld.shared::cluster.v2.f32 {%0, %1}, [%2];" : "=f"(ml.x), "=f"(ml.y) : "r"(cluster_addr(&s_ml[rl], lane)) : "memory");
             float v[kMaxCluster][D / 32], o[D / 32];
 #pragma unroll
             for (int u = 0; u < kMaxCluster; ++u) {
 #pragma unroll
                 for (int c = 0; c < D / 32; ++c) v[u][c] = 0.f;
                 if (u >= P.n_splits) continue;
-                const uint32_t from = in_block(s_o + rl * D + lane * (D / 32), u);
+                const uint32_t from = cluster_addr(s_o + rl * D + lane * (D / 32), u);
                 if constexpr (D == 128)
                     asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v[u][0]), "=f"(v[u][1]), "=f"(v[u][2]), "=f"(v[u][3]) : "r"(from) : "memory");
                 else
@@ -282,20 +273,18 @@ __global__ void __launch_bounds__(kThreads) tree_attn_fp32_kernel(const AttnPara
             if (a.lse != nullptr && lane == 0) a.lse[((int64_t)b * Hq + hq) * kMaxNodes + node] = mx + logf(den);
         }
         cluster_barrier();                              // no block leaves while another reads from it
-        return;
-    }
-
-    // ---- partial results ----
+    } else {                                            // partial results
 #pragma unroll
-    for (int i = 0; i < kRowsPerWarp; ++i) {
-        const int r = row0 + warp * kRowsPerWarp + i;
-        if (r >= R) continue;
-        const int node = r / G, hq = g * G + r % G;
-        const int64_t rec = (((int64_t)b * Hq + hq) * kMaxNodes + node) * P.n_splits + split;
-        if (lane == 0) P.part_ml[rec] = make_float2(m_run[i], l_run[i]);
-        float* dst = P.part_o + rec * D + lane * (D / 32);
+        for (int i = 0; i < kRowsPerWarp; ++i) {
+            const int r = row0 + warp * kRowsPerWarp + i;
+            if (r >= R) continue;
+            const int node = r / G, hq = g * G + r % G;
+            const int64_t rec = (((int64_t)b * Hq + hq) * kMaxNodes + node) * P.n_splits + split;
+            if (lane == 0) P.part_ml[rec] = make_float2(m_run[i], l_run[i]);
+            float* dst = P.part_o + rec * D + lane * (D / 32);
 #pragma unroll
-        for (int c = 0; c < D / 32; ++c) dst[c] = acc[i][c];
+            for (int c = 0; c < D / 32; ++c) dst[c] = acc[i][c];
+        }
     }
 }
 

@@ -40,16 +40,6 @@ __device__ __forceinline__ float max_nan(float a, float b) {
     return y;
 }
 
-// best (value desc, index asc) pair over the warp, in every lane
-__device__ __forceinline__ void warp_best(float& v, int& i) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        const float ov = __shfl_xor_sync(kFull, v, o);
-        const int oi = __shfl_xor_sync(kFull, i, o);
-        if (precedes(ov, oi, v, i)) { v = ov; i = oi; }
-    }
-}
-
 // EPT = values per thread kept in registers (a multiple of the vector width), chunk = kThreads * EPT
 template <typename T, int EPT>
 __global__ void __launch_bounds__(kThreads, 5) vocab_pass_kernel(const VocabPassParams p) {
