@@ -82,10 +82,10 @@ struct radar_launch_scope {
     }
 };
 
-// Every kernel of the library is launched with programmatic stream serialization and begins with
+// Every kernel of the library is launched with programmatic stream serialization, and most begin with
 // chain_wait(): the next kernel's launch and block scheduling overlap the tail of the previous one, and
-// nothing of a kernel touches memory before its predecessor (and, transitively, every earlier kernel of
-// the stream) has completed and flushed.
+// nothing of such a kernel touches memory before its predecessor (and, transitively, every earlier kernel
+// of the stream) has completed and flushed.
 template <typename... KArgs, typename... Args>
 inline cudaError_t launch_chained(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream,
                                   Args&&... args) {
@@ -109,8 +109,14 @@ __device__ __forceinline__ void chain_wait() {
 // it.  Rules that keep the chain sound: (1) every block runs chain_sync() in at least one thread
 // before it exits, so "kernel N complete" always implies "kernel N-1 complete"; (2) nothing written by
 // the immediate predecessor is read, and nothing it reads is written, before chain_sync() (or a block
-// barrier behind a thread that ran it).  Whatever kernels before the predecessor wrote is complete
-// when the block starts, because the predecessor's blocks trigger only after their own wait.
+// barrier behind a thread that ran it); (3) what kernels ahead of the predecessor wrote may be read before
+// chain_sync() only if that is complete when the block starts: the predecessor triggers behind its own wait,
+// or its own predecessor does and all that is read is older than that one.
+// Ahead of their own wait trigger: row_merge_kernel, expand_select_gate_kernel (but not where it is launched on
+// its own) and the tensor-core attention.  Read before their wait: row_merge_kernel, nothing but L2 prefetches;
+// expand_select_gate_kernel (again not on its own) and expand_calls_kernel, the weights and the state that earlier
+// calls have left: both always stand behind row_topk_kernel, which triggers behind its wait, or behind
+// row_merge_kernel, whose predecessor row_pass_kernel does.  Whatever follows one of the early triggers waits first.
 __device__ __forceinline__ void chain_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void chain_sync() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 

@@ -7,12 +7,13 @@
 //
 // The read is bound by HBM as long as nothing but loads and exponentials is in it: no selection, and no barrier behind the
 // loads.  (With a selection of each chunk's k best in the pass, four block barriers and a ranking behind every 32 KB, its blocks
-// spent as long on those as on their loads, whatever their number: the reads of 320 rows of 128256 took 39 us, now 25.)  The merge is a chain of
-// dependent steps, which other rows hide.  Two forms:
+// spent as long on those as on their loads, whatever their number: the reads of 320 rows of 128256 took 39 us, now 25.)  The merge
+// is a chain of dependent steps, which other rows hide.  Two forms:
 //
 //   row_topk_kernel     a row to a cluster, whose warps send what they leave into the first CTA's shared memory; that CTA merges.
-//                       For launches whose clusters are all resident at once: no second kernel, which costs a call 1.6 us from one
-//                       kernel's last store to the next one's first load, and the reads of what the pass has left.
+//                       For launches of up to two CTAs per SM, so that all clusters are resident at once or nearly (a cluster
+//                       needs its SMs in one GPC): no second kernel, which costs a call 1.6 us from one kernel's last store to
+//                       the next one's first load, and the reads of what the pass has left.
 //   row_pass_kernel,    all warps of all rows, then a block per row.  Once clusters queue for SMs, a merging CTA keeps the
 //   row_merge_kernel    reads of the next ones waiting (both kernels 12.9 us for 80 rows of 128256, 31.8 for 320; clusters
 //                       16.3 and 47.4).  The pass lets the merge start at its end: earlier, the waiting blocks gather on the

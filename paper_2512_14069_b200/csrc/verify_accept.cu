@@ -1113,8 +1113,9 @@ extern "C" int radar_verify_accept(radar_ctx* ctx, const radar_accept_args* a, v
     sp.tab = exp_table();
     // Cluster size: as many CTAs per sequence as keep the whole batch resident at once, two to an SM, while a CTA's slice
     // of the vocabulary is worth an exchange between them.  One CTA per SM where that still leaves SMs over (clusters need
-    // their SMs in one GPC, so not all SMs can be used that way): B = 4, V = 32000 28 / 34 us for one / two; B = 16,
-    // V = 17000 42 / 35; B = 32, V = 128256 128 (clusters of 4) / 107.
+    // their SMs in one GPC, so not all SMs can be used that way).  us for one / two at clusters of eight: B = 4, V = 32000 21.2 /
+    // 27.5; 8, 128256 45.6 / 57.4; 14, 128256 60.4 / 66.9; 16, 17000 25.0 / 25.4; 16, 50256 41.9 / 37.9; 16, 128256 80.4 / 77.9;
+    // B = 32, V = 128256 157 (clusters of four, one) / 106.  (Off the rule: B = 24, V = 32000 38 with clusters of four, one per SM, 41 so.)
     int cs = 1;
     while (cs < kMaxCluster && (long long)a->B * cs * 2 <= 2 * ctx->sm_count && a->V >= cs * 2 * kMinSlice) cs *= 2;
     const bool one = 4ll * a->B * cs <= 3ll * ctx->sm_count;
@@ -1186,9 +1187,9 @@ extern "C" int radar_accept_length_distribution(radar_ctx* ctx, const radar_accl
     P.status = ctx->d_status;
     P.tab = exp_table();
     // One CTA per SM while the rows (about twenty with children to a tree) are few waves, two when their passes are what
-    // takes the time.  us for one / two, by trees times CTAs a row: 8 (1 tree, V = 128256) 42 / 47; 16 (4, 32000) 29 / 36, (8, 16000)
-    // 29 / 37, (2, 128256) 43 / 50; 20 (5, 32000) 33 / 37; 24 (6, 32000) 39 / 37, (3, 70000) 41 / 39, (3, 128256) 66 / 55; 32 (4, 70000)
-    // 47 / 41; 64 (16, 32000) 88 / 72, (8, 128256) 191 / 135.  (Short vocabularies cross later: 16 trees, V = 16000 47 / 65.)
+    // takes the time.  us for one / two, by trees times CTAs a row: 8 (1 tree, V = 128256) 34 / 41; 16 (4, 32000) 24 / 31, (8, 16000)
+    // 24 / 31, (2, 128256) 35 / 45; 20 (5, 32000) 30 / 31; 24 (6, 32000) 35 / 32, (3, 70000) 37 / 33, (3, 128256) 55 / 48; 32 (4, 70000)
+    // 42 / 35; 64 (16, 32000) 76 / 61, (8, 128256) 126 / 101.  (Short vocabularies cross later: 16 trees, V = 16000 44 / 57.)
     const bool one = a->B * cs <= 16;
     if (a->logits_dtype == RADAR_F32) RADAR_CUDA_CHECK((one ? launch_acclen<float, 1>(ctx, P, cs, max_clusters, stream) : launch_acclen<float, 2>(ctx, P, cs, max_clusters, stream)));
     else RADAR_CUDA_CHECK((one ? launch_acclen<__nv_bfloat16, 1>(ctx, P, cs, max_clusters, stream) : launch_acclen<__nv_bfloat16, 2>(ctx, P, cs, max_clusters, stream)));
