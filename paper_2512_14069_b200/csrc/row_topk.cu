@@ -488,31 +488,38 @@ __device__ __forceinline__ void merge_row(const RowTopkParams& p, const Row<T>& 
 }
 
 // The mask may be written while this runs (a sequence that stops meanwhile is read in vain): the first CTA's look at it decides
-// for the cluster, whose blocks would else wait for messages of blocks that have left, or send to one.  Each thread's own look
-// only decides whether its span is asked for ahead of that.
+// for the cluster, whose blocks would else wait for messages of blocks that have left, or send to one.  It sends the others
+// what it saw; a thread's own look only decides whether its span is asked for ahead of that.
 template <typename T>
 __global__ void __launch_bounds__(kThreads, 2) row_topk_kernel(const RowTopkParams p) {
     __shared__ MergeShared S;
     __shared__ __align__(16) float s_gmax[kMaxSlots * 32];           // the first CTA's: what all warps of the cluster leave
     __shared__ __align__(16) float2 s_part[kMaxSlots];
-    __shared__ __align__(8) uint64_t s_bar;                          // completes when they have sent it
-    __shared__ uint32_t s_live;
+    __shared__ __align__(8) uint64_t s_bar;                          // the first CTA's completes when they have sent it,
+    __shared__ uint32_t s_live;                                      // the others' with what the first CTA saw in the mask
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, n = gridDim.x, rank = blockIdx.x, f = blockIdx.y, seq = blockIdx.z;
-    if (rank == 0 && threadIdx.x == 0) init_message_barrier(&s_bar, (uint32_t)(n * kWarps * (32 * sizeof(float) + sizeof(float2))));
+    if (threadIdx.x == 0) init_message_barrier(&s_bar, rank == 0 ? (uint32_t)(n * kWarps * (32 * sizeof(float) + sizeof(float2))) : (uint32_t)sizeof(s_live));
+    if (n > 1) cluster_barrier();                     // every CTA has started and its barrier word is initialised
+    else __syncthreads();
     chain_wait();
     const bool ahead = p.seq_active == nullptr || p.seq_active[seq] != 0;
-    if (threadIdx.x == 0) s_live = ahead;
     const Row<T> r(p, seq, f);
     const int slot = rank * kWarps + warp;
     Span<T> x;
     if (ahead) x.load(r, slot);                       // (past the row's end: -inf, nothing is read)
-    if (n > 1) cluster_barrier();                     // the first CTA has started and its barrier word is initialised
-    else __syncthreads();
     if (p.seq_active != nullptr) {
-        if (load_u32(cluster_addr(&s_live, 0)) == 0) {
-            if (n > 1) cluster_barrier();             // the first CTA stays until all have looked
+        if (rank == 0) {
+            if (warp == 0) {
+                const uint32_t look = __shfl_sync(kFull, ahead ? 1u : 0u, 0);
+                if (lane == 0) s_live = look;
+                else if (lane < n) send_f32(cluster_addr(&s_live, lane), cluster_addr(&s_bar, lane), __uint_as_float(look));
+            }
+            __syncthreads();
+        } else if (!cluster_wait(&s_bar, 0)) {
+            set_status(p.status, RADAR_ERR_TIMEOUT);
             return;
         }
+        if (s_live == 0) return;
         if (!ahead) x.load(r, slot);
     }
     float gmax, m, s;

@@ -53,11 +53,6 @@ __device__ __forceinline__ bool cluster_wait(const uint64_t* bar, uint32_t parit
     for (uint32_t it = 0; it < (1u << 22) && !(ok = mbar_try_wait_cluster(bar, parity)); ++it) {}
     return ok;
 }
-__device__ __forceinline__ uint32_t load_u32(uint32_t addr) {
-    uint32_t v;
-    asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(v) : "r"(addr) : "memory");
-    return v;
-}
 // a word into another block's shared memory, counted by a barrier there: the message needs no release of what came before it
 __device__ __forceinline__ void send_f32(uint32_t addr, uint32_t bar, float v) {
     asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.b32 [%0], %1, [%2];" ::"r"(addr), "r"(__float_as_uint(v)), "r"(bar) : "memory");
