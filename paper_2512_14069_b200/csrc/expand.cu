@@ -180,6 +180,14 @@ __global__ void __launch_bounds__(kSelThreads, 1) expand_select_gate_kernel(cons
     cp_async_wait_all();
     chain_sync();
     if (base + n_cand > a.pool_capacity) {             // never write past the pool
+        if (mine) {
+            const size_t q = (size_t)b * n_cand + e;
+            const int tk = P.row_tok[q];
+            if (tk < 0) set_status(P.status, RADAR_ERR_NUMERIC);
+            a.topk_tok[q] = tk & ~kNanRow;
+            a.topk_logp[q] = (float)P.row_logp[q];
+        }
+        __syncthreads();
         if (tid == 0) {
             if (kHelpers) cluster_wait(&s_bar, 0);     // what the helpers send has landed
             set_status(P.status, RADAR_ERR_INVALID_ARG);
