@@ -6,7 +6,7 @@
 // Call by call, a step is a chain of two dozen launches whose blocks each reload the gate's weights and hand the state on through
 // global memory: 8 us a call, whatever the size.  Here the passes, which depend on nothing the calls decide, run once over all
 // rows of a range of calls, and the calls themselves are a loop whose weights and state stay on chip, 2.3 us a call (B = 1,
-// V = 128256, 8 calls: 71 us call by call, 31 together).  What it costs: rows of calls that a sequence never makes are read
+// V = 128256, 8 calls: 65 us call by call, 32 together).  What it costs: rows of calls that a sequence never makes are read
 // too, so with long passes a step is made in several ranges; what one range leaves, the next one starts from.  It takes
 // draft logits that exist before the range's first call (recorded ones, or a draft model that does not look at the frontier);
 // where the draft model runs between the calls, radar_expand_step is the form.
